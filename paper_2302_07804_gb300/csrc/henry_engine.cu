@@ -32,6 +32,7 @@
 #include "henry_kernels.cuh"
 #include "henry_misc.cuh"
 #include "henry_cta.cuh"
+#include "henry_tail.cuh"
 #include "henry_kl.cuh"
 #include "henry_adjoint.cuh"
 #include "henry_vc.cuh"
@@ -509,13 +510,6 @@ bool fused_eligible(const henry_config& c, int level, CtaLayout* L) {
   return L->bytes <= optin;
 }
 
-int smem_optin();
-// Dynamic shared memory the tail kernel may use: the opt-in limit less a
-// small margin (the kernel declares no static shared memory; the margin
-// keeps room should it ever declare some).
-constexpr int TAIL_STATIC_RESERVE = 256;
-int tail_dyn_max() { return std::max(0, smem_optin() - TAIL_STATIC_RESERVE); }
-
 // The device's opt-in shared memory per CTA (cached per device; 0 on error).
 int smem_optin() {
   int dev = 0;
@@ -528,8 +522,25 @@ int smem_optin() {
   return optin;
 }
 
-// Let the fused multigrid tail kernel use up to the opt-in shared memory
-// (once per device and precision; outside any stream capture).
+// Runs f(std::integral_constant<int, NX0>{}) for a tail that starts on a grid
+// nx cells wide (4 .. 64).
+template <typename F>
+void with_tail_width(int nx, F&& f) {
+  switch (nx) {
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+    case 16: f(std::integral_constant<int, 16>()); break;
+    case 32: f(std::integral_constant<int, 32>()); break;
+    default: f(std::integral_constant<int, 64>()); break;
+  }
+}
+template <typename T>
+constexpr int tail_bytes(int nx0) {
+  return tail_smem_v2(nx0) * (int)sizeof(typename VT<T>::v2);
+}
+
+// Let the tail from 64 x 32 cells use its dynamic shared memory (above the
+// default limit; once per device and precision, outside any stream capture).
 template <typename T>
 int ensure_tail_attr() {
   static std::atomic<int> done[64] = {};
@@ -537,8 +548,8 @@ int ensure_tail_attr() {
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return set_err(HENRY_EINVAL, "device %d outside [0, 64)", dev);
   if (done[dev].load(std::memory_order_relaxed)) return HENRY_OK;
-  const int dmax = tail_dyn_max();
-  if (dmax > 0) CK(cudaFuncSetAttribute(k_vcycle_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, dmax));
+  static_assert(tail_bytes<T>(32) <= 48 * 1024, "the narrower tails fit the default shared-memory limit");
+  CK(cudaFuncSetAttribute(k_vcycle_tail<T, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_bytes<T>(64)));
   done[dev].store(1, std::memory_order_relaxed);
   return HENRY_OK;
 }
@@ -731,26 +742,27 @@ int restrict_states(henry_handle* H, Group<T>& G, int B, bool old, const int* ac
 }
 
 // First multigrid level of the fused tail: the first coarse level (k >= 1)
-// with at most mg_tail_cells cells per sample (-1: 2048 with FP32 linear
-// algebra on fine grids of 128 x 64 cells or more, else 128, as measured),
-// if the tail below it has at
-// least two levels, its shared-memory layout fits and the batch is small
-// enough (B x cells of that level <= mg_tail_batch_cells; larger batches keep
-// those levels as separate kernels, which then are large launches and fill
-// the FP64 pipe better than the tail's partly idle warps); -1: no tail.
+// with at most mg_tail_cells cells per sample, and at most 2048 (-1: 2048 with
+// FP32 linear algebra on fine grids of 128 x 64 cells or more, else 128, as
+// measured), if the batch is small enough (B x cells of that level <=
+// mg_tail_batch_cells; larger batches keep those levels as separate kernels,
+// which then are large launches and fill the FP64 pipe better than the tail's
+// partly idle warps); -1: no tail.
+// Measured per launch with the two-threads-per-cell kernel (henry_tail.cuh)
+// against the one-thread-per-cell one it replaced, by event timer: FP64 from
+// 16 x 8 cells 42.4 -> 18.6 us (64 samples) and 404 -> 182 us (8192 samples);
+// FP32 from 64 x 32 cells 54.9 -> 18.7 us (2 samples), 55 -> 21 us (20 to 50
+// samples).  Level-0 FP64 solves: 37.4 -> 30.3 ms (64 samples), 518 -> 445 ms
+// (8192); level 2 with partners, 33 samples: 315 -> 279 ms.
 template <typename T>
-int tail_level(const henry_config& c, const Group<T>& G, int B, CtaLayout* L) {
+int tail_level(const henry_config& c, const Group<T>& G, int B) {
   const int cells =
-      c.mg_tail_cells >= 0 ? c.mg_tail_cells : (sizeof(T) == sizeof(float) && G.lv[0].N >= 8192 ? 2048 : 128);
+      c.mg_tail_cells >= 0 ? std::min(c.mg_tail_cells, 2048) : (sizeof(T) == sizeof(float) && G.lv[0].N >= 8192 ? 2048 : 128);
   if (cells <= 0) return -1;
   for (int k = 1; k < G.K; ++k) {
     if (G.lv[k].N > cells) continue;
     if (c.mg_tail_batch_cells > 0 && (double)B * G.lv[k].N > (double)c.mg_tail_batch_cells) return -1;
-    // the finest tail levels read their operators from global memory (L2)
-    // when the layout does not fit otherwise
-    for (int ns = 0; ns < G.K - k; ++ns)
-      if (tail_layout(G.lv[k].nx, G.lv[k].ny, (int)sizeof(T), L, ns) && L->bytes <= tail_dyn_max()) return k;
-    return -1;
+    return k;
   }
   return -1;
 }
@@ -765,8 +777,7 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
   const int* act = G.lin_active;
   const double na = H->nact;
   const double b4 = sizeof(B4), v2 = sizeof(V2);
-  CtaLayout TL;
-  const int kt = tail_level<T>(H->cfg, G, B, &TL);
+  const int kt = tail_level<T>(H->cfg, G, B);
   const int kend = kt > 0 ? kt : G.K;  // levels 0 .. kend - 1 run as separate kernels
   const int mnt = H->cfg.mg_threads;
   for (int k = 0; k < kend; ++k) {
@@ -837,9 +848,14 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
     A.b = G.lv[kt].mgb;
     A.x = G.lv[kt].mgx;
     A.ainv = G.Ainv;
-    const int thr = std::min(TAIL_MAX_THREADS, std::max(32, ((G.lv[kt].N / 2 + 31) / 32) * 32));
+    A.active = act;
+    A.nu1 = nu1;
+    A.nu2 = nu2;
     launch(H, st, HENRY_K_MG_TAIL, na * tb, na * (tf + 32.0), [&] {
-      k_vcycle_tail<T><<<B, thr, TL.bytes, st>>>(TL, A, B, nu1, nu2, act);
+      with_tail_width(G.lv[kt].nx, [&](auto w) {
+        constexpr int NX0 = decltype(w)::value;
+        k_vcycle_tail<T, NX0><<<B, tail_threads(NX0), tail_bytes<T>(NX0), st>>>(A, B);
+      });
     });
     CKL();
   } else {

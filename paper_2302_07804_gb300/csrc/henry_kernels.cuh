@@ -218,6 +218,12 @@ __device__ __forceinline__ void bmv(const B4& A, T x0, T x1, T& y0, T& y1) {
   y0 = fma_(A.a00, x0, A.a01 * x1);
   y1 = fma_(A.a10, x0, A.a11 * x1);
 }
+// One row of the coarsest grid's explicit inverse times its four unknowns
+// (every solver of that grid uses this order).
+template <typename T>
+__device__ __forceinline__ T coarse_row(const T* m, T v0, T v1, T v2, T v3) {
+  return fma_(m[3], v3, fma_(m[2], v2, fma_(m[1], v1, m[0] * v0)));
+}
 template <typename B4>
 __device__ __forceinline__ B4 mkblk(double a00, double a01, double a10, double a11) {
   B4 b;
@@ -860,7 +866,7 @@ __global__ void k_coarse_solve(int B, const T* __restrict__ Ainv, const typename
   const T* M = Ainv + (int64_t)s * 16;
   T o[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) o[i] = M[4 * i] * v[0] + M[4 * i + 1] * v[1] + M[4 * i + 2] * v[2] + M[4 * i + 3] * v[3];
+  for (int i = 0; i < 4; ++i) o[i] = coarse_row(M + 4 * i, v[0], v[1], v[2], v[3]);
   x[2 * (int64_t)s] = mk2<V2>(o[0], o[1]);
   x[2 * (int64_t)s + 1] = mk2<V2>(o[2], o[3]);
 }
