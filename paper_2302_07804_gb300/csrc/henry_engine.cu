@@ -2890,8 +2890,37 @@ int mlmc_accumulate(int level, int n, int n_qoi, const double* qoi_fine_dev, con
   if (level < 0) return set_err(HENRY_EINVAL, "level %d < 0", level);
   if (n <= 0 || n_qoi <= 0) return set_err(HENRY_EINVAL, "n = %d and n_qoi = %d must be positive", n, n_qoi);
   if (!qoi_fine_dev || !sums_dev) return set_err(HENRY_EINVAL, "NULL device pointer");
-  k_mlmc_accumulate<<<dim3(n_qoi, 2), 1024, 0, (cudaStream_t)stream>>>(n, n_qoi, qoi_fine_dev, qoi_coarse_dev,
-                                                                        status_dev, sums_dev);
+  // Columns per cluster: the widest group (at most 16) that still leaves 16
+  // groups (x 8 CTAs: most of the chip); rows: a cluster CTA for every two
+  // steps of its 8 warps, at most 8.  Clusters of 8 whole-SM CTAs fit only
+  // twice into a GPC (17 of them ran as two waves: 358 us instead of 180), so
+  // the CTAs are small enough for four to share an SM.
+  int cw = 16;
+  while (cw > 1 && (n_qoi + cw - 1) / cw < 16) cw /= 2;
+  const int rows = ACC_THREADS / cw;
+  const int cy = std::max(1, std::min(ACC_MAX_CLUSTER, (int)(((int64_t)n + 2 * rows - 1) / (2 * rows))));
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((n_qoi + cw - 1) / cw, cy);
+  lc.blockDim = dim3(ACC_THREADS);
+  lc.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = cy;
+  at[0].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  auto go = [&](auto w) {
+    return cudaLaunchKernelEx(&lc, k_mlmc_accumulate<decltype(w)::value>, n, n_qoi, qoi_fine_dev, qoi_coarse_dev,
+                              status_dev, sums_dev);
+  };
+  switch (cw) {
+    case 16: CK(go(std::integral_constant<int, 16>())); break;
+    case 8: CK(go(std::integral_constant<int, 8>())); break;
+    case 4: CK(go(std::integral_constant<int, 4>())); break;
+    case 2: CK(go(std::integral_constant<int, 2>())); break;
+    default: CK(go(std::integral_constant<int, 1>())); break;
+  }
   CKL();
   return HENRY_OK;
 }
