@@ -68,6 +68,23 @@ int set_err(int code, const char* fmt, ...) {
 
 inline unsigned nblk(int64_t n, int tpb = TPB) { return (unsigned)((n + tpb - 1) / tpb); }
 
+// Launch a kernel of the solve's chain with the programmatic-serialisation
+// attribute (the rules stand at grid_wait in henry_kernels.cuh).
+template <typename... P, typename... A>
+void chain(cudaStream_t st, unsigned grid, unsigned tpb, size_t smem, void (*k)(P...), A&&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(tpb);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute a[1];
+  a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = a;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, k, std::forward<A>(args)...);
+}
+
 struct Level {
   int nx, ny, N;
   double h;
@@ -423,6 +440,20 @@ auto assemble_kernel(const henry_config& c, int nx, int ny) -> decltype(&k_assem
   return &k_assemble<T, FINE, FIELDS, DROP, JAC>;
 }
 
+// Whether a launch of `threads` threads (one per cell) takes the PRE form of
+// its kernel, which loads the operands that the previous kernel does not write
+// before it waits for that kernel.  That shortens a launch of one wave (level
+// 2 with partners, 33 samples, FP64: 268 -> 237 ms; with the line at 3 CTAs an
+// SM 252 ms; level-5 KL mixed, 2 samples: 149 -> 133 ms) and costs a large one
+// occupancy (level 0, 8192 samples, FP64: 445 -> 456 ms), so the line is what
+// 8 CTAs of 256 threads on each of 152 SMs hold.
+constexpr int64_t PRELOAD_THREADS = (int64_t)152 * 8 * TPB;
+template <typename F>
+void with_preload(int64_t threads, F&& f) {
+  if (threads <= PRELOAD_THREADS) f(std::true_type());
+  else f(std::false_type());
+}
+
 // Runs f(std::integral_constant<int, NT>{}) for the multigrid kernels' CTA
 // size nt: 64, 128, 256 or 512 threads (anything else: TPB).
 template <typename F>
@@ -700,17 +731,17 @@ int build_coarse_ops(henry_handle* H, Group<T>& G, int B, double inv_tau, double
     if (H->cfg.coarse_op == HENRY_COARSE_GALERKIN && !DROP) {
       Level& Lf = G.lv[k - 1];
       launch(H, st, HENRY_K_COARSE_OPS, na * L.N * 26.0 * sizeof(B4), [&] {
-        k_galerkin<T><<<nblk((int64_t)B * L.N), TPB, 0, st>>>(B, L.nx, L.ny, (const B4*)Lf.J, Lf.plane, (B4*)L.J,
+        chain(st, nblk((int64_t)B * L.N), TPB, 0, k_galerkin<T>, B, L.nx, L.ny, (const B4*)Lf.J, Lf.plane, (B4*)L.J,
                                                                L.plane, G.lin_active);
       });
     } else {
       launch(H, st, HENRY_K_COARSE_OPS, na * L.N * (32.0 + 6.0 * sizeof(B4)), [&] {
         if (L.cc)
-          assemble_kernel<T, false, true, DROP>(H->cfg, L.nx, L.ny)<<<nblk((int64_t)B * L.N), TPB, 0, st>>>(
+          chain(st, nblk((int64_t)B * L.N), TPB, 0, assemble_kernel<T, false, true, DROP>(H->cfg, L.nx, L.ny), 
               ph, G.coef, B, L.nx, L.ny, L.h, 1.0 / L.h, L.h * L.h * inv_tau * inv_s, inv_s, L.x, L.xo, G.lin_active,
               nullptr, (B4*)L.J, L.plane, nullptr, L.cc, L.fc);
         else
-          assemble_kernel<T, false>(H->cfg, L.nx, L.ny)<<<nblk((int64_t)B * L.N), TPB, 0, st>>>(ph, G.coef, B, L.nx, L.ny, L.h, 1.0 / L.h,
+          chain(st, nblk((int64_t)B * L.N), TPB, 0, assemble_kernel<T, false>(H->cfg, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, L.h, 1.0 / L.h,
                                                                         L.h * L.h * inv_tau * inv_s, inv_s, L.x,
                                                                         L.xo, G.lin_active, nullptr, (B4*)L.J,
                                                                         L.plane, nullptr, nullptr, nullptr);
@@ -720,7 +751,7 @@ int build_coarse_ops(henry_handle* H, Group<T>& G, int B, double inv_tau, double
   }
   Level& Lc = G.lv[G.K];
   launch(H, st, HENRY_K_COARSE_OPS, na * (4.0 * sizeof(B4) + 16.0 * sizeof(T)), [&] {
-    k_coarse_inverse<T><<<nblk(B, 64), 64, 0, st>>>(B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
+    chain(st, nblk(B, 64), 64, 0, k_coarse_inverse<T>, B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
   });
   CKL();
   return HENRY_OK;
@@ -733,7 +764,7 @@ int restrict_states(henry_handle* H, Group<T>& G, int B, bool old, const int* ac
     Level& Lf = G.lv[k];
     Level& Lc = G.lv[k + 1];
     launch(H, st, HENRY_K_STATE_RESTRICT, (double)H->nact * Lc.N * 80.0, [&] {
-      k_restrict_state<<<nblk((int64_t)B * Lc.N), TPB, 0, st>>>(B, Lc.nx, Lc.ny, old ? Lf.xo : Lf.x,
+      chain(st, nblk((int64_t)B * Lc.N), TPB, 0, k_restrict_state, B, Lc.nx, Lc.ny, old ? Lf.xo : Lf.x,
                                                                 old ? Lc.xo : Lc.x, active);
     });
     CKL();
@@ -793,7 +824,10 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
       constexpr int MODE = decltype(mode)::value;
       with_mg_threads(mnt, [&](auto nt) {
         constexpr int NT = decltype(nt)::value;
-        k_sweep<T, MODE, NT><<<nblk(hn, NT), NT, 0, st>>>(B, L.nx, L.ny, col, J, L.plane, b, x, nullptr, act);
+        with_preload(hn, [&](auto pre) {
+          chain(st, nblk(hn, NT), NT, 0, k_sweep<T, MODE, NT, decltype(pre)::value>, B, L.nx, L.ny, col, J, L.plane, b,
+                x, nullptr, act);
+        });
       });
     };
     if (nu1 > 0) {
@@ -809,21 +843,23 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
       launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * Lc.N * (10 * b4 + 7 * v2), na * restrict_flops(L.nx, L.ny), [&] {
         with_mg_threads(mnt, [&](auto nt) {
           constexpr int NT = decltype(nt)::value;
-          k_residual_restrict<T, 0, NT><<<nblk((int64_t)B * Lc.N, NT), NT, 0, st>>>(B, Lc.nx, Lc.ny, J, L.plane, b,
-                                                                                   x, (V2*)Lc.mgb, act);
+          with_preload((int64_t)B * Lc.N, [&](auto pre) {
+            chain(st, nblk((int64_t)B * Lc.N, NT), NT, 0, k_residual_restrict<T, 0, NT, decltype(pre)::value>, B, Lc.nx,
+                  Lc.ny, J, L.plane, b, x, (V2*)Lc.mgb, act);
+          });
         });
       });
     } else {
       launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * L.N * v2, [&] {
         with_mg_threads(mnt, [&](auto nt) {
           constexpr int NT = decltype(nt)::value;
-          k_zero<T, NT><<<nblk((int64_t)B * L.N, NT), NT, 0, st>>>((int64_t)B * L.N, x);
+          chain(st, nblk((int64_t)B * L.N, NT), NT, 0, k_zero<T, NT>, (int64_t)B * L.N, x);
         });
       });
       launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * Lc.N * 5 * v2, [&] {
         with_mg_threads(mnt, [&](auto nt) {
           constexpr int NT = decltype(nt)::value;
-          k_residual_restrict<T, 1, NT><<<nblk((int64_t)B * Lc.N, NT), NT, 0, st>>>(B, Lc.nx, Lc.ny, J, L.plane, b,
+          chain(st, nblk((int64_t)B * Lc.N, NT), NT, 0, k_residual_restrict<T, 1, NT>, B, Lc.nx, Lc.ny, J, L.plane, b,
                                                                                    x, (V2*)Lc.mgb, act);
         });
       });
@@ -854,14 +890,14 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
     launch(H, st, HENRY_K_MG_TAIL, na * tb, na * (tf + 32.0), [&] {
       with_tail_width(G.lv[kt].nx, [&](auto w) {
         constexpr int NX0 = decltype(w)::value;
-        k_vcycle_tail<T, NX0><<<B, tail_threads(NX0), tail_bytes<T>(NX0), st>>>(A, B);
+        chain(st, B, tail_threads(NX0), tail_bytes<T>(NX0), k_vcycle_tail<T, NX0>, A, B);
       });
     });
     CKL();
   } else {
     Level& Lc = G.lv[G.K];
     launch(H, st, HENRY_K_COARSE_SOLVE, na * (16.0 * sizeof(T) + 4 * v2), [&] {
-      k_coarse_solve<T><<<nblk(B, 64), 64, 0, st>>>(B, G.Ainv, (const V2*)Lc.mgb, (V2*)Lc.mgx, act);
+      chain(st, nblk(B, 64), 64, 0, k_coarse_solve<T>, B, G.Ainv, (const V2*)Lc.mgb, (V2*)Lc.mgx, act);
     });
     CKL();
   }
@@ -878,8 +914,10 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
       constexpr int MODE = decltype(mode)::value;
       with_mg_threads(mnt, [&](auto nt) {
         constexpr int NT = decltype(nt)::value;
-        k_sweep<T, MODE, NT><<<nblk(hn, NT), NT, 0, st>>>(B, L.nx, L.ny, col, J, L.plane, b, x,
-                                                          MODE == 2 ? (const V2*)Lc.mgx : nullptr, act);
+        with_preload(hn, [&](auto pre) {
+          chain(st, nblk(hn, NT), NT, 0, k_sweep<T, MODE, NT, decltype(pre)::value>, B, L.nx, L.ny, col, J, L.plane, b,
+                x, MODE == 2 ? (const V2*)Lc.mgx : nullptr, act);
+        });
       });
     };
     if (nu2 > 0) {
@@ -896,7 +934,7 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
       launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * L.N * 2.25 * v2, [&] {
         with_mg_threads(mnt, [&](auto nt) {
           constexpr int NT = decltype(nt)::value;
-          k_prolong_add<T, NT><<<nblk((int64_t)B * L.N, NT), NT, 0, st>>>(B, L.nx, L.ny, x, (const V2*)Lc.mgx, act);
+          chain(st, nblk((int64_t)B * L.N, NT), NT, 0, k_prolong_add<T, NT>, B, L.nx, L.ny, x, (const V2*)Lc.mgx, act);
         });
       });
     }
@@ -934,7 +972,7 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
   const unsigned g = nblk((int64_t)B * N);
   const double b4 = sizeof(B4), v2 = sizeof(V2);
   launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * v2), [&] {
-    k_bicg_init<T><<<g, TPB, 0, st>>>(B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
+    chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
   });
   CKL();
   // Large grids: reduce each sample's partials once (one warp per sample)
@@ -943,7 +981,7 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
   auto finalize = [&](int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
-           [&] { k_finalize<<<nblk((int64_t)B * 32, 128), 128, 0, ss>>>(B, G.nct, G.part, a, b, fin); });
+           [&] { chain(ss, nblk((int64_t)B * 32, 128), 128, 0, k_finalize, B, G.nct, G.part, a, b, fin); });
   };
   finalize(P_RR, P_RN, st);
   const double rt = rtol > 0.0 ? rtol : H->cfg.lin_rtol;
@@ -957,23 +995,29 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
     int rc = vcycle<T>(H, G, B, G.p, G.ph, ss, Jpre0);
     if (rc) return rc;
     launch(H, ss, HENRY_K_SPMV, nc * (5 * b4 + 3 * v2), n_act * spmv_flops(L.nx, L.ny, 1), [&] {
-      k_spmv<T, 1><<<g, TPB, 0, ss>>>(B, L.nx, L.ny, (const B4*)L.J, L.plane, G.ph, G.v, G.rh, G.part, P_RV, 0,
-                                       G.lin_active);
+      with_preload((int64_t)B * N, [&](auto pre) {
+        chain(ss, g, TPB, 0, k_spmv<T, 1, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.ph, G.v, G.rh, G.part, P_RV, 0,
+              G.lin_active);
+      });
     });
     finalize(P_RV, -1, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 3 * v2,
-           [&] { k_bicg_s<T><<<g, TPB, 0, ss>>>(B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin); });
+           [&] { chain(ss, g, TPB, 0, k_bicg_s<T>, B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin); });
     CKL();
     rc = vcycle<T>(H, G, B, G.s, G.sh, ss, Jpre0);
     if (rc) return rc;
     launch(H, ss, HENRY_K_SPMV, nc * (5 * b4 + 3 * v2), n_act * spmv_flops(L.nx, L.ny, 2), [&] {
-      k_spmv<T, 2><<<g, TPB, 0, ss>>>(B, L.nx, L.ny, (const B4*)L.J, L.plane, G.sh, G.t, G.s, G.part, P_TS, P_TT,
-                                       G.lin_active);
+      with_preload((int64_t)B * N, [&](auto pre) {
+        chain(ss, g, TPB, 0, k_spmv<T, 2, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.sh, G.t, G.s, G.part, P_TS, P_TT,
+              G.lin_active);
+      });
     });
     finalize(P_TS, P_TT, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 8 * v2, [&] {
-      k_bicg_update<T><<<g, TPB, 0, ss>>>(B, N, G.dx, G.ph, G.sh, G.s, G.t, G.rh, G.r, G.part, G.sc, G.lin_active,
-                                           fin);
+      with_preload((int64_t)B * N, [&](auto pre) {
+        chain(ss, g, TPB, 0, k_bicg_update<T, decltype(pre)::value>, B, N, G.dx, G.ph, G.sh, G.s, G.t, G.rh, G.r, G.part,
+              G.sc, G.lin_active, fin);
+      });
     });
     finalize(P_RR, P_RN, ss);
     CKL();
@@ -1011,7 +1055,7 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
   for (int it = 0; it <= mi; ++it) {
     CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * v2, [&] {
-      k_bicg_p<T><<<g, TPB, 0, st>>>(B, N, it, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
+      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
                                       G.iters, G.status, G.counter + 1, G.totals + 1, fin);
     });
     CKL();
@@ -1038,7 +1082,7 @@ int retry_linear_solve(henry_handle* H, Group<T>& G, int B, double inv_tau, doub
   const LevelGeom lg = geom(c, G.level);
   Level& L = G.lv[0];
   CK(cudaMemsetAsync(G.counter + 2, 0, sizeof(int), st));
-  k_mark_retry<<<nblk(B, 128), 128, 0, st>>>(B, G.newton_active, G.iters, G.lin_active, G.counter + 2);
+  chain(st, nblk(B, 128), 128, 0, k_mark_retry, B, G.newton_active, G.iters, G.lin_active, G.counter + 2);
   CKL();
   int n_retry = 0;
   int rc = read_counter(H, G.counter + 2, st, &n_retry);
@@ -1047,7 +1091,7 @@ int retry_linear_solve(henry_handle* H, Group<T>& G, int B, double inv_tau, doub
   if (n_retry == 0) return HENRY_OK;
   H->nact = n_retry;
   double* pscratch = G.part + P_MAX * (int64_t)B * G.nct;
-  assemble_kernel<T, true, true, true>(H->cfg, L.nx, L.ny)<<<nblk((int64_t)B * L.N), TPB, 0, st>>>(
+  chain(st, nblk((int64_t)B * L.N), TPB, 0, assemble_kernel<T, true, true, true>(H->cfg, L.nx, L.ny), 
       phys_of(c), G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
       G.lin_active, nullptr, (B4*)G.Jp, L.plane, pscratch, L.cc, L.fc);
   CKL();
@@ -1079,15 +1123,15 @@ int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st
     // quadratic predictor from step 2 on (three states), linear at step 1
     const bool quad = c.newton_predictor_order == 2 && G.xoo;
     if (step > 1 && quad && c.newton_predictor > 0.0) {
-      k_step_begin_predict2<<<nblk(n0), TPB, 0, st>>>(n0, c.newton_predictor, L.x, L.xo, G.xoo);
+      chain(st, nblk(n0), TPB, 0, k_step_begin_predict2, n0, c.newton_predictor, L.x, L.xo, G.xoo);
     } else {
-      if (quad) k_copy_d2<<<nblk(n0), TPB, 0, st>>>(n0, L.xo, G.xoo);
+      if (quad) chain(st, nblk(n0), TPB, 0, k_copy_d2, n0, L.xo, G.xoo);
       if (step > 0 && c.newton_predictor > 0.0)
-        k_step_begin_predict<<<nblk(n0), TPB, 0, st>>>(n0, c.newton_predictor, L.x, L.xo);
+        chain(st, nblk(n0), TPB, 0, k_step_begin_predict, n0, c.newton_predictor, L.x, L.xo);
       else
-        k_step_begin<<<nblk(n0), TPB, 0, st>>>(n0, L.x, L.xo);
+        chain(st, nblk(n0), TPB, 0, k_step_begin, n0, L.x, L.xo);
     }
-    k_step_flags<<<nblk(B, 128), 128, 0, st>>>(B, G.status, G.newton_active, G.newton_it);
+    chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.newton_active, G.newton_it);
   });
   CKL();
   int rc = restrict_states<T>(H, G, B, true, G.newton_active, st);
@@ -1099,22 +1143,22 @@ int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st
     if (jac)
       launch(H, st, HENRY_K_ASSEMBLE, (double)H->nact * N * (48.0 + 6.0 * sizeof(B4)), [&] {
         if (L.cc)
-          assemble_kernel<T, true, true>(c, L.nx, L.ny)<<<nblk(n0), TPB, 0, st>>>(
+          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, true>(c, L.nx, L.ny), 
               ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo, G.newton_active, G.F, (B4*)L.J,
               L.plane, pmax, L.cc, L.fc);
         else
-          assemble_kernel<T, true>(c, L.nx, L.ny)<<<nblk(n0), TPB, 0, st>>>(ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h,
+          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true>(c, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h,
                                                                       vt, inv_s, L.x, L.xo, G.newton_active, G.F,
                                                                       (B4*)L.J, L.plane, pmax, nullptr, nullptr);
       });
     else
       launch(H, st, HENRY_K_RESIDUAL, (double)H->nact * N * 48.0, [&] {
         if (L.cc)
-          assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny)<<<nblk(n0), TPB, 0, st>>>(
+          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny), 
               ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo, G.newton_active, G.F, nullptr,
               L.plane, pmax, L.cc, L.fc);
         else
-          assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny)<<<nblk(n0), TPB, 0, st>>>(
+          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny), 
               ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo, G.newton_active, G.F, nullptr,
               L.plane, pmax, nullptr, nullptr);
       });
@@ -1137,7 +1181,7 @@ int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st
     CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
     assemble_fine(!res_first);
     launch(H, st, HENRY_K_NEWTON, (double)B * 8 * G.nct, [&] {
-      k_newton_res_check<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(B, G.nct, c.newton_atol, c.newton_maxit, pmax,
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, G.nct, c.newton_atol, c.newton_maxit, pmax,
                                                        G.newton_active, G.lin_active, G.newton_it, G.status,
                                                        G.counter, G.totals);
     });
@@ -1172,10 +1216,10 @@ int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st
     H->nact = n_act;
     launch(H, st, HENRY_K_NEWTON, (double)n_act * N * (32.0 + sizeof(V2)), [&] {
       double* pdc = G.part + P_DC * (int64_t)B * G.nct;
-      k_newton_step_max<T><<<nblk(n0), TPB, 0, st>>>(B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
-      k_newton_theta<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(B, G.nct, c.newton_dc_limit, pdc, G.newton_active, G.theta);
-      k_newton_update<T><<<nblk(n0), TPB, 0, st>>>(B, N, L.x, G.dx, G.theta, G.newton_active);
-      k_newton_dx_check<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(B, G.nct, c.newton_dxtol, pmax, G.newton_active, G.status);
+      chain(st, nblk(n0), TPB, 0, k_newton_step_max<T>, B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active, G.theta);
+      chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta, G.newton_active);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active, G.status);
     });
     CKL();
   }
@@ -1482,14 +1526,14 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
   const unsigned g = nblk((int64_t)B * N);
   const double b4 = sizeof(B4), v2 = sizeof(V2);
   launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * v2), [&] {
-    k_bicg_init<T><<<g, TPB, 0, st>>>(B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
+    chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
   });
   CKL();
   double* fin = (H->cfg.finalize_nct > 0 && G.nct >= H->cfg.finalize_nct) ? G.fin : nullptr;
   auto finalize = [&](int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
-           [&] { k_finalize<<<nblk((int64_t)B * 32, 128), 128, 0, ss>>>(B, G.nct, G.part, a, b, fin); });
+           [&] { chain(ss, nblk((int64_t)B * 32, 128), 128, 0, k_finalize, B, G.nct, G.part, a, b, fin); });
   };
   finalize(P_RR, P_RN, st);
   const double rt = rtol > 0.0 ? rtol : H->cfg.lin_rtol;
@@ -1504,7 +1548,7 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
     });
     finalize(P_RV, -1, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 3 * v2,
-           [&] { k_bicg_s<T><<<g, TPB, 0, ss>>>(B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin); });
+           [&] { chain(ss, g, TPB, 0, k_bicg_s<T>, B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin); });
     CKL();
     rc = vc_vcycle<T>(H, G, B, G.s, G.sh, ss);
     if (rc) return rc;
@@ -1513,7 +1557,7 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
     });
     finalize(P_TS, P_TT, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 8 * v2, [&] {
-      k_bicg_update<T><<<g, TPB, 0, ss>>>(B, N, G.dx, G.ph, G.sh, G.s, G.t, G.rh, G.r, G.part, G.sc, G.lin_active,
+      chain(ss, g, TPB, 0, k_bicg_update<T, false>, B, N, G.dx, G.ph, G.sh, G.s, G.t, G.rh, G.r, G.part, G.sc, G.lin_active,
                                            fin);
     });
     finalize(P_RR, P_RN, ss);
@@ -1547,7 +1591,7 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
   for (int it = 0; it <= mi; ++it) {
     CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * v2, [&] {
-      k_bicg_p<T><<<g, TPB, 0, st>>>(B, N, it, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
+      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
                                       G.status, G.counter + 1, G.totals + 1, fin);
     });
     CKL();
@@ -1619,15 +1663,15 @@ int vc_implicit_step(henry_handle* H, VcGroup<T>& G, int B, int step, cudaStream
     // the predictor as in implicit_step (quadratic from step 2 on)
     const bool quad = c.newton_predictor_order == 2 && G.xoo;
     if (step > 1 && quad && c.newton_predictor > 0.0) {
-      k_step_begin_predict2<<<nblk(n0), TPB, 0, st>>>(n0, c.newton_predictor, L.x, L.xo, G.xoo);
+      chain(st, nblk(n0), TPB, 0, k_step_begin_predict2, n0, c.newton_predictor, L.x, L.xo, G.xoo);
     } else {
-      if (quad) k_copy_d2<<<nblk(n0), TPB, 0, st>>>(n0, L.xo, G.xoo);
+      if (quad) chain(st, nblk(n0), TPB, 0, k_copy_d2, n0, L.xo, G.xoo);
       if (step > 0 && c.newton_predictor > 0.0)
-        k_step_begin_predict<<<nblk(n0), TPB, 0, st>>>(n0, c.newton_predictor, L.x, L.xo);
+        chain(st, nblk(n0), TPB, 0, k_step_begin_predict, n0, c.newton_predictor, L.x, L.xo);
       else
-        k_step_begin<<<nblk(n0), TPB, 0, st>>>(n0, L.x, L.xo);
+        chain(st, nblk(n0), TPB, 0, k_step_begin, n0, L.x, L.xo);
     }
-    k_step_flags<<<nblk(B, 128), 128, 0, st>>>(B, G.status, G.newton_active, G.newton_it);
+    chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.newton_active, G.newton_it);
   });
   CKL();
   int rc = vc_inject<T>(H, G, B, true, G.newton_active, st);
@@ -1644,7 +1688,7 @@ int vc_implicit_step(henry_handle* H, VcGroup<T>& G, int B, int step, cudaStream
     int nct_f = 0;
     const double* fmax_parts = vc_max_parts<T>(H, G, B, &nct_f);
     launch(H, st, HENRY_K_NEWTON, (double)B * 8 * nct_f, [&] {
-      k_newton_res_check<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(B, nct_f, c.newton_atol, c.newton_maxit, fmax_parts,
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, nct_f, c.newton_atol, c.newton_maxit, fmax_parts,
                                                        G.newton_active, G.lin_active, G.newton_it, G.status,
                                                        G.counter, G.totals);
     });
@@ -1665,10 +1709,10 @@ int vc_implicit_step(henry_handle* H, VcGroup<T>& G, int B, int step, cudaStream
     H->nact = n_act;
     launch(H, st, HENRY_K_NEWTON, (double)n_act * N * (32.0 + sizeof(V2)), [&] {
       double* pdc = G.part + P_DC * (int64_t)B * G.nct;
-      k_newton_step_max<T><<<nblk(n0), TPB, 0, st>>>(B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
-      k_newton_theta<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(B, G.nct, c.newton_dc_limit, pdc, G.newton_active, G.theta);
-      k_newton_update<T><<<nblk(n0), TPB, 0, st>>>(B, N, L.x, G.dx, G.theta, G.newton_active);
-      k_newton_dx_check<<<nblk((int64_t)B * 32, 128), 128, 0, st>>>(B, G.nct, c.newton_dxtol, pmax, G.newton_active, G.status);
+      chain(st, nblk(n0), TPB, 0, k_newton_step_max<T>, B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active, G.theta);
+      chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta, G.newton_active);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active, G.status);
     });
     CKL();
   }
@@ -1782,7 +1826,7 @@ int vc_step_entry(henry_handle* H, int which, int level, const double* xi, int n
   const double inv_s = 1.0 / (H->cfg.rho0 * lg.h * lg.h / lg.tau);
   k_vc_to_storage<double2><<<nblk(nv), TPB, 0, st>>>(n, L.nx, L.ny, L.stride, (const double2*)state, L.x);
   k_vc_to_storage<double2><<<nblk(nv), TPB, 0, st>>>(n, L.nx, L.ny, L.stride, (const double2*)state_old, L.xo);
-  k_step_flags<<<nblk(n, 128), 128, 0, st>>>(n, G.status, G.newton_active, G.newton_it);
+  chain(st, nblk(n, 128), 128, 0, k_step_flags, n, G.status, G.newton_active, G.newton_it);
   CK(cudaMemcpyAsync(G.lin_active, G.newton_active, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
   CKL();
   rc = vc_assemble_fine<T>(H, G, n, lg.tau, inv_s, st);
@@ -1872,7 +1916,7 @@ int setup_from_states(henry_handle* H, int level, const double* xi, int n, const
   const int64_t n0 = (int64_t)n * L.N;
   k_to_storage<double2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)state, L.x);
   k_to_storage<double2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)state_old, L.xo);
-  k_step_flags<<<nblk(n, 128), 128, 0, st>>>(n, G->status, G->newton_active, G->newton_it);
+  chain(st, nblk(n, 128), 128, 0, k_step_flags, n, G->status, G->newton_active, G->newton_it);
   CK(cudaMemcpyAsync(G->lin_active, G->newton_active, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
   CKL();
   *out = G;
@@ -1892,22 +1936,22 @@ int assemble_all(henry_handle* H, Group<T>& G, int n, bool coarse, cudaStream_t 
   if (!jac) {
     double* pm = G.part + P_MAX * (int64_t)n * G.nct;
     if (L.cc)
-      assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny)<<<nblk((int64_t)n * L.N), TPB, 0, st>>>(
+      chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny), 
           phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
           G.newton_active, G.F, nullptr, L.plane, pm, L.cc, L.fc);
     else
-      assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny)<<<nblk((int64_t)n * L.N), TPB, 0, st>>>(
+      chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny), 
           phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
           G.newton_active, G.F, nullptr, L.plane, pm, nullptr, nullptr);
     CKL();
     return HENRY_OK;
   }
   if (L.cc)
-    assemble_kernel<T, true, true>(H->cfg, L.nx, L.ny)<<<nblk((int64_t)n * L.N), TPB, 0, st>>>(
+    chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true, true>(H->cfg, L.nx, L.ny), 
         phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
         G.newton_active, G.F, (B4*)L.J, L.plane, G.part + P_MAX * (int64_t)n * G.nct, L.cc, L.fc);
   else
-    assemble_kernel<T, true>(H->cfg, L.nx, L.ny)<<<nblk((int64_t)n * L.N), TPB, 0, st>>>(phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h,
+    chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true>(H->cfg, L.nx, L.ny), phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h,
                                                                  lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
                                                                  G.newton_active, G.F, (B4*)L.J, L.plane,
                                                                  G.part + P_MAX * (int64_t)n * G.nct, nullptr, nullptr);
@@ -2000,7 +2044,7 @@ int adjoint_group(henry_handle* H, Group<double>& G, int B, const double* xi, co
                              qoi_spec(c));
   CKL();
   // backward
-  k_step_flags<<<nblk(B, 128), 128, 0, st>>>(B, G.status, G.lin_active, G.newton_it);
+  chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.lin_active, G.newton_it);
   k_adj_start<<<nblk(n0), TPB, 0, st>>>(B, L.nx, L.ny, lg.h, c.rho0, c.rho1 - c.rho0, G.coef, L.cc, w, L.x, rhs, S,
                                          G.lin_active);
   CKL();
@@ -2021,16 +2065,16 @@ int adjoint_group(henry_handle* H, Group<double>& G, int B, const double* xi, co
       const double2* xm1 = step == s0 ? ck + (int64_t)(cw * k) * n0 : seg + (int64_t)(step - s0 - 1) * n0;
       CK(cudaMemcpyAsync(L.x, xm, vbytes, cudaMemcpyDeviceToDevice, st));
       CK(cudaMemcpyAsync(L.xo, xm1, vbytes, cudaMemcpyDeviceToDevice, st));
-      k_step_flags<<<nblk(B, 128), 128, 0, st>>>(B, G.status, G.lin_active, G.newton_it);
+      chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.lin_active, G.newton_it);
       CKL();
       H->nact = B;
       launch(H, st, HENRY_K_ASSEMBLE, (double)n0 * (48.0 + 6.0 * sizeof(B4)), [&] {
         if (L.cc)
-          assemble_kernel<double, true, true>(H->cfg, L.nx, L.ny)<<<nblk(n0), TPB, 0, st>>>(ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt,
+          chain(st, nblk(n0), TPB, 0, assemble_kernel<double, true, true>(H->cfg, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt,
                                                                   inv_s, L.x, L.xo, G.lin_active, G.F, (B4*)L.J,
                                                                   L.plane, pmax, L.cc, L.fc);
         else
-          assemble_kernel<double, true>(H->cfg, L.nx, L.ny)<<<nblk(n0), TPB, 0, st>>>(ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s,
+          chain(st, nblk(n0), TPB, 0, assemble_kernel<double, true>(H->cfg, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s,
                                                             L.x, L.xo, G.lin_active, G.F, (B4*)L.J, L.plane, pmax, nullptr, nullptr);
       });
       CKL();
@@ -2049,7 +2093,7 @@ int adjoint_group(henry_handle* H, Group<double>& G, int B, const double* xi, co
                                                                             G.lin_active);
       }
       Level& Lc = G.lv[G.K];
-      k_coarse_inverse<double><<<nblk(B, 64), 64, 0, st>>>(B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
+      chain(st, nblk(B, 64), 64, 0, k_coarse_inverse<double>, B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
       k_adj_neg<<<nblk(n0), TPB, 0, st>>>(n0, rhs, G.F);
       CKL();
       rc = linear_solve<double>(H, G, B, st, nullptr, c.adj_rtol, c.adj_maxit);

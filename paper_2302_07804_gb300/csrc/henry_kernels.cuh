@@ -67,12 +67,40 @@ enum { P_RR = 0, P_RN = 1, P_RV = 2, P_TS = 3, P_TT = 4, P_MAX = 5, P_DC = 6, NP
 __host__ __device__ __forceinline__ int st_of(int ix, int iy, int nx) {
   return iy * nx + (((ix + iy) & 1) ? (nx >> 1) : 0) + (ix >> 1);
 }
+// Grid widths and cells per sample are powers of two: indices are split by
+// shifts (a 64-bit division is some 70 instructions, a noticeable part of a
+// small launch).
+__device__ __forceinline__ int lg2(int pow2) { return 31 - __clz(pow2); }
+__device__ __forceinline__ int sample_of(int64_t e, int N) { return (int)(e >> lg2(N)); }
 __device__ __forceinline__ void xy_of(int st, int nx, int& ix, int& iy) {
-  iy = st / nx;
+  iy = st >> lg2(nx);
   const int r = st - iy * nx, half = nx >> 1;
   const int col = r >= half ? 1 : 0;
   const int j = r - col * half;
   ix = 2 * j + ((col ^ iy) & 1);
+}
+
+// Programmatic dependent launch.  The kernels of a solve form one chain; each
+// is launched with the programmatic-serialisation attribute, so that its CTAs
+// start, split their indices and load what does not come from the kernel
+// before while that one drains (measured on GB300 between dependent launches
+// of a small kernel: 4.1 -> 1.4 us on a stream, 1.3 -> 0.95 us as graph nodes).
+// Rules that keep this safe:
+//  * every CTA of every kernel of the chain waits (grid_wait) before it ends,
+//    also where its sample has stopped, so a kernel's completion implies its
+//    predecessors';
+//  * a kernel lets its successor start (grid_start_next) only after its own
+//    wait, so when a kernel starts, all kernels but its direct predecessor
+//    have completed: what those wrote (operators, right-hand sides, flags) may
+//    be read before the wait, what the predecessor writes only after it;
+//  * nothing is written before the wait, and pointers to what the
+//    predecessor writes carry no __restrict__ (their loads must not become
+//    read-only ones that could be moved across the wait).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_enter() {
+  grid_wait();
+  grid_start_next();
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -152,7 +180,7 @@ __device__ __forceinline__ double block_max_nonneg(double v, double* sh) {
 }
 // Sum of a sample's nct partials, computed identically by every CTA of the
 // sample (fixed order), returned to every thread.
-__device__ __forceinline__ double sample_sum(const double* __restrict__ p, int nct, double* sh) {
+__device__ __forceinline__ double sample_sum(const double* p, int nct, double* sh) {
   double v = 0.0;
   if (threadIdx.x < 32) {
     for (int i = threadIdx.x; i < nct; i += 32) v += p[i];
@@ -166,15 +194,16 @@ __device__ __forceinline__ double sample_sum(const double* __restrict__ p, int n
 }
 // The same sum read from the finalised per-sample values when `fin` is set
 // (large grids: one warp per sample summed the partials in the same order).
-__device__ __forceinline__ double sample_sum_or_fin(const double* __restrict__ part, const double* __restrict__ fin,
+__device__ __forceinline__ double sample_sum_or_fin(const double* part, const double* fin,
                                                     int slot, int64_t stride, int s, int nct, double* sh) {
   if (fin) return fin[(int64_t)s * NPART + slot];
   return sample_sum(part + slot * stride + (int64_t)s * nct, nct, sh);
 }
 // One warp per sample: fin[s][slot] = sum of the sample's partials of up to
 // two slots (slot_b < 0: one), in the order sample_sum uses.
-__global__ void k_finalize(int B, int nct, const double* __restrict__ part, int slot_a, int slot_b,
+__global__ void k_finalize(int B, int nct, const double* part, int slot_a, int slot_b,
                            double* __restrict__ fin) {
+  grid_enter();
   const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (s >= B) return;
@@ -192,7 +221,7 @@ __global__ void k_finalize(int B, int nct, const double* __restrict__ part, int 
 // Max of a sample's nct non-negative partial maxima, by one warp (lanes
 // stride over the partials; a max does not depend on the order), returned
 // to every lane.  Wide grids have thousands of partials per sample.
-__device__ __forceinline__ double warp_sample_max(const double* __restrict__ p, int nct, int lane) {
+__device__ __forceinline__ double warp_sample_max(const double* p, int nct, int lane) {
   double v = 0.0;
   for (int i = lane; i < nct; i += 32) v = fmax(v, p[i]);
   return warp_max(v);
@@ -391,8 +420,8 @@ __device__ __forceinline__ void store_blocks(typename VT<T>::b4* J, int64_t ps, 
 template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true>
 __global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restrict__ coef, int B, int nx, int ny,
                                                   double h, double inv_h, double vt_s, double inv_s,
-                                                  const double2* __restrict__ x, const double2* __restrict__ xo,
-                                                  const int* __restrict__ active, double2* __restrict__ F,
+                                                  const double2* x, const double2* xo,
+                                                  const int* active, double2* __restrict__ F,
                                                   typename VT<T>::b4* __restrict__ J, int64_t plane,
                                                   double* __restrict__ rmax_part, const double2* __restrict__ cc = nullptr,
                                                   const double4_32a* __restrict__ fc = nullptr) {
@@ -401,7 +430,8 @@ __global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restric
   const int N = nx * ny;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int64_t total = (int64_t)B * N;
-  const int s = (int)(e / N);
+  const int s = sample_of(e, N);
+  grid_enter();
   if (FINE) {
     if (!active[s]) return;  // uniform over the CTA
   } else {
@@ -525,8 +555,8 @@ __device__ __forceinline__ void add_face(const FaceData<T, S, JAC>& f, bool cell
 template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true>
 __global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __restrict__ coef, int B, int nx, int ny,
                                                        double h, double inv_h, double vt_s, double inv_s,
-                                                       const double2* __restrict__ x, const double2* __restrict__ xo,
-                                                       const int* __restrict__ active, double2* __restrict__ F,
+                                                       const double2* x, const double2* xo,
+                                                       const int* active, double2* __restrict__ F,
                                                        typename VT<T>::b4* __restrict__ J, int64_t plane,
                                                        double* __restrict__ rmax_part,
                                                        const double2* __restrict__ cc = nullptr,
@@ -537,7 +567,8 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __re
   const int N = nx * ny;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int64_t total = (int64_t)B * N;
-  const int s = (int)(e / N);
+  const int s = sample_of(e, N);
+  grid_enter();
   if (FINE) {
     if (!active[s]) return;  // uniform over the CTA
   }
@@ -547,7 +578,7 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __re
   xy_of(st, nx, ix, iy);
   const int64_t base = e - st;
   // tile slot of the cell (ix, row r of the tile); rows hold nx consecutive storage entries
-  const int r = threadIdx.x / nx;
+  const int r = threadIdx.x >> lg2(nx);
   const int slot = r * nx + ix;
   const S hS = (S)h, ihS = (S)inv_h;
   const Coef cf = on ? coef[s] : Coef{};
@@ -646,8 +677,8 @@ constexpr int TILE_W_DEFAULT = 128;  // for grids wider than TPB cells
 template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true, int TILE_W = TILE_W_DEFAULT>
 __global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __restrict__ coef, int B, int nx,
                                                          int ny, double h, double inv_h, double vt_s, double inv_s,
-                                                         const double2* __restrict__ x, const double2* __restrict__ xo,
-                                                         const int* __restrict__ active, double2* __restrict__ F,
+                                                         const double2* x, const double2* xo,
+                                                         const int* active, double2* __restrict__ F,
                                                          typename VT<T>::b4* __restrict__ J, int64_t plane,
                                                          double* __restrict__ rmax_part,
                                                          const double2* __restrict__ cc = nullptr,
@@ -658,12 +689,13 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __
   __shared__ double sh[40];
   const int N = nx * ny;
   const int tiles = N / TPB;  // per sample
-  const int s = (int)(blockIdx.x / tiles);
+  const int s = blockIdx.x >> lg2(tiles);
   const int tile = (int)(blockIdx.x - (int64_t)s * tiles);
+  grid_enter();
   if (s >= B || !active[s]) return;  // uniform over the CTA
   const int tx = threadIdx.x % TILE_W, ty = threadIdx.x / TILE_W;
   const int tpr = nx / TILE_W;  // tiles per row band
-  const int ix = (tile % tpr) * TILE_W + tx, iy = (tile / tpr) * TH + ty;
+  const int ix = (tile & (tpr - 1)) * TILE_W + tx, iy = (tile >> lg2(tpr)) * TH + ty;
   const int st = st_of(ix, iy, nx);
   const int64_t base = (int64_t)s * N;
   const int slot = threadIdx.x;
@@ -756,12 +788,13 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __
 }
 
 // Coarse states: mean of the 2x2 children (both the iterate and the old state).
-__global__ void __launch_bounds__(TPB) k_restrict_state(int B, int ncx, int ncy, const double2* __restrict__ xf,
-                                                        double2* __restrict__ xc, const int* __restrict__ active) {
+__global__ void __launch_bounds__(TPB) k_restrict_state(int B, int ncx, int ncy, const double2* xf,
+                                                        double2* __restrict__ xc, const int* active) {
   const int Nc = ncx * ncy;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  grid_enter();
   if (e >= (int64_t)B * Nc) return;
-  const int s = (int)(e / Nc);
+  const int s = sample_of(e, Nc);
   if (!active[s]) return;
   const int stc = (int)(e - (int64_t)s * Nc);
   int IX, IY;
@@ -777,14 +810,15 @@ __global__ void __launch_bounds__(TPB) k_restrict_state(int B, int ncx, int ncy,
 
 // a5 (Galerkin option): A_c = R A P with piecewise-constant P, R = P^T.
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_galerkin(int B, int ncx, int ncy, const typename VT<T>::b4* __restrict__ Jf,
+__global__ void __launch_bounds__(TPB) k_galerkin(int B, int ncx, int ncy, const typename VT<T>::b4* Jf,
                                                   int64_t plane_f, typename VT<T>::b4* __restrict__ Jc,
-                                                  int64_t plane_c, const int* __restrict__ active) {
+                                                  int64_t plane_c, const int* active) {
   typedef typename VT<T>::b4 B4;
   const int Nc = ncx * ncy;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  grid_enter();
   if (e >= (int64_t)B * Nc) return;
-  const int s = (int)(e / Nc);
+  const int s = sample_of(e, Nc);
   if (!active[s]) return;
   const int stc = (int)(e - (int64_t)s * Nc);
   int IX, IY;
@@ -816,8 +850,9 @@ __global__ void __launch_bounds__(TPB) k_galerkin(int B, int ncx, int ncy, const
 // Coarsest grid (2 x 1 cells, 4 unknowns): explicit inverse per sample by
 // Gauss-Jordan elimination with partial pivoting in FP64.
 template <typename T>
-__global__ void k_coarse_inverse(int B, const typename VT<T>::b4* __restrict__ J, int64_t plane,
-                                 T* __restrict__ Ainv, const int* __restrict__ active) {
+__global__ void k_coarse_inverse(int B, const typename VT<T>::b4* J, int64_t plane,
+                                 T* __restrict__ Ainv, const int* active) {
+  grid_enter();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= B || !active[s]) return;
   // cells: st 0 = (0,0) colour 0, st 1 = (1,0) colour 1
@@ -856,9 +891,10 @@ __global__ void k_coarse_inverse(int B, const typename VT<T>::b4* __restrict__ J
 }
 
 template <typename T>
-__global__ void k_coarse_solve(int B, const T* __restrict__ Ainv, const typename VT<T>::v2* __restrict__ b,
+__global__ void k_coarse_solve(int B, const T* __restrict__ Ainv, const typename VT<T>::v2* b,
                                typename VT<T>::v2* __restrict__ x, const int* __restrict__ active) {
   typedef typename VT<T>::v2 V2;
+  grid_enter();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= B || !active[s]) return;
   const V2 b0 = b[2 * (int64_t)s], b1 = b[2 * (int64_t)s + 1];
@@ -912,25 +948,71 @@ __device__ __forceinline__ typename VT<T>::v2 sweep_cell(int nx, int ny, int ix,
   return mk2<V2>(y0, y1);
 }
 
-// NT: threads per CTA (any multiple of 32 up to 1024; every thread owns one cell).
-template <typename T, int MODE, int NT = TPB>
+// NT: threads per CTA (any multiple of 32 up to 1024; every thread owns one
+// cell).  Every sweep but the first of a level (MODE 0) follows another kernel
+// of the cycle, so its blocks and right-hand side are complete when it starts.
+// PRE: they are loaded before the wait, which leaves only the neighbours' x on
+// the critical path of a small launch but takes 76 registers instead of 32 in
+// FP64; the rule stands at preload (henry_engine.cu).
+template <typename T, int MODE, int NT = TPB, bool PRE = false>
 __global__ void __launch_bounds__(NT) k_sweep(int B, int nx, int ny, int col, const typename VT<T>::b4* __restrict__ J,
-                                               int64_t plane, const typename VT<T>::v2* __restrict__ b,
-                                               typename VT<T>::v2* __restrict__ x,
-                                               const typename VT<T>::v2* __restrict__ xc,
-                                               const int* __restrict__ active) {
+                                               int64_t plane, const typename VT<T>::v2* b,
+                                               typename VT<T>::v2* x, const typename VT<T>::v2* xc,
+                                               const int* active) {
+  typedef typename VT<T>::v2 V2;
+  typedef typename VT<T>::b4 B4;
   const int N = nx * ny, halfN = N >> 1, half = nx >> 1;
   const int64_t t = (int64_t)blockIdx.x * NT + threadIdx.x;
-  if (t >= (int64_t)B * halfN) return;
-  const int s = (int)(t / halfN);
-  if (!active[s]) return;
+  const bool in = t < (int64_t)B * halfN;
+  const int s = in ? sample_of(t, halfN) : 0;
   const int u = (int)(t - (int64_t)s * halfN);
-  const int iy = u / half, j = u - iy * half;
+  const int iy = u >> lg2(half), j = u - iy * half;
   const int ix = 2 * j + ((col ^ iy) & 1);
   const int64_t base = (int64_t)s * N;
   const int i = iy * nx + col * half + j;
-  x[base + i] = sweep_cell<T, MODE>(nx, ny, ix, iy, i, J + base, plane, b + base, x + base,
-                                    MODE == 2 ? xc + (int64_t)s * (N >> 2) : nullptr);
+  if constexpr (MODE == 0 || !PRE) {
+    grid_enter();
+    if (!in || !active[s]) return;
+    x[base + i] = sweep_cell<T, MODE>(nx, ny, ix, iy, i, J + base, plane, b + base, x + base,
+                                      MODE == 2 ? xc + (int64_t)s * (N >> 2) : nullptr);
+  } else {
+    const bool on = in && active[s];
+    const bool has[4] = {ix > 0, ix + 1 < nx, iy > 0, iy + 1 < ny};
+    B4 A[4], Ci;
+    V2 bb = mk2<V2>((T)0, (T)0);
+    if (on) {
+      const B4* Js = J + base + i;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (has[k]) A[k] = Js[(k + 1) * plane];
+      Ci = Js[5 * plane];
+      bb = b[base + i];
+    }
+    grid_enter();
+    if (!on) return;
+    // sweep_cell's arithmetic
+    const V2* xs = x + base;
+    const V2* xcs = MODE == 2 ? xc + (int64_t)s * (N >> 2) : nullptr;
+    const int ncx = nx >> 1;
+    V2 xn[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (!has[k]) continue;
+      const int jx = ix + (k == 0 ? -1 : (k == 1 ? 1 : 0)), jy = iy + (k == 2 ? -1 : (k == 3 ? 1 : 0));
+      xn[k] = xs[st_of(jx, jy, nx)];
+      if (MODE == 2) {
+        const V2 cc = xcs[st_of(jx >> 1, jy >> 1, ncx)];
+        xn[k].x += cc.x;
+        xn[k].y += cc.y;
+      }
+    }
+    T r0 = bb.x, r1 = bb.y, y0, y1;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (has[k]) bmv_sub(A[k], xn[k].x, xn[k].y, r0, r1);
+    bmv(Ci, r0, r1, y0, y1);
+    x[base + i] = mk2<V2>(y0, y1);
+  }
 }
 // ---- smoother source end
 
@@ -986,35 +1068,82 @@ __device__ __forceinline__ typename VT<T>::v2 restrict_cell(int ncx, int ncy, in
   return mk2<V2>(s0, s1);
 }
 
-template <typename T, int MODE, int NT = TPB>  // MODE 0: RED_ONLY, 1: ZERO_X
+// PRE as in k_sweep (the residual form follows a sweep).
+template <typename T, int MODE, int NT = TPB, bool PRE = false>  // MODE 0: RED_ONLY, 1: ZERO_X
 __global__ void __launch_bounds__(NT) k_residual_restrict(int B, int ncx, int ncy,
                                                            const typename VT<T>::b4* __restrict__ J, int64_t plane,
-                                                           const typename VT<T>::v2* __restrict__ b,
-                                                           const typename VT<T>::v2* __restrict__ x,
+                                                           const typename VT<T>::v2* b,
+                                                           const typename VT<T>::v2* x,
                                                            typename VT<T>::v2* __restrict__ bc,
-                                                           const int* __restrict__ active) {
+                                                           const int* active) {
+  typedef typename VT<T>::v2 V2;
+  typedef typename VT<T>::b4 B4;
   const int Nc = ncx * ncy;
   const int64_t e = (int64_t)blockIdx.x * NT + threadIdx.x;
-  if (e >= (int64_t)B * Nc) return;
-  const int s = (int)(e / Nc);
-  if (!active[s]) return;
+  const bool in = e < (int64_t)B * Nc;
+  const int s = in ? sample_of(e, Nc) : 0;
   const int stc = (int)(e - (int64_t)s * Nc);
   int IX, IY;
   xy_of(stc, ncx, IX, IY);
   const int64_t base = (int64_t)s * Nc * 4;
-  bc[e] = restrict_cell<T, MODE>(ncx, ncy, IX, IY, J + base, plane, b + base, x + base);
+  if constexpr (MODE == 1 || !PRE) {
+    grid_enter();
+    if (!in || !active[s]) return;
+    bc[e] = restrict_cell<T, MODE>(ncx, ncy, IX, IY, J + base, plane, b + base, x + base);
+  } else {
+    const bool on = in && active[s];
+    const int nx = 2 * ncx, ny = 2 * ncy;
+    B4 A[2][5];
+    V2 bb[2];
+    if (on) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int ix = 2 * IX + c, iy = 2 * IY + c, i = st_of(ix, iy, nx);
+        const bool has[4] = {ix > 0, ix + 1 < nx, iy > 0, iy + 1 < ny};
+        const B4* Js = J + base + i;
+        A[c][0] = Js[0];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (has[k]) A[c][k + 1] = Js[(k + 1) * plane];
+        bb[c] = b[base + i];
+      }
+    }
+    grid_enter();
+    if (!on) return;
+    // restrict_cell's arithmetic
+    const V2* xs = x + base;
+    T s0 = 0, s1 = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int ix = 2 * IX + c, iy = 2 * IY + c;
+      const bool has[4] = {ix > 0, ix + 1 < nx, iy > 0, iy + 1 < ny};
+      T r0 = bb[c].x, r1 = bb[c].y;
+      const V2 xx = xs[st_of(ix, iy, nx)];
+      bmv_sub(A[c][0], xx.x, xx.y, r0, r1);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (!has[k]) continue;
+        const V2 xn = xs[st_of(ix + (k == 0 ? -1 : (k == 1 ? 1 : 0)), iy + (k == 2 ? -1 : (k == 3 ? 1 : 0)), nx)];
+        bmv_sub(A[c][k + 1], xn.x, xn.y, r0, r1);
+      }
+      s0 += r0;
+      s1 += r1;
+    }
+    bc[e] = mk2<V2>(s0, s1);
+  }
 }
 
 // x += P x_c (used only when there is no post-smoothing to fuse it into).
 template <typename T, int NT = TPB>
-__global__ void __launch_bounds__(NT) k_prolong_add(int B, int nx, int ny, typename VT<T>::v2* __restrict__ x,
-                                                    const typename VT<T>::v2* __restrict__ xc,
-                                                    const int* __restrict__ active) {
+__global__ void __launch_bounds__(NT) k_prolong_add(int B, int nx, int ny, typename VT<T>::v2* x,
+                                                    const typename VT<T>::v2* xc,
+                                                    const int* active) {
   typedef typename VT<T>::v2 V2;
   const int N = nx * ny;
   const int64_t e = (int64_t)blockIdx.x * NT + threadIdx.x;
+  grid_enter();
   if (e >= (int64_t)B * N) return;
-  const int s = (int)(e / N);
+  const int s = sample_of(e, N);
   if (!active[s]) return;
   int ix, iy;
   xy_of((int)(e - (int64_t)s * N), nx, ix, iy);
@@ -1027,6 +1156,7 @@ __global__ void __launch_bounds__(NT) k_prolong_add(int B, int nx, int ny, typen
 
 template <typename T, int NT = TPB>
 __global__ void __launch_bounds__(NT) k_zero(int64_t n, typename VT<T>::v2* __restrict__ x) {
+  grid_enter();
   const int64_t e = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (e < n) x[e] = mk2<typename VT<T>::v2>((T)0, (T)0);
 }
@@ -1054,27 +1184,58 @@ __device__ __forceinline__ typename VT<T>::v2 spmv_cell(int nx, int ny, int ix, 
 
 // y = A x (fine level, all cells) with per-CTA partial dot products:
 //   NDOT 1: <w1, y>;  NDOT 2: <w1, y>, <y, y>.
-template <typename T, int NDOT>
+// PRE as in k_sweep (the kernel follows the sweep that ends a V-cycle).
+template <typename T, int NDOT, bool PRE = false>
 __global__ void __launch_bounds__(TPB) k_spmv(int B, int nx, int ny, const typename VT<T>::b4* __restrict__ J,
-                                              int64_t plane, const typename VT<T>::v2* __restrict__ x,
+                                              int64_t plane, const typename VT<T>::v2* x,
                                               typename VT<T>::v2* __restrict__ y,
-                                              const typename VT<T>::v2* __restrict__ w1, double* __restrict__ part,
-                                              int slot1, int slot2, const int* __restrict__ active) {
+                                              const typename VT<T>::v2* w1, double* __restrict__ part,
+                                              int slot1, int slot2, const int* active) {
   typedef typename VT<T>::v2 V2;
+  typedef typename VT<T>::b4 B4;
   __shared__ double sh[TPB + 1];
   const int N = nx * ny, nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
-  if (!active[s]) return;  // uniform over the CTA
+  const int s = sample_of(e, N);
+  const bool on = active[s];  // uniform over the CTA
   const int st = (int)(e - (int64_t)s * N);
   int ix, iy;
   xy_of(st, nx, ix, iy);
   const int64_t base = e - st;
-  const V2 yy = spmv_cell<T>(nx, ny, ix, iy, st, J + base, plane, x + base);
+  V2 ww = mk2<V2>((T)0, (T)0), yy;
+  if constexpr (PRE) {
+    const bool has[4] = {ix > 0, ix + 1 < nx, iy > 0, iy + 1 < ny};
+    B4 A[5];
+    if (on) {
+      A[0] = J[e];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (has[k]) A[k + 1] = J[(k + 1) * plane + e];
+      if (NDOT >= 1 && part) ww = w1[e];
+    }
+    grid_enter();
+    if (!on) return;
+    // spmv_cell's arithmetic
+    const V2* xs = x + base;
+    const V2 xx = xs[st];
+    T r0, r1;
+    bmv(A[0], xx.x, xx.y, r0, r1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (!has[k]) continue;
+      const V2 xn = xs[st_of(ix + (k == 0 ? -1 : (k == 1 ? 1 : 0)), iy + (k == 2 ? -1 : (k == 3 ? 1 : 0)), nx)];
+      bmv_add(A[k + 1], xn.x, xn.y, r0, r1);
+    }
+    yy = mk2<V2>(r0, r1);
+  } else {
+    grid_enter();
+    if (!on) return;
+    yy = spmv_cell<T>(nx, ny, ix, iy, st, J + base, plane, x + base);
+    if (NDOT >= 1 && part) ww = w1[e];
+  }
   y[e] = yy;
   if (NDOT >= 1 && part) {
     // per-cell products in T, widened once for the FP64 CTA reduction
-    const V2 ww = w1[e];
     const double d1 = block_sum_tree((double)fma_(ww.x, yy.x, ww.y * yy.y), sh);
     double d2 = 0.0;
     if (NDOT == 2) d2 = block_sum_tree((double)fma_(yy.x, yy.x, yy.y * yy.y), sh);
@@ -1092,17 +1253,18 @@ __global__ void __launch_bounds__(TPB) k_spmv(int B, int nx, int ny, const typen
 
 // r = r_hat = b (= -F), p = v = dx = 0; partials <r_hat, r>, <r, r>.
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_bicg_init(int B, int N, const double2* __restrict__ F,
+__global__ void __launch_bounds__(TPB) k_bicg_init(int B, int N, const double2* F,
                                                    typename VT<T>::v2* __restrict__ r,
                                                    typename VT<T>::v2* __restrict__ rh,
                                                    typename VT<T>::v2* __restrict__ p, typename VT<T>::v2* __restrict__ v,
                                                    typename VT<T>::v2* __restrict__ dx, double* __restrict__ part,
-                                                   const int* __restrict__ active) {
+                                                   const int* active) {
   typedef typename VT<T>::v2 V2;
   __shared__ double sh[TPB + 1];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
+  const int s = blockIdx.x / (unsigned)nct;
+  grid_enter();
   if (!active[s]) return;
   const double2 f = F[e];
   const V2 rr = mk2<V2>((T)(-f.x), (T)(-f.y));
@@ -1126,19 +1288,17 @@ __global__ void __launch_bounds__(TPB) k_bicg_init(int B, int N, const double2* 
 // still-active samples in *n_active and per-sample iterations in iters.
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, int maxit, double rtol2,
-                                                const typename VT<T>::v2* __restrict__ r,
-                                                typename VT<T>::v2* __restrict__ p,
-                                                const typename VT<T>::v2* __restrict__ v,
-                                                const double* __restrict__ part, LinScal* __restrict__ sc,
-                                                int* __restrict__ lin_active, int* __restrict__ iters,
+                                                const typename VT<T>::v2* r, typename VT<T>::v2* p,
+                                                const typename VT<T>::v2* v, const double* part, LinScal* sc,
+                                                int* lin_active, int* __restrict__ iters,
                                                 int* __restrict__ status, int* __restrict__ n_active,
-                                                unsigned long long* __restrict__ lin_total,
-                                                const double* __restrict__ fin) {
+                                                unsigned long long* __restrict__ lin_total, const double* fin) {
   typedef typename VT<T>::v2 V2;
   __shared__ double sh[40];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
+  const int s = blockIdx.x / (unsigned)nct;
+  grid_enter();
   if (!lin_active[s]) return;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
@@ -1188,16 +1348,15 @@ __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, int maxit,
 
 // alpha = rho / <r_hat, v>; s = r - alpha v.  CTA 0 stores rho and alpha.
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_bicg_s(int B, int N, const typename VT<T>::v2* __restrict__ r,
-                                                const typename VT<T>::v2* __restrict__ v,
-                                                typename VT<T>::v2* __restrict__ sv, const double* __restrict__ part,
-                                                LinScal* __restrict__ sc, const int* __restrict__ lin_active,
-                                                const double* __restrict__ fin) {
+__global__ void __launch_bounds__(TPB) k_bicg_s(int B, int N, const typename VT<T>::v2* r, const typename VT<T>::v2* v,
+                                                typename VT<T>::v2* __restrict__ sv, const double* part,
+                                                LinScal* sc, const int* lin_active, const double* fin) {
   typedef typename VT<T>::v2 V2;
   __shared__ double sh[40];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
+  const int s = blockIdx.x / (unsigned)nct;
+  grid_enter();
   if (!lin_active[s]) return;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
@@ -1218,22 +1377,30 @@ __global__ void __launch_bounds__(TPB) k_bicg_s(int B, int N, const typename VT<
 
 // omega = <t, s> / <t, t>; dx += alpha p_hat + omega s_hat; r = s - omega t;
 // partials <r_hat, r>, <r, r>.  CTA 0 stores omega.
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T>::v2* __restrict__ dx,
-                                                     const typename VT<T>::v2* __restrict__ ph,
-                                                     const typename VT<T>::v2* __restrict__ shv,
-                                                     const typename VT<T>::v2* __restrict__ sv,
-                                                     const typename VT<T>::v2* __restrict__ t,
-                                                     const typename VT<T>::v2* __restrict__ rh,
-                                                     typename VT<T>::v2* __restrict__ r, double* __restrict__ part,
-                                                     LinScal* __restrict__ sc, const int* __restrict__ lin_active,
-                                                     const double* __restrict__ fin) {
+// PRE: everything but t and the matvec's sums is loaded before the wait.
+template <typename T, bool PRE = false>
+__global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T>::v2* dx, const typename VT<T>::v2* ph,
+                                                     const typename VT<T>::v2* shv, const typename VT<T>::v2* sv,
+                                                     const typename VT<T>::v2* t, const typename VT<T>::v2* rh,
+                                                     typename VT<T>::v2* __restrict__ r, double* part, LinScal* sc,
+                                                     const int* lin_active, const double* fin) {
   typedef typename VT<T>::v2 V2;
   __shared__ double sh[TPB + 1];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
-  if (!lin_active[s]) return;
+  const int s = blockIdx.x / (unsigned)nct;
+  const bool on = lin_active[s];
+  V2 x0, p0, s0, sv0, rh0;
+  auto load = [&] {
+    x0 = dx[e];
+    p0 = ph[e];
+    s0 = shv[e];
+    sv0 = sv[e];
+    rh0 = rh[e];
+  };
+  if (PRE && on) load();
+  grid_enter();
+  if (!on) return;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
   const double ts = sample_sum_or_fin(part, fin, P_TS, stride, s, nct, sh);
@@ -1245,7 +1412,8 @@ __global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T
   const double alpha = sc[s].alpha;
   if (threadIdx.x == 0 && ct == 0) sc[s].omega = omega;
   const T a = (T)alpha, w = (T)omega;
-  const V2 x0 = dx[e], p0 = ph[e], s0 = shv[e], sv0 = sv[e], t0 = t[e], rh0 = rh[e];
+  if (!PRE) load();
+  const V2 t0 = t[e];
   dx[e] = mk2<V2>(x0.x + a * p0.x + w * s0.x, x0.y + a * p0.y + w * s0.y);
   const V2 rn = mk2<V2>(sv0.x - w * t0.x, sv0.y - w * t0.y);
   r[e] = rn;
@@ -1260,8 +1428,9 @@ __global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T
 
 // Samples whose BiCGStab did not converge (or broke down) in this Newton
 // iteration get a second linear solve with the fallback preconditioner.
-__global__ void k_mark_retry(int B, const int* __restrict__ newton_active, const int* __restrict__ iters,
-                             int* __restrict__ lin_active, int* __restrict__ n_retry) {
+__global__ void k_mark_retry(int B, const int* newton_active, const int* iters,
+                             int* __restrict__ lin_active, int* n_retry) {
+  grid_enter();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= B) return;
   const int r = newton_active[s] && iters[s] < 0;
@@ -1274,10 +1443,10 @@ __global__ void k_mark_retry(int B, const int* __restrict__ newton_active, const
 
 // Per sample, after the fine assembly: converged if max |F| <= atol; a
 // non-finite residual fails the sample; counts samples still iterating.
-__global__ void k_newton_res_check(int B, int nct, double atol, int maxit, const double* __restrict__ rmax_part,
-                                   int* __restrict__ newton_active, int* __restrict__ lin_active,
-                                   int* __restrict__ newton_it, int* __restrict__ status,
-                                   int* __restrict__ n_active, unsigned long long* __restrict__ it_total) {
+__global__ void k_newton_res_check(int B, int nct, double atol, int maxit, const double* rmax_part,
+                                   int* newton_active, int* lin_active, int* newton_it, int* status,
+                                   int* n_active, unsigned long long* it_total) {
+  grid_enter();
   // one warp per sample
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (s >= B) return;
@@ -1307,13 +1476,14 @@ __global__ void k_newton_res_check(int B, int nct, double atol, int maxit, const
 // test) and max |dc| (the step limiter).
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_newton_step_max(int B, int N, double inv_pref,
-                                                         const typename VT<T>::v2* __restrict__ dx,
+                                                         const typename VT<T>::v2* dx,
                                                          double* __restrict__ dmax_part, double* __restrict__ dc_part,
-                                                         const int* __restrict__ newton_active) {
+                                                         const int* newton_active) {
   __shared__ double sh[40];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
+  const int s = blockIdx.x / (unsigned)nct;
+  grid_enter();
   if (!newton_active[s]) return;
   const auto d = dx[e];
   double dc = fabs((double)d.y);
@@ -1331,8 +1501,9 @@ __global__ void __launch_bounds__(TPB) k_newton_step_max(int B, int N, double in
 
 // Per sample: theta = min(1, dc_limit / max |dc|) (a step that would change a
 // mass fraction by more than dc_limit is shortened; dc_limit <= 0: theta = 1).
-__global__ void k_newton_theta(int B, int nct, double dc_limit, const double* __restrict__ dc_part,
-                               const int* __restrict__ newton_active, double* __restrict__ theta) {
+__global__ void k_newton_theta(int B, int nct, double dc_limit, const double* dc_part,
+                               const int* newton_active, double* __restrict__ theta) {
+  grid_enter();
   // one warp per sample
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (s >= B || !newton_active[s]) return;
@@ -1346,12 +1517,11 @@ __global__ void k_newton_theta(int B, int nct, double dc_limit, const double* __
 
 // a9: x += theta dx.
 template <typename T>
-__global__ void __launch_bounds__(TPB) k_newton_update(int B, int N, double2* __restrict__ x,
-                                                       const typename VT<T>::v2* __restrict__ dx,
-                                                       const double* __restrict__ theta,
-                                                       const int* __restrict__ newton_active) {
+__global__ void __launch_bounds__(TPB) k_newton_update(int B, int N, double2* x, const typename VT<T>::v2* dx,
+                                                       const double* theta, const int* newton_active) {
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = (int)(e / N);
+  const int s = blockIdx.x / (unsigned)(N / TPB);
+  grid_enter();
   if (!newton_active[s]) return;
   const double th = theta[s];
   const auto d = dx[e];
@@ -1361,8 +1531,9 @@ __global__ void __launch_bounds__(TPB) k_newton_update(int B, int N, double2* __
   x[e] = xx;
 }
 
-__global__ void k_newton_dx_check(int B, int nct, double dxtol, const double* __restrict__ dmax_part,
-                                  int* __restrict__ newton_active, int* __restrict__ status) {
+__global__ void k_newton_dx_check(int B, int nct, double dxtol, const double* dmax_part,
+                                  int* newton_active, int* status) {
+  grid_enter();
   // one warp per sample
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (s >= B || !newton_active[s]) return;
@@ -1377,7 +1548,8 @@ __global__ void k_newton_dx_check(int B, int nct, double dxtol, const double* __
 }
 
 // Start of a time step: old state = state; samples that have not failed iterate.
-__global__ void __launch_bounds__(TPB) k_step_begin(int64_t n, const double2* __restrict__ x, double2* __restrict__ xo) {
+__global__ void __launch_bounds__(TPB) k_step_begin(int64_t n, const double2* x, double2* __restrict__ xo) {
+  grid_enter();
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e < n) xo[e] = x[e];
 }
@@ -1385,8 +1557,8 @@ __global__ void __launch_bounds__(TPB) k_step_begin(int64_t n, const double2* __
 // first iterate: x_old <- x^n, x <- x^n + w (x^n - x^{n-1}) (x^{n-1} is the
 // old state of the previous step).  Only the starting point changes; Newton
 // still stops on the residual and update tests of the step.
-__global__ void __launch_bounds__(TPB) k_step_begin_predict(int64_t n, double w, double2* __restrict__ x,
-                                                            double2* __restrict__ xo) {
+__global__ void __launch_bounds__(TPB) k_step_begin_predict(int64_t n, double w, double2* x, double2* xo) {
+  grid_enter();
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e >= n) return;
   const double2 a = x[e], b = xo[e];
@@ -1396,8 +1568,9 @@ __global__ void __launch_bounds__(TPB) k_step_begin_predict(int64_t n, double w,
 // The quadratic predictor: x^{n+1} ~ x^n + w (2 (x^n - x^{n-1}) - (x^{n-1} -
 // x^{n-2})), i.e. 3 x^n - 3 x^{n-1} + x^{n-2} for w = 1 (extrapolation of the
 // parabola through the last three states); xoo <- x^{n-1}, xo <- x^n.
-__global__ void __launch_bounds__(TPB) k_step_begin_predict2(int64_t n, double w, double2* __restrict__ x,
-                                                             double2* __restrict__ xo, double2* __restrict__ xoo) {
+__global__ void __launch_bounds__(TPB) k_step_begin_predict2(int64_t n, double w, double2* x, double2* xo,
+                                                             double2* xoo) {
+  grid_enter();
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e >= n) return;
   const double2 a = x[e], b = xo[e], c = xoo[e];
@@ -1408,12 +1581,14 @@ __global__ void __launch_bounds__(TPB) k_step_begin_predict2(int64_t n, double w
 }
 // xoo <- x^{n-1} ahead of a step that still uses the linear predictor, so
 // that the next step has three states.
-__global__ void __launch_bounds__(TPB) k_copy_d2(int64_t n, const double2* __restrict__ src, double2* __restrict__ dst) {
+__global__ void __launch_bounds__(TPB) k_copy_d2(int64_t n, const double2* src, double2* __restrict__ dst) {
+  grid_enter();
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e < n) dst[e] = src[e];
 }
-__global__ void k_step_flags(int B, const int* __restrict__ status, int* __restrict__ newton_active,
+__global__ void k_step_flags(int B, const int* status, int* __restrict__ newton_active,
                              int* __restrict__ newton_it) {
+  grid_enter();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= B) return;
   newton_active[s] = status[s] == 0 ? 1 : 0;

@@ -21,7 +21,8 @@
 //    or divides an index.
 //  * A thread reads each block row it will need once per launch, the first
 //    level's into registers, the coarser levels' into its own slots of shared
-//    memory, all before the first phase; levels of one warp (8 x 4 and below)
+//    memory, all before the first phase and before the wait for the kernel
+//    that writes b; levels of one warp (8 x 4 and below)
 //    synchronise by __syncwarp, the 16 x 8 level by a barrier of its own four
 //    warps.
 // The times before and after stand at tail_level (henry_engine.cu).
@@ -188,6 +189,7 @@ struct TailLevel {
     const int x0 = xi(ix0, iy0), x1 = xi(ix1, iy1);
     T b0, b1;
     if constexpr (FIRST) {
+      grid_enter();
       const T* bg = reinterpret_cast<const T*>(reinterpret_cast<const V2*>(A.b) + (int64_t)s * (NX * NY));
       b0 = bg[2 * st_of(ix0, iy0, NX) + row];
       b1 = bg[2 * st_of(ix1, iy1, NX) + row];
@@ -325,6 +327,7 @@ struct TailWide {
     __syncthreads();
   }
   __device__ __forceinline__ void run(const TailArgs& A, int s, int Q, const T* ainv) {
+    grid_enter();
     const V2* bg = reinterpret_cast<const V2*>(A.b) + (int64_t)s * (NX * NY);
 #pragma unroll
     for (int col = 0; col < 2; ++col)
@@ -414,7 +417,10 @@ __global__ void __launch_bounds__(tail_threads(NX0)) k_vcycle_tail(const __grid_
   extern __shared__ __align__(16) unsigned char tail_smem[];
   V2* sm = reinterpret_cast<V2*>(tail_smem);
   const int s = blockIdx.x;
-  if (s >= B || !A.active[s]) return;
+  if (s >= B || !A.active[s]) {
+    grid_enter();
+    return;
+  }
   // The one- and four-warp levels run in the logical warps 0 and 0-3: rotate
   // those over the sub-partitions from CTA to CTA.
   const int t = (threadIdx.x + 32 * (blockIdx.x & 3)) & (NT - 1);
