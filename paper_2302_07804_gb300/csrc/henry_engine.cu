@@ -11,9 +11,11 @@
 // arXiv 2302.07804); each step runs Newton iterations, each Newton iteration
 // assembles the residual and the Jacobian on the fine grid and the coarse
 // operators, and solves the Newton system with BiCGStab right-preconditioned
-// by one V-cycle.  Per-sample convergence decisions are taken on the device;
-// the host only reads "how many samples are still iterating" once per Newton
-// and once per BiCGStab iteration to decide when to stop launching.
+// by one V-cycle.  Per-sample convergence decisions are taken on the device,
+// and so are the loops': a step is one CUDA graph with conditional nodes (see
+// "Device-driven loops"; with cuda_graphs = 0, the kernel timer on, or the
+// allocation-free entry point the host reads how many samples are still
+// iterating once per Newton and once per BiCGStab iteration instead).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -70,6 +72,9 @@ inline unsigned nblk(int64_t n, int tpb = TPB) { return (unsigned)((n + tpb - 1)
 
 // Launch a kernel of the solve's chain with the programmatic-serialisation
 // attribute (the rules stand at grid_wait in henry_kernels.cuh).
+// Set before capturing nodes that follow a conditional node: the next kernel
+// is launched without the attribute (a full dependency).
+thread_local bool g_full_dependency = false;
 template <typename... P, typename... A>
 void chain(cudaStream_t st, unsigned grid, unsigned tpb, size_t smem, void (*k)(P...), A&&... args) {
   cudaLaunchConfig_t c = {};
@@ -81,7 +86,8 @@ void chain(cudaStream_t st, unsigned grid, unsigned tpb, size_t smem, void (*k)(
   a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   a[0].val.programmaticStreamSerializationAllowed = 1;
   c.attrs = a;
-  c.numAttrs = 1;
+  c.numAttrs = g_full_dependency ? 0 : 1;
+  g_full_dependency = false;
   cudaLaunchKernelEx(&c, k, std::forward<A>(args)...);
 }
 
@@ -123,18 +129,19 @@ struct Group {
   V2 *r, *rh, *p, *v, *s, *t, *ph, *sh, *dx;
   Coef* coef;
   double* part;
-  int *newton_active, *lin_active, *newton_it, *status, *iters, *counter;
+  int *newton_active, *lin_active, *newton_it, *status, *iters;
+  int* counter;  // samples iterating: [0] Newton, [1] BiCGStab, [2] retries; [3] the BiCGStab iteration index
   double* theta;  // per-sample Newton step factor
   double* fin;    // finalised per-sample reduction values [B][NPART] (large grids)
   unsigned long long* totals;  // [0] Newton iterations, [1] BiCGStab iterations
   LinScal* sc;
   T* Ainv;
   void* Jp = nullptr;  // fine-level fallback preconditioner operator (field models only)
-  // Instantiated CUDA graphs of one BiCGStab iteration's body, by batch size,
-  // preconditioner operator and every setting that changes the body's
-  // launches (nu1, nu2, mg_tail_cells, mg_threads); they hold this
-  // workspace's pointers and are dropped with it.
-  std::map<std::tuple<int, const void*, int, int, int, int>, cudaGraphExec_t> gexec;
+  // Instantiated CUDA graphs (a whole implicit step, or a linear solve), by
+  // what they run, the batch size and the whole configuration (every setting
+  // that changes their launches); they hold this workspace's pointers and are
+  // dropped with it.
+  std::map<std::string, cudaGraphExec_t> gexec;
   bool graphs = true;  // false: never capture (the allocation-free entry point)
   void drop_graphs() {
     for (auto& kv : gexec) cudaGraphExecDestroy(kv.second);
@@ -959,45 +966,169 @@ int read_counter(henry_handle* H, const int* dev, cudaStream_t st, int* out) {
   return HENRY_OK;
 }
 
-// BiCGStab on the fine level for the samples with lin_active set; right-hand
-// side -F; solution in G.dx.  rtol / maxit > 0 override the configuration's
-// lin_rtol / lin_maxit.
+// ---------------------------------------------------------------------------
+// Device-driven loops.  The Newton and BiCGStab loops of an implicit step run
+// as conditional (WHILE / IF) nodes of one CUDA graph: the kernels count the
+// samples still iterating and a one-thread kernel (k_loop_gate) sets the
+// node's condition, so the host launches one graph a step and never waits
+// for a count.  A host-driven turn costs some 19 us beyond its kernels (copy
+// of the count, synchronisation, launches), a WHILE turn 4.4 us, and the
+// launches outside the iteration's body 1.4 - 4 us each instead of ~1 us.
+// Against one graph per BiCGStab iteration between host turns: level-0 FP64
+// 64 samples 24.6 -> 20.3 ms, level 2 with partners (33 samples) 237 -> 219
+// ms, two-layer level 1 (50) 67 -> 59 ms, 8192 level-0 samples 444 -> 440 ms.
+// A graph under construction and the nodes its next node will follow.
+struct GraphBuild {
+  henry_handle* H;
+  cudaGraph_t g;
+  std::vector<cudaGraphNode_t> deps;
+
+  // Append the launches f(stream) makes.
+  template <typename F>
+  int seg(F&& f) {
+    cudaStream_t cs = H->cap_stream;
+    g_full_dependency = true;
+    CK(cudaStreamBeginCaptureToGraph(cs, g, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(),
+                                     cudaStreamCaptureModeThreadLocal));
+    int rc = f(cs);
+    g_full_dependency = false;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t* d = nullptr;
+    const cudaGraphEdgeData* ed = nullptr;
+    size_t nd = 0;
+    const cudaError_t e1 = cudaStreamGetCaptureInfo(cs, &status, nullptr, nullptr, &d, &ed, &nd);
+    if (e1 == cudaSuccess && status == cudaStreamCaptureStatusActive) deps.assign(d, d + nd);
+    cudaGraph_t out = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(cs, &out);
+    if (rc) return rc;
+    if (e1 != cudaSuccess || e2 != cudaSuccess || status != cudaStreamCaptureStatusActive)
+      return set_err(HENRY_ECUDA, "graph capture failed: %s", cudaGetErrorString(e2 != cudaSuccess ? e2 : e1));
+    return HENRY_OK;
+  }
+  int handle(cudaGraphConditionalHandle* h) {
+    CK(cudaGraphConditionalHandleCreate(h, g, 0, cudaGraphCondAssignDefault));
+    return HENRY_OK;
+  }
+  // Append a conditional node; *body is the graph it runs.
+  int cond(cudaGraphConditionalNodeType type, cudaGraphConditionalHandle h, GraphBuild* body) {
+    cudaGraphNodeParams p = {};
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = h;
+    p.conditional.type = type;
+    p.conditional.size = 1;
+    cudaGraphNode_t n = nullptr;
+    CK(cudaGraphAddNode(&n, g, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(), &p));
+    deps.assign(1, n);
+    body->H = H;
+    body->g = p.conditional.phGraph_out[0];
+    body->deps.clear();
+    return HENRY_OK;
+  }
+};
+
+// Launch the graph that emit(GraphBuild&) describes on `st`, building it on
+// first use (key: what it is; the batch size and the configuration are added
+// here).  Captured on the handle's own stream, of st's priority (capturing the
+// legacy default stream is not allowed; capture executes nothing).
+constexpr size_t MAX_GRAPHS = 16;
+template <typename T, typename F>
+int run_graph(henry_handle* H, Group<T>& G, int B, const std::string& what, cudaStream_t st, F&& emit) {
+  std::string key = what;
+  key.append(reinterpret_cast<const char*>(&B), sizeof B);
+  key.append(reinterpret_cast<const char*>(&H->cfg), sizeof H->cfg);
+  auto f = G.gexec.find(key);
+  if (f == G.gexec.end()) {
+    if (G.gexec.size() >= MAX_GRAPHS) {  // e.g. an autotuner's candidates
+      CK(cudaStreamSynchronize(st));
+      G.drop_graphs();
+    }
+    if (!H->cap_stream) {
+      int prio = 0;
+      CK(cudaStreamGetPriority(st, &prio));
+      CK(cudaStreamCreateWithPriority(&H->cap_stream, cudaStreamNonBlocking, prio));
+    }
+    cudaGraph_t gr = nullptr;
+    CK(cudaGraphCreate(&gr, 0));
+    GraphBuild b{H, gr, {}};
+    const int rc = emit(b);
+    if (rc) {
+      cudaGraphDestroy(gr);
+      return rc;
+    }
+    cudaGraphExec_t ex = nullptr;
+    const cudaError_t e = cudaGraphInstantiate(&ex, gr, 0);
+    cudaGraphDestroy(gr);
+    if (e != cudaSuccess) return set_err(HENRY_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e));
+    f = G.gexec.emplace(key, ex).first;
+  }
+  CK(cudaGraphLaunch(f->second, st));
+  return HENRY_OK;
+}
+// Graphs are used unless the configuration says no, the workspace may not
+// allocate (instantiation would) or the kernel timer brackets every launch.
 template <typename T>
-int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const void* Jpre0 = nullptr,
-                 double rtol = -1.0, int maxit = -1) {
+bool graphs_on(const henry_handle* H, const Group<T>& G) {
+  return H->cfg.cuda_graphs && G.graphs && !H->prof.on;
+}
+
+// BiCGStab on the fine level for the samples with lin_active set; right-hand
+// side -F; solution in G.dx.  Jpre0: fine operator of the preconditioner
+// (NULL: the Jacobian).  The pieces of the loop, and the loop as nodes of a
+// graph.
+template <typename T>
+struct Krylov {
   typedef typename VT<T>::v2 V2;
   typedef typename VT<T>::b4 B4;
-  Level& L = G.lv[0];
-  const int N = L.N;
-  const unsigned g = nblk((int64_t)B * N);
-  const double b4 = sizeof(B4), v2 = sizeof(V2);
-  launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * v2), [&] {
-    chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
-  });
-  CKL();
-  // Large grids: reduce each sample's partials once (one warp per sample)
-  // instead of in every CTA of the consumer kernel.
-  double* fin = (H->cfg.finalize_nct > 0 && G.nct >= H->cfg.finalize_nct) ? G.fin : nullptr;
-  auto finalize = [&](int a, int b, cudaStream_t ss) {
+  henry_handle* H;
+  Group<T>& G;
+  int B;
+  const void* Jpre0;
+  double rtol2;
+  int maxit;
+  Level& L;
+  int N;
+  unsigned g;
+  double* fin;  // large grids: each sample's partials reduced once, not in every CTA of the consumer kernel
+
+  Krylov(henry_handle* h, Group<T>& grp, int b, const void* jpre0, double rtol, int mi)
+      : H(h), G(grp), B(b), Jpre0(jpre0), rtol2(rtol * rtol), maxit(mi), L(grp.lv[0]), N(grp.lv[0].N),
+        g(nblk((int64_t)b * grp.lv[0].N)),
+        fin((h->cfg.finalize_nct > 0 && grp.nct >= h->cfg.finalize_nct) ? grp.fin : nullptr) {}
+
+  void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
            [&] { chain(ss, nblk((int64_t)B * 32, 128), 128, 0, k_finalize, B, G.nct, G.part, a, b, fin); });
-  };
-  finalize(P_RR, P_RN, st);
-  const double rt = rtol > 0.0 ? rtol : H->cfg.lin_rtol;
-  const int mi = maxit > 0 ? maxit : H->cfg.lin_maxit;
-  const double rtol2 = rt * rt;
-  // One iteration after the convergence test: two preconditioned matvecs and
-  // the vector updates (every argument fixed for this group and B; the
-  // samples' activity is read from lin_active on the device).
-  auto body = [&](int n_act, cudaStream_t ss) -> int {
-    const double nc = (double)n_act * N;
+  }
+  int init(cudaStream_t st, int* loop) {
+    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * sizeof(V2)), [&] {
+      chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, loop);
+    });
+    finalize(P_RR, P_RN, st);
+    CKL();
+    return HENRY_OK;
+  }
+  // The convergence test and the new search direction of iteration `it` (or
+  // *it_dev), counting the samples that go on in G.counter[1].
+  int head(int it, const int* it_dev, cudaStream_t st) {
+    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * sizeof(V2), [&] {
+      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
+            G.iters, G.status, G.counter + 1, G.totals + 1, fin);
+    });
+    CKL();
+    return HENRY_OK;
+  }
+  // The rest of an iteration: two preconditioned matvecs and the vector
+  // updates (every argument fixed for this group and B; the samples' activity
+  // is read from lin_active on the device).
+  int body(int n_act, cudaStream_t ss) {
+    const double nc = (double)n_act * N, b4 = sizeof(B4), v2 = sizeof(V2);
     int rc = vcycle<T>(H, G, B, G.p, G.ph, ss, Jpre0);
     if (rc) return rc;
     launch(H, ss, HENRY_K_SPMV, nc * (5 * b4 + 3 * v2), n_act * spmv_flops(L.nx, L.ny, 1), [&] {
       with_preload((int64_t)B * N, [&](auto pre) {
-        chain(ss, g, TPB, 0, k_spmv<T, 1, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.ph, G.v, G.rh, G.part, P_RV, 0,
-              G.lin_active);
+        chain(ss, g, TPB, 0, k_spmv<T, 1, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.ph, G.v, G.rh,
+              G.part, P_RV, 0, G.lin_active);
       });
     });
     finalize(P_RV, -1, ss);
@@ -1008,8 +1139,8 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
     if (rc) return rc;
     launch(H, ss, HENRY_K_SPMV, nc * (5 * b4 + 3 * v2), n_act * spmv_flops(L.nx, L.ny, 2), [&] {
       with_preload((int64_t)B * N, [&](auto pre) {
-        chain(ss, g, TPB, 0, k_spmv<T, 2, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.sh, G.t, G.s, G.part, P_TS, P_TT,
-              G.lin_active);
+        chain(ss, g, TPB, 0, k_spmv<T, 2, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.sh, G.t, G.s,
+              G.part, P_TS, P_TT, G.lin_active);
       });
     });
     finalize(P_TS, P_TT, ss);
@@ -1022,208 +1153,324 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
     finalize(P_RR, P_RN, ss);
     CKL();
     return HENRY_OK;
-  };
-  // The body is captured once into a CUDA graph and replayed: one launch
-  // instead of ~80 at level 0, which matters on launch-bound groups (small
-  // grids, coarse levels).  Captured on the handle's own stream (capturing
-  // the legacy default stream is not allowed; capture executes nothing) and
-  // launched on `st`.  Off while the kernel timer runs.
-  const bool use_graph = H->cfg.cuda_graphs && G.graphs && !H->prof.on;
-  auto run_graph = [&]() -> int {
-    const auto key = std::make_tuple(B, Jpre0, H->cfg.nu1, H->cfg.nu2, H->cfg.mg_tail_cells, H->cfg.mg_threads);
-    auto f = G.gexec.find(key);
-    if (f == G.gexec.end()) {
-      if (!H->cap_stream) CK(cudaStreamCreateWithFlags(&H->cap_stream, cudaStreamNonBlocking));
-      cudaGraph_t gr = nullptr;
-      CK(cudaStreamBeginCapture(H->cap_stream, cudaStreamCaptureModeThreadLocal));
-      const int rc = body(B, H->cap_stream);
-      const cudaError_t e = cudaStreamEndCapture(H->cap_stream, &gr);
-      if (rc) {
-        if (e == cudaSuccess && gr) cudaGraphDestroy(gr);
-        return rc;
-      }
-      if (e != cudaSuccess) return set_err(HENRY_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
-      cudaGraphExec_t ex = nullptr;
-      const cudaError_t e2 = cudaGraphInstantiate(&ex, gr, 0);
-      cudaGraphDestroy(gr);
-      if (e2 != cudaSuccess) return set_err(HENRY_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e2));
-      f = G.gexec.emplace(key, ex).first;
-    }
-    CK(cudaGraphLaunch(f->second, st));
-    return HENRY_OK;
-  };
-  for (int it = 0; it <= mi; ++it) {
-    CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
-    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * v2, [&] {
-      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
-                                      G.iters, G.status, G.counter + 1, G.totals + 1, fin);
-    });
-    CKL();
-    int n_act = 0;
-    int rc = read_counter(H, G.counter + 1, st, &n_act);
-    if (rc) return rc;
-    if (n_act == 0) break;
-    H->nact = n_act;
-    rc = use_graph ? run_graph() : body(n_act, st);
-    if (rc) return rc;
   }
-  return HENRY_OK;
+  // The whole solve as nodes of a graph.
+  int emit(GraphBuild& b) {
+    cudaGraphConditionalHandle h;
+    int rc = b.handle(&h);
+    if (rc) return rc;
+    auto test = [&](cudaStream_t s) {
+      const int r = head(0, G.counter + 3, s);
+      chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 1, G.counter + 3);
+      return r;
+    };
+    rc = b.seg([&](cudaStream_t s) {
+      const int r = init(s, G.counter + 1);
+      return r ? r : test(s);
+    });
+    GraphBuild it;
+    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &it);
+    if (!rc)
+      rc = it.seg([&](cudaStream_t s) {
+        const int r = body(B, s);
+        return r ? r : test(s);
+      });
+    return rc;
+  }
+  // The whole solve driven from the host.
+  int run(cudaStream_t st) {
+    int rc = init(st, nullptr);
+    for (int it = 0; !rc && it <= maxit; ++it) {
+      CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
+      rc = head(it, nullptr, st);
+      int n_act = 0;
+      if (!rc) rc = read_counter(H, G.counter + 1, st, &n_act);
+      if (rc || n_act == 0) return rc;
+      H->nact = n_act;
+      rc = body(n_act, st);
+    }
+    return rc;
+  }
+};
+
+// rtol / maxit > 0 override the configuration's lin_rtol / lin_maxit.
+template <typename T>
+int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const void* Jpre0 = nullptr,
+                 double rtol = -1.0, int maxit = -1) {
+  const double rt = rtol > 0.0 ? rtol : H->cfg.lin_rtol;
+  const int mi = maxit > 0 ? maxit : H->cfg.lin_maxit;
+  Krylov<T> k(H, G, B, Jpre0, rt, mi);
+  if (!graphs_on(H, G)) return k.run(st);
+  std::string what = "linear";
+  what.append(reinterpret_cast<const char*>(&Jpre0), sizeof Jpre0);
+  what.append(reinterpret_cast<const char*>(&rt), sizeof rt);
+  what.append(reinterpret_cast<const char*>(&mi), sizeof mi);
+  return run_graph<T>(H, G, B, what, st, [&](GraphBuild& b) { return k.emit(b); });
 }
 
-// Second linear solve for the samples whose BiCGStab failed: the V-cycle
-// runs on the operator without the density derivatives (DROP), fine and
-// coarse, while the Krylov matvec keeps the exact Jacobian.  The coarse
-// operators of the retried samples are rebuilt by the next Newton iteration.
+// One implicit-Euler step (Sec. 2.3) of the B samples of a group: the state
+// x^n in lv[0].x (and x^{n-1} in lv[0].xo, for the predictor) becomes x^{n+1},
+// with Newton iterations as described at the top of this file.
+//
+// Newton's choices (the same in both drives): the Jacobian and the coarse
+// operators are assembled at iterations 0, k, 2k, ... of the step, k =
+// newton_jacobian_every (chord Newton; and after a fallback-preconditioner
+// retry, which rebuilt coarse operators for its samples), the others evaluate
+// the residual alone and reuse them.  From iteration newton_residual_first on
+// a sample is most likely converged: its residual is evaluated alone first,
+// and the Jacobian is assembled only for the samples that go on iterating
+// (the residual is recomputed with it, bit-identically).  The FP64 residual
+// test decides convergence.
 template <typename T>
-int retry_linear_solve(henry_handle* H, Group<T>& G, int B, double inv_tau, double inv_s, cudaStream_t st,
-                       int* retried = nullptr) {
-  typedef typename VT<T>::b4 B4;
-  const henry_config& c = H->cfg;
-  const LevelGeom lg = geom(c, G.level);
-  Level& L = G.lv[0];
-  CK(cudaMemsetAsync(G.counter + 2, 0, sizeof(int), st));
-  chain(st, nblk(B, 128), 128, 0, k_mark_retry, B, G.newton_active, G.iters, G.lin_active, G.counter + 2);
-  CKL();
-  int n_retry = 0;
-  int rc = read_counter(H, G.counter + 2, st, &n_retry);
-  if (rc) return rc;
-  if (retried) *retried = n_retry;
-  if (n_retry == 0) return HENRY_OK;
-  H->nact = n_retry;
-  double* pscratch = G.part + P_MAX * (int64_t)B * G.nct;
-  chain(st, nblk((int64_t)B * L.N), TPB, 0, assemble_kernel<T, true, true, true>(H->cfg, L.nx, L.ny), 
-      phys_of(c), G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
-      G.lin_active, nullptr, (B4*)G.Jp, L.plane, pscratch, L.cc, L.fc);
-  CKL();
-  rc = build_coarse_ops<T, true>(H, G, B, inv_tau, inv_s, st);
-  if (rc) return rc;
-  return linear_solve<T>(H, G, B, st, G.Jp);
-}
-
-// One implicit-Euler step (Sec. 2.3) of the B samples of a group: the
-// state x^n in lv[0].x (and x^{n-1} in lv[0].xo, for the predictor) becomes
-// x^{n+1}, with Newton iterations as described at the top of this file.
-// `step` is the step's index (the predictor is used from step 1 on).
-template <typename T>
-int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st) {
+struct NewtonStep {
   typedef typename VT<T>::b4 B4;
   typedef typename VT<T>::v2 V2;
-  const henry_config& c = H->cfg;
-  const LevelGeom lg = geom(c, G.level);
-  const Phys ph = phys_of(c);
-  Level& L = G.lv[0];
-  const int N = L.N;
-  const int64_t n0 = (int64_t)B * N;
-  const double inv_tau = 1.0 / lg.tau;
-  const double inv_s = 1.0 / (c.rho0 * lg.h * lg.h * inv_tau);
-  const double inv_pref = 1.0 / (c.rho0 * c.g * c.Ly);
-  double* pmax = G.part + P_MAX * (int64_t)B * G.nct;
-  H->nact = B;
-  launch(H, st, HENRY_K_NEWTON, (double)n0 * 32, [&] {
-    // quadratic predictor from step 2 on (three states), linear at step 1
-    const bool quad = c.newton_predictor_order == 2 && G.xoo;
-    if (step > 1 && quad && c.newton_predictor > 0.0) {
-      chain(st, nblk(n0), TPB, 0, k_step_begin_predict2, n0, c.newton_predictor, L.x, L.xo, G.xoo);
-    } else {
-      if (quad) chain(st, nblk(n0), TPB, 0, k_copy_d2, n0, L.xo, G.xoo);
-      if (step > 0 && c.newton_predictor > 0.0)
-        chain(st, nblk(n0), TPB, 0, k_step_begin_predict, n0, c.newton_predictor, L.x, L.xo);
-      else
-        chain(st, nblk(n0), TPB, 0, k_step_begin, n0, L.x, L.xo);
-    }
-    chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.newton_active, G.newton_it);
-  });
-  CKL();
-  int rc = restrict_states<T>(H, G, B, true, G.newton_active, st);
-  if (rc) return rc;
-  const double vt = lg.h * lg.h * inv_tau * inv_s;
-  // Fine residual and Jacobian (JAC), or the residual alone, of the samples
+  henry_handle* H;
+  Group<T>& G;
+  int B;
+  const henry_config& c;
+  LevelGeom lg;
+  Phys ph;
+  Level& L;
+  int N;
+  int64_t n0;
+  double inv_tau, inv_s, inv_pref, vt;
+  double* pmax;
+  int jac_every, res_from;  // newton_jacobian_every; newton_residual_first (< 0: never)
+
+  NewtonStep(henry_handle* h, Group<T>& g, int b)
+      : H(h), G(g), B(b), c(h->cfg), lg(geom(h->cfg, g.level)), ph(phys_of(h->cfg)), L(g.lv[0]), N(g.lv[0].N),
+        n0((int64_t)b * g.lv[0].N) {
+    inv_tau = 1.0 / lg.tau;
+    inv_s = 1.0 / (c.rho0 * lg.h * lg.h * inv_tau);
+    inv_pref = 1.0 / (c.rho0 * c.g * c.Ly);
+    vt = lg.h * lg.h * inv_tau * inv_s;
+    pmax = G.part + P_MAX * (int64_t)B * G.nct;
+    jac_every = std::max(1, c.newton_jacobian_every);
+    res_from = c.newton_residual_first;
+  }
+  bool retries() const { return G.Jp && c.lin_retry; }
+  // Step start: old states and Newton's first iterate (the predictor is used
+  // from step 1 on: linear at step 1, quadratic with three states).
+  int begin(int step, cudaStream_t st) {
+    H->nact = B;
+    launch(H, st, HENRY_K_NEWTON, (double)n0 * 32, [&] {
+      const bool quad = c.newton_predictor_order == 2 && G.xoo;
+      if (step > 1 && quad && c.newton_predictor > 0.0) {
+        chain(st, nblk(n0), TPB, 0, k_step_begin_predict2, n0, c.newton_predictor, L.x, L.xo, G.xoo);
+      } else {
+        if (quad) chain(st, nblk(n0), TPB, 0, k_copy_d2, n0, L.xo, G.xoo);
+        if (step > 0 && c.newton_predictor > 0.0)
+          chain(st, nblk(n0), TPB, 0, k_step_begin_predict, n0, c.newton_predictor, L.x, L.xo);
+        else
+          chain(st, nblk(n0), TPB, 0, k_step_begin, n0, L.x, L.xo);
+      }
+    });
+    CKL();
+    return HENRY_OK;
+  }
+  // Flags of the step and the coarse levels' old states.
+  int start(cudaStream_t st) {
+    launch(H, st, HENRY_K_NEWTON, (double)B * 12,
+           [&] { chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.newton_active, G.newton_it); });
+    CKL();
+    return restrict_states<T>(H, G, B, true, G.newton_active, st);
+  }
+  // Fine residual and Jacobian (jac), or the residual alone, of the samples
   // with newton_active set; F and the per-CTA max |F| into pmax.
-  auto assemble_fine = [&](bool jac) {
+  int assemble(bool jac, cudaStream_t st) {
+    auto go = [&](auto* k, B4* J) {
+      chain(st, nblk(n0), TPB, 0, k, ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo,
+            G.newton_active, G.F, J, L.plane, pmax, L.cc, L.fc);
+    };
     if (jac)
       launch(H, st, HENRY_K_ASSEMBLE, (double)H->nact * N * (48.0 + 6.0 * sizeof(B4)), [&] {
-        if (L.cc)
-          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, true>(c, L.nx, L.ny), 
-              ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo, G.newton_active, G.F, (B4*)L.J,
-              L.plane, pmax, L.cc, L.fc);
-        else
-          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true>(c, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h,
-                                                                      vt, inv_s, L.x, L.xo, G.newton_active, G.F,
-                                                                      (B4*)L.J, L.plane, pmax, nullptr, nullptr);
+        if (L.cc) go(assemble_kernel<T, true, true>(c, L.nx, L.ny), (B4*)L.J);
+        else go(assemble_kernel<T, true>(c, L.nx, L.ny), (B4*)L.J);
       });
     else
       launch(H, st, HENRY_K_RESIDUAL, (double)H->nact * N * 48.0, [&] {
-        if (L.cc)
-          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny), 
-              ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo, G.newton_active, G.F, nullptr,
-              L.plane, pmax, L.cc, L.fc);
-        else
-          chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny), 
-              ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo, G.newton_active, G.F, nullptr,
-              L.plane, pmax, nullptr, nullptr);
+        if (L.cc) go(assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny), nullptr);
+        else go(assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny), nullptr);
       });
-  };
-  // Chord Newton (newton_jacobian_every = k > 1): the Jacobian and the
-  // coarse operators are assembled at iterations 0, k, 2k, ... of the step
-  // (and after a fallback-preconditioner retry, which rebuilt coarse
-  // operators for its samples); the other iterations evaluate the residual
-  // alone and reuse them.  The FP64 residual test still decides convergence.
-  const int jac_every = std::max(1, c.newton_jacobian_every);
-  int last_jac = -1;
-  bool force_jac = false;
-  for (int it = 0; it <= c.newton_maxit; ++it) {
-    const bool jac_now = force_jac || last_jac < 0 || it - last_jac >= jac_every;
-    // From iteration newton_residual_first on, a sample is most likely
-    // converged: its residual is evaluated alone first, and the Jacobian is
-    // assembled only for the samples that go on iterating (the residual is
-    // recomputed with it, bit-identically).
-    const bool res_first = !jac_now || (c.newton_residual_first >= 0 && it >= c.newton_residual_first);
-    CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
-    assemble_fine(!res_first);
+    CKL();
+    return HENRY_OK;
+  }
+  bool jac_at(int it) const { return it % jac_every == 0; }
+  bool res_first_at(int it, bool jac_now) const { return !jac_now || (res_from >= 0 && it >= res_from); }
+  // The evaluation of an iteration and its residual test; `count` (nullable):
+  // the samples that go on are added to it.
+  int evaluate(bool res_first, int* count, cudaStream_t st) {
+    const int rc = assemble(!res_first, st);
     launch(H, st, HENRY_K_NEWTON, (double)B * 8 * G.nct, [&] {
       chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, G.nct, c.newton_atol, c.newton_maxit, pmax,
-                                                       G.newton_active, G.lin_active, G.newton_it, G.status,
-                                                       G.counter, G.totals);
+            G.newton_active, G.lin_active, G.newton_it, G.status, count, G.totals);
     });
     CKL();
-    int n_act = 0;
-    rc = read_counter(H, G.counter, st, &n_act);
-    if (rc) return rc;
-    if (n_act == 0) break;
-    H->nact = n_act;
-    if (jac_now) {
-      if (res_first) {
-        assemble_fine(true);
-        CKL();
-      }
-      if (c.coarse_op == HENRY_COARSE_REDISCRETISE) {
-        rc = restrict_states<T>(H, G, B, false, G.lin_active, st);
-        if (rc) return rc;
-      }
-      rc = build_coarse_ops<T>(H, G, B, inv_tau, inv_s, st);
-      if (rc) return rc;
-      last_jac = it;
-      force_jac = false;
-    }
-    rc = linear_solve<T>(H, G, B, st);
-    if (rc) return rc;
-    if (G.Jp && c.lin_retry) {  // fallback preconditioner for the samples whose solve failed
-      int retried = 0;
-      rc = retry_linear_solve<T>(H, G, B, inv_tau, inv_s, st, &retried);
-      if (rc) return rc;
-      if (retried) force_jac = true;
-    }
-    H->nact = n_act;
+    return rc;
+  }
+  // The Jacobian (if the evaluation took the residual alone) and the coarse
+  // operators.
+  int operators(bool res_first, cudaStream_t st) {
+    int rc = res_first ? assemble(true, st) : HENRY_OK;
+    if (!rc && c.coarse_op == HENRY_COARSE_REDISCRETISE) rc = restrict_states<T>(H, G, B, false, G.lin_active, st);
+    return rc ? rc : build_coarse_ops<T>(H, G, B, inv_tau, inv_s, st);
+  }
+  // Second linear solve for the samples whose BiCGStab failed: the V-cycle
+  // runs on the operator without the density derivatives (DROP), fine and
+  // coarse, while the Krylov matvec keeps the exact Jacobian.  The coarse
+  // operators of the retried samples are rebuilt by the next Newton iteration.
+  int mark_retry(cudaStream_t st) {
+    chain(st, nblk(B, 128), 128, 0, k_mark_retry, B, G.newton_active, G.iters, G.lin_active, G.counter + 2);
+    CKL();
+    return HENRY_OK;
+  }
+  int retry_operators(cudaStream_t st) {
+    double* pscratch = G.part + P_MAX * (int64_t)B * G.nct;
+    chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, true, true>(c, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h,
+          1.0 / lg.h, vt, inv_s, L.x, L.xo, G.lin_active, nullptr, (B4*)G.Jp, L.plane, pscratch, L.cc, L.fc);
+    CKL();
+    return build_coarse_ops<T, true>(H, G, B, inv_tau, inv_s, st);
+  }
+  int update(int n_act, cudaStream_t st) {
     launch(H, st, HENRY_K_NEWTON, (double)n_act * N * (32.0 + sizeof(V2)), [&] {
       double* pdc = G.part + P_DC * (int64_t)B * G.nct;
       chain(st, nblk(n0), TPB, 0, k_newton_step_max<T>, B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active, G.theta);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active,
+            G.theta);
       chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active, G.status);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active,
+            G.status);
     });
     CKL();
+    return HENRY_OK;
   }
-  return HENRY_OK;
+
+  // --- host-driven
+  int run(cudaStream_t st) {
+    int rc = start(st);
+    int last_jac = -1;
+    bool force_jac = false;
+    for (int it = 0; !rc && it <= c.newton_maxit; ++it) {
+      const bool jac_now = force_jac || last_jac < 0 || it - last_jac >= jac_every;
+      const bool res_first = res_first_at(it, jac_now);
+      CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
+      rc = evaluate(res_first, G.counter, st);
+      int n_act = 0;
+      if (!rc) rc = read_counter(H, G.counter, st, &n_act);
+      if (rc || n_act == 0) return rc;
+      H->nact = n_act;
+      if (jac_now) {
+        rc = operators(res_first, st);
+        if (rc) return rc;
+        last_jac = it;
+        force_jac = false;
+      }
+      rc = linear_solve<T>(H, G, B, st);
+      if (!rc && retries()) {
+        CK(cudaMemsetAsync(G.counter + 2, 0, sizeof(int), st));
+        rc = mark_retry(st);
+        int n_retry = 0;
+        if (!rc) rc = read_counter(H, G.counter + 2, st, &n_retry);
+        if (!rc && n_retry > 0) {
+          H->nact = n_retry;
+          rc = retry_operators(st);
+          if (!rc) rc = linear_solve<T>(H, G, B, st, G.Jp);
+          force_jac = true;
+        }
+      }
+      H->nact = n_act;
+      if (!rc) rc = update(n_act, st);
+    }
+    return rc;
+  }
+
+  // --- as a graph
+  // From this iteration on the pattern of evaluations repeats every jac_every
+  // iterations.
+  int steady() const { return res_from <= 0 ? 0 : ((res_from + jac_every - 1) / jac_every) * jac_every; }
+  // Whether the step can run as one graph: few iterations before the steady
+  // pattern, and no retries that would shift a chord pattern.
+  bool graphable() const { return steady() <= 6 && jac_every <= 8 && !(retries() && jac_every > 1); }
+  int emit_work(GraphBuild& b, int it) {
+    int rc = HENRY_OK;
+    if (jac_at(it)) rc = b.seg([&](cudaStream_t s) { return operators(res_first_at(it, true), s); });
+    if (!rc) rc = Krylov<T>(H, G, B, nullptr, c.lin_rtol, c.lin_maxit).emit(b);
+    if (!rc && retries()) {
+      cudaGraphConditionalHandle h;
+      rc = b.handle(&h);
+      if (!rc)
+        rc = b.seg([&](cudaStream_t s) {
+          const int r = mark_retry(s);
+          chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 2, (int*)nullptr);
+          return r;
+        });
+      GraphBuild r;
+      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &r);
+      if (!rc) rc = r.seg([&](cudaStream_t s) { return retry_operators(s); });
+      if (!rc) rc = Krylov<T>(H, G, B, G.Jp, c.lin_rtol, c.lin_maxit).emit(r);
+    }
+    return rc ? rc : b.seg([&](cudaStream_t s) { return update(B, s); });
+  }
+  // Iteration `it`: evaluate, then set the conditions h1 (and h2) to whether
+  // any sample goes on.
+  int emit_test(GraphBuild& b, int it, cudaGraphConditionalHandle h1, cudaGraphConditionalHandle h2, int two) {
+    return b.seg([&](cudaStream_t s) {
+      const int r = evaluate(res_first_at(it, jac_at(it)), G.counter, s);
+      chain(s, 1, 1, 0, k_loop_gate, h1, h2, two, G.counter, (int*)nullptr);
+      return r;
+    });
+  }
+  // The iterations from `it` on.  The first two run unconditionally (their
+  // kernels skip samples that have converged; hardly any step is done by
+  // then), the following ones up to the steady pattern inside IF nodes, then
+  // a WHILE node runs jac_every iterations a turn.
+  int emit_from(GraphBuild& b, int it) {
+    const int S = steady();
+    if (it < S && it < 2) {
+      int rc = b.seg([&](cudaStream_t s) { return evaluate(res_first_at(it, jac_at(it)), nullptr, s); });
+      if (!rc) rc = emit_work(b, it);
+      return rc ? rc : emit_from(b, it + 1);
+    }
+    cudaGraphConditionalHandle h;
+    int rc = b.handle(&h);
+    if (!rc) rc = emit_test(b, it, h, h, 0);
+    GraphBuild in;
+    if (it < S) {
+      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
+      if (!rc) rc = emit_work(in, it);
+      return rc ? rc : emit_from(in, it + 1);
+    }
+    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &in);
+    return rc ? rc : emit_turn(in, S, 0, h);
+  }
+  // Iterations S + j .. S + jac_every - 1 of a turn of the WHILE node (condition w).
+  int emit_turn(GraphBuild& b, int S, int j, cudaGraphConditionalHandle w) {
+    int rc = emit_work(b, S + j);
+    if (rc) return rc;
+    if (j == jac_every - 1) return emit_test(b, S + j + 1, w, w, 0);
+    cudaGraphConditionalHandle h;
+    rc = b.handle(&h);
+    if (!rc) rc = emit_test(b, S + j + 1, h, w, 1);
+    GraphBuild in;
+    if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
+    return rc ? rc : emit_turn(in, S, j + 1, w);
+  }
+  int emit(GraphBuild& b) {
+    const int rc = b.seg([&](cudaStream_t s) { return start(s); });
+    return rc ? rc : emit_from(b, 0);
+  }
+};
+
+// `step` is the step's index.
+template <typename T>
+int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st) {
+  NewtonStep<T> n(H, G, B);
+  const int rc = n.begin(step, st);
+  if (rc) return rc;
+  if (!graphs_on(H, G) || !n.graphable()) return n.run(st);
+  if (step == 0) CK(cudaMemsetAsync(G.counter, 0, 4 * sizeof(int), st));
+  return run_graph<T>(H, G, B, "step", st, [&](GraphBuild& b) { return n.emit(b); });
 }
 
 // Full scenario solves of B samples whose coefficients and status are set.
@@ -1526,7 +1773,7 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
   const unsigned g = nblk((int64_t)B * N);
   const double b4 = sizeof(B4), v2 = sizeof(V2);
   launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * v2), [&] {
-    chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
+    chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, (int*)nullptr);
   });
   CKL();
   double* fin = (H->cfg.finalize_nct > 0 && G.nct >= H->cfg.finalize_nct) ? G.fin : nullptr;
@@ -1591,7 +1838,7 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
   for (int it = 0; it <= mi; ++it) {
     CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * v2, [&] {
-      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
+      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, (const int*)nullptr, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
                                       G.status, G.counter + 1, G.totals + 1, fin);
     });
     CKL();
