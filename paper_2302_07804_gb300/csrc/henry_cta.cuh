@@ -13,6 +13,7 @@
 // summation order of the dot products.
 #pragma once
 #include "henry_kernels.cuh"
+#include "henry_misc.cuh"
 
 namespace hk {
 
@@ -273,6 +274,14 @@ __global__ void __launch_bounds__(CTA_THREADS) k_cta_solve(const __grid_constant
   V2 *r = S.vec(L.r), *rh = S.vec(L.rh), *p = S.vec(L.p), *v = S.vec(L.v), *t = S.vec(L.t);
   V2 *ph = S.vec(L.ph), *dx = S.vec(L.dx);
   const double inv_tau = 1.0 / P.tau;
+  __shared__ LevelCoef lcoef[CTA_MAX_LEVELS];
+  if (threadIdx.x <= K) {
+    const double hk = P.h0 * (double)(1 << threadIdx.x);
+    lcoef[threadIdx.x] = level_coef(P.ph, cf, hk, hk * hk * inv_tau * P.inv_s, P.inv_s);
+  }
+  __syncthreads();
+  CellCoefs<double, false> K0;
+  K0.load(P.ph, lcoef, nullptr, 0, 0.0, 0.0, 0.0, nullptr, 0);
   unsigned long long newton_total = 0, lin_total = 0;
   int fail = 0;
 
@@ -326,16 +335,13 @@ __global__ void __launch_bounds__(CTA_THREADS) k_cta_solve(const __grid_constant
       for (int i = threadIdx.x; i < N0; i += blockDim.x) {
         int ix, iy;
         xy_of(i, nx0, ix, iy);
-        CellSys<T, double> o;
-        assemble_cell<T, double>(P.ph, cf, nx0, ny0, P.h0, 1.0 / P.h0, P.h0 * P.h0 * inv_tau * P.inv_s, P.inv_s, x,
-                                 xo, i, ix, iy, o);
+        CellSum<T, double> o;
+        assemble_cell<T, double>(P.ph, K0, nx0, ny0, P.h0, x, xo, i, ix, iy, o);
         store_blocks<T>(S.J(0), N0, i, o.C, o.Nb);
-        const V2 ri = mk2<V2>((T)(-o.fm), (T)(-o.fs));
+        const V2 ri = mk2<V2>((T)(-o.Rm), (T)(-o.Rs));
         r[i] = ri;
         rh[i] = ri;
-        double l = fmax(fabs(o.fm), fabs(o.fs));
-        if (!(l <= 1.0e300)) l = INFINITY;
-        rloc = fmax(rloc, l);
+        rloc = abs_max_or_inf(rloc, abs_max_or_inf(o.Rm, o.Rs));
         rrT = fma_(ri.x, ri.x, fma_(ri.y, ri.y, rrT));
       }
       const double rmax = cta_max(rloc, sh);
@@ -363,12 +369,13 @@ __global__ void __launch_bounds__(CTA_THREADS) k_cta_solve(const __grid_constant
         }
         __syncthreads();
         const double hk = P.h0 * (double)(1 << k);
+        CellCoefs<SC, false> Kk;
+        Kk.load(P.ph, lcoef + k, nullptr, 0, 0.0, 0.0, 0.0, nullptr, 0);
         for (int c = threadIdx.x; c < Nc; c += blockDim.x) {
           int IX, IY;
           xy_of(c, ncx, IX, IY);
-          CellSys<T, SC> o;
-          assemble_cell<T, SC>(P.ph, cf, ncx, ncy, hk, 1.0 / hk, hk * hk * inv_tau * P.inv_s, P.inv_s, xc,
-                               S.XO(k), c, IX, IY, o);
+          CellSum<T, SC> o;
+          assemble_cell<T, SC>(P.ph, Kk, ncx, ncy, hk, xc, S.XO(k), c, IX, IY, o);
           store_blocks<T>(S.J(k), Nc, c, o.C, o.Nb);
         }
       }

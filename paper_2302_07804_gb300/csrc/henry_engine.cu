@@ -97,6 +97,7 @@ struct Level {
   double2 *x, *xo;  // state (fine: Newton iterate; coarse: restricted) and old state
   double2* cc;      // per-cell (phi, K / mu) of the field models (else null)
   double4_32a* fc;      // per-cell east/north face harmonic means of the field models (else null)
+  LevelCoef* lc;    // per-sample scaled coefficients of the constant-coefficient model (else null)
   void* J;          // 6 planes of B4
   void *mgx, *mgb;  // multigrid vectors (coarse levels)
   int64_t plane;
@@ -164,6 +165,7 @@ struct Group {
       l.J = l.mgx = l.mgb = nullptr;
       l.cc = nullptr;
       l.fc = nullptr;
+      l.lc = (fields || light_ws) ? nullptr : c.take<LevelCoef>(sizeof(LevelCoef) * B);
       if (fields) {
         l.cc = c.take<double2>(sizeof(double2) * l.plane);
         l.fc = c.take<double4_32a>(sizeof(double4_32a) * l.plane);
@@ -497,6 +499,7 @@ Phys phys_of(const henry_config& c) {
 
   Phys p;
   p.rho0 = c.rho0; p.rho1 = c.rho1; p.drho = c.rho1 - c.rho0; p.g = c.g; p.Ly = c.Ly; p.Dm = c.Dm;
+  p.rho1g = c.rho1 * c.g;
   return p;
 }
 
@@ -687,10 +690,23 @@ int ensure_kl_tables(henry_handle* H, int level, KLTables** out) {
 template <typename T>
 int set_coefficients(henry_handle* H, Group<T>& G, const double* xi, int B, cudaStream_t st) {
   const henry_config& c = H->cfg;
+  const LevelGeom lg = geom(c, G.level);
+  const double inv_tau = 1.0 / lg.tau;
+  const double inv_s = 1.0 / (c.rho0 * lg.h * lg.h * inv_tau);
   if (!has_fields(c)) {
     CoefModel m{c.phi_mean, c.K_mean, c.qin_mean, c.phi_amp, c.logK_amp, c.qin_amp, c.mu, c.Dm};
-    launch(H, st, HENRY_K_QOI, (double)B * (24 + 32 + 4),
-           [&] { k_coefficients<<<nblk(B, 128), 128, 0, st>>>(m, B, xi, G.coef, G.status); });
+    LevelList LL;
+    std::memset(&LL, 0, sizeof LL);
+    LL.ph = phys_of(c);
+    LL.inv_s = inv_s;
+    for (Level& L : G.lv) {
+      if (!L.lc) continue;  // the fused solver forms its own
+      LL.h[LL.n] = L.h;
+      LL.vt_s[LL.n] = L.h * L.h * inv_tau * inv_s;
+      LL.lc[LL.n++] = L.lc;
+    }
+    launch(H, st, HENRY_K_QOI, (double)B * (24 + 32 + 4 + LL.n * 64),
+           [&] { k_coefficients<<<nblk(B, 128), 128, 0, st>>>(m, B, xi, G.coef, G.status, LL); });
     CKL();
     return HENRY_OK;
   }
@@ -718,12 +734,29 @@ int set_coefficients(henry_handle* H, Group<T>& G, const double* xi, int B, cuda
       k_restrict_cc<<<nblk((int64_t)B * L.N), TPB, 0, st>>>(B, L.nx, L.ny, G.lv[k - 1].cc, L.cc);
       CKL();
     }
-    k_face_coefs<<<nblk((int64_t)B * L.N), TPB, 0, st>>>(B, L.nx, L.ny, c.Dm, L.cc, L.fc);
+    k_face_coefs<<<nblk((int64_t)B * L.N), TPB, 0, st>>>(B, L.nx, L.ny, c.Dm, inv_s, L.cc, L.fc);
     CKL();
   }
   return HENRY_OK;
 }
 
+
+// Residual and Jacobian blocks (JAC; else the residual alone) of one multigrid
+// level for the samples with active[s] set; FINE: F and the per-CTA max |F|.
+template <typename T, bool FINE, bool DROP = false, bool JAC = true>
+void assemble_level(const henry_config& c, Group<T>& G, const Level& L, int B, double inv_tau, double inv_s,
+                    const int* active, double2* F, void* J, double* rmax_part, cudaStream_t st) {
+  typedef typename VT<T>::b4 B4;
+  auto go = [&](auto* k) {
+    chain(st, nblk((int64_t)B * L.N), TPB, 0, k, phys_of(c), G.coef, L.lc, B, L.nx, L.ny, L.h,
+          L.h * L.h * inv_tau * inv_s, inv_s, L.x, L.xo, active, F, (B4*)J, L.plane, rmax_part, L.cc, L.fc);
+  };
+  if (L.cc) {
+    go(assemble_kernel<T, FINE, true, DROP, JAC>(c, L.nx, L.ny));
+  } else if constexpr (!DROP) {
+    go(assemble_kernel<T, FINE, false, false, JAC>(c, L.nx, L.ny));
+  }
+}
 
 // Coarse-grid operators for every multigrid level below the fine one, plus
 // the coarsest inverse.  Expects lv[k].x for k >= 1 up to date when
@@ -731,7 +764,6 @@ int set_coefficients(henry_handle* H, Group<T>& G, const double* xi, int B, cuda
 template <typename T, bool DROP = false>
 int build_coarse_ops(henry_handle* H, Group<T>& G, int B, double inv_tau, double inv_s, cudaStream_t st) {
   typedef typename VT<T>::b4 B4;
-  const Phys ph = phys_of(H->cfg);
   const double na = H->nact;
   for (int k = 1; k <= G.K; ++k) {
     Level& L = G.lv[k];
@@ -743,15 +775,7 @@ int build_coarse_ops(henry_handle* H, Group<T>& G, int B, double inv_tau, double
       });
     } else {
       launch(H, st, HENRY_K_COARSE_OPS, na * L.N * (32.0 + 6.0 * sizeof(B4)), [&] {
-        if (L.cc)
-          chain(st, nblk((int64_t)B * L.N), TPB, 0, assemble_kernel<T, false, true, DROP>(H->cfg, L.nx, L.ny), 
-              ph, G.coef, B, L.nx, L.ny, L.h, 1.0 / L.h, L.h * L.h * inv_tau * inv_s, inv_s, L.x, L.xo, G.lin_active,
-              nullptr, (B4*)L.J, L.plane, nullptr, L.cc, L.fc);
-        else
-          chain(st, nblk((int64_t)B * L.N), TPB, 0, assemble_kernel<T, false>(H->cfg, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, L.h, 1.0 / L.h,
-                                                                        L.h * L.h * inv_tau * inv_s, inv_s, L.x,
-                                                                        L.xo, G.lin_active, nullptr, (B4*)L.J,
-                                                                        L.plane, nullptr, nullptr, nullptr);
+        assemble_level<T, false, DROP>(H->cfg, G, L, B, inv_tau, inv_s, G.lin_active, nullptr, L.J, nullptr, st);
       });
     }
     CKL();
@@ -1230,21 +1254,19 @@ struct NewtonStep {
   int B;
   const henry_config& c;
   LevelGeom lg;
-  Phys ph;
   Level& L;
   int N;
   int64_t n0;
-  double inv_tau, inv_s, inv_pref, vt;
+  double inv_tau, inv_s, inv_pref;
   double* pmax;
   int jac_every, res_from;  // newton_jacobian_every; newton_residual_first (< 0: never)
 
   NewtonStep(henry_handle* h, Group<T>& g, int b)
-      : H(h), G(g), B(b), c(h->cfg), lg(geom(h->cfg, g.level)), ph(phys_of(h->cfg)), L(g.lv[0]), N(g.lv[0].N),
+      : H(h), G(g), B(b), c(h->cfg), lg(geom(h->cfg, g.level)), L(g.lv[0]), N(g.lv[0].N),
         n0((int64_t)b * g.lv[0].N) {
     inv_tau = 1.0 / lg.tau;
     inv_s = 1.0 / (c.rho0 * lg.h * lg.h * inv_tau);
     inv_pref = 1.0 / (c.rho0 * c.g * c.Ly);
-    vt = lg.h * lg.h * inv_tau * inv_s;
     pmax = G.part + P_MAX * (int64_t)B * G.nct;
     jac_every = std::max(1, c.newton_jacobian_every);
     res_from = c.newton_residual_first;
@@ -1279,19 +1301,13 @@ struct NewtonStep {
   // Fine residual and Jacobian (jac), or the residual alone, of the samples
   // with newton_active set; F and the per-CTA max |F| into pmax.
   int assemble(bool jac, cudaStream_t st) {
-    auto go = [&](auto* k, B4* J) {
-      chain(st, nblk(n0), TPB, 0, k, ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s, L.x, L.xo,
-            G.newton_active, G.F, J, L.plane, pmax, L.cc, L.fc);
-    };
     if (jac)
       launch(H, st, HENRY_K_ASSEMBLE, (double)H->nact * N * (48.0 + 6.0 * sizeof(B4)), [&] {
-        if (L.cc) go(assemble_kernel<T, true, true>(c, L.nx, L.ny), (B4*)L.J);
-        else go(assemble_kernel<T, true>(c, L.nx, L.ny), (B4*)L.J);
+        assemble_level<T, true>(c, G, L, B, inv_tau, inv_s, G.newton_active, G.F, L.J, pmax, st);
       });
     else
       launch(H, st, HENRY_K_RESIDUAL, (double)H->nact * N * 48.0, [&] {
-        if (L.cc) go(assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny), nullptr);
-        else go(assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny), nullptr);
+        assemble_level<T, true, false, false>(c, G, L, B, inv_tau, inv_s, G.newton_active, G.F, nullptr, pmax, st);
       });
     CKL();
     return HENRY_OK;
@@ -1327,8 +1343,7 @@ struct NewtonStep {
   }
   int retry_operators(cudaStream_t st) {
     double* pscratch = G.part + P_MAX * (int64_t)B * G.nct;
-    chain(st, nblk(n0), TPB, 0, assemble_kernel<T, true, true, true>(c, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h,
-          1.0 / lg.h, vt, inv_s, L.x, L.xo, G.lin_active, nullptr, (B4*)G.Jp, L.plane, pscratch, L.cc, L.fc);
+    assemble_level<T, true, true>(c, G, L, B, inv_tau, inv_s, G.lin_active, nullptr, G.Jp, pscratch, st);
     CKL();
     return build_coarse_ops<T, true>(H, G, B, inv_tau, inv_s, st);
   }
@@ -2161,10 +2176,8 @@ int setup_from_states(henry_handle* H, int level, const double* xi, int n, const
   if (rc) return rc;
   Level& L = G->lv[0];
   const int64_t n0 = (int64_t)n * L.N;
-  k_to_storage<double2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)state, L.x);
-  k_to_storage<double2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)state_old, L.xo);
-  chain(st, nblk(n, 128), 128, 0, k_step_flags, n, G->status, G->newton_active, G->newton_it);
-  CK(cudaMemcpyAsync(G->lin_active, G->newton_active, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
+  chain(st, nblk(n0), TPB, 0, k_states_in, n, L.nx, L.ny, (const double2*)state, (const double2*)state_old, L.x, L.xo,
+        G->status, G->newton_active, G->lin_active, G->newton_it);
   CKL();
   *out = G;
   return HENRY_OK;
@@ -2180,29 +2193,11 @@ int assemble_all(henry_handle* H, Group<T>& G, int n, bool coarse, cudaStream_t 
   const double inv_tau = 1.0 / lg.tau;
   const double inv_s = 1.0 / (c.rho0 * lg.h * lg.h * inv_tau);
   Level& L = G.lv[0];
-  if (!jac) {
-    double* pm = G.part + P_MAX * (int64_t)n * G.nct;
-    if (L.cc)
-      chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true, true, false, false>(c, L.nx, L.ny), 
-          phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
-          G.newton_active, G.F, nullptr, L.plane, pm, L.cc, L.fc);
-    else
-      chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true, false, false, false>(c, L.nx, L.ny), 
-          phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
-          G.newton_active, G.F, nullptr, L.plane, pm, nullptr, nullptr);
-    CKL();
-    return HENRY_OK;
-  }
-  if (L.cc)
-    chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true, true>(H->cfg, L.nx, L.ny), 
-        phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h, lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
-        G.newton_active, G.F, (B4*)L.J, L.plane, G.part + P_MAX * (int64_t)n * G.nct, L.cc, L.fc);
-  else
-    chain(st, nblk((int64_t)n * L.N), TPB, 0, assemble_kernel<T, true>(H->cfg, L.nx, L.ny), phys_of(c), G.coef, n, L.nx, L.ny, lg.h, 1.0 / lg.h,
-                                                                 lg.h * lg.h * inv_tau * inv_s, inv_s, L.x, L.xo,
-                                                                 G.newton_active, G.F, (B4*)L.J, L.plane,
-                                                                 G.part + P_MAX * (int64_t)n * G.nct, nullptr, nullptr);
+  double* pm = G.part + P_MAX * (int64_t)n * G.nct;
+  if (jac) assemble_level<T, true>(c, G, L, n, inv_tau, inv_s, G.newton_active, G.F, L.J, pm, st);
+  else assemble_level<T, true, false, false>(c, G, L, n, inv_tau, inv_s, G.newton_active, G.F, nullptr, pm, st);
   CKL();
+  if (!jac) return HENRY_OK;
   if (!coarse) return HENRY_OK;
   int rc = restrict_states<T>(H, G, n, true, G.lin_active, st);
   if (rc) return rc;
@@ -2316,13 +2311,7 @@ int adjoint_group(henry_handle* H, Group<double>& G, int B, const double* xi, co
       CKL();
       H->nact = B;
       launch(H, st, HENRY_K_ASSEMBLE, (double)n0 * (48.0 + 6.0 * sizeof(B4)), [&] {
-        if (L.cc)
-          chain(st, nblk(n0), TPB, 0, assemble_kernel<double, true, true>(H->cfg, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt,
-                                                                  inv_s, L.x, L.xo, G.lin_active, G.F, (B4*)L.J,
-                                                                  L.plane, pmax, L.cc, L.fc);
-        else
-          chain(st, nblk(n0), TPB, 0, assemble_kernel<double, true>(H->cfg, L.nx, L.ny), ph, G.coef, B, L.nx, L.ny, lg.h, 1.0 / lg.h, vt, inv_s,
-                                                            L.x, L.xo, G.lin_active, G.F, (B4*)L.J, L.plane, pmax, nullptr, nullptr);
+        assemble_level<double, true>(c, G, L, B, inv_tau, inv_s, G.lin_active, G.F, L.J, pmax, st);
       });
       CKL();
       int rc;
@@ -2421,30 +2410,31 @@ int step_entry(henry_handle* H, int which, int level, const double* xi, int n, c
   if (rc) return rc;
   switch (which) {
     case 0:  // assemble
-      k_from_storage<double2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, G->F, (double2*)out);
-      if (out2) k_blocks_out<B4><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const B4*)L.J, L.plane, out2);
+      chain(st, nblk(n0), TPB, 0, k_from_storage<double2>, n, L.nx, L.ny, G->F, (double2*)out);
+      if (out2)
+        chain(st, nblk(n0 * 10), TPB, 0, k_blocks_out<V2>, n, L.nx, L.ny, (const V2*)L.J, L.plane, (double2*)out2);
       break;
     case 1:  // apply
-      k_to_storage<V2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)in, G->p);
-      k_spmv<T, 0><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const B4*)L.J, L.plane, G->p, G->v, nullptr, nullptr,
-                                             0, 0, G->lin_active);
-      k_from_storage<V2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, G->v, (double2*)out);
+      chain(st, nblk(n0), TPB, 0, k_to_storage<V2>, n, L.nx, L.ny, (const double2*)in, G->p);
+      chain(st, nblk(n0), TPB, 0, k_spmv<T, 0>, n, L.nx, L.ny, (const B4*)L.J, L.plane, G->p, G->v, nullptr, nullptr, 0,
+            0, G->lin_active);
+      chain(st, nblk(n0), TPB, 0, k_from_storage<V2>, n, L.nx, L.ny, G->v, (double2*)out);
       break;
     case 2:  // precondition
-      k_to_storage<V2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)in, G->p);
+      chain(st, nblk(n0), TPB, 0, k_to_storage<V2>, n, L.nx, L.ny, (const double2*)in, G->p);
       CKL();
       rc = vcycle<T>(H, *G, n, G->p, G->ph, st);
       if (rc) return rc;
-      k_from_storage<V2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, G->ph, (double2*)out);
+      chain(st, nblk(n0), TPB, 0, k_from_storage<V2>, n, L.nx, L.ny, G->ph, (double2*)out);
       break;
     case 3:  // linear solve: F := -b, BiCGStab, dx out
-      k_to_storage<double2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, (const double2*)in, G->F);
-      k_scale_d2<<<nblk(n0), TPB, 0, st>>>(n0, -1.0, G->F);
+      chain(st, nblk(n0), TPB, 0, k_to_storage<double2>, n, L.nx, L.ny, (const double2*)in, G->F);
+      chain(st, nblk(n0), TPB, 0, k_scale_d2, n0, -1.0, G->F);
       CKL();
       CK(cudaMemsetAsync(G->totals, 0, 4 * sizeof(unsigned long long), st));
       rc = linear_solve<T>(H, *G, n, st);
       if (rc) return rc;
-      k_from_storage<V2><<<nblk(n0), TPB, 0, st>>>(n, L.nx, L.ny, G->dx, (double2*)out);
+      chain(st, nblk(n0), TPB, 0, k_from_storage<V2>, n, L.nx, L.ny, G->dx, (double2*)out);
       if (iters) CK(cudaMemcpyAsync(iters, G->iters, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
       break;
   }

@@ -49,6 +49,7 @@ __device__ __forceinline__ V2 mk2(T a, T b) { V2 v; v.x = a; v.y = b; return v; 
 // Physics constants passed by value.
 struct Phys {
   double rho0, rho1, drho, g, Ly, Dm;
+  double rho1g;  // rho1 g
 };
 
 // Per-sample coefficients: porosity, K / mu, phi * Dm, inflow velocity.
@@ -260,147 +261,293 @@ __device__ __forceinline__ B4 mkblk(double a00, double a01, double a10, double a
   return b;
 }
 
-// Land (ix = 0) and seaside (ix = nx - 1) boundary terms of one cell, added
-// to its scaled residuals and centre block (assemble_cell and the tile
-// assembly share them).
-template <typename T, typename S, bool DROP, bool JAC = true>
-__device__ __forceinline__ void boundary_terms(const Phys& ph, double qin, double inv_s, S kmu, S PD, int nx, int ix,
-                                               int iy, S hS, S ihS, S rhoP, S pP, S cP, S& Rm, S& Rs, T& C00,
-                                               T& C01, T& C10, T& C11) {
-  const S drho = (S)ph.drho, rho0 = (S)ph.rho0;
-  const T kmuP_T = (T)kmu, PDP_T = (T)PD, hT = (T)hS, hdT = (T)(0.5 * ph.drho);
-  if (ix == 0) {  // land side: prescribed inflow of fresh water, c_b = 0
-    const S Fl = -rho0 * (S)(qin * inv_s) * hS;
-    const S rb = (S)0.5 * (rhoP + rho0);
-    const bool up = Fl >= (S)0;
-    Rm += Fl;
-    Rs += fma_(Fl, up ? cP : (S)0, (S)2 * rb * PD * cP);
-    if constexpr (JAC) C11 += (up ? (T)Fl : (T)0) + PDP_T * (T)fma_(drho, cP, (S)2 * rb);
-  }
-  if (ix == nx - 1) {  // seaside: hydrostatic brine pressure, c_b = 1
-    const S yP = ((S)iy + (S)0.5) * hS;
-    const S pb = (S)ph.rho1 * (S)ph.g * ((S)ph.Ly - yP);
-    const S rb = (S)0.5 * (rhoP + (S)ph.rho1);
-    const S q = -kmu * (pb - pP) * ((S)2 * ihS);
-    const S Fr = rb * q * hS;
-    const bool up = Fr >= (S)0;
-    const S cup = up ? cP : (S)1;
-    const S dif = PD * ((S)1 - cP);
-    Rm += Fr;
-    Rs += fma_(Fr, cup, -(S)2 * rb * dif);
-    if constexpr (JAC) {
-      const T dFdp = (T)2 * (T)rb * kmuP_T;
-      const T dFdc = DROP ? (T)0 : hdT * (T)q * hT;
-      C00 += dFdp;
-      C01 += dFdc;
-      C10 = fma_(dFdp, (T)cup, C10);
-      C11 += fma_(dFdc, (T)cup, (up ? (T)Fr : (T)0) - ((T)drho * (T)dif - (T)2 * (T)rb * PDP_T));
-    }
-  }
+// Products that the compiler must not contract into multiply-adds, so that the
+// assembly's arithmetic is the same at every call site; sign changes and
+// comparisons on the integer pipes (an FP64 compare or negation takes the
+// FP64 pipe's 64 cycles a warp).
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double neg_(double a) {
+  return __hiloint2double(__double2hiint(a) ^ 0x80000000, __double2loint(a));
+}
+__device__ __forceinline__ float neg_(float a) { return -a; }
+__device__ __forceinline__ bool nonneg(double a) {  // a >= 0 (-0 included)
+  const long long u = __double_as_longlong(a);
+  return u >= 0 || (u << 1) == 0;
+}
+__device__ __forceinline__ bool nonneg(float a) { return a >= 0.f; }
+// max(|a|, |b|) as a non-negative double; +inf for anything beyond 1e300 or NaN.
+__device__ __forceinline__ double abs_max_or_inf(double a, double b) {
+  const unsigned long long m = 0x7fffffffffffffffull, lim = 0x7e37e43c8800759cull;  // the bits of 1e300
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a) & m;
+  const unsigned long long y = (unsigned long long)__double_as_longlong(b) & m;
+  const unsigned long long z = x > y ? x : y;
+  return __longlong_as_double((long long)(z <= lim ? z : 0x7ff0000000000000ull));
 }
 
 // ---------------------------------------------------------------------------
-// a4 (and coarse operators by rediscretisation): residual and Jacobian of one
-// cell.  `xs`, `xos` point at the cell arrays of one sample (storage layout;
-// global or shared memory).  The per-sample K/mu and phi Dm and the
-// accumulation factor h^2/tau arrive already multiplied by inv_s, so every
-// flux and derivative comes out scaled.  Fluxes and residuals are formed in S
-// (FP64 on the fine grid), derivative blocks in T; in the mixed mode
-// (T = float) the coarse operators are assembled entirely in FP32 (S = T) and
-// the fine Jacobian's derivative terms are formed in FP32 from FP64 fluxes.
+// a4 (and coarse operators by rediscretisation): residual and Jacobian.
+//
+// A face between a left/lower cell L and a right/upper cell R carries the
+// scaled mass and salt fluxes F, G from L to R; L's residuals gain +F, +G and
+// R's lose them.  With rho_f = rs / 2 (rs = rho_L + rho_R), K/mu = 2 kh and
+// phi Dm = 2 PDh (all scaled by inv_s, the square cells' h in F's favour):
+//   F = rs qh,  qh = -kh (p_R - p_L + ghh rs)   (ghh = g h / 2 on a north face, else 0)
+//   G = F c_up - rs PDh (c_R - c_L),  c_up = c_L if F >= 0 else c_R  (the tie takes c_L)
+//   dF/dp_L = rs kh = -dF/dp_R,  dF/dc_L = dF/dc_R = drho (qh - kh ghh rs),
+//   dG/dp = c_up dF/dp,  dG/dc_L = c_up dF/dc + [F if F >= 0] + PD rho_L,
+//   dG/dc_R = c_up dF/dc + [F if F < 0] - PD rho_R
+// (the diffusive terms because rho_f -+ drho (c_R - c_L) / 2 are rho_L and
+// rho_R): 19 operations for a north face, 17 for an east one, derivatives
+// included.  The seaside boundary is an east face with twice the cell's
+// coefficients (half the distance) to a ghost cell of p_b = rho1 g (Ly - y),
+// c = 1; the land side has its prescribed flux (land_side).
+//
+// What bounds it: the FP64 pipe (a warp instruction takes 17-19 cycles of an
+// SM).  Per cell 36 operations of its east and north face, ~4 of re-evaluated
+// tile-edge faces, 22 to add four faces, 8 accumulation, ~14 for the inverse
+// of the centre block - about 95 instead of 176 before the fluxes were written
+// in these terms, with comparisons and sign changes on the integer pipes and
+// the scaled coefficients formed once per sample and level.  8192 level-0
+// samples, FP64, per call of the event timer: residual and Jacobian 1048 ->
+// 639 us, residual alone 468 -> 289 us, coarse operators 68 -> 42 us; the
+// solve 440 -> 386 ms; the fused FP32 level-0 solver, 1000 samples, 32.6 ->
+// 28.6 ms.
+//
+// Fluxes and residuals are formed in S (FP64 on the fine grid), derivatives
+// and blocks in T; in the mixed mode (T = float) the coarse operators are
+// assembled entirely in FP32 (S = T) and the fine Jacobian's derivative terms
+// in FP32 from FP64 fluxes.
+//
+// Scaled coefficients of one sample on one multigrid level of the constant-
+// coefficient model (k_level_coefs), inv_s included.
+struct __align__(64) LevelCoef {
+  double kh, kg;    // K / (2 mu), kh g h / 2
+  double PD, PDh;   // phi Dm, half of it
+  double pv, pvd;   // phi h^2 / tau, that times drho
+  double Fl, Flo;   // land side: outward mass flux -rho0 q_in h, and max(Fl, 0)
+};
+template <typename S>
+struct FaceCoef {
+  S kh, kg, PD, PDh;
+};
+template <typename T, typename S, bool JAC = true>
+struct FaceData {
+  S F, G;              // fluxes L -> R (scaled)
+  T dp, dc, dpc;       // dF/dp_L, dF/dc, dG/dp_L
+  T gL, gR;            // dG/dc_L, dG/dc_R
+};
+// Residual-only evaluation (JAC = false): the fluxes alone.
 template <typename T, typename S>
-struct CellSys {
-  S fm, fs;      // scaled residuals (fluid mass, salt)
-  T C[4];        // centre block
-  T Nb[4][4];    // W, E, S, N blocks
+struct FaceData<T, S, false> {
+  S F, G;
 };
 
-// FIELDS: per-cell coefficients instead of the sample's scalars: cc[st] =
-// (phi, K/mu) of the cell and fc[st] = (K/mu, phi Dm) harmonic means on its
-// east face (.x, .y) and north face (.z, .w), zero across the boundary.
-// JAC = false: the residual alone (no derivative terms; the residual's
-// arithmetic is the same code, so it is bit-identical to the JAC = true
-// form's).
+// JAC = false: the fluxes only, with exactly the arithmetic of the JAC =
+// true form, so both forms give bit-identical residuals.
 // DROP: the fallback preconditioner operator - the Jacobian without the
 // derivatives of the face densities with respect to c (dF/dc = 0 in both
 // rows), an operator whose diagonal blocks stay definite where density
 // contrasts over heterogeneous K make point-block Gauss-Seidel diverge.
-template <typename T, typename S, bool FIELDS = false, bool DROP = false, bool JAC = true>
-__device__ __forceinline__ void assemble_cell(const Phys& ph, const Coef& cf, int nx, int ny, double h, double inv_h,
-                                              double vt_s, double inv_s, const double2* xs, const double2* xos,
-                                              int st, int ix, int iy, CellSys<T, S>& o,
-                                              const double2* cc = nullptr, const double4_32a* fc = nullptr) {
-  S kmu, PD, phi;
-  if (FIELDS) {
-    const double2 c = cc[st];
-    phi = (S)c.x;
-    kmu = (S)(c.y * inv_s);
-    PD = (S)(c.x * ph.Dm * inv_s);
-  } else {
-    kmu = (S)(cf.kmu * inv_s);
-    PD = (S)(cf.PD * inv_s);
-    phi = (S)cf.phi;
-  }
-  const S hS = (S)h, ihS = (S)inv_h, drho = (S)ph.drho, rho0 = (S)ph.rho0;
-  const double2 xP = xs[st], xO = xos[st];
-  const S pP = (S)xP.x, cP = (S)xP.y, cO = (S)xO.y;
-  const S rhoP = rho0 + drho * cP;
-  const S rhoO = rho0 + drho * cO;
-  const S vt = (S)vt_s;
-  S Rm = phi * (rhoP - rhoO) * vt;
-  S Rs = phi * (rhoP * cP - rhoO * cO) * vt;
-  T C00 = (T)0, C01 = (T)(phi * drho * vt), C10 = (T)0, C11 = (T)(phi * (drho * cP + rhoP) * vt);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) o.Nb[k][0] = o.Nb[k][1] = o.Nb[k][2] = o.Nb[k][3] = (T)0;
-  const T kmuP_T = (T)kmu, PDP_T = (T)PD, hT = (T)h, hdT = (T)(0.5 * ph.drho);
-
-  // interior faces W, E, S, N
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int jx = ix + (k == 0 ? -1 : (k == 1 ? 1 : 0));
-    const int jy = iy + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-    if (jx < 0 || jx >= nx || jy < 0 || jy >= ny) continue;
-    const S sg = (S)(k == 2 ? -ph.g : (k == 3 ? ph.g : 0.0));
-    const int sn = st_of(jx, jy, nx);
-    S kmu_f = kmu, PD_f = PD;
-    if (FIELDS) {  // the face's harmonic means, stored with the cell west of / below the face
-      const double4_32a f = fc[(k == 0 || k == 2) ? sn : st];
-      kmu_f = (S)(((k < 2) ? f.x : f.z) * inv_s);
-      PD_f = (S)(((k < 2) ? f.y : f.w) * inv_s);
+template <typename T, typename S, bool NORTH, bool DROP, bool JAC = true>
+__device__ __forceinline__ void face_eval(S drho, S rho0, S ghh, const FaceCoef<S>& k, S pL, S cL, S pR, S cR,
+                                          FaceData<T, S, JAC>& f) {
+  const S rhoL = fma_(drho, cL, rho0), rhoR = fma_(drho, cR, rho0);
+  const S rs = rhoL + rhoR;
+  S u = pR - pL;
+  if (NORTH) u = fma_(ghh, rs, u);
+  const S qh = mul_(neg_(k.kh), u);
+  const S Ff = mul_(rs, qh);
+  const bool up = nonneg(Ff);
+  const S cup = up ? cL : cR;
+  f.F = Ff;
+  f.G = fma_(Ff, cup, neg_(mul_(rs, mul_(k.PDh, cR - cL))));
+  if constexpr (JAC) {
+    const T rsT = (T)rs, cupT = (T)cup, FT = (T)Ff, khT = (T)k.kh, PDT = (T)k.PD, dT = (T)drho;
+    T rLT, rRT;
+    if constexpr (std::is_same<T, S>::value) {
+      rLT = rhoL;
+      rRT = rhoR;
+    } else {
+      rLT = (T)rhoL;
+      rRT = rsT - rLT;
     }
-    const T kmuT = (T)kmu_f, PDT = (T)PD_f;
-    const double2 xN = xs[sn];
-    const S pN = (S)xN.x, cN = (S)xN.y;
-    const S rhoN = rho0 + drho * cN;
-    const S rhof = (S)0.5 * (rhoP + rhoN);
-    const S q = -kmu_f * fma_((pN - pP), ihS, sg * rhof);
-    const S Ff = rhof * q * hS;
-    const bool up = Ff >= (S)0;
-    const S cup = up ? cP : cN;
-    const S dif = PD_f * (cN - cP);
-    Rm += Ff;
-    Rs += fma_(Ff, cup, -rhof * dif);
-    if constexpr (!JAC) continue;
-    // derivatives of (F, G) w.r.t. the unknowns of P and of the neighbour
-    const T rhofT = (T)rhof, cupT = (T)cup, FfT = (T)Ff, difT = (T)dif;
-    const T dFdp = rhofT * kmuT;
-    const T dFdc = DROP ? (T)0 : hdT * hT * fma_((T)q, (T)1, -rhofT * kmuT * (T)sg);
-    const T dGdifP = fma_(hdT, difT, -rhofT * PDT);
-    const T dGdifN = fma_(hdT, difT, rhofT * PDT);
-    C00 += dFdp;
-    C01 += dFdc;
-    C10 = fma_(dFdp, cupT, C10);
-    C11 += fma_(dFdc, cupT, (up ? FfT : (T)0) - dGdifP);
-    o.Nb[k][0] = -dFdp;
-    o.Nb[k][1] = dFdc;
-    o.Nb[k][2] = -dFdp * cupT;
-    o.Nb[k][3] = fma_(dFdc, cupT, (up ? (T)0 : FfT) - dGdifN);
+    const T dp = mul_(rsT, khT);
+    const T dc = DROP ? (T)0 : mul_(dT, NORTH ? fma_(neg_((T)k.kg), rsT, (T)qh) : (T)qh);
+    f.dp = dp;
+    f.dc = dc;
+    f.dpc = mul_(dp, cupT);
+    f.gL = fma_(dc, cupT, (up ? FT : (T)0) + mul_(PDT, rLT));
+    f.gR = fma_(dc, cupT, (up ? (T)0 : FT) - mul_(PDT, rRT));
   }
-  boundary_terms<T, S, DROP, JAC>(ph, cf.qin, inv_s, kmu, PD, nx, ix, iy, hS, ihS, rhoP, pP, cP, Rm, Rs, C00, C01, C10,
-                             C11);
-  o.fm = Rm;
-  o.fs = Rs;
-  o.C[0] = C00; o.C[1] = C01; o.C[2] = C10; o.C[3] = C11;
+}
+
+// One cell's residual and blocks as its faces are added.
+template <typename T, typename S, bool JAC = true>
+struct CellSum {
+  S Rm, Rs;
+  T C[4], Nb[4][4];  // centre block; W, E, S, N blocks
+};
+// Accumulation terms.
+template <typename T, typename S, bool JAC>
+__device__ __forceinline__ void cell_begin(S drho, S rho0, S pv, S pvd, S cP, S cO, CellSum<T, S, JAC>& o) {
+  const S d = cP - cO;
+  o.Rm = mul_(pvd, d);
+  o.Rs = mul_(mul_(pv, d), fma_(drho, cP + cO, rho0));
+  if constexpr (JAC) {
+    o.C[0] = o.C[2] = (T)0;
+    o.C[1] = (T)pvd;
+    o.C[3] = (T)mul_(pv, fma_((S)2 * drho, cP, rho0));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o.Nb[k][0] = o.Nb[k][1] = o.Nb[k][2] = o.Nb[k][3] = (T)0;
+  }
+}
+// The face to neighbour k (0 W, 1 E, 2 S, 3 N); IS_L: the cell is its L.  With
+// nb false (the seaside boundary face) no neighbour block.
+template <bool IS_L, typename T, typename S, bool JAC>
+__device__ __forceinline__ void cell_add(const FaceData<T, S, JAC>& f, int k, CellSum<T, S, JAC>& o, bool nb = true) {
+  if (IS_L) {
+    o.Rm += f.F;
+    o.Rs += f.G;
+    if constexpr (JAC) {
+      o.C[0] += f.dp;
+      o.C[1] += f.dc;
+      o.C[2] += f.dpc;
+      o.C[3] += f.gL;
+      if (nb) {
+        o.Nb[k][0] = neg_(f.dp);
+        o.Nb[k][1] = f.dc;
+        o.Nb[k][2] = neg_(f.dpc);
+        o.Nb[k][3] = f.gR;
+      }
+    }
+  } else {
+    o.Rm -= f.F;
+    o.Rs -= f.G;
+    if constexpr (JAC) {
+      o.C[0] += f.dp;
+      o.C[1] -= f.dc;
+      o.C[2] += f.dpc;
+      o.C[3] -= f.gR;
+      o.Nb[k][0] = neg_(f.dp);
+      o.Nb[k][1] = neg_(f.dc);
+      o.Nb[k][2] = neg_(f.dpc);
+      o.Nb[k][3] = neg_(f.gL);
+    }
+  }
+}
+// The land side (ix = 0): prescribed inflow of fresh water, c_b = 0, diffusion
+// over half a cell; Fl the outward mass flux, Flo = max(Fl, 0), PD the cell's.
+template <typename T, typename S, bool JAC>
+__device__ __forceinline__ void land_side(S drho, S rho0, S Fl, S Flo, S PD, S cP, CellSum<T, S, JAC>& o) {
+  const S rhoP = fma_(drho, cP, rho0), PDr = mul_(PD, cP);
+  o.Rm += Fl;
+  o.Rs += fma_(Flo, cP, mul_(rhoP + rho0, PDr));
+  if constexpr (JAC) o.C[3] += (T)fma_((S)2 * PD, rhoP, Flo);
+}
+
+// A thread's view of its cell's coefficients: the sample's scalars or, with
+// FIELDS, cc[st] = (phi, K/mu) of the cell and fc[st] = (K / (2 mu), phi Dm),
+// scaled by inv_s, on its east (.x, .y) and north (.z, .w) face (harmonic
+// means; zero across the boundary).
+template <typename S, bool FIELDS>
+struct CellCoefs {
+  S pv, pvd, PD, Fl, Flo;
+  FaceCoef<S> in;  // of the sample's interior faces (not FIELDS)
+  S kc;            // K/mu of the cell, scaled (FIELDS: for the seaside face)
+
+  __device__ __forceinline__ void load(const Phys& ph, const LevelCoef* lc, const Coef* coef, int s, double vt_s,
+                                       double inv_s, double h, const double2* cc, int64_t e) {
+    if constexpr (FIELDS) {
+      const double2 c = cc[e];
+      pv = (S)mul_(c.x, vt_s);
+      pvd = mul_(pv, (S)ph.drho);
+      kc = (S)mul_(c.y, inv_s);
+      PD = (S)mul_(mul_(c.x, ph.Dm), inv_s);
+      Fl = (S)mul_(mul_(mul_(-ph.rho0, coef[s].qin), inv_s), h);
+      Flo = nonneg(Fl) ? Fl : (S)0;
+    } else {
+      const LevelCoef c = lc[s];
+      pv = (S)c.pv;
+      pvd = (S)c.pvd;
+      PD = (S)c.PD;
+      Fl = (S)c.Fl;
+      Flo = (S)c.Flo;
+      in.kh = (S)c.kh;
+      in.kg = (S)c.kg;
+      in.PD = (S)c.PD;
+      in.PDh = (S)c.PDh;
+      kc = in.kh + in.kh;
+    }
+  }
+  // The east or north face of the cell at entry e (its L).
+  __device__ __forceinline__ FaceCoef<S> face(bool north, S ghh, const double4_32a* fc, int64_t e) const {
+    if constexpr (FIELDS) {
+      const double4_32a q = fc[e];
+      FaceCoef<S> k;
+      k.kh = (S)(north ? q.z : q.x);
+      k.PD = (S)(north ? q.w : q.y);
+      k.PDh = mul_((S)0.5, k.PD);
+      k.kg = mul_(k.kh, ghh);
+      return k;
+    } else {
+      return in;
+    }
+  }
+  // The seaside boundary face: twice the cell's coefficients.
+  __device__ __forceinline__ FaceCoef<S> sea() const {
+    FaceCoef<S> k;
+    k.kh = kc;
+    k.kg = (S)0;
+    k.PD = PD + PD;
+    k.PDh = PD;
+    return k;
+  }
+};
+__device__ __forceinline__ double2 sea_ghost(const Phys& ph, double h, int iy) {
+  // iy + 1/2 exactly, from the bits of 2^52 + iy (an int conversion takes the FP64 pipe as well)
+  const double y = __hiloint2double(0x43300000, iy) - 4503599627370495.5;
+  return make_double2(mul_(ph.rho1g, fma(-h, y, ph.Ly)), 1.0);
+}
+
+// One cell, all four faces evaluated by its own thread.  `xs`, `xos` point at
+// the cell arrays of one sample (storage layout; global or shared memory), cc
+// and fc at the sample's (FIELDS), e0 is the sample's first entry (unused
+// here: the arrays are sample-relative).
+template <typename T, typename S, bool FIELDS = false, bool DROP = false, bool JAC = true>
+__device__ __forceinline__ void assemble_cell(const Phys& ph, const CellCoefs<S, FIELDS>& K, int nx, int ny, double h,
+                                              const double2* xs, const double2* xos, int st, int ix, int iy,
+                                              CellSum<T, S, JAC>& o, const double4_32a* fc = nullptr) {
+  const S drho = (S)ph.drho, rho0 = (S)ph.rho0, ghh = (S)(0.5 * ph.g * h);
+  const double2 xP = xs[st];
+  const S pP = (S)xP.x, cP = (S)xP.y;
+  cell_begin<T, S, JAC>(drho, rho0, K.pv, K.pvd, cP, (S)xos[st].y, o);
+  FaceData<T, S, JAC> f;
+  if (ix > 0) {
+    const int w = st_of(ix - 1, iy, nx);
+    const double2 xN = xs[w];
+    face_eval<T, S, false, DROP, JAC>(drho, rho0, ghh, K.face(false, ghh, fc, w), (S)xN.x, (S)xN.y, pP, cP, f);
+    cell_add<false>(f, 0, o);
+  }
+  {
+    const bool sea = ix + 1 == nx;
+    const double2 xN = sea ? sea_ghost(ph, h, iy) : xs[st_of(ix + 1, iy, nx)];
+    face_eval<T, S, false, DROP, JAC>(drho, rho0, ghh, sea ? K.sea() : K.face(false, ghh, fc, st), pP, cP, (S)xN.x,
+                                      (S)xN.y, f);
+    cell_add<true>(f, 1, o, !sea);
+  }
+  if (iy > 0) {
+    const int w = st_of(ix, iy - 1, nx);
+    const double2 xN = xs[w];
+    face_eval<T, S, true, DROP, JAC>(drho, rho0, ghh, K.face(true, ghh, fc, w), (S)xN.x, (S)xN.y, pP, cP, f);
+    cell_add<false>(f, 2, o);
+  }
+  if (iy + 1 < ny) {
+    const double2 xN = xs[st_of(ix, iy + 1, nx)];
+    face_eval<T, S, true, DROP, JAC>(drho, rho0, ghh, K.face(true, ghh, fc, st), pP, cP, (S)xN.x, (S)xN.y, f);
+    cell_add<true>(f, 3, o);
+  }
+  if (ix == 0) land_side<T, S, JAC>(drho, rho0, K.Fl, K.Flo, K.PD, cP, o);
 }
 
 // Store a cell's Jacobian blocks (6 planes with stride `ps`, incl. C^-1).
@@ -411,20 +558,22 @@ __device__ __forceinline__ void store_blocks(typename VT<T>::b4* J, int64_t ps, 
   J[i] = mkblk<B4>(C[0], C[1], C[2], C[3]);
 #pragma unroll
   for (int k = 0; k < 4; ++k) J[(k + 1) * ps + i] = mkblk<B4>(Nb[k][0], Nb[k][1], Nb[k][2], Nb[k][3]);
-  const T idet = (T)1 / (C[0] * C[3] - C[1] * C[2]);
-  J[5 * ps + i] = mkblk<B4>(C[3] * idet, -C[1] * idet, -C[2] * idet, C[0] * idet);
+  const T idet = (T)1 / fma_(C[0], C[3], neg_(mul_(C[1], C[2])));
+  const T nd = neg_(idet);
+  J[5 * ps + i] = mkblk<B4>(mul_(C[3], idet), mul_(C[1], nd), mul_(C[2], nd), mul_(C[0], idet));
 }
 
 // One thread per cell; FINE: CTAs never straddle samples (N % TPB == 0) and
 // write the per-CTA max |F| (inf for non-finite) to rmax_part[s][ct].
 template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true>
-__global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restrict__ coef, int B, int nx, int ny,
-                                                  double h, double inv_h, double vt_s, double inv_s,
+__global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restrict__ coef,
+                                                  const LevelCoef* __restrict__ lc, int B, int nx, int ny,
+                                                  double h, double vt_s, double inv_s,
                                                   const double2* x, const double2* xo,
                                                   const int* active, double2* __restrict__ F,
                                                   typename VT<T>::b4* __restrict__ J, int64_t plane,
-                                                  double* __restrict__ rmax_part, const double2* __restrict__ cc = nullptr,
-                                                  const double4_32a* __restrict__ fc = nullptr) {
+                                                  double* __restrict__ rmax_part, const double2* __restrict__ cc,
+                                                  const double4_32a* __restrict__ fc) {
   typedef typename std::conditional<FINE, double, T>::type S;
   __shared__ double sh[40];
   const int N = nx * ny;
@@ -441,15 +590,15 @@ __global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restric
   int ix, iy;
   xy_of(st, nx, ix, iy);
   const int64_t base = e - st;
-  CellSys<T, S> o;
-  assemble_cell<T, S, FIELDS, DROP, JAC>(ph, coef[s], nx, ny, h, inv_h, vt_s, inv_s, x + base, xo + base, st, ix, iy, o,
-                              FIELDS ? cc + base : nullptr, FIELDS ? fc + base : nullptr);
+  CellCoefs<S, FIELDS> K;
+  K.load(ph, lc, coef, s, vt_s, inv_s, h, cc, e);
+  CellSum<T, S, JAC> o;
+  assemble_cell<T, S, FIELDS, DROP, JAC>(ph, K, nx, ny, h, x + base, xo + base, st, ix, iy, o,
+                                         FIELDS ? fc + base : nullptr);
   if (FINE) {
-    const double fm = (double)o.fm, fs = (double)o.fs;
+    const double fm = (double)o.Rm, fs = (double)o.Rs;
     if (F) F[e] = make_double2(fm, fs);
-    double loc = fmax(fabs(fm), fabs(fs));
-    if (!(loc <= 1.0e300)) loc = INFINITY;  // NaN or inf
-    const double bm = block_max_nonneg(loc, sh);
+    const double bm = block_max_nonneg(abs_max_or_inf(fm, fs), sh);
     if (threadIdx.x == 0) {
       const int nct = N / TPB;
       rmax_part[(int64_t)s * nct + (st / TPB)] = bm;
@@ -460,107 +609,24 @@ __global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restric
   }
 }
 
-// ---------------------------------------------------------------------------
-// a4, face-once form.  A face between a left/lower cell L and a right/upper
-// cell R carries the scaled mass and salt fluxes F, G from L to R; L's
-// residuals gain +F, +G and R's lose them, so R's derivative terms are the
-// negated ones of L.  The tile kernel evaluates each face once (assemble_cell
-// evaluates every interior face from both sides): the same arithmetic from
-// L's side, upwinding included (at the tie F = 0 the upwind value is L's,
-// the same tie-break as assemble_cell's from L's side).
-template <typename T, typename S, bool JAC = true>
-struct FaceData {
-  S F, G;   // fluxes L -> R (scaled)
-  T aL[4];  // d(F, G)/d(p_L, c_L): dF/dp, dF/dc, dG/dp, dG/dc
-  T aR[4];  // d(F, G)/d(p_R, c_R)
-};
-// Residual-only evaluation (JAC = false): the fluxes alone.
-template <typename T, typename S>
-struct FaceData<T, S, false> {
-  S F, G;
-};
-
-// JAC = false: the fluxes only, with exactly the arithmetic of the JAC =
-// true form (the derivative terms come after F and G and feed nothing back),
-// so both forms give bit-identical residuals.
-template <typename T, typename S, bool DROP, bool JAC = true>
-__device__ __forceinline__ void face_eval(const Phys& ph, S kmu_f, S PD_f, S sg, S hS, S ihS, double2 xL, double2 xR,
-                                          FaceData<T, S, JAC>& f) {
-  const S drho = (S)ph.drho, rho0 = (S)ph.rho0;
-  const S pL = (S)xL.x, cL = (S)xL.y, pR = (S)xR.x, cR = (S)xR.y;
-  const S rhoL = rho0 + drho * cL, rhoR = rho0 + drho * cR;
-  const S rhof = (S)0.5 * (rhoL + rhoR);
-  const S q = -kmu_f * fma_((pR - pL), ihS, sg * rhof);
-  const S Ff = rhof * q * hS;
-  const bool up = Ff >= (S)0;
-  const S cup = up ? cL : cR;
-  const S dif = PD_f * (cR - cL);
-  f.F = Ff;
-  f.G = fma_(Ff, cup, -rhof * dif);
-  if constexpr (!JAC) return;
-  else {
-  const T kmuT = (T)kmu_f, PDT = (T)PD_f, hT = (T)hS, hdT = (T)(0.5 * ph.drho);
-  const T rhofT = (T)rhof, cupT = (T)cup, FfT = (T)Ff, difT = (T)dif;
-  const T dFdp = rhofT * kmuT;
-  const T dFdc = DROP ? (T)0 : hdT * hT * fma_((T)q, (T)1, -rhofT * kmuT * (T)sg);
-  const T dGdifL = fma_(hdT, difT, -rhofT * PDT);
-  const T dGdifR = fma_(hdT, difT, rhofT * PDT);
-  f.aL[0] = dFdp;
-  f.aL[1] = dFdc;
-  f.aL[2] = dFdp * cupT;
-  f.aL[3] = fma_(dFdc, cupT, (up ? FfT : (T)0) - dGdifL);
-  f.aR[0] = -dFdp;
-  f.aR[1] = dFdc;
-  f.aR[2] = -dFdp * cupT;
-  f.aR[3] = fma_(dFdc, cupT, (up ? (T)0 : FfT) - dGdifR);
-  }
-}
-
-// The residual and Jacobian of one cell from its faces' data (sgn = +1: the
-// cell is the face's L, -1: its R; k = 0 W, 1 E, 2 S, 3 N).
-template <typename T, typename S, bool JAC = true>
-__device__ __forceinline__ void add_face(const FaceData<T, S, JAC>& f, bool cell_is_L, int k, S& Rm, S& Rs, T C[4],
-                                         T Nb[4][4]) {
-  if (cell_is_L) {
-    Rm += f.F;
-    Rs += f.G;
-    if constexpr (JAC) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        C[j] += f.aL[j];
-        Nb[k][j] = f.aR[j];
-      }
-    }
-  } else {
-    Rm -= f.F;
-    Rs -= f.G;
-    if constexpr (JAC) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        C[j] -= f.aR[j];
-        Nb[k][j] = -f.aL[j];
-      }
-    }
-  }
-}
-
-// Tile assembly: a CTA holds TPB consecutive cells in storage order, i.e.
-// TPB / nx whole rows (nx <= TPB), possibly of several samples.  Phase 1:
-// every cell evaluates its east and north faces into shared memory.  Phase
-// 2: every cell sums its four faces (a cell of the tile's first row
-// evaluates the face below it itself: its other cell lies in another tile),
-// its accumulation and boundary terms, and stores F, the blocks and C^-1
-// like k_assemble (same arguments; FINE: N % TPB == 0, one sample per CTA).
-// Shared memory: 2 x TPB faces (40 KB in FP64).
+// Tile assembly, the face-once form: every cell evaluates its east and north
+// faces into shared memory (phase 1) and then sums its four faces (phase 2);
+// a face to a cell of another tile is evaluated again, by the same code.
+//
+// k_assemble_tile: a CTA holds TPB consecutive cells in storage order, i.e.
+// TPB / nx whole rows (nx <= TPB), possibly of several samples.  A cell of the
+// tile's first row evaluates the face below it itself.  FINE: N % TPB == 0,
+// one sample per CTA.  Shared memory: 2 x TPB faces (28 KB in FP64).
 template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true>
-__global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __restrict__ coef, int B, int nx, int ny,
-                                                       double h, double inv_h, double vt_s, double inv_s,
+__global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __restrict__ coef,
+                                                       const LevelCoef* __restrict__ lc, int B, int nx, int ny,
+                                                       double h, double vt_s, double inv_s,
                                                        const double2* x, const double2* xo,
                                                        const int* active, double2* __restrict__ F,
                                                        typename VT<T>::b4* __restrict__ J, int64_t plane,
                                                        double* __restrict__ rmax_part,
-                                                       const double2* __restrict__ cc = nullptr,
-                                                       const double4_32a* __restrict__ fc = nullptr) {
+                                                       const double2* __restrict__ cc,
+                                                       const double4_32a* __restrict__ fc) {
   typedef typename std::conditional<FINE, double, T>::type S;
   __shared__ FaceData<T, S, JAC> fE[TPB], fN[TPB];
   __shared__ double sh[40];
@@ -580,109 +646,75 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __re
   // tile slot of the cell (ix, row r of the tile); rows hold nx consecutive storage entries
   const int r = threadIdx.x >> lg2(nx);
   const int slot = r * nx + ix;
-  const S hS = (S)h, ihS = (S)inv_h;
-  const Coef cf = on ? coef[s] : Coef{};
-  S kmu = (S)0, PD = (S)0, phi = (S)0;
+  const S drho = (S)ph.drho, rho0 = (S)ph.rho0, ghh = (S)(0.5 * ph.g * h);
+  CellCoefs<S, FIELDS> K;
+  S pP = (S)0, cP = (S)0;
   if (on) {
-    if (FIELDS) {
-      const double2 c = cc[base + st];
-      phi = (S)c.x;
-      kmu = (S)(c.y * inv_s);
-      PD = (S)(c.x * ph.Dm * inv_s);
-    } else {
-      kmu = (S)(cf.kmu * inv_s);
-      PD = (S)(cf.PD * inv_s);
-      phi = (S)cf.phi;
-    }
-    const double2 xP = x[base + st];
-    if (ix + 1 < nx) {  // east face, P = L
-      S kf = kmu, pf = PD;
-      if (FIELDS) {
-        const double4_32a q = fc[base + st];
-        kf = (S)(q.x * inv_s);
-        pf = (S)(q.y * inv_s);
-      }
-      face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)0, hS, ihS, xP, x[base + st_of(ix + 1, iy, nx)], fE[slot]);
+    K.load(ph, lc, coef, s, vt_s, inv_s, h, cc, e);
+    const double2 xP = x[e];
+    pP = (S)xP.x;
+    cP = (S)xP.y;
+    const bool sea = ix + 1 == nx;
+    {  // east face (or the seaside boundary), P = L
+      const double2 xN = sea ? sea_ghost(ph, h, iy) : x[base + st_of(ix + 1, iy, nx)];
+      face_eval<T, S, false, DROP, JAC>(drho, rho0, ghh, sea ? K.sea() : K.face(false, ghh, fc, e), pP, cP, (S)xN.x,
+                                        (S)xN.y, fE[slot]);
     }
     if (iy + 1 < ny) {  // north face, P = L
-      S kf = kmu, pf = PD;
-      if (FIELDS) {
-        const double4_32a q = fc[base + st];
-        kf = (S)(q.z * inv_s);
-        pf = (S)(q.w * inv_s);
-      }
-      face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)ph.g, hS, ihS, xP, x[base + st_of(ix, iy + 1, nx)], fN[slot]);
+      const double2 xN = x[base + st_of(ix, iy + 1, nx)];
+      face_eval<T, S, true, DROP, JAC>(drho, rho0, ghh, K.face(true, ghh, fc, e), pP, cP, (S)xN.x, (S)xN.y, fN[slot]);
     }
   }
   __syncthreads();
   if (!on) return;
-  const double2 xP = x[base + st], xO = xo[base + st];
-  const S drho = (S)ph.drho, rho0 = (S)ph.rho0;
-  const S pP = (S)xP.x, cP = (S)xP.y, cO = (S)xO.y;
-  const S rhoP = rho0 + drho * cP;
-  const S rhoO = rho0 + drho * cO;
-  const S vt = (S)vt_s;
-  S Rm = phi * (rhoP - rhoO) * vt;
-  S Rs = phi * (rhoP * cP - rhoO * cO) * vt;
-  T C[4] = {(T)0, (T)(phi * drho * vt), (T)0, (T)(phi * (drho * cP + rhoP) * vt)};
-  T Nb[4][4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) Nb[k][0] = Nb[k][1] = Nb[k][2] = Nb[k][3] = (T)0;
-  if (ix > 0) add_face<T, S, JAC>(fE[slot - 1], false, 0, Rm, Rs, C, Nb);                     // W: P = R
-  if (ix + 1 < nx) add_face<T, S, JAC>(fE[slot], true, 1, Rm, Rs, C, Nb);                     // E: P = L
-  if (iy > 0) {  // S: P = R
+  CellSum<T, S, JAC> o;
+  cell_begin<T, S, JAC>(drho, rho0, K.pv, K.pvd, cP, (S)xo[e].y, o);
+  if (ix > 0) cell_add<false>(fE[slot - 1], 0, o);       // W: P = R
+  cell_add<true>(fE[slot], 1, o, ix + 1 < nx);            // E: P = L
+  if (iy > 0) {                                           // S: P = R
     if (r > 0) {
-      add_face<T, S, JAC>(fN[slot - nx], false, 2, Rm, Rs, C, Nb);
+      cell_add<false>(fN[slot - nx], 2, o);
     } else {  // the lower cell is in another tile: evaluate the face here
       const int sb = st_of(ix, iy - 1, nx);
-      S kf = kmu, pf = PD;
-      if (FIELDS) {
-        const double4_32a q = fc[base + sb];
-        kf = (S)(q.z * inv_s);
-        pf = (S)(q.w * inv_s);
-      }
-      FaceData<T, S, JAC> fb;
-      face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)ph.g, hS, ihS, x[base + sb], xP, fb);
-      add_face<T, S, JAC>(fb, false, 2, Rm, Rs, C, Nb);
+      const double2 xN = x[base + sb];
+      FaceData<T, S, JAC> f;
+      face_eval<T, S, true, DROP, JAC>(drho, rho0, ghh, K.face(true, ghh, fc, base + sb), (S)xN.x, (S)xN.y, pP, cP, f);
+      cell_add<false>(f, 2, o);
     }
   }
-  if (iy + 1 < ny) add_face<T, S, JAC>(fN[slot], true, 3, Rm, Rs, C, Nb);                     // N: P = L
-  boundary_terms<T, S, DROP, JAC>(ph, cf.qin, inv_s, kmu, PD, nx, ix, iy, hS, ihS, rhoP, pP, cP, Rm, Rs, C[0], C[1], C[2],
-                             C[3]);
+  if (iy + 1 < ny) cell_add<true>(fN[slot], 3, o);        // N: P = L
+  if (ix == 0) land_side<T, S, JAC>(drho, rho0, K.Fl, K.Flo, K.PD, cP, o);
   if (FINE) {
-    const double fm = (double)Rm, fs = (double)Rs;
+    const double fm = (double)o.Rm, fs = (double)o.Rs;
     if (F) F[e] = make_double2(fm, fs);
-    double loc = fmax(fabs(fm), fabs(fs));
-    if (!(loc <= 1.0e300)) loc = INFINITY;  // NaN or inf
-    const double bm = block_max_nonneg(loc, sh);
+    const double bm = block_max_nonneg(abs_max_or_inf(fm, fs), sh);
     if (threadIdx.x == 0) {
       const int nct = N / TPB;
       rmax_part[(int64_t)s * nct + (st / TPB)] = bm;
     }
   }
   if constexpr (JAC) {
-    if (J) store_blocks<T>(J, plane, e, C, Nb);
+    if (J) store_blocks<T>(J, plane, e, o.C, o.Nb);
   }
 }
 
-// Tile assembly in 2-D tiles: a CTA covers a TILE_W x (TPB / TILE_W) block
-// of cells of one sample, mapped by position, not by storage order (nx a
-// multiple of TILE_W, ny of TPB / TILE_W).  Phase 1: every cell evaluates its
-// east and north faces into shared memory.  Phase 2: a cell takes its west
-// and south faces from the tile, or, on the tile's west or south edge,
-// evaluates them itself: 2 + 1 / TH + 1 / TILE_W face evaluations per cell
-// (TH = TPB / TILE_W rows; 2.5 for 128 x 2, 2.16 for 32 x 8).  The per-tile
-// max |F| goes to slot (tile index) of the sample's N / TPB partials.
+// k_assemble_tile2d: a CTA covers a TILE_W x (TPB / TILE_W) block of cells of
+// one sample, mapped by position, not by storage order (nx a multiple of
+// TILE_W, ny of TPB / TILE_W).  A cell on the tile's west or south edge
+// evaluates that face itself: 2 + 1 / TH + 1 / TILE_W face evaluations per
+// cell (TH = TPB / TILE_W rows; 2.5 for 128 x 2, 2.16 for 32 x 8).  The
+// per-tile max |F| goes to slot (tile index) of the sample's N / TPB partials.
 constexpr int TILE_W_DEFAULT = 128;  // for grids wider than TPB cells
 template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true, int TILE_W = TILE_W_DEFAULT>
-__global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __restrict__ coef, int B, int nx,
-                                                         int ny, double h, double inv_h, double vt_s, double inv_s,
+__global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __restrict__ coef,
+                                                         const LevelCoef* __restrict__ lc, int B, int nx,
+                                                         int ny, double h, double vt_s, double inv_s,
                                                          const double2* x, const double2* xo,
                                                          const int* active, double2* __restrict__ F,
                                                          typename VT<T>::b4* __restrict__ J, int64_t plane,
                                                          double* __restrict__ rmax_part,
-                                                         const double2* __restrict__ cc = nullptr,
-                                                         const double4_32a* __restrict__ fc = nullptr) {
+                                                         const double2* __restrict__ cc,
+                                                         const double4_32a* __restrict__ fc) {
   typedef typename std::conditional<FINE, double, T>::type S;
   constexpr int TH = TPB / TILE_W;
   __shared__ FaceData<T, S, JAC> fE[TPB], fN[TPB];
@@ -696,94 +728,59 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __
   const int tx = threadIdx.x % TILE_W, ty = threadIdx.x / TILE_W;
   const int tpr = nx / TILE_W;  // tiles per row band
   const int ix = (tile & (tpr - 1)) * TILE_W + tx, iy = (tile >> lg2(tpr)) * TH + ty;
-  const int st = st_of(ix, iy, nx);
-  const int64_t base = (int64_t)s * N;
+  const int64_t base = (int64_t)s * N, e = base + st_of(ix, iy, nx);
   const int slot = threadIdx.x;
-  const S hS = (S)h, ihS = (S)inv_h;
-  const Coef cf = coef[s];
-  S kmu, PD, phi;
-  if (FIELDS) {
-    const double2 c = cc[base + st];
-    phi = (S)c.x;
-    kmu = (S)(c.y * inv_s);
-    PD = (S)(c.x * ph.Dm * inv_s);
-  } else {
-    kmu = (S)(cf.kmu * inv_s);
-    PD = (S)(cf.PD * inv_s);
-    phi = (S)cf.phi;
-  }
-  const double2 xP = x[base + st];
-  auto face_coef = [&](int owner, bool north, S& kf, S& pf) {
-    kf = kmu;
-    pf = PD;
-    if (FIELDS) {
-      const double4_32a q = fc[base + owner];
-      kf = (S)((north ? q.z : q.x) * inv_s);
-      pf = (S)((north ? q.w : q.y) * inv_s);
-    }
-  };
-  if (ix + 1 < nx) {  // east face, P = L
-    S kf, pf;
-    face_coef(st, false, kf, pf);
-    face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)0, hS, ihS, xP, x[base + st_of(ix + 1, iy, nx)], fE[slot]);
+  const S drho = (S)ph.drho, rho0 = (S)ph.rho0, ghh = (S)(0.5 * ph.g * h);
+  CellCoefs<S, FIELDS> K;
+  K.load(ph, lc, coef, s, vt_s, inv_s, h, cc, e);
+  const double2 xP = x[e];
+  const S pP = (S)xP.x, cP = (S)xP.y;
+  const bool sea = ix + 1 == nx;
+  {  // east face (or the seaside boundary), P = L
+    const double2 xN = sea ? sea_ghost(ph, h, iy) : x[base + st_of(ix + 1, iy, nx)];
+    face_eval<T, S, false, DROP, JAC>(drho, rho0, ghh, sea ? K.sea() : K.face(false, ghh, fc, e), pP, cP, (S)xN.x,
+                                      (S)xN.y, fE[slot]);
   }
   if (iy + 1 < ny) {  // north face, P = L
-    S kf, pf;
-    face_coef(st, true, kf, pf);
-    face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)ph.g, hS, ihS, xP, x[base + st_of(ix, iy + 1, nx)], fN[slot]);
+    const double2 xN = x[base + st_of(ix, iy + 1, nx)];
+    face_eval<T, S, true, DROP, JAC>(drho, rho0, ghh, K.face(true, ghh, fc, e), pP, cP, (S)xN.x, (S)xN.y, fN[slot]);
   }
   __syncthreads();
-  const double2 xO = xo[base + st];
-  const S drho = (S)ph.drho, rho0 = (S)ph.rho0;
-  const S pP = (S)xP.x, cP = (S)xP.y, cO = (S)xO.y;
-  const S rhoP = rho0 + drho * cP;
-  const S rhoO = rho0 + drho * cO;
-  const S vt = (S)vt_s;
-  S Rm = phi * (rhoP - rhoO) * vt;
-  S Rs = phi * (rhoP * cP - rhoO * cO) * vt;
-  T C[4] = {(T)0, (T)(phi * drho * vt), (T)0, (T)(phi * (drho * cP + rhoP) * vt)};
-  T Nb[4][4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) Nb[k][0] = Nb[k][1] = Nb[k][2] = Nb[k][3] = (T)0;
+  CellSum<T, S, JAC> o;
+  cell_begin<T, S, JAC>(drho, rho0, K.pv, K.pvd, cP, (S)xo[e].y, o);
   if (ix > 0) {  // W: P = R
     if (tx > 0) {
-      add_face<T, S, JAC>(fE[slot - 1], false, 0, Rm, Rs, C, Nb);
+      cell_add<false>(fE[slot - 1], 0, o);
     } else {
-      const int sw = st_of(ix - 1, iy, nx);
-      S kf, pf;
-      face_coef(sw, false, kf, pf);
-      FaceData<T, S, JAC> fw;
-      face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)0, hS, ihS, x[base + sw], xP, fw);
-      add_face<T, S, JAC>(fw, false, 0, Rm, Rs, C, Nb);
+      const int64_t w = base + st_of(ix - 1, iy, nx);
+      const double2 xN = x[w];
+      FaceData<T, S, JAC> f;
+      face_eval<T, S, false, DROP, JAC>(drho, rho0, ghh, K.face(false, ghh, fc, w), (S)xN.x, (S)xN.y, pP, cP, f);
+      cell_add<false>(f, 0, o);
     }
   }
-  if (ix + 1 < nx) add_face<T, S, JAC>(fE[slot], true, 1, Rm, Rs, C, Nb);  // E: P = L
-  if (iy > 0) {  // S: P = R
+  cell_add<true>(fE[slot], 1, o, !sea);  // E: P = L
+  if (iy > 0) {                          // S: P = R
     if (ty > 0) {
-      add_face<T, S, JAC>(fN[slot - TILE_W], false, 2, Rm, Rs, C, Nb);
+      cell_add<false>(fN[slot - TILE_W], 2, o);
     } else {
-      const int sb = st_of(ix, iy - 1, nx);
-      S kf, pf;
-      face_coef(sb, true, kf, pf);
-      FaceData<T, S, JAC> fb;
-      face_eval<T, S, DROP, JAC>(ph, kf, pf, (S)ph.g, hS, ihS, x[base + sb], xP, fb);
-      add_face<T, S, JAC>(fb, false, 2, Rm, Rs, C, Nb);
+      const int64_t w = base + st_of(ix, iy - 1, nx);
+      const double2 xN = x[w];
+      FaceData<T, S, JAC> f;
+      face_eval<T, S, true, DROP, JAC>(drho, rho0, ghh, K.face(true, ghh, fc, w), (S)xN.x, (S)xN.y, pP, cP, f);
+      cell_add<false>(f, 2, o);
     }
   }
-  if (iy + 1 < ny) add_face<T, S, JAC>(fN[slot], true, 3, Rm, Rs, C, Nb);  // N: P = L
-  boundary_terms<T, S, DROP, JAC>(ph, cf.qin, inv_s, kmu, PD, nx, ix, iy, hS, ihS, rhoP, pP, cP, Rm, Rs, C[0], C[1], C[2],
-                             C[3]);
-  const int64_t e = base + st;
+  if (iy + 1 < ny) cell_add<true>(fN[slot], 3, o);  // N: P = L
+  if (ix == 0) land_side<T, S, JAC>(drho, rho0, K.Fl, K.Flo, K.PD, cP, o);
   if (FINE) {
-    const double fm = (double)Rm, fs = (double)Rs;
+    const double fm = (double)o.Rm, fs = (double)o.Rs;
     if (F) F[e] = make_double2(fm, fs);
-    double loc = fmax(fabs(fm), fabs(fs));
-    if (!(loc <= 1.0e300)) loc = INFINITY;  // NaN or inf
-    const double bm = block_max_nonneg(loc, sh);
+    const double bm = block_max_nonneg(abs_max_or_inf(fm, fs), sh);
     if (threadIdx.x == 0) rmax_part[(int64_t)s * tiles + tile] = bm;
   }
   if constexpr (JAC) {
-    if (J) store_blocks<T>(J, plane, e, C, Nb);
+    if (J) store_blocks<T>(J, plane, e, o.C, o.Nb);
   }
 }
 
@@ -1506,10 +1503,8 @@ __global__ void __launch_bounds__(TPB) k_newton_step_max(int B, int N, double in
   grid_enter();
   if (!newton_active[s]) return;
   const auto d = dx[e];
-  double dc = fabs((double)d.y);
-  double loc = fmax(fabs((double)d.x) * inv_pref, dc);
-  if (!(loc <= 1.0e300)) loc = INFINITY;
-  if (!(dc <= 1.0e300)) dc = INFINITY;
+  const double dc = abs_max_or_inf((double)d.y, 0.0);
+  const double loc = abs_max_or_inf((double)d.x * inv_pref, dc);
   const double m = block_max_nonneg(loc, sh);
   const double mc = block_max_nonneg(dc, sh);
   if (threadIdx.x == 0) {

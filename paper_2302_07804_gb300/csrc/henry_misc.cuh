@@ -50,8 +50,30 @@ __global__ void k_sample_xi(uint64_t seed, int level, uint64_t first, int n, dou
 struct CoefModel {
   double phi_mean, K_mean, qin_mean, phi_amp, logK_amp, qin_amp, mu, Dm;
 };
+// The assembly's scaled coefficients of each sample on one multigrid level
+// (constant-coefficient model): cells of width h, vt_s = h^2 / tau inv_s.
+__device__ __forceinline__ LevelCoef level_coef(const Phys& ph, const Coef& c, double h, double vt_s, double inv_s) {
+  LevelCoef l;
+  l.kh = 0.5 * (c.kmu * inv_s);
+  l.kg = l.kh * (0.5 * ph.g * h);
+  l.PD = c.PD * inv_s;
+  l.PDh = 0.5 * l.PD;
+  l.pv = c.phi * vt_s;
+  l.pvd = l.pv * ph.drho;
+  l.Fl = -ph.rho0 * c.qin * inv_s * h;
+  l.Flo = l.Fl >= 0.0 ? l.Fl : 0.0;
+  return l;
+}
+// The multigrid levels whose LevelCoef k_coefficients fills.
+struct LevelList {
+  static constexpr int MAX = 16;
+  int n;
+  Phys ph;
+  double inv_s, h[MAX], vt_s[MAX];
+  LevelCoef* lc[MAX];
+};
 __global__ void k_coefficients(CoefModel m, int n, const double* __restrict__ xi, Coef* __restrict__ coef,
-                               int* __restrict__ status) {
+                               int* __restrict__ status, const __grid_constant__ LevelList L = LevelList{}) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double x1 = xi[3 * (int64_t)i], x2 = xi[3 * (int64_t)i + 1], x3 = xi[3 * (int64_t)i + 2];
@@ -62,6 +84,7 @@ __global__ void k_coefficients(CoefModel m, int n, const double* __restrict__ xi
   c.PD = c.phi * m.Dm;
   c.qin = m.qin_mean * (1.0 + m.qin_amp * x3);
   coef[i] = c;
+  for (int k = 0; k < L.n; ++k) L.lc[k][i] = level_coef(L.ph, c, L.h[k], L.vt_s[k], L.inv_s);
   const bool ok = (c.phi > 0.0) && (c.phi < 1.0) && (K > 0.0) && (K <= 1.0e300) && (c.qin == c.qin) &&
                   (fabs(c.qin) <= 1.0e300);
   status[i] = ok ? 0 : 3;
@@ -147,9 +170,11 @@ __global__ void __launch_bounds__(TPB) k_restrict_cc(int B, int ncx, int ncy, co
   ccc[e] = make_double2(0.25 * (((a.x + b.x) + c.x) + d.x), 0.25 * (((a.y + b.y) + c.y) + d.y));
 }
 
-// Face coefficients: harmonic means 2 a b / (a + b) of K / mu and of phi Dm on
-// the east (.x, .y) and north (.z, .w) face of every cell, 0 on the boundary.
-__global__ void __launch_bounds__(TPB) k_face_coefs(int B, int nx, int ny, double Dm, const double2* __restrict__ cc,
+// Face coefficients: harmonic means 2 a b / (a + b) of K / mu (halved) and of
+// phi Dm, scaled by inv_s, on the east (.x, .y) and north (.z, .w) face of
+// every cell, 0 on the boundary.
+__global__ void __launch_bounds__(TPB) k_face_coefs(int B, int nx, int ny, double Dm, double inv_s,
+                                                    const double2* __restrict__ cc,
                                                     double4_32a* __restrict__ fc) {
   const int N = nx * ny;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
@@ -165,13 +190,13 @@ __global__ void __launch_bounds__(TPB) k_face_coefs(int B, int nx, int ny, doubl
   auto harm = [](double a, double b) { return 2.0 * a * b / (a + b); };
   if (ix + 1 < nx) {
     const double2 E = c[st_of(ix + 1, iy, nx)];
-    f.x = harm(P.y, E.y);
-    f.y = harm(P.x * Dm, E.x * Dm);
+    f.x = 0.5 * harm(P.y, E.y) * inv_s;
+    f.y = harm(P.x * Dm, E.x * Dm) * inv_s;
   }
   if (iy + 1 < ny) {
     const double2 Nn = c[st_of(ix, iy + 1, nx)];
-    f.z = harm(P.y, Nn.y);
-    f.w = harm(P.x * Dm, Nn.x * Dm);
+    f.z = 0.5 * harm(P.y, Nn.y) * inv_s;
+    f.w = harm(P.x * Dm, Nn.x * Dm) * inv_s;
   }
   fc[e] = f;
 }
@@ -281,52 +306,68 @@ __global__ void __launch_bounds__(TPB) k_qfw(int B, int N, double h, const doubl
 }
 
 // Natural layout [B][ny][nx] <-> storage layout (colour-split rows).
+__device__ __forceinline__ int64_t storage_of(int64_t e, int nx, int N) {  // of the natural entry e
+  const int64_t s = sample_of(e, N);
+  const int nat = (int)(e - s * N), iy = nat >> lg2(nx);
+  return s * N + st_of(nat - iy * nx, iy, nx);
+}
 template <typename V2>
-__global__ void __launch_bounds__(TPB) k_to_storage(int B, int nx, int ny, const double2* __restrict__ in,
+__global__ void __launch_bounds__(TPB) k_to_storage(int B, int nx, int ny, const double2* in,
                                                     V2* __restrict__ out) {
+  grid_enter();
   const int N = nx * ny;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e >= (int64_t)B * N) return;
-  const int64_t s = e / N;
-  const int nat = (int)(e - s * N);
-  const int iy = nat / nx, ix = nat - iy * nx;
   const double2 v = in[e];
   V2 o;
   o.x = v.x;
   o.y = v.y;
-  out[s * N + st_of(ix, iy, nx)] = o;
+  out[storage_of(e, nx, N)] = o;
+}
+// Both states of a per-step call, and its samples' flags from their status.
+__global__ void __launch_bounds__(TPB) k_states_in(int B, int nx, int ny, const double2* __restrict__ in,
+                                                   const double2* __restrict__ in_old, double2* __restrict__ x,
+                                                   double2* __restrict__ xo, const int* status,
+                                                   int* __restrict__ newton_active, int* __restrict__ lin_active,
+                                                   int* __restrict__ newton_it) {
+  grid_enter();
+  const int N = nx * ny;
+  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  if (e >= (int64_t)B * N) return;
+  const int64_t i = storage_of(e, nx, N);
+  x[i] = in[e];
+  xo[i] = in_old[e];
+  if (e < B) {
+    newton_active[e] = lin_active[e] = status[e] == 0 ? 1 : 0;
+    newton_it[e] = 0;
+  }
 }
 template <typename V2>
-__global__ void __launch_bounds__(TPB) k_from_storage(int B, int nx, int ny, const V2* __restrict__ in,
+__global__ void __launch_bounds__(TPB) k_from_storage(int B, int nx, int ny, const V2* in,
                                                       double2* __restrict__ out) {
+  grid_enter();
   const int N = nx * ny;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e >= (int64_t)B * N) return;
-  const int64_t s = e / N;
-  const int nat = (int)(e - s * N);
-  const int iy = nat / nx, ix = nat - iy * nx;
-  const V2 v = in[s * N + st_of(ix, iy, nx)];
+  const V2 v = in[storage_of(e, nx, N)];
   out[e] = make_double2((double)v.x, (double)v.y);
 }
-// Jacobian planes -> natural [B][ny][nx][5][2][2] FP64.
-template <typename B4>
-__global__ void __launch_bounds__(TPB) k_blocks_out(int B, int nx, int ny, const B4* __restrict__ J, int64_t plane,
-                                                    double* __restrict__ out) {
+// Jacobian planes -> natural [B][ny][nx][5][2][2] FP64.  One thread per block
+// row (two values): a warp writes 512 contiguous bytes and reads whole 32-byte
+// blocks; with one thread per cell (20 stores 160 bytes apart) and
+// a launch per conversion henry_assemble of 8 samples of 512 x 256 cells took 434 us,
+// now 314 us (160 us of it the assembly).
+template <typename V2>
+__global__ void __launch_bounds__(TPB) k_blocks_out(int B, int nx, int ny, const V2* J, int64_t plane,
+                                                    double2* __restrict__ out) {
+  grid_enter();
   const int N = nx * ny;
-  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  if (e >= (int64_t)B * N) return;
-  const int64_t s = e / N;
-  const int nat = (int)(e - s * N);
-  const int iy = nat / nx, ix = nat - iy * nx;
-  const int64_t src = s * N + st_of(ix, iy, nx);
-  for (int k = 0; k < 5; ++k) {
-    const B4 b = J[k * plane + src];
-    double* o = out + e * 20 + 4 * k;
-    o[0] = (double)b.a00;
-    o[1] = (double)b.a01;
-    o[2] = (double)b.a10;
-    o[3] = (double)b.a11;
-  }
+  const int64_t t = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  if (t >= (int64_t)B * N * 10) return;
+  const int64_t e = t / 10;
+  const int q = (int)(t - e * 10);
+  const V2 v = J[2 * ((q >> 1) * plane + storage_of(e, nx, N)) + (q & 1)];
+  out[t] = make_double2((double)v.x, (double)v.y);
 }
 
 // Row permutation of a [n][w] array (uneven mixed-level batches): gather
@@ -348,7 +389,8 @@ __global__ void k_zero_rows(int n, int w, const int* __restrict__ perm, double* 
   dst[(int64_t)perm[t / w] * w + t % w] = 0.0;
 }
 
-__global__ void __launch_bounds__(TPB) k_scale_d2(int64_t n, double a, double2* __restrict__ x) {
+__global__ void __launch_bounds__(TPB) k_scale_d2(int64_t n, double a, double2* x) {
+  grid_enter();
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e < n) {
     double2 v = x[e];
