@@ -177,13 +177,14 @@ typedef struct {
                             sample (and at most 2048, 64 x 32) down to the coarsest run as one kernel, one CTA
                             per sample with those levels' vectors in shared memory and their operators in
                             registers and shared memory (FP64 from 64 x 32 cells reads that level's operator
-                            from global memory at each use); -1 (default): 2048 cells (64 x 32) with FP32
-                            linear algebra on fine grids of 128 x 64 cells or more, else 128 (16 x 8), the
-                            faster choice measured on the MLMC levels' batches; 0: every level as separate
-                            kernels.  Same values either way */
+                            from global memory at each use); -1 (default): with FP32 linear algebra from 64 x
+                            32 cells, a fine grid of that size included (32 x 16 fine grids: up to 1024
+                            samples, else 128 cells); with FP64 512 cells (32 x 16) up to 304 samples, that
+                            fine grid included up to 152, else 128 (16 x 8), the faster choices measured; 0:
+                            every level as separate kernels.  Same values either way */
   int32_t mg_tail_batch_cells; /* ... only while the batch times that level's cells per sample is at most this
-                                  (default 2^20; 0: no limit): large batches of small grids run those levels
-                                  as separate, large launches */
+                                  (default 2^20; 0: no limit): larger batches run those levels as separate,
+                                  large launches.  The default start with FP32 linear algebra has no limit */
   int32_t scheme; /* HENRY_SCHEME_CELL (default) or HENRY_SCHEME_VERTEX */
   int32_t newton_jacobian_every; /* Newton assembles the Jacobian and the coarse operators at
                                     iterations 0, k, 2k, ... of a time step and reuses them in between (chord
@@ -200,8 +201,8 @@ typedef struct {
                               contracts multiply-adds per call site, and tile-edge faces are evaluated
                               at another call site) */
   int32_t mg_threads; /* threads per CTA of the multigrid smoother, restriction and prolongation kernels of
-                         the cell-centred scheme: 64, 128, 256 or 512 (0, the default: 256).  Identical
-                         values for every size */
+                         the cell-centred scheme: 64, 128, 256 or 512; 0 (default): 256, and 64 or 128 for
+                         small FP64 launches.  Identical values for every size */
   int32_t newton_predictor_order; /* Newton's first iterate of step n+1 (with weight newton_predictor): 1
                                      linear extrapolation from x^n and x^{n-1}; 2 (default) quadratic, x^n +
                                      w (2 (x^n - x^{n-1}) - (x^{n-1} - x^{n-2})), from step 2 on (linear at

@@ -463,6 +463,19 @@ void with_preload(int64_t threads, F&& f) {
   else f(std::false_type());
 }
 
+// CTA size of the multigrid kernels where mg_threads leaves it open.  Small FP64
+// launches take small CTAs: an SM's FP64 pipe needs 19 cycles for a warp
+// instruction, so a launch of few CTAs is faster on more SMs (against 256
+// threads everywhere: level 2 with partners, 33 samples, 206 -> 193 ms; two-
+// layer level 1, 50 samples, 55.6 -> 51.2 ms; level 0, 64 samples, 18.8 -> 18.0
+// ms).  FP32 launches gain nothing (level 3, 20 samples: 311 ms either way; 64
+// threads up to the PRELOAD_THREADS line: 319 ms).
+template <typename T>
+int mg_cta(int mg_threads, int64_t threads) {
+  if (mg_threads || sizeof(T) == sizeof(float)) return mg_threads;
+  return threads <= PRELOAD_THREADS / 4 ? 64 : (threads <= PRELOAD_THREADS ? 128 : TPB);
+}
+
 // Runs f(std::integral_constant<int, NT>{}) for the multigrid kernels' CTA
 // size nt: 64, 128, 256 or 512 threads (anything else: TPB).
 template <typename F>
@@ -803,30 +816,65 @@ int restrict_states(henry_handle* H, Group<T>& G, int B, bool old, const int* ac
   return HENRY_OK;
 }
 
-// First multigrid level of the fused tail: the first coarse level (k >= 1)
-// with at most mg_tail_cells cells per sample, and at most 2048 (-1: 2048 with
-// FP32 linear algebra on fine grids of 128 x 64 cells or more, else 128, as
-// measured), if the batch is small enough (B x cells of that level <=
-// mg_tail_batch_cells; larger batches keep those levels as separate kernels,
-// which then are large launches and fill the FP64 pipe better than the tail's
-// partly idle warps); -1: no tail.
-// Measured per launch with the two-threads-per-cell kernel (henry_tail.cuh)
-// against the one-thread-per-cell one it replaced, by event timer: FP64 from
-// 16 x 8 cells 42.4 -> 18.6 us (64 samples) and 404 -> 182 us (8192 samples);
-// FP32 from 64 x 32 cells 54.9 -> 18.7 us (2 samples), 55 -> 21 us (20 to 50
-// samples).  Level-0 FP64 solves: 37.4 -> 30.3 ms (64 samples), 518 -> 445 ms
-// (8192); level 2 with partners, 33 samples: 315 -> 279 ms.
+// Where the fused tail (henry_tail.cuh) starts: the first multigrid level it
+// runs, -1 for no tail.  With mg_tail_cells >= 0: the first coarse level (k >=
+// 1) with at most that many cells per sample, and at most 2048, if the batch is
+// small enough (B x cells of that level <= mg_tail_batch_cells; larger batches
+// keep those levels as separate kernels, which then are large launches).  By
+// default (-1), as measured:
+//  * FP32: from 64 x 32 cells, the whole cycle where that is the fine grid -
+//    the kernel reads a sample's operator once where the separate sweeps read
+//    it nine times - for any batch (level 1 against a tail from 16 x 8: 200
+//    samples 25.9 / 30.4 ms, 884 80.8 / 97.3, 2500 208 / 256; level 2: 500
+//    samples 351 / 368 ms); fine grids of 32 x 16 up to 1024 samples, beyond
+//    that from 16 x 8 (4000 samples: 106 against 116 ms).
+//  * FP64: from 32 x 16 cells while every sample's CTA has an SM or half of
+//    one to itself (its half-sweep there keeps the SM's FP64 pipe busy for
+//    1.5 us; level 1: 300 samples 46.4 against 48.6 ms from 16 x 8), the whole
+//    cycle of a 32 x 16 fine grid up to 152 samples (7.9 against 9.8 ms); else
+//    from 16 x 8 within mg_tail_batch_cells.
+// The kernel itself against the one-thread-per-cell one it replaced, by event
+// timer: FP64 from 16 x 8 cells 42.4 -> 18.6 us (64 samples) and 404 -> 182 us
+// (8192 samples); FP32 from 64 x 32 cells 54.9 -> 18.7 us (2 samples), 55 ->
+// 21 us (20 to 50 samples).
 template <typename T>
 int tail_level(const henry_config& c, const Group<T>& G, int B) {
-  const int cells =
-      c.mg_tail_cells >= 0 ? std::min(c.mg_tail_cells, 2048) : (sizeof(T) == sizeof(float) && G.lv[0].N >= 8192 ? 2048 : 128);
+  const int N0 = G.lv[0].N;
+  int cells = std::min(c.mg_tail_cells, 2048), k0 = 1;
+  bool limit = true;
+  if (cells < 0) {
+    if (sizeof(T) == sizeof(float)) {
+      const bool all = N0 > 512 || B <= 1024;
+      cells = all ? 2048 : 128;
+      k0 = all ? 0 : 1;
+      limit = !all;
+    } else {
+      cells = B <= 304 ? 512 : 128;
+      k0 = B <= 152 ? 0 : 1;
+    }
+  }
   if (cells <= 0) return -1;
-  for (int k = 1; k < G.K; ++k) {
+  for (int k = k0; k < G.K; ++k) {
     if (G.lv[k].N > cells) continue;
-    if (c.mg_tail_batch_cells > 0 && (double)B * G.lv[k].N > (double)c.mg_tail_batch_cells) return -1;
+    if (limit && c.mg_tail_batch_cells > 0 && (double)B * G.lv[k].N > (double)c.mg_tail_batch_cells) return -1;
     return k;
   }
   return -1;
+}
+
+// Launch one half-sweep of colour col (MODE as in sweep_cell) of a level.
+template <typename T, int MODE>
+void launch_sweep(int mg_threads, int B, const Level& L, int col, const typename VT<T>::b4* J,
+                  const typename VT<T>::v2* b, typename VT<T>::v2* x, const typename VT<T>::v2* xc, const int* act,
+                  cudaStream_t st) {
+  const int64_t hn = (int64_t)B * L.N / 2;  // swept cells
+  with_mg_threads(mg_cta<T>(mg_threads, hn), [&](auto nt) {
+    constexpr int NT = decltype(nt)::value;
+    with_preload(hn, [&](auto pre) {
+      chain(st, nblk(hn, NT), NT, 0, k_sweep<T, MODE, NT, decltype(pre)::value>, B, L.nx, L.ny, col, J, L.plane, b, x,
+            xc, act);
+    });
+  });
 }
 
 // One V(nu1, nu2) cycle: x0 = M^{-1} b0 on the fine level (active = lin_active).
@@ -840,26 +888,18 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
   const double na = H->nact;
   const double b4 = sizeof(B4), v2 = sizeof(V2);
   const int kt = tail_level<T>(H->cfg, G, B);
-  const int kend = kt > 0 ? kt : G.K;  // levels 0 .. kend - 1 run as separate kernels
+  const int kend = kt >= 0 ? kt : G.K;  // levels 0 .. kend - 1 run as separate kernels
   const int mnt = H->cfg.mg_threads;
   for (int k = 0; k < kend; ++k) {
     Level& L = G.lv[k];
     const V2* b = k == 0 ? b0 : (const V2*)L.mgb;
     V2* x = k == 0 ? x0 : (V2*)L.mgx;
     const B4* J = (const B4*)((k == 0 && J0) ? J0 : L.J);
-    const int64_t hn = (int64_t)B * L.N / 2;  // threads per half-sweep
     const double hc = na * L.N / 2;  // swept cells per half-sweep
     const int sm = k == 0 ? HENRY_K_SMOOTH : HENRY_K_SMOOTH_COARSE;
     Level& Lc = G.lv[k + 1];
     auto sweep = [&](int col, auto mode) {
-      constexpr int MODE = decltype(mode)::value;
-      with_mg_threads(mnt, [&](auto nt) {
-        constexpr int NT = decltype(nt)::value;
-        with_preload(hn, [&](auto pre) {
-          chain(st, nblk(hn, NT), NT, 0, k_sweep<T, MODE, NT, decltype(pre)::value>, B, L.nx, L.ny, col, J, L.plane, b,
-                x, nullptr, act);
-        });
-      });
+      launch_sweep<T, decltype(mode)::value>(mnt, B, L, col, J, b, x, nullptr, act, st);
     };
     if (nu1 > 0) {
       launch(H, st, sm, hc * (b4 + 2 * v2), na * sweep_flops(L.nx, L.ny, 0),
@@ -872,11 +912,12 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
                  [&] { sweep(col, std::integral_constant<int, 1>()); });
       }
       launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * Lc.N * (10 * b4 + 7 * v2), na * restrict_flops(L.nx, L.ny), [&] {
-        with_mg_threads(mnt, [&](auto nt) {
+        const int64_t nc = (int64_t)B * Lc.N;
+        with_mg_threads(mg_cta<T>(mnt, nc), [&](auto nt) {
           constexpr int NT = decltype(nt)::value;
-          with_preload((int64_t)B * Lc.N, [&](auto pre) {
-            chain(st, nblk((int64_t)B * Lc.N, NT), NT, 0, k_residual_restrict<T, 0, NT, decltype(pre)::value>, B, Lc.nx,
-                  Lc.ny, J, L.plane, b, x, (V2*)Lc.mgb, act);
+          with_preload(nc, [&](auto pre) {
+            chain(st, nblk(nc, NT), NT, 0, k_residual_restrict<T, 0, NT, decltype(pre)::value>, B, Lc.nx, Lc.ny, J,
+                  L.plane, b, x, (V2*)Lc.mgb, act);
           });
         });
       });
@@ -897,13 +938,13 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
     }
     CKL();
   }
-  if (kt > 0) {  // levels kt .. K: one CTA per sample in shared memory
+  if (kt >= 0) {  // levels kt .. K: one CTA per sample in shared memory
     TailArgs A;
     std::memset(&A, 0, sizeof A);
     double tb = 2.0 * G.lv[kt].N * v2 + 16.0 * sizeof(T), tf = 0.0;
     for (int k = kt; k <= G.K; ++k) {
       const Level& L = G.lv[k];
-      A.J[k - kt] = L.J;
+      A.J[k - kt] = (k == 0 && J0) ? J0 : L.J;
       A.plane[k - kt] = L.plane;
       tb += 6.0 * L.N * b4;
       if (k < G.K)
@@ -912,8 +953,8 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
                        : 0.0) +
               2 * nu2 * sweep_flops(L.nx, L.ny, 1) + (nu2 > 0 ? L.N : 0);
     }
-    A.b = G.lv[kt].mgb;
-    A.x = G.lv[kt].mgx;
+    A.b = kt == 0 ? (const void*)b0 : G.lv[kt].mgb;
+    A.x = kt == 0 ? (void*)x0 : G.lv[kt].mgx;
     A.ainv = G.Ainv;
     A.active = act;
     A.nu1 = nu1;
@@ -938,18 +979,10 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
     const V2* b = k == 0 ? b0 : (const V2*)L.mgb;
     V2* x = k == 0 ? x0 : (V2*)L.mgx;
     const B4* J = (const B4*)((k == 0 && J0) ? J0 : L.J);
-    const int64_t hn = (int64_t)B * L.N / 2;
     const double hc = na * L.N / 2;
     const int sm = k == 0 ? HENRY_K_SMOOTH : HENRY_K_SMOOTH_COARSE;
     auto sweep = [&](int col, auto mode) {
-      constexpr int MODE = decltype(mode)::value;
-      with_mg_threads(mnt, [&](auto nt) {
-        constexpr int NT = decltype(nt)::value;
-        with_preload(hn, [&](auto pre) {
-          chain(st, nblk(hn, NT), NT, 0, k_sweep<T, MODE, NT, decltype(pre)::value>, B, L.nx, L.ny, col, J, L.plane, b,
-                x, MODE == 2 ? (const V2*)Lc.mgx : nullptr, act);
-        });
-      });
+      launch_sweep<T, decltype(mode)::value>(mnt, B, L, col, J, b, x, (const V2*)Lc.mgx, act, st);
     };
     if (nu2 > 0) {
       launch(H, st, sm, hc * (5 * b4 + 3.5 * v2), na * (sweep_flops(L.nx, L.ny, 1) + L.N),
