@@ -161,9 +161,8 @@ typedef struct {
   int32_t adj_maxit; /* henry_adjoint: BiCGStab iteration cap of each adjoint solve (default 200) */
   int32_t cuda_graphs; /* 1 (default): each implicit step (Newton and BiCGStab loops included, as conditional
                           nodes) is captured once per workspace, batch size and settings into a CUDA graph
-                          and replayed without host synchronisation (vertex-centred scheme: each BiCGStab
-                          iteration's body); 0: plain launches driven by the host.  Same values either way;
-                          off while profiling */
+                          and replayed without host synchronisation; 0: plain launches driven by the host.
+                          Same values either way; off while profiling */
   int32_t qoi_set;     /* HENRY_QOI_* (default STANDARD); sets other than STANDARD use the multi-kernel path */
   int32_t tile_assembly; /* 1 (default): face-once assembly in tiles of 256 cells (whole rows up to 256 cells
                             wide, else 128 x 2 blocks), every face inside a tile evaluated once; 0: every
@@ -181,7 +180,8 @@ typedef struct {
                             32 cells, a fine grid of that size included (32 x 16 fine grids: up to 1024
                             samples, else 128 cells); with FP64 512 cells (32 x 16) up to 304 samples, that
                             fine grid included up to 152, else 128 (16 x 8), the faster choices measured; 0:
-                            every level as separate kernels.  Same values either way */
+                            every level as separate kernels.  The vertex-centred scheme's tail starts at 32 x
+                            16 elements unless this is 0.  Same values either way */
   int32_t mg_tail_batch_cells; /* ... only while the batch times that level's cells per sample is at most this
                                   (default 2^20; 0: no limit): larger batches run those levels as separate,
                                   large launches.  The default start with FP32 linear algebra has no limit */

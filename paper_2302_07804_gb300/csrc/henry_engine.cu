@@ -27,7 +27,6 @@
 #include <map>
 #include <string>
 #include <thread>
-#include <tuple>
 #include <vector>
 
 #include "henry.h"
@@ -39,6 +38,7 @@
 #include "henry_adjoint.cuh"
 #include "henry_vc.cuh"
 #include "henry_vc_solve.cuh"
+#include "henry_vc_tail.cuh"
 
 using namespace hk;
 
@@ -251,7 +251,8 @@ struct VcGroup {
   unsigned long long* totals;
   LinScal* sc;
   T* Ainv;
-  std::map<std::tuple<int, int, int>, cudaGraphExec_t> gexec;  // (B, nu1, nu2)
+  std::map<std::string, cudaGraphExec_t> gexec;  // as Group's
+  bool graphs = true;
   void drop_graphs() {
     for (auto& kv : gexec) cudaGraphExecDestroy(kv.second);
     gexec.clear();
@@ -1088,8 +1089,8 @@ struct GraphBuild {
 // here).  Captured on the handle's own stream, of st's priority (capturing the
 // legacy default stream is not allowed; capture executes nothing).
 constexpr size_t MAX_GRAPHS = 16;
-template <typename T, typename F>
-int run_graph(henry_handle* H, Group<T>& G, int B, const std::string& what, cudaStream_t st, F&& emit) {
+template <typename GRP, typename F>
+int run_graph(henry_handle* H, GRP& G, int B, const std::string& what, cudaStream_t st, F&& emit) {
   std::string key = what;
   key.append(reinterpret_cast<const char*>(&B), sizeof B);
   key.append(reinterpret_cast<const char*>(&H->cfg), sizeof H->cfg);
@@ -1123,17 +1124,64 @@ int run_graph(henry_handle* H, Group<T>& G, int B, const std::string& what, cuda
 }
 // Graphs are used unless the configuration says no, the workspace may not
 // allocate (instantiation would) or the kernel timer brackets every launch.
-template <typename T>
-bool graphs_on(const henry_handle* H, const Group<T>& G) {
+template <typename GRP>
+bool graphs_on(const henry_handle* H, const GRP& G) {
   return H->cfg.cuda_graphs && G.graphs && !H->prof.on;
 }
 
+// The BiCGStab loop over a solver D's pieces - init(stream, loop words), head
+// (iteration, its index in device memory, stream), body(samples, stream) - on
+// group D::G.
+template <typename D>
+struct KrylovDrive {
+  D& d() { return static_cast<D&>(*this); }
+  // As nodes of a graph.
+  int emit(GraphBuild& b) {
+    auto& G = d().G;
+    cudaGraphConditionalHandle h;
+    int rc = b.handle(&h);
+    if (rc) return rc;
+    auto test = [&](cudaStream_t s) {
+      const int r = d().head(0, G.counter + 3, s);
+      chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 1, G.counter + 3);
+      return r;
+    };
+    rc = b.seg([&](cudaStream_t s) {
+      const int r = d().init(s, G.counter + 1);
+      return r ? r : test(s);
+    });
+    GraphBuild it;
+    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &it);
+    if (!rc)
+      rc = it.seg([&](cudaStream_t s) {
+        const int r = d().body(d().B, s);
+        return r ? r : test(s);
+      });
+    return rc;
+  }
+  // Driven from the host.
+  int run(cudaStream_t st) {
+    auto& G = d().G;
+    henry_handle* H = d().H;
+    int rc = d().init(st, nullptr);
+    for (int it = 0; !rc && it <= d().maxit; ++it) {
+      CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
+      rc = d().head(it, nullptr, st);
+      int n_act = 0;
+      if (!rc) rc = read_counter(H, G.counter + 1, st, &n_act);
+      if (rc || n_act == 0) return rc;
+      H->nact = n_act;
+      rc = d().body(n_act, st);
+    }
+    return rc;
+  }
+};
+
 // BiCGStab on the fine level for the samples with lin_active set; right-hand
 // side -F; solution in G.dx.  Jpre0: fine operator of the preconditioner
-// (NULL: the Jacobian).  The pieces of the loop, and the loop as nodes of a
-// graph.
+// (NULL: the Jacobian).
 template <typename T>
-struct Krylov {
+struct Krylov : KrylovDrive<Krylov<T>> {
   typedef typename VT<T>::v2 V2;
   typedef typename VT<T>::b4 B4;
   henry_handle* H;
@@ -1211,43 +1259,6 @@ struct Krylov {
     CKL();
     return HENRY_OK;
   }
-  // The whole solve as nodes of a graph.
-  int emit(GraphBuild& b) {
-    cudaGraphConditionalHandle h;
-    int rc = b.handle(&h);
-    if (rc) return rc;
-    auto test = [&](cudaStream_t s) {
-      const int r = head(0, G.counter + 3, s);
-      chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 1, G.counter + 3);
-      return r;
-    };
-    rc = b.seg([&](cudaStream_t s) {
-      const int r = init(s, G.counter + 1);
-      return r ? r : test(s);
-    });
-    GraphBuild it;
-    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &it);
-    if (!rc)
-      rc = it.seg([&](cudaStream_t s) {
-        const int r = body(B, s);
-        return r ? r : test(s);
-      });
-    return rc;
-  }
-  // The whole solve driven from the host.
-  int run(cudaStream_t st) {
-    int rc = init(st, nullptr);
-    for (int it = 0; !rc && it <= maxit; ++it) {
-      CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
-      rc = head(it, nullptr, st);
-      int n_act = 0;
-      if (!rc) rc = read_counter(H, G.counter + 1, st, &n_act);
-      if (rc || n_act == 0) return rc;
-      H->nact = n_act;
-      rc = body(n_act, st);
-    }
-    return rc;
-  }
 };
 
 // rtol / maxit > 0 override the configuration's lin_rtol / lin_maxit.
@@ -1262,12 +1273,12 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
   what.append(reinterpret_cast<const char*>(&Jpre0), sizeof Jpre0);
   what.append(reinterpret_cast<const char*>(&rt), sizeof rt);
   what.append(reinterpret_cast<const char*>(&mi), sizeof mi);
-  return run_graph<T>(H, G, B, what, st, [&](GraphBuild& b) { return k.emit(b); });
+  return run_graph(H, G, B, what, st, [&](GraphBuild& b) { return k.emit(b); });
 }
 
-// One implicit-Euler step (Sec. 2.3) of the B samples of a group: the state
-// x^n in lv[0].x (and x^{n-1} in lv[0].xo, for the predictor) becomes x^{n+1},
-// with Newton iterations as described at the top of this file.
+// Newton's loop over a step D's pieces - start, evaluate(residual first, count,
+// stream), operators, krylov / solve(fallback), mark_retry and retry_operators
+// where retries(), update - on group D::G.
 //
 // Newton's choices (the same in both drives): the Jacobian and the coarse
 // operators are assembled at iterations 0, k, 2k, ... of the step, k =
@@ -1278,8 +1289,142 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
 // and the Jacobian is assembled only for the samples that go on iterating
 // (the residual is recomputed with it, bit-identically).  The FP64 residual
 // test decides convergence.
+template <typename D>
+struct NewtonDrive {
+  int jac_every, res_from;  // newton_jacobian_every; newton_residual_first (< 0: never)
+  explicit NewtonDrive(const henry_config& c)
+      : jac_every(std::max(1, c.newton_jacobian_every)), res_from(c.newton_residual_first) {}
+  D& d() { return static_cast<D&>(*this); }
+  bool jac_at(int it) const { return it % jac_every == 0; }
+  bool res_first_at(int it, bool jac_now) const { return !jac_now || (res_from >= 0 && it >= res_from); }
+
+  // --- host-driven
+  int run(cudaStream_t st) {
+    D& n = d();
+    henry_handle* H = n.H;
+    auto& G = n.G;
+    const henry_config& c = n.c;
+    int rc = n.start(st);
+    int last_jac = -1;
+    bool force_jac = false;
+    for (int it = 0; !rc && it <= c.newton_maxit; ++it) {
+      const bool jac_now = force_jac || last_jac < 0 || it - last_jac >= jac_every;
+      const bool res_first = res_first_at(it, jac_now);
+      CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
+      rc = n.evaluate(res_first, G.counter, st);
+      int n_act = 0;
+      if (!rc) rc = read_counter(H, G.counter, st, &n_act);
+      if (rc || n_act == 0) return rc;
+      H->nact = n_act;
+      if (jac_now) {
+        rc = n.operators(res_first, st);
+        if (rc) return rc;
+        last_jac = it;
+        force_jac = false;
+      }
+      rc = n.solve(false, st);
+      if (!rc && n.retries()) {
+        CK(cudaMemsetAsync(G.counter + 2, 0, sizeof(int), st));
+        rc = n.mark_retry(st);
+        int n_retry = 0;
+        if (!rc) rc = read_counter(H, G.counter + 2, st, &n_retry);
+        if (!rc && n_retry > 0) {
+          H->nact = n_retry;
+          rc = n.retry_operators(st);
+          if (!rc) rc = n.solve(true, st);
+          force_jac = true;
+        }
+      }
+      H->nact = n_act;
+      if (!rc) rc = n.update(n_act, st);
+    }
+    return rc;
+  }
+
+  // --- as a graph
+  // From this iteration on the pattern of evaluations repeats every jac_every
+  // iterations.
+  int steady() const { return res_from <= 0 ? 0 : ((res_from + jac_every - 1) / jac_every) * jac_every; }
+  // Whether the step can run as one graph: few iterations before the steady
+  // pattern, and no retries that would shift a chord pattern.
+  bool graphable() { return steady() <= 6 && jac_every <= 8 && !(d().retries() && jac_every > 1); }
+  int emit_work(GraphBuild& b, int it) {
+    D& n = d();
+    auto& G = n.G;
+    int rc = HENRY_OK;
+    if (jac_at(it)) rc = b.seg([&](cudaStream_t s) { return n.operators(res_first_at(it, true), s); });
+    if (!rc) rc = n.krylov(false).emit(b);
+    if (!rc && n.retries()) {
+      cudaGraphConditionalHandle h;
+      rc = b.handle(&h);
+      if (!rc)
+        rc = b.seg([&](cudaStream_t s) {
+          const int r = n.mark_retry(s);
+          chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 2, (int*)nullptr);
+          return r;
+        });
+      GraphBuild r;
+      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &r);
+      if (!rc) rc = r.seg([&](cudaStream_t s) { return n.retry_operators(s); });
+      if (!rc) rc = n.krylov(true).emit(r);
+    }
+    return rc ? rc : b.seg([&](cudaStream_t s) { return n.update(n.B, s); });
+  }
+  // Iteration `it`: evaluate, then set the conditions h1 (and h2) to whether
+  // any sample goes on.
+  int emit_test(GraphBuild& b, int it, cudaGraphConditionalHandle h1, cudaGraphConditionalHandle h2, int two) {
+    return b.seg([&](cudaStream_t s) {
+      const int r = d().evaluate(res_first_at(it, jac_at(it)), d().G.counter, s);
+      chain(s, 1, 1, 0, k_loop_gate, h1, h2, two, d().G.counter, (int*)nullptr);
+      return r;
+    });
+  }
+  // The iterations from `it` on.  The first two run unconditionally (their
+  // kernels skip samples that have converged; hardly any step is done by
+  // then), the following ones up to the steady pattern inside IF nodes, then
+  // a WHILE node runs jac_every iterations a turn.
+  int emit_from(GraphBuild& b, int it) {
+    const int S = steady();
+    if (it < S && it < 2) {
+      int rc = b.seg([&](cudaStream_t s) { return d().evaluate(res_first_at(it, jac_at(it)), nullptr, s); });
+      if (!rc) rc = emit_work(b, it);
+      return rc ? rc : emit_from(b, it + 1);
+    }
+    cudaGraphConditionalHandle h;
+    int rc = b.handle(&h);
+    if (!rc) rc = emit_test(b, it, h, h, 0);
+    GraphBuild in;
+    if (it < S) {
+      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
+      if (!rc) rc = emit_work(in, it);
+      return rc ? rc : emit_from(in, it + 1);
+    }
+    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &in);
+    return rc ? rc : emit_turn(in, S, 0, h);
+  }
+  // Iterations S + j .. S + jac_every - 1 of a turn of the WHILE node (condition w).
+  int emit_turn(GraphBuild& b, int S, int j, cudaGraphConditionalHandle w) {
+    int rc = emit_work(b, S + j);
+    if (rc) return rc;
+    if (j == jac_every - 1) return emit_test(b, S + j + 1, w, w, 0);
+    cudaGraphConditionalHandle h;
+    rc = b.handle(&h);
+    if (!rc) rc = emit_test(b, S + j + 1, h, w, 1);
+    GraphBuild in;
+    if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
+    return rc ? rc : emit_turn(in, S, j + 1, w);
+  }
+  int emit(GraphBuild& b) {
+    const int rc = b.seg([&](cudaStream_t s) { return d().start(s); });
+    return rc ? rc : emit_from(b, 0);
+  }
+};
+
+// One implicit-Euler step (Sec. 2.3) of the B samples of a group: the state
+// x^n in lv[0].x (and x^{n-1} in lv[0].xo, for the predictor) becomes x^{n+1},
+// with Newton iterations as described at the top of this file.
 template <typename T>
-struct NewtonStep {
+struct NewtonStep : NewtonDrive<NewtonStep<T>> {
   typedef typename VT<T>::b4 B4;
   typedef typename VT<T>::v2 V2;
   henry_handle* H;
@@ -1292,17 +1437,14 @@ struct NewtonStep {
   int64_t n0;
   double inv_tau, inv_s, inv_pref;
   double* pmax;
-  int jac_every, res_from;  // newton_jacobian_every; newton_residual_first (< 0: never)
 
   NewtonStep(henry_handle* h, Group<T>& g, int b)
-      : H(h), G(g), B(b), c(h->cfg), lg(geom(h->cfg, g.level)), L(g.lv[0]), N(g.lv[0].N),
+      : NewtonDrive<NewtonStep<T>>(h->cfg), H(h), G(g), B(b), c(h->cfg), lg(geom(h->cfg, g.level)), L(g.lv[0]), N(g.lv[0].N),
         n0((int64_t)b * g.lv[0].N) {
     inv_tau = 1.0 / lg.tau;
     inv_s = 1.0 / (c.rho0 * lg.h * lg.h * inv_tau);
     inv_pref = 1.0 / (c.rho0 * c.g * c.Ly);
     pmax = G.part + P_MAX * (int64_t)B * G.nct;
-    jac_every = std::max(1, c.newton_jacobian_every);
-    res_from = c.newton_residual_first;
   }
   bool retries() const { return G.Jp && c.lin_retry; }
   // Step start: old states and Newton's first iterate (the predictor is used
@@ -1345,8 +1487,8 @@ struct NewtonStep {
     CKL();
     return HENRY_OK;
   }
-  bool jac_at(int it) const { return it % jac_every == 0; }
-  bool res_first_at(int it, bool jac_now) const { return !jac_now || (res_from >= 0 && it >= res_from); }
+  Krylov<T> krylov(bool fallback) { return Krylov<T>(H, G, B, fallback ? G.Jp : nullptr, c.lin_rtol, c.lin_maxit); }
+  int solve(bool fallback, cudaStream_t st) { return linear_solve<T>(H, G, B, st, fallback ? G.Jp : nullptr); }
   // The evaluation of an iteration and its residual test; `count` (nullable):
   // the samples that go on are added to it.
   int evaluate(bool res_first, int* count, cudaStream_t st) {
@@ -1393,121 +1535,6 @@ struct NewtonStep {
     CKL();
     return HENRY_OK;
   }
-
-  // --- host-driven
-  int run(cudaStream_t st) {
-    int rc = start(st);
-    int last_jac = -1;
-    bool force_jac = false;
-    for (int it = 0; !rc && it <= c.newton_maxit; ++it) {
-      const bool jac_now = force_jac || last_jac < 0 || it - last_jac >= jac_every;
-      const bool res_first = res_first_at(it, jac_now);
-      CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
-      rc = evaluate(res_first, G.counter, st);
-      int n_act = 0;
-      if (!rc) rc = read_counter(H, G.counter, st, &n_act);
-      if (rc || n_act == 0) return rc;
-      H->nact = n_act;
-      if (jac_now) {
-        rc = operators(res_first, st);
-        if (rc) return rc;
-        last_jac = it;
-        force_jac = false;
-      }
-      rc = linear_solve<T>(H, G, B, st);
-      if (!rc && retries()) {
-        CK(cudaMemsetAsync(G.counter + 2, 0, sizeof(int), st));
-        rc = mark_retry(st);
-        int n_retry = 0;
-        if (!rc) rc = read_counter(H, G.counter + 2, st, &n_retry);
-        if (!rc && n_retry > 0) {
-          H->nact = n_retry;
-          rc = retry_operators(st);
-          if (!rc) rc = linear_solve<T>(H, G, B, st, G.Jp);
-          force_jac = true;
-        }
-      }
-      H->nact = n_act;
-      if (!rc) rc = update(n_act, st);
-    }
-    return rc;
-  }
-
-  // --- as a graph
-  // From this iteration on the pattern of evaluations repeats every jac_every
-  // iterations.
-  int steady() const { return res_from <= 0 ? 0 : ((res_from + jac_every - 1) / jac_every) * jac_every; }
-  // Whether the step can run as one graph: few iterations before the steady
-  // pattern, and no retries that would shift a chord pattern.
-  bool graphable() const { return steady() <= 6 && jac_every <= 8 && !(retries() && jac_every > 1); }
-  int emit_work(GraphBuild& b, int it) {
-    int rc = HENRY_OK;
-    if (jac_at(it)) rc = b.seg([&](cudaStream_t s) { return operators(res_first_at(it, true), s); });
-    if (!rc) rc = Krylov<T>(H, G, B, nullptr, c.lin_rtol, c.lin_maxit).emit(b);
-    if (!rc && retries()) {
-      cudaGraphConditionalHandle h;
-      rc = b.handle(&h);
-      if (!rc)
-        rc = b.seg([&](cudaStream_t s) {
-          const int r = mark_retry(s);
-          chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 2, (int*)nullptr);
-          return r;
-        });
-      GraphBuild r;
-      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &r);
-      if (!rc) rc = r.seg([&](cudaStream_t s) { return retry_operators(s); });
-      if (!rc) rc = Krylov<T>(H, G, B, G.Jp, c.lin_rtol, c.lin_maxit).emit(r);
-    }
-    return rc ? rc : b.seg([&](cudaStream_t s) { return update(B, s); });
-  }
-  // Iteration `it`: evaluate, then set the conditions h1 (and h2) to whether
-  // any sample goes on.
-  int emit_test(GraphBuild& b, int it, cudaGraphConditionalHandle h1, cudaGraphConditionalHandle h2, int two) {
-    return b.seg([&](cudaStream_t s) {
-      const int r = evaluate(res_first_at(it, jac_at(it)), G.counter, s);
-      chain(s, 1, 1, 0, k_loop_gate, h1, h2, two, G.counter, (int*)nullptr);
-      return r;
-    });
-  }
-  // The iterations from `it` on.  The first two run unconditionally (their
-  // kernels skip samples that have converged; hardly any step is done by
-  // then), the following ones up to the steady pattern inside IF nodes, then
-  // a WHILE node runs jac_every iterations a turn.
-  int emit_from(GraphBuild& b, int it) {
-    const int S = steady();
-    if (it < S && it < 2) {
-      int rc = b.seg([&](cudaStream_t s) { return evaluate(res_first_at(it, jac_at(it)), nullptr, s); });
-      if (!rc) rc = emit_work(b, it);
-      return rc ? rc : emit_from(b, it + 1);
-    }
-    cudaGraphConditionalHandle h;
-    int rc = b.handle(&h);
-    if (!rc) rc = emit_test(b, it, h, h, 0);
-    GraphBuild in;
-    if (it < S) {
-      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
-      if (!rc) rc = emit_work(in, it);
-      return rc ? rc : emit_from(in, it + 1);
-    }
-    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &in);
-    return rc ? rc : emit_turn(in, S, 0, h);
-  }
-  // Iterations S + j .. S + jac_every - 1 of a turn of the WHILE node (condition w).
-  int emit_turn(GraphBuild& b, int S, int j, cudaGraphConditionalHandle w) {
-    int rc = emit_work(b, S + j);
-    if (rc) return rc;
-    if (j == jac_every - 1) return emit_test(b, S + j + 1, w, w, 0);
-    cudaGraphConditionalHandle h;
-    rc = b.handle(&h);
-    if (!rc) rc = emit_test(b, S + j + 1, h, w, 1);
-    GraphBuild in;
-    if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
-    return rc ? rc : emit_turn(in, S, j + 1, w);
-  }
-  int emit(GraphBuild& b) {
-    const int rc = b.seg([&](cudaStream_t s) { return start(s); });
-    return rc ? rc : emit_from(b, 0);
-  }
 };
 
 // `step` is the step's index.
@@ -1518,7 +1545,7 @@ int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st
   if (rc) return rc;
   if (!graphs_on(H, G) || !n.graphable()) return n.run(st);
   if (step == 0) CK(cudaMemsetAsync(G.counter, 0, 4 * sizeof(int), st));
-  return run_graph<T>(H, G, B, "step", st, [&](GraphBuild& b) { return n.emit(b); });
+  return run_graph(H, G, B, "step", st, [&](GraphBuild& b) { return n.emit(b); });
 }
 
 // Full scenario solves of B samples whose coefficients and status are set.
@@ -1621,6 +1648,14 @@ size_t vc_bytes_per_sample(const henry_config& c, int level) {
 // shared memory with the Jacobian (the per-vertex kernel is used where the
 // device grants less).
 constexpr int VC_TILE_NT = 128;
+template <typename T>
+constexpr int vc_tail_bytes(int nx0) {
+  return vc_tail_smem_v2(nx0) * (int)sizeof(typename VT<T>::v2);
+}
+template <typename T>
+bool vc_tail_fits() {
+  return smem_optin() >= vc_tail_bytes<T>(32);
+}
 bool vc_tile_fits() { return smem_optin() >= vc_tile_smem<true, VC_TILE_NT>() + 1024; }
 template <typename T>
 int ensure_vc_tile_attr() {
@@ -1628,7 +1663,15 @@ int ensure_vc_tile_attr() {
   int dev = 0;
   CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return set_err(HENRY_EINVAL, "device %d outside [0, 64)", dev);
-  if (done[dev].load(std::memory_order_relaxed) || !vc_tile_fits()) return HENRY_OK;
+  if (done[dev].load(std::memory_order_relaxed)) return HENRY_OK;
+  if (vc_tail_fits<T>()) {
+    CK(cudaFuncSetAttribute(k_vc_tail<T, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, vc_tail_bytes<T>(32)));
+    CK(cudaFuncSetAttribute(k_vc_tail<T, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, vc_tail_bytes<T>(16)));
+  }
+  if (!vc_tile_fits()) {
+    done[dev].store(1, std::memory_order_relaxed);
+    return HENRY_OK;
+  }
   CK(cudaFuncSetAttribute(k_vc_assemble_tile<T, true, true, VC_TILE_NT>,
                           cudaFuncAttributeMaxDynamicSharedMemorySize, vc_tile_smem<true, VC_TILE_NT>()));
   CK(cudaFuncSetAttribute(k_vc_assemble_tile<T, false, true, VC_TILE_NT>,
@@ -1647,12 +1690,11 @@ void vc_assemble_launch(const henry_config& c, cudaStream_t st, const VcParams& 
                         int stride, int64_t plane, double inv_s, const double2* x, const double2* xo,
                         const int* active, double2* F, typename VT<T>::b4* J, double* rmax_part) {
   if (vc_use_tile(c))
-    k_vc_assemble_tile<T, FINE, JAC, VC_TILE_NT>
-        <<<nblk((int64_t)B * stride, VC_TILE_NT), VC_TILE_NT, vc_tile_smem<JAC, VC_TILE_NT>(), st>>>(
-            P, coef, B, stride, plane, inv_s, x, xo, active, F, J, rmax_part);
+    chain(st, nblk((int64_t)B * stride, VC_TILE_NT), VC_TILE_NT, vc_tile_smem<JAC, VC_TILE_NT>(),
+          k_vc_assemble_tile<T, FINE, JAC, VC_TILE_NT>, P, coef, B, stride, plane, inv_s, x, xo, active, F, J, rmax_part);
   else
-    k_vc_assemble_st<T, FINE, JAC><<<nblk((int64_t)B * stride), TPB, 0, st>>>(P, coef, B, stride, plane, inv_s, x,
-                                                                              xo, active, F, J, rmax_part);
+    chain(st, nblk((int64_t)B * stride), TPB, 0, k_vc_assemble_st<T, FINE, JAC>, P, coef, B, stride, plane, inv_s, x, xo,
+          active, F, J, rmax_part);
 }
 
 template <typename T>
@@ -1706,7 +1748,7 @@ int vc_inject(henry_handle* H, VcGroup<T>& G, int B, bool old, const int* active
     auto& Lf = G.lv[k - 1];
     auto& Lc = G.lv[k];
     launch(H, st, HENRY_K_STATE_RESTRICT, (double)H->nact * Lc.NV * 32.0, [&] {
-      k_vc_inject<<<nblk((int64_t)B * Lc.NV), TPB, 0, st>>>(B, Lc.nx, Lc.ny, Lf.stride, Lc.stride,
+      chain(st, nblk((int64_t)B * Lc.NV), TPB, 0, k_vc_inject, B, Lc.nx, Lc.ny, Lf.stride, Lc.stride,
                                                              old ? Lf.xo : Lf.x, old ? Lc.xo : Lc.x, active);
     });
     CKL();
@@ -1729,10 +1771,23 @@ int vc_coarse_ops(henry_handle* H, VcGroup<T>& G, int B, double tau, double inv_
   }
   auto& Lc = G.lv[G.K];
   launch(H, st, HENRY_K_COARSE_OPS, (double)H->nact * (9.0 * 6 * sizeof(B4) + 144.0 * sizeof(T)), [&] {
-    k_vc_coarse_inverse<T><<<nblk(B, 64), 64, 0, st>>>(B, vc_args<T>(Lc), (const B4*)Lc.J, G.Ainv, G.lin_active);
+    chain(st, nblk(B, 64), 64, 0, k_vc_coarse_inverse<T>, B, vc_args<T>(Lc), (const B4*)Lc.J, G.Ainv, G.lin_active);
   });
   CKL();
   return HENRY_OK;
+}
+
+// The first level of the fused tail (henry_vc_tail.cuh), -1 for none: the first
+// coarse one of at most 32 x 16 elements, whatever the batch (10 steps of
+// level 1, 400 samples, FP64: 235 ms, 246 ms from 16 x 8 elements, 290 ms
+// without; 4096 samples of level 0, whose first coarse grid is 16 x 8: 351 and
+// 353 ms); mg_tail_cells = 0: none.
+template <typename T>
+int vc_tail_level(const henry_config& c, const VcGroup<T>& G) {
+  if (c.mg_tail_cells == 0 || !vc_tail_fits<T>()) return -1;
+  for (int k = 1; k < G.K; ++k)
+    if (G.lv[k].nx <= 32) return k;
+  return -1;
 }
 
 // One V(nu1, nu2) cycle on the vertex hierarchy: x0 = M^{-1} b0 (fine level,
@@ -1754,11 +1809,13 @@ int vc_vcycle(henry_handle* H, VcGroup<T>& G, int B, const typename VT<T>::v2* b
     const int nv = vc_colour_rows(L.ny + 1, CJ[col]) * vc_colour_cols(L.nx + 1, CI[col]);
     launch(H, st, k == 0 ? HENRY_K_SMOOTH : HENRY_K_SMOOTH_COARSE, na * nv * (9 * b4 + 3 * v2),
            na * nv * (8 * 8.0 + 6.0), [&] {
-             k_vc_sweep<T, 1><<<nblk((int64_t)B * nv), TPB, 0, st>>>(B, A, CI[col], CJ[col], (const B4*)L.J, b, x,
+             chain(st, nblk((int64_t)B * nv), TPB, 0, k_vc_sweep<T, 1>, B, A, CI[col], CJ[col], (const B4*)L.J, b, x,
                                                                      act);
            });
   };
-  for (int k = 0; k < G.K; ++k) {
+  const int kt = vc_tail_level<T>(H->cfg, G);
+  const int kend = kt > 0 ? kt : G.K;  // levels 0 .. kend - 1 run as separate kernels
+  for (int k = 0; k < kend; ++k) {
     auto& L = G.lv[k];
     auto& Lc = G.lv[k + 1];
     const VcLevelArgs A = vc_args<T>(L), Ac = vc_args<T>(Lc);
@@ -1767,39 +1824,70 @@ int vc_vcycle(henry_handle* H, VcGroup<T>& G, int B, const typename VT<T>::v2* b
     const int sm = k == 0 ? HENRY_K_SMOOTH : HENRY_K_SMOOTH_COARSE;
     if (nu1 > 0) {
       launch(H, st, sm, na * L.NV * (0.25 * (b4 + v2) + v2), na * L.NV * 1.5, [&] {
-        k_vc_sweep<T, 0><<<nblk((int64_t)B * L.NV), TPB, 0, st>>>(B, A, 0, 0, (const B4*)L.J, b, x, act);
+        chain(st, nblk((int64_t)B * L.NV), TPB, 0, k_vc_sweep<T, 0>, B, A, 0, 0, (const B4*)L.J, b, x, act);
       });
       for (int col = 1; col < 4; ++col) sweep(k, col, b, x);
       for (int i = 1; i < nu1; ++i)
         for (int col = 0; col < 4; ++col) sweep(k, col, b, x);
     } else {
       launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * L.NV * v2, [&] {
-        k_vc_sweep<T, 2><<<nblk((int64_t)B * L.NV), TPB, 0, st>>>(B, A, 0, 0, (const B4*)L.J, b, x, act);
+        chain(st, nblk((int64_t)B * L.NV), TPB, 0, k_vc_sweep<T, 2>, B, A, 0, 0, (const B4*)L.J, b, x, act);
       });
     }
     launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * L.NV * (9 * b4 + 3 * v2) + na * Lc.NV * v2,
            na * L.NV * 74.0, [&] {
-             k_vc_residual<T><<<nblk((int64_t)B * L.NV), TPB, 0, st>>>(B, A, (const B4*)L.J, b, x, (V2*)L.mgr, act);
-             k_vc_restrict<T><<<nblk((int64_t)B * Lc.NV), TPB, 0, st>>>(B, A, Ac, (const V2*)L.mgr, (V2*)Lc.mgb,
+             chain(st, nblk((int64_t)B * L.NV), TPB, 0, k_vc_residual<T>, B, A, (const B4*)L.J, b, x, (V2*)L.mgr, act);
+             chain(st, nblk((int64_t)B * Lc.NV), TPB, 0, k_vc_restrict<T>, B, A, Ac, (const V2*)L.mgr, (V2*)Lc.mgb,
                                                                         act);
            });
     CKL();
   }
-  {
+  if (kt > 0) {
+    VcTailArgs A;
+    std::memset(&A, 0, sizeof A);
+    double nv = 0.0;
+    for (int k = kt; k < G.K; ++k) {
+      auto& L = G.lv[k];
+      A.J[k - kt] = L.J;
+      A.plane[k - kt] = L.plane;
+      A.stride[k - kt] = L.stride;
+      nv += L.NV;
+    }
+    A.b = G.lv[kt].mgb;
+    A.x = G.lv[kt].mgx;
+    A.ainv = G.Ainv;
+    A.active = act;
+    A.nu1 = nu1;
+    A.nu2 = nu2;
+    launch(H, st, HENRY_K_MG_TAIL, na * (nv * 10 * b4 + 2.0 * G.lv[kt].NV * v2 + 144.0 * sizeof(T)),
+           na * nv * ((nu1 + nu2) * 70.0 + 74.0), [&] {
+             auto go = [&](auto w) {
+               constexpr int NX0 = decltype(w)::value;
+               chain(st, B, vc_tail_threads(NX0), vc_tail_bytes<T>(NX0), k_vc_tail<T, NX0>, A, B);
+             };
+             switch (G.lv[kt].nx) {
+               case 4: go(std::integral_constant<int, 4>()); break;
+               case 8: go(std::integral_constant<int, 8>()); break;
+               case 16: go(std::integral_constant<int, 16>()); break;
+               default: go(std::integral_constant<int, 32>()); break;
+             }
+           });
+    CKL();
+  } else {
     auto& Lc = G.lv[G.K];
     launch(H, st, HENRY_K_COARSE_SOLVE, na * (144.0 * sizeof(T) + 24 * v2), [&] {
-      k_vc_coarse_solve<T><<<nblk(B, 64), 64, 0, st>>>(B, vc_args<T>(Lc), G.Ainv, (const V2*)Lc.mgb, (V2*)Lc.mgx,
+      chain(st, nblk(B, 64), 64, 0, k_vc_coarse_solve<T>, B, vc_args<T>(Lc), G.Ainv, (const V2*)Lc.mgb, (V2*)Lc.mgx,
                                                        act);
     });
     CKL();
   }
-  for (int k = G.K - 1; k >= 0; --k) {
+  for (int k = kend - 1; k >= 0; --k) {
     auto& L = G.lv[k];
     auto& Lc = G.lv[k + 1];
     const V2* b = k == 0 ? b0 : (const V2*)L.mgb;
     V2* x = k == 0 ? x0 : (V2*)L.mgx;
     launch(H, st, HENRY_K_RESIDUAL_RESTRICT, na * (L.NV * 2.0 * v2 + Lc.NV * v2), [&] {
-      k_vc_prolong_add<T><<<nblk((int64_t)B * L.NV), TPB, 0, st>>>(B, vc_args<T>(L), vc_args<T>(Lc), x,
+      chain(st, nblk((int64_t)B * L.NV), TPB, 0, k_vc_prolong_add<T>, B, vc_args<T>(L), vc_args<T>(Lc), x,
                                                                    (const V2*)Lc.mgx, act);
     });
     for (int i = 0; i < nu2; ++i)
@@ -1810,36 +1898,53 @@ int vc_vcycle(henry_handle* H, VcGroup<T>& G, int B, const typename VT<T>::v2* b
 }
 
 // BiCGStab on the fine vertex grid for the samples with lin_active set;
-// right-hand side -F, solution in G.dx (linear_solve's kernels and order).
+// right-hand side -F, solution in G.dx (Krylov's kernels and order).
 template <typename T>
-int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, double rtol = -1.0, int maxit = -1) {
+struct VcKrylov : KrylovDrive<VcKrylov<T>> {
   typedef typename VT<T>::v2 V2;
   typedef typename VT<T>::b4 B4;
-  auto& L = G.lv[0];
-  const int N = L.stride;
-  const VcLevelArgs A = vc_args<T>(L);
-  const unsigned g = nblk((int64_t)B * N);
-  const double b4 = sizeof(B4), v2 = sizeof(V2);
-  launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * v2), [&] {
-    chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, (int*)nullptr);
-  });
-  CKL();
-  double* fin = (H->cfg.finalize_nct > 0 && G.nct >= H->cfg.finalize_nct) ? G.fin : nullptr;
-  auto finalize = [&](int a, int b, cudaStream_t ss) {
+  henry_handle* H;
+  VcGroup<T>& G;
+  int B;
+  double rtol2;
+  int maxit;
+  const typename VcGroup<T>::Lv& L;
+  int N;
+  unsigned g;
+  double* fin;
+
+  VcKrylov(henry_handle* h, VcGroup<T>& grp, int b)
+      : H(h), G(grp), B(b), rtol2(h->cfg.lin_rtol * h->cfg.lin_rtol), maxit(h->cfg.lin_maxit), L(grp.lv[0]),
+        N(grp.lv[0].stride), g(nblk((int64_t)b * grp.lv[0].stride)),
+        fin((h->cfg.finalize_nct > 0 && grp.nct >= h->cfg.finalize_nct) ? grp.fin : nullptr) {}
+  void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
            [&] { chain(ss, nblk((int64_t)B * 32, 128), 128, 0, k_finalize, B, G.nct, G.part, a, b, fin); });
-  };
-  finalize(P_RR, P_RN, st);
-  const double rt = rtol > 0.0 ? rtol : H->cfg.lin_rtol;
-  const int mi = maxit > 0 ? maxit : H->cfg.lin_maxit;
-  const double rtol2 = rt * rt;
-  auto body = [&](int n_act, cudaStream_t ss) -> int {
-    const double nc = (double)n_act * L.NV;
+  }
+  int init(cudaStream_t st, int* loop) {
+    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * sizeof(V2)), [&] {
+      chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, loop);
+    });
+    finalize(P_RR, P_RN, st);
+    CKL();
+    return HENRY_OK;
+  }
+  int head(int it, const int* it_dev, cudaStream_t st) {
+    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * sizeof(V2), [&] {
+      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
+            G.iters, G.status, G.counter + 1, G.totals + 1, fin);
+    });
+    CKL();
+    return HENRY_OK;
+  }
+  int body(int n_act, cudaStream_t ss) {
+    const double nc = (double)n_act * L.NV, b4 = sizeof(B4), v2 = sizeof(V2);
+    const VcLevelArgs A = vc_args<T>(L);
     int rc = vc_vcycle<T>(H, G, B, G.p, G.ph, ss);
     if (rc) return rc;
     launch(H, ss, HENRY_K_SPMV, nc * (9 * b4 + 3 * v2), nc * (9 * 8.0 + 4.0), [&] {
-      k_vc_spmv<T, 1><<<g, TPB, 0, ss>>>(B, A, (const B4*)L.J, G.ph, G.v, G.rh, G.part, P_RV, 0, G.lin_active);
+      chain(ss, g, TPB, 0, k_vc_spmv<T, 1>, B, A, (const B4*)L.J, G.ph, G.v, G.rh, G.part, P_RV, 0, G.lin_active);
     });
     finalize(P_RV, -1, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 3 * v2,
@@ -1848,57 +1953,23 @@ int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st, doub
     rc = vc_vcycle<T>(H, G, B, G.s, G.sh, ss);
     if (rc) return rc;
     launch(H, ss, HENRY_K_SPMV, nc * (9 * b4 + 3 * v2), nc * (9 * 8.0 + 8.0), [&] {
-      k_vc_spmv<T, 2><<<g, TPB, 0, ss>>>(B, A, (const B4*)L.J, G.sh, G.t, G.s, G.part, P_TS, P_TT, G.lin_active);
+      chain(ss, g, TPB, 0, k_vc_spmv<T, 2>, B, A, (const B4*)L.J, G.sh, G.t, G.s, G.part, P_TS, P_TT, G.lin_active);
     });
     finalize(P_TS, P_TT, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 8 * v2, [&] {
-      chain(ss, g, TPB, 0, k_bicg_update<T, false>, B, N, G.dx, G.ph, G.sh, G.s, G.t, G.rh, G.r, G.part, G.sc, G.lin_active,
-                                           fin);
+      chain(ss, g, TPB, 0, k_bicg_update<T, false>, B, N, G.dx, G.ph, G.sh, G.s, G.t, G.rh, G.r, G.part, G.sc,
+            G.lin_active, fin);
     });
     finalize(P_RR, P_RN, ss);
     CKL();
     return HENRY_OK;
-  };
-  const bool use_graph = H->cfg.cuda_graphs && !H->prof.on;
-  auto run_graph = [&]() -> int {
-    const auto key = std::make_tuple(B, H->cfg.nu1, H->cfg.nu2);
-    auto f = G.gexec.find(key);
-    if (f == G.gexec.end()) {
-      if (!H->cap_stream) CK(cudaStreamCreateWithFlags(&H->cap_stream, cudaStreamNonBlocking));
-      cudaGraph_t gr = nullptr;
-      CK(cudaStreamBeginCapture(H->cap_stream, cudaStreamCaptureModeThreadLocal));
-      const int rc = body(B, H->cap_stream);
-      const cudaError_t e = cudaStreamEndCapture(H->cap_stream, &gr);
-      if (rc) {
-        if (e == cudaSuccess && gr) cudaGraphDestroy(gr);
-        return rc;
-      }
-      if (e != cudaSuccess) return set_err(HENRY_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
-      cudaGraphExec_t ex = nullptr;
-      const cudaError_t e2 = cudaGraphInstantiate(&ex, gr, 0);
-      cudaGraphDestroy(gr);
-      if (e2 != cudaSuccess) return set_err(HENRY_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e2));
-      f = G.gexec.emplace(key, ex).first;
-    }
-    CK(cudaGraphLaunch(f->second, st));
-    return HENRY_OK;
-  };
-  for (int it = 0; it <= mi; ++it) {
-    CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
-    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * v2, [&] {
-      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, (const int*)nullptr, mi, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
-                                      G.status, G.counter + 1, G.totals + 1, fin);
-    });
-    CKL();
-    int n_act = 0;
-    int rc = read_counter(H, G.counter + 1, st, &n_act);
-    if (rc) return rc;
-    if (n_act == 0) break;
-    H->nact = n_act;
-    rc = use_graph ? run_graph() : body(n_act, st);
-    if (rc) return rc;
   }
-  return HENRY_OK;
+};
+template <typename T>
+int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st) {
+  VcKrylov<T> k(H, G, B);
+  if (!graphs_on(H, G)) return k.run(st);
+  return run_graph(H, G, B, "linear", st, [&](GraphBuild& b) { return k.emit(b); });
 }
 
 // Where the fine assembly leaves its per-CTA maxima of |F| and how many a
@@ -1940,78 +2011,96 @@ int vc_assemble_fine(henry_handle* H, VcGroup<T>& G, int B, double tau, double i
   return HENRY_OK;
 }
 
-// One implicit-Euler step of the vertex-centred scheme (implicit_step's
-// Newton iteration and tests).
+// One implicit-Euler step of the vertex-centred scheme (NewtonStep's iteration
+// and tests).
 template <typename T>
-int vc_implicit_step(henry_handle* H, VcGroup<T>& G, int B, int step, cudaStream_t st) {
+struct VcNewtonStep : NewtonDrive<VcNewtonStep<T>> {
   typedef typename VT<T>::v2 V2;
-  const henry_config& c = H->cfg;
-  const LevelGeom lg = geom(c, G.level);
-  auto& L = G.lv[0];
-  const int N = L.stride;
-  const int64_t n0 = (int64_t)B * N;
-  const double inv_s = 1.0 / (c.rho0 * lg.h * lg.h / lg.tau);
-  const double inv_pref = 1.0 / (c.rho0 * c.g * c.Ly);
-  double* pmax = G.part + P_MAX * (int64_t)B * G.nct;
-  H->nact = B;
-  launch(H, st, HENRY_K_NEWTON, (double)n0 * 32, [&] {
-    // the predictor as in implicit_step (quadratic from step 2 on)
-    const bool quad = c.newton_predictor_order == 2 && G.xoo;
-    if (step > 1 && quad && c.newton_predictor > 0.0) {
-      chain(st, nblk(n0), TPB, 0, k_step_begin_predict2, n0, c.newton_predictor, L.x, L.xo, G.xoo);
-    } else {
-      if (quad) chain(st, nblk(n0), TPB, 0, k_copy_d2, n0, L.xo, G.xoo);
-      if (step > 0 && c.newton_predictor > 0.0)
-        chain(st, nblk(n0), TPB, 0, k_step_begin_predict, n0, c.newton_predictor, L.x, L.xo);
-      else
-        chain(st, nblk(n0), TPB, 0, k_step_begin, n0, L.x, L.xo);
-    }
-    chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.newton_active, G.newton_it);
-  });
-  CKL();
-  int rc = vc_inject<T>(H, G, B, true, G.newton_active, st);
-  if (rc) return rc;
-  // residual-first test and chord Newton as in implicit_step
-  const int jac_every = std::max(1, c.newton_jacobian_every);
-  int last_jac = -1;
-  for (int it = 0; it <= c.newton_maxit; ++it) {
-    const bool jac_now = last_jac < 0 || it - last_jac >= jac_every;
-    const bool res_first = !jac_now || (c.newton_residual_first >= 0 && it >= c.newton_residual_first);
-    CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
-    rc = vc_assemble_fine<T>(H, G, B, lg.tau, inv_s, st, !res_first);
-    if (rc) return rc;
+  henry_handle* H;
+  VcGroup<T>& G;
+  int B;
+  const henry_config& c;
+  LevelGeom lg;
+  const typename VcGroup<T>::Lv& L;
+  int N;
+  int64_t n0;
+  double inv_s, inv_pref;
+  double* pmax;
+
+  VcNewtonStep(henry_handle* h, VcGroup<T>& g, int b)
+      : NewtonDrive<VcNewtonStep<T>>(h->cfg), H(h), G(g), B(b), c(h->cfg), lg(geom(h->cfg, g.level)), L(g.lv[0]),
+        N(g.lv[0].stride), n0((int64_t)b * g.lv[0].stride) {
+    inv_s = 1.0 / (c.rho0 * lg.h * lg.h / lg.tau);
+    inv_pref = 1.0 / (c.rho0 * c.g * c.Ly);
+    pmax = G.part + P_MAX * (int64_t)B * G.nct;
+  }
+  int begin(int step, cudaStream_t st) {
+    H->nact = B;
+    launch(H, st, HENRY_K_NEWTON, (double)n0 * 32, [&] {
+      // the predictor as in NewtonStep (quadratic from step 2 on)
+      const bool quad = c.newton_predictor_order == 2 && G.xoo;
+      if (step > 1 && quad && c.newton_predictor > 0.0) {
+        chain(st, nblk(n0), TPB, 0, k_step_begin_predict2, n0, c.newton_predictor, L.x, L.xo, G.xoo);
+      } else {
+        if (quad) chain(st, nblk(n0), TPB, 0, k_copy_d2, n0, L.xo, G.xoo);
+        if (step > 0 && c.newton_predictor > 0.0)
+          chain(st, nblk(n0), TPB, 0, k_step_begin_predict, n0, c.newton_predictor, L.x, L.xo);
+        else
+          chain(st, nblk(n0), TPB, 0, k_step_begin, n0, L.x, L.xo);
+      }
+    });
+    CKL();
+    return HENRY_OK;
+  }
+  int start(cudaStream_t st) {
+    launch(H, st, HENRY_K_NEWTON, (double)B * 12,
+           [&] { chain(st, nblk(B, 128), 128, 0, k_step_flags, B, G.status, G.newton_active, G.newton_it); });
+    CKL();
+    return vc_inject<T>(H, G, B, true, G.newton_active, st);
+  }
+  VcKrylov<T> krylov(bool) { return VcKrylov<T>(H, G, B); }
+  int solve(bool, cudaStream_t st) { return vc_linear_solve<T>(H, G, B, st); }
+  int evaluate(bool res_first, int* count, cudaStream_t st) {
+    const int rc = vc_assemble_fine<T>(H, G, B, lg.tau, inv_s, st, !res_first);
     int nct_f = 0;
     const double* fmax_parts = vc_max_parts<T>(H, G, B, &nct_f);
     launch(H, st, HENRY_K_NEWTON, (double)B * 8 * nct_f, [&] {
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, nct_f, c.newton_atol, c.newton_maxit, fmax_parts,
-                                                       G.newton_active, G.lin_active, G.newton_it, G.status,
-                                                       G.counter, G.totals);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, nct_f, c.newton_atol, c.newton_maxit,
+            fmax_parts, G.newton_active, G.lin_active, G.newton_it, G.status, count, G.totals);
     });
     CKL();
-    int n_act = 0;
-    rc = read_counter(H, G.counter, st, &n_act);
-    if (rc) return rc;
-    if (n_act == 0) break;
-    H->nact = n_act;
-    if (jac_now) {
-      if (res_first) rc = vc_assemble_fine<T>(H, G, B, lg.tau, inv_s, st);
-      if (!rc) rc = vc_inject<T>(H, G, B, false, G.lin_active, st);
-      if (!rc) rc = vc_coarse_ops<T>(H, G, B, lg.tau, inv_s, st);
-      last_jac = it;
-    }
-    if (!rc) rc = vc_linear_solve<T>(H, G, B, st);
-    if (rc) return rc;
-    H->nact = n_act;
+    return rc;
+  }
+  int operators(bool res_first, cudaStream_t st) {
+    int rc = res_first ? vc_assemble_fine<T>(H, G, B, lg.tau, inv_s, st) : HENRY_OK;
+    if (!rc) rc = vc_inject<T>(H, G, B, false, G.lin_active, st);
+    return rc ? rc : vc_coarse_ops<T>(H, G, B, lg.tau, inv_s, st);
+  }
+  bool retries() const { return false; }
+  int mark_retry(cudaStream_t) { return HENRY_OK; }
+  int retry_operators(cudaStream_t) { return HENRY_OK; }
+  int update(int n_act, cudaStream_t st) {
     launch(H, st, HENRY_K_NEWTON, (double)n_act * N * (32.0 + sizeof(V2)), [&] {
       double* pdc = G.part + P_DC * (int64_t)B * G.nct;
       chain(st, nblk(n0), TPB, 0, k_newton_step_max<T>, B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active, G.theta);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active,
+            G.theta);
       chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active, G.status);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active,
+            G.status);
     });
     CKL();
+    return HENRY_OK;
   }
-  return HENRY_OK;
+};
+template <typename T>
+int vc_implicit_step(henry_handle* H, VcGroup<T>& G, int B, int step, cudaStream_t st) {
+  VcNewtonStep<T> n(H, G, B);
+  const int rc = n.begin(step, st);
+  if (rc) return rc;
+  if (!graphs_on(H, G) || !n.graphable()) return n.run(st);
+  if (step == 0) CK(cudaMemsetAsync(G.counter, 0, 4 * sizeof(int), st));
+  return run_graph(H, G, B, "step", st, [&](GraphBuild& b) { return n.emit(b); });
 }
 
 // Full scenario solves of B samples of the vertex-centred scheme whose

@@ -69,8 +69,8 @@ __host__ __device__ __forceinline__ int vc_colour_cols(int nxv, int ci) { return
 // false: the residual alone (bit-identical to the JAC = true residual).
 template <typename T, bool FINE, bool JAC = true>
 __global__ void __launch_bounds__(TPB) k_vc_assemble_st(VcParams P, const Coef* __restrict__ coef, int B, int stride,
-                                                        int64_t plane, double inv_s, const double2* __restrict__ x,
-                                                        const double2* __restrict__ xo, const int* __restrict__ active,
+                                                        int64_t plane, double inv_s, const double2* x,
+                                                        const double2* xo, const int* active,
                                                         double2* __restrict__ F, typename VT<T>::b4* __restrict__ J,
                                                         double* __restrict__ rmax_part) {
   typedef typename VT<T>::b4 B4;
@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(TPB) k_vc_assemble_st(VcParams P, const Coef* 
   const int nxv = P.nx + 1, NV = nxv * (P.ny + 1);
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int s = (int)(e / stride);
+  grid_enter();
   if (FINE) {
     if (!active[s]) return;  // uniform over the CTA
   } else {
@@ -158,9 +159,8 @@ __device__ __forceinline__ void vc_eval_face(const VcParams& P, const VcCoef& C,
 template <typename T, bool FINE, bool JAC = true, int NT = 128>
 __global__ void __launch_bounds__(NT) k_vc_assemble_tile(VcParams P, const Coef* __restrict__ coef, int B,
                                                           int stride, int64_t plane, double inv_s,
-                                                          const double2* __restrict__ x,
-                                                          const double2* __restrict__ xo,
-                                                          const int* __restrict__ active, double2* __restrict__ F,
+                                                          const double2* x, const double2* xo,
+                                                          const int* active, double2* __restrict__ F,
                                                           typename VT<T>::b4* __restrict__ J,
                                                           double* __restrict__ rmax_part) {
   typedef typename VT<T>::b4 B4;
@@ -172,6 +172,7 @@ __global__ void __launch_bounds__(NT) k_vc_assemble_tile(VcParams P, const Coef*
   const int64_t t0 = (int64_t)blockIdx.x * NT;
   const int64_t e = t0 + threadIdx.x;
   const int s = (int)(e / stride);
+  grid_enter();
   if (FINE) {
     if (!active[s]) return;  // uniform over the CTA (stride % NT == 0)
   }
@@ -286,8 +287,9 @@ constexpr int vc_tile_smem() {
 // Coarse states by injection: x_c(J, I) = x_f(2J, 2I), for the iterate and
 // (old != 0) the old state.
 __global__ void __launch_bounds__(TPB) k_vc_inject(int B, int ncx, int ncy, int stride_f, int stride_c,
-                                                   const double2* __restrict__ xf, double2* __restrict__ xc,
-                                                   const int* __restrict__ active) {
+                                                   const double2* xf, double2* __restrict__ xc,
+                                                   const int* active) {
+  grid_enter();
   const int ncxv = ncx + 1, NVc = ncxv * (ncy + 1), nfxv = 2 * ncx + 1;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (e >= (int64_t)B * NVc) return;
@@ -322,11 +324,12 @@ __device__ __forceinline__ void vc_offdiag(int nxv, int nyv, int j, int i, int s
 template <typename T, int MODE>
 __global__ void __launch_bounds__(TPB) k_vc_sweep(int B, VcLevelArgs L, int ci, int cj,
                                                   const typename VT<T>::b4* __restrict__ J,
-                                                  const typename VT<T>::v2* __restrict__ b,
-                                                  typename VT<T>::v2* __restrict__ x, const int* __restrict__ active) {
+                                                  const typename VT<T>::v2* b, typename VT<T>::v2* x,
+                                                  const int* active) {
   typedef typename VT<T>::v2 V2;
   const int nxv = L.nx + 1, nyv = L.ny + 1, NV = nxv * nyv;
   const int64_t t = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  grid_enter();
   int s, j, i, st;
   if (MODE == 1) {
     const int nr = vc_colour_rows(nyv, cj), nc = vc_colour_cols(nxv, ci), per = nr * nc;
@@ -359,9 +362,9 @@ __global__ void __launch_bounds__(TPB) k_vc_sweep(int B, VcLevelArgs L, int ci, 
 // r = b - A x on every vertex of a level.
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_vc_residual(int B, VcLevelArgs L, const typename VT<T>::b4* __restrict__ J,
-                                                     const typename VT<T>::v2* __restrict__ b,
-                                                     const typename VT<T>::v2* __restrict__ x,
-                                                     typename VT<T>::v2* __restrict__ r, const int* __restrict__ active) {
+                                                     const typename VT<T>::v2* b, const typename VT<T>::v2* x,
+                                                     typename VT<T>::v2* __restrict__ r, const int* active) {
+  grid_enter();
   const int nxv = L.nx + 1, nyv = L.ny + 1, NV = nxv * nyv;
   const int64_t t = (int64_t)blockIdx.x * TPB + threadIdx.x;
   if (t >= (int64_t)B * NV) return;
@@ -383,8 +386,9 @@ __global__ void __launch_bounds__(TPB) k_vc_residual(int B, VcLevelArgs L, const
 // Dirichlet equations (p and c at x = Lx, c at x = 0) are set to zero.
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_vc_restrict(int B, VcLevelArgs Lf, VcLevelArgs Lc,
-                                                     const typename VT<T>::v2* __restrict__ rf,
-                                                     typename VT<T>::v2* __restrict__ bc, const int* __restrict__ active) {
+                                                     const typename VT<T>::v2* rf,
+                                                     typename VT<T>::v2* __restrict__ bc, const int* active) {
+  grid_enter();
   typedef typename VT<T>::v2 V2;
   const int ncxv = Lc.nx + 1, NVc = ncxv * (Lc.ny + 1), nfxv = Lf.nx + 1, nfyv = Lf.ny + 1;
   const int64_t t = (int64_t)blockIdx.x * TPB + threadIdx.x;
@@ -415,9 +419,9 @@ __global__ void __launch_bounds__(TPB) k_vc_restrict(int B, VcLevelArgs Lf, VcLe
 // x_f += P x_c (bilinear interpolation from the coarse vertices).
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_vc_prolong_add(int B, VcLevelArgs Lf, VcLevelArgs Lc,
-                                                        typename VT<T>::v2* __restrict__ xf,
-                                                        const typename VT<T>::v2* __restrict__ xc,
-                                                        const int* __restrict__ active) {
+                                                        typename VT<T>::v2* xf, const typename VT<T>::v2* xc,
+                                                        const int* active) {
+  grid_enter();
   typedef typename VT<T>::v2 V2;
   const int nfxv = Lf.nx + 1, NVf = nfxv * (Lf.ny + 1), ncxv = Lc.nx + 1;
   const int64_t t = (int64_t)blockIdx.x * TPB + threadIdx.x;
@@ -458,8 +462,9 @@ __global__ void __launch_bounds__(TPB) k_vc_prolong_add(int B, VcLevelArgs Lf, V
 // + var): the dense matrix from the 9-point blocks, inverted per sample by
 // Gauss-Jordan elimination with partial pivoting in FP64; Ainv[s][12][12].
 template <typename T>
-__global__ void k_vc_coarse_inverse(int B, VcLevelArgs L, const typename VT<T>::b4* __restrict__ J,
-                                    T* __restrict__ Ainv, const int* __restrict__ active) {
+__global__ void k_vc_coarse_inverse(int B, VcLevelArgs L, const typename VT<T>::b4* J,
+                                    T* __restrict__ Ainv, const int* active) {
+  grid_enter();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= B || !active[s]) return;
   constexpr int n = VC_COARSE_N;
@@ -506,8 +511,9 @@ __global__ void k_vc_coarse_inverse(int B, VcLevelArgs L, const typename VT<T>::
 
 template <typename T>
 __global__ void k_vc_coarse_solve(int B, VcLevelArgs L, const T* __restrict__ Ainv,
-                                  const typename VT<T>::v2* __restrict__ b, typename VT<T>::v2* __restrict__ x,
-                                  const int* __restrict__ active) {
+                                  const typename VT<T>::v2* b, typename VT<T>::v2* __restrict__ x,
+                                  const int* active) {
+  grid_enter();
   typedef typename VT<T>::v2 V2;
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= B || !active[s]) return;
@@ -536,10 +542,10 @@ __global__ void k_vc_coarse_solve(int B, VcLevelArgs L, const T* __restrict__ Ai
 //   NDOT 1: <w1, y>;  NDOT 2: <w1, y>, <y, y>.
 template <typename T, int NDOT>
 __global__ void __launch_bounds__(TPB) k_vc_spmv(int B, VcLevelArgs L, const typename VT<T>::b4* __restrict__ J,
-                                                 const typename VT<T>::v2* __restrict__ x,
-                                                 typename VT<T>::v2* __restrict__ y,
-                                                 const typename VT<T>::v2* __restrict__ w1, double* __restrict__ part,
-                                                 int slot1, int slot2, const int* __restrict__ active) {
+                                                 const typename VT<T>::v2* x, typename VT<T>::v2* __restrict__ y,
+                                                 const typename VT<T>::v2* w1, double* __restrict__ part,
+                                                 int slot1, int slot2, const int* active) {
+  grid_enter();
   typedef typename VT<T>::v2 V2;
   __shared__ double sh[TPB + 1];
   const int nxv = L.nx + 1, nyv = L.ny + 1, NV = nxv * nyv, nct = L.stride / TPB;

@@ -76,3 +76,32 @@ def test_step_graph_with_retries_equals_host_driven_loops(hl):
     ok = out[0][2] == 0
     assert torch.equal(out[0][2], out[1][2]) and out[0][3] == out[1][3]
     assert torch.equal(out[0][0][ok], out[1][0][ok])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("level,n,nu", [(0, 1, (2, 2)), (0, 3, (1, 2)), (1, 3, (2, 2)), (1, 2, (0, 1)), (1, 2, (1, 0)),
+                                        (3, 2, (2, 1))])
+def test_vertex_tail_is_bit_identical_to_separate_kernels(hl, precision, level, n, nu):
+    ny, nx = 16 << level, 32 << level
+    xi = torch.as_tensor(inputs.uniform_xi(9400 + level, n), device="cuda")
+    b = torch.as_tensor(inputs.rng(9401 + n).standard_normal((n, ny + 1, nx + 1, 2)), device="cuda")
+    z = []
+    for tail in (-1, 0):
+        s = hl.Solver(scheme=hl.HENRY_SCHEME_VERTEX, precision=precision, mg_tail_cells=tail, nu1=nu[0], nu2=nu[1])
+        z.append(s.precondition(level, xi, _wedge(n, ny + 1, nx + 1, 0.0), _wedge(n, ny + 1, nx + 1, 0.02), b))
+        s.close()
+    assert bool(torch.isfinite(z[0]).all()) and torch.equal(z[0], z[1])
+
+
+@pytest.mark.parametrize("res_first,every,maxit", [(2, 1, 30), (-1, 2, 30), (3, 2, 30), (2, 1, 1)])
+def test_vertex_step_graph_equals_host_driven_loops(hl, res_first, every, maxit):
+    xi = torch.as_tensor(inputs.uniform_xi(9500, 4), device="cuda")
+    out = []
+    for graphs in (1, 0):
+        s = hl.Solver(scheme=hl.HENRY_SCHEME_VERTEX, cuda_graphs=graphs, newton_residual_first=res_first,
+                      newton_jacobian_every=every, newton_maxit=maxit, steps0=4, T=4 * 360.0)
+        out.append(s.level_batch_solve(0, xi, allow_failures=True))
+        s.close()
+    ok = out[0][2] == 0
+    assert (maxit == 1) == bool((~ok).all())
+    assert torch.equal(out[0][2], out[1][2]) and torch.equal(out[0][0][ok], out[1][0][ok]) and out[0][3] == out[1][3]
