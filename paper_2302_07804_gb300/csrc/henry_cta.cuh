@@ -194,45 +194,15 @@ __device__ void cta_vcycle(const CtaSmem<T>& S, int nu1, int nu2, const typename
   }
 }
 
-// Coarsest 4 x 4 inverse (thread 0), FP64 Gauss-Jordan with partial pivoting.
+// Coarsest 4 x 4 inverse (the first warp).
 template <typename T>
 __device__ void cta_coarse_inverse(const CtaSmem<T>& S) {
-  if (threadIdx.x != 0) return;
-  const int K = S.L->K;
-  const typename VT<T>::b4* J = S.J(K);
-  const int ps = 2;
-  const auto Ca = J[0], Ea = J[2 * ps + 0], Wb = J[ps + 1], Cb = J[1];
-  double M[4][8];
-  const double blk[4][4] = {{Ca.a00, Ca.a01, Ea.a00, Ea.a01},
-                            {Ca.a10, Ca.a11, Ea.a10, Ea.a11},
-                            {Wb.a00, Wb.a01, Cb.a00, Cb.a01},
-                            {Wb.a10, Wb.a11, Cb.a10, Cb.a11}};
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      M[i][j] = blk[i][j];
-      M[i][4 + j] = (i == j) ? 1.0 : 0.0;
-    }
-  for (int col = 0; col < 4; ++col) {
-    int piv = col;
-    for (int r = col + 1; r < 4; ++r)
-      if (fabs(M[r][col]) > fabs(M[piv][col])) piv = r;
-    if (piv != col)
-      for (int j = 0; j < 8; ++j) {
-        const double tt = M[col][j];
-        M[col][j] = M[piv][j];
-        M[piv][j] = tt;
-      }
-    const double inv = 1.0 / M[col][col];
-    for (int j = 0; j < 8; ++j) M[col][j] *= inv;
-    for (int r = 0; r < 4; ++r) {
-      if (r == col) continue;
-      const double f = M[r][col];
-      for (int j = 0; j < 8; ++j) M[r][j] -= f * M[col][j];
-    }
-  }
-  T* A = S.ainv();
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) A[i * 4 + j] = (T)M[i][4 + j];
+  if (threadIdx.x >= 32) return;
+  const int c = threadIdx.x & 7;
+  double M[4];
+  coarse_inverse_lanes(S.J(S.L->K), 2, c, M);
+  if (threadIdx.x >= 4 && threadIdx.x < 8)
+    for (int i = 0; i < 4; ++i) S.ainv()[i * 4 + c - 4] = (T)M[i];
 }
 
 // The fused scenario solve: one CTA per sample.  xo_g: the sample's old state

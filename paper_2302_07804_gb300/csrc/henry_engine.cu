@@ -778,25 +778,62 @@ void assemble_level(const henry_config& c, Group<T>& G, const Level& L, int B, d
 template <typename T, bool DROP = false>
 int build_coarse_ops(henry_handle* H, Group<T>& G, int B, double inv_tau, double inv_s, cudaStream_t st) {
   typedef typename VT<T>::b4 B4;
+  const henry_config& c = H->cfg;
   const double na = H->nact;
-  for (int k = 1; k <= G.K; ++k) {
-    Level& L = G.lv[k];
-    if (H->cfg.coarse_op == HENRY_COARSE_GALERKIN && !DROP) {
+  if (c.coarse_op == HENRY_COARSE_GALERKIN && !DROP) {
+    for (int k = 1; k <= G.K; ++k) {
+      Level& L = G.lv[k];
       Level& Lf = G.lv[k - 1];
       launch(H, st, HENRY_K_COARSE_OPS, na * L.N * 26.0 * sizeof(B4), [&] {
         chain(st, nblk((int64_t)B * L.N), TPB, 0, k_galerkin<T>, B, L.nx, L.ny, (const B4*)Lf.J, Lf.plane, (B4*)L.J,
-                                                               L.plane, G.lin_active);
+              L.plane, G.lin_active);
       });
-    } else {
-      launch(H, st, HENRY_K_COARSE_OPS, na * L.N * (32.0 + 6.0 * sizeof(B4)), [&] {
-        assemble_level<T, false, DROP>(H->cfg, G, L, B, inv_tau, inv_s, G.lin_active, nullptr, L.J, nullptr, st);
-      });
+      CKL();
     }
+  } else {
+    // The levels of whole-row tiles go into one launch (8192 level-0 samples
+    // and single samples alike); others, and other tile settings, one by one.
+    AssembleLevels A;
+    std::memset(&A, 0, sizeof A);
+    double cells = 0.0;
+    for (int k = 1; k <= G.K; ++k) {
+      Level& L = G.lv[k];
+      if (c.tile_assembly && c.assembly_tile_w == 0 && L.nx <= TPB && A.n < AssembleLevels::MAX) {
+        const int i = A.n++;
+        A.nx[i] = L.nx;
+        A.ny[i] = L.ny;
+        A.h[i] = L.h;
+        A.vt_s[i] = L.h * L.h * inv_tau * inv_s;
+        A.lc[i] = L.lc;
+        A.x[i] = L.x;
+        A.xo[i] = L.xo;
+        A.J[i] = L.J;
+        A.plane[i] = L.plane;
+        A.cc[i] = L.cc;
+        A.fc[i] = L.fc;
+        A.first[i + 1] = A.first[i] + nblk((int64_t)B * L.N);
+        cells += L.N;
+        continue;
+      }
+      launch(H, st, HENRY_K_COARSE_OPS, na * L.N * (32.0 + 6.0 * sizeof(B4)), [&] {
+        assemble_level<T, false, DROP>(c, G, L, B, inv_tau, inv_s, G.lin_active, nullptr, L.J, nullptr, st);
+      });
+      CKL();
+    }
+    if (A.n)
+      launch(H, st, HENRY_K_COARSE_OPS, na * cells * (32.0 + 6.0 * sizeof(B4)), [&] {
+        if (G.lv[0].cc)
+          chain(st, A.first[A.n], TPB, 0, k_assemble_levels<T, true, DROP>, phys_of(c), G.coef, A, B, inv_s,
+                G.lin_active);
+        else if constexpr (!DROP)
+          chain(st, A.first[A.n], TPB, 0, k_assemble_levels<T, false, false>, phys_of(c), G.coef, A, B, inv_s,
+                G.lin_active);
+      });
     CKL();
   }
   Level& Lc = G.lv[G.K];
   launch(H, st, HENRY_K_COARSE_OPS, na * (4.0 * sizeof(B4) + 16.0 * sizeof(T)), [&] {
-    chain(st, nblk(B, 64), 64, 0, k_coarse_inverse<T>, B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
+    chain(st, nblk((int64_t)B * 8, 64), 64, 0, k_coarse_inverse<T>, B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
   });
   CKL();
   return HENRY_OK;
@@ -805,14 +842,23 @@ int build_coarse_ops(henry_handle* H, Group<T>& G, int B, double inv_tau, double
 // x_k -> x_{k+1} (mean of children) for all levels; `old` selects xo.
 template <typename T>
 int restrict_states(henry_handle* H, Group<T>& G, int B, bool old, const int* active, cudaStream_t st) {
-  for (int k = 0; k < G.K; ++k) {
-    Level& Lf = G.lv[k];
-    Level& Lc = G.lv[k + 1];
-    launch(H, st, HENRY_K_STATE_RESTRICT, (double)H->nact * Lc.N * 80.0, [&] {
-      chain(st, nblk((int64_t)B * Lc.N), TPB, 0, k_restrict_state, B, Lc.nx, Lc.ny, old ? Lf.xo : Lf.x,
-                                                                old ? Lc.xo : Lc.x, active);
+  for (int k = 0; k < G.K;) {
+    Level& L = G.lv[k];
+    const int tw = std::min(32, L.nx);  // tile width: halved level by level down to 2 cells
+    RestrictLevels A;
+    std::memset(&A, 0, sizeof A);
+    double cells = 0.0;
+    while (A.n < 4 && k + A.n < G.K && (tw >> (A.n + 1)) >= 2) {
+      Level& Lc = G.lv[k + A.n + 1];
+      A.xc[A.n++] = old ? Lc.xo : Lc.x;
+      cells += Lc.N;
+    }
+    launch(H, st, HENRY_K_STATE_RESTRICT, (double)H->nact * cells * 80.0, [&] {
+      chain(st, (unsigned)((int64_t)B * (L.N / (tw * tw / 2))), RESTRICT_THREADS, 0, k_restrict_states, B, L.nx, L.ny,
+            old ? L.xo : L.x, A, active);
     });
     CKL();
+    k += A.n;
   }
   return HENRY_OK;
 }
@@ -1526,11 +1572,9 @@ struct NewtonStep : NewtonDrive<NewtonStep<T>> {
     launch(H, st, HENRY_K_NEWTON, (double)n_act * N * (32.0 + sizeof(V2)), [&] {
       double* pdc = G.part + P_DC * (int64_t)B * G.nct;
       chain(st, nblk(n0), TPB, 0, k_newton_step_max<T>, B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active,
-            G.theta);
-      chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active,
-            G.status);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc,
+            c.newton_dxtol, pmax, G.newton_active, G.status, G.theta);
+      chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta);
     });
     CKL();
     return HENRY_OK;
@@ -2083,11 +2127,9 @@ struct VcNewtonStep : NewtonDrive<VcNewtonStep<T>> {
     launch(H, st, HENRY_K_NEWTON, (double)n_act * N * (32.0 + sizeof(V2)), [&] {
       double* pdc = G.part + P_DC * (int64_t)B * G.nct;
       chain(st, nblk(n0), TPB, 0, k_newton_step_max<T>, B, N, inv_pref, G.dx, pmax, pdc, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc, G.newton_active,
-            G.theta);
-      chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta, G.newton_active);
-      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_dx_check, B, G.nct, c.newton_dxtol, pmax, G.newton_active,
-            G.status);
+      chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_theta, B, G.nct, c.newton_dc_limit, pdc,
+            c.newton_dxtol, pmax, G.newton_active, G.status, G.theta);
+      chain(st, nblk(n0), TPB, 0, k_newton_update<T>, B, N, L.x, G.dx, G.theta);
     });
     CKL();
     return HENRY_OK;
@@ -2451,7 +2493,7 @@ int adjoint_group(henry_handle* H, Group<double>& G, int B, const double* xi, co
                                                                             G.lin_active);
       }
       Level& Lc = G.lv[G.K];
-      chain(st, nblk(B, 64), 64, 0, k_coarse_inverse<double>, B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
+      chain(st, nblk((int64_t)B * 8, 64), 64, 0, k_coarse_inverse<double>, B, (const B4*)Lc.J, Lc.plane, G.Ainv, G.lin_active);
       k_adj_neg<<<nblk(n0), TPB, 0, st>>>(n0, rhs, G.F);
       CKL();
       rc = linear_solve<double>(H, G, B, st, nullptr, c.adj_rtol, c.adj_maxit);

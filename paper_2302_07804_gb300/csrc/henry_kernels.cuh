@@ -223,9 +223,17 @@ __global__ void k_finalize(int B, int nct, const double* part, int slot_a, int s
 // stride over the partials; a max does not depend on the order), returned
 // to every lane.  Wide grids have thousands of partials per sample.
 __device__ __forceinline__ double warp_sample_max(const double* p, int nct, int lane) {
-  double v = 0.0;
-  for (int i = lane; i < nct; i += 32) v = fmax(v, p[i]);
-  return warp_max(v);
+  unsigned long long v = 0;  // the bit patterns of non-negative values order like the values
+  for (int i = lane; i < nct; i += 32) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(p[i]);
+    v = u > v ? u : v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u > v ? u : v;
+  }
+  return __longlong_as_double((long long)v);
 }
 
 // 2x2 block helpers as explicit fused multiply-add chains: two FMAs per row
@@ -617,24 +625,21 @@ __global__ void __launch_bounds__(TPB) k_assemble(Phys ph, const Coef* __restric
 // TPB / nx whole rows (nx <= TPB), possibly of several samples.  A cell of the
 // tile's first row evaluates the face below it itself.  FINE: N % TPB == 0,
 // one sample per CTA.  Shared memory: 2 x TPB faces (28 KB in FP64).
-template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true>
-__global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __restrict__ coef,
-                                                       const LevelCoef* __restrict__ lc, int B, int nx, int ny,
-                                                       double h, double vt_s, double inv_s,
-                                                       const double2* x, const double2* xo,
-                                                       const int* active, double2* __restrict__ F,
-                                                       typename VT<T>::b4* __restrict__ J, int64_t plane,
-                                                       double* __restrict__ rmax_part,
-                                                       const double2* __restrict__ cc,
-                                                       const double4_32a* __restrict__ fc) {
+template <typename T, bool FINE, bool FIELDS, bool DROP, bool JAC>
+__device__ __forceinline__ void assemble_tile(unsigned blk, const Phys& ph, const Coef* __restrict__ coef,
+                                              const LevelCoef* __restrict__ lc, int B, int nx, int ny, double h,
+                                              double vt_s, double inv_s, const double2* x, const double2* xo,
+                                              const int* active, double2* __restrict__ F,
+                                              typename VT<T>::b4* __restrict__ J, int64_t plane,
+                                              double* __restrict__ rmax_part, const double2* __restrict__ cc,
+                                              const double4_32a* __restrict__ fc) {
   typedef typename std::conditional<FINE, double, T>::type S;
   __shared__ FaceData<T, S, JAC> fE[TPB], fN[TPB];
   __shared__ double sh[40];
   const int N = nx * ny;
-  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  const int64_t e = (int64_t)blk * TPB + threadIdx.x;
   const int64_t total = (int64_t)B * N;
   const int s = sample_of(e, N);
-  grid_enter();
   if (FINE) {
     if (!active[s]) return;  // uniform over the CTA
   }
@@ -696,6 +701,49 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __re
   if constexpr (JAC) {
     if (J) store_blocks<T>(J, plane, e, o.C, o.Nb);
   }
+}
+
+template <typename T, bool FINE, bool FIELDS = false, bool DROP = false, bool JAC = true>
+__global__ void __launch_bounds__(TPB) k_assemble_tile(Phys ph, const Coef* __restrict__ coef,
+                                                       const LevelCoef* __restrict__ lc, int B, int nx, int ny,
+                                                       double h, double vt_s, double inv_s,
+                                                       const double2* x, const double2* xo,
+                                                       const int* active, double2* __restrict__ F,
+                                                       typename VT<T>::b4* __restrict__ J, int64_t plane,
+                                                       double* __restrict__ rmax_part,
+                                                       const double2* __restrict__ cc,
+                                                       const double4_32a* __restrict__ fc) {
+  grid_enter();
+  assemble_tile<T, FINE, FIELDS, DROP, JAC>(blockIdx.x, ph, coef, lc, B, nx, ny, h, vt_s, inv_s, x, xo, active, F, J,
+                                            plane, rmax_part, cc, fc);
+}
+
+// The coarse operators of several levels (nx <= TPB) in one launch: a level's
+// assembly is one dependent chain of some 95 operations a cell (3 us in FP64
+// whatever the grid), and the levels do not depend on one another.
+struct AssembleLevels {
+  static constexpr int MAX = 12;
+  int n;
+  unsigned first[MAX + 1];  // first block of each level
+  int nx[MAX], ny[MAX];
+  double h[MAX], vt_s[MAX];
+  const LevelCoef* lc[MAX];
+  const double2 *x[MAX], *xo[MAX];
+  void* J[MAX];
+  int64_t plane[MAX];
+  const double2* cc[MAX];
+  const double4_32a* fc[MAX];
+};
+template <typename T, bool FIELDS, bool DROP>
+__global__ void __launch_bounds__(TPB) k_assemble_levels(Phys ph, const Coef* __restrict__ coef,
+                                                         const __grid_constant__ AssembleLevels A, int B,
+                                                         double inv_s, const int* active) {
+  grid_enter();
+  int l = 0;
+  while (l + 1 < A.n && blockIdx.x >= A.first[l + 1]) ++l;
+  assemble_tile<T, false, FIELDS, DROP, true>(blockIdx.x - A.first[l], ph, coef, A.lc[l], B, A.nx[l], A.ny[l], A.h[l],
+                                              A.vt_s[l], inv_s, A.x[l], A.xo[l], active, nullptr,
+                                              (typename VT<T>::b4*)A.J[l], A.plane[l], nullptr, A.cc[l], A.fc[l]);
 }
 
 // k_assemble_tile2d: a CTA covers a TILE_W x (TPB / TILE_W) block of cells of
@@ -784,25 +832,54 @@ __global__ void __launch_bounds__(TPB) k_assemble_tile2d(Phys ph, const Coef* __
   }
 }
 
-// Coarse states: mean of the 2x2 children (both the iterate and the old state).
-__global__ void __launch_bounds__(TPB) k_restrict_state(int B, int ncx, int ncy, const double2* xf,
-                                                        double2* __restrict__ xc, const int* active) {
-  const int Nc = ncx * ncy;
-  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+// Coarse states: means of the 2x2 children, up to four levels in one launch.
+// A CTA takes a tile of TW x TW/2 cells (TW = min(32, nx)) of one sample's
+// grid and halves it level by level in shared memory; xc[k] are the sample-
+// major arrays of the next levels.
+struct RestrictLevels {
+  int n;
+  double2* xc[4];
+};
+constexpr int RESTRICT_THREADS = 128;
+__global__ void __launch_bounds__(RESTRICT_THREADS) k_restrict_states(int B, int nx, int ny, const double2* xf,
+                                                                      const __grid_constant__ RestrictLevels A,
+                                                                      const int* active) {
+  __shared__ double2 buf[2][RESTRICT_THREADS];
   grid_enter();
-  if (e >= (int64_t)B * Nc) return;
-  const int s = sample_of(e, Nc);
-  if (!active[s]) return;
-  const int stc = (int)(e - (int64_t)s * Nc);
-  int IX, IY;
-  xy_of(stc, ncx, IX, IY);
-  const int nxf = 2 * ncx;
-  const int64_t bf = (int64_t)s * Nc * 4;
-  const double2 a = xf[bf + st_of(2 * IX, 2 * IY, nxf)];
-  const double2 b = xf[bf + st_of(2 * IX + 1, 2 * IY, nxf)];
-  const double2 c = xf[bf + st_of(2 * IX, 2 * IY + 1, nxf)];
-  const double2 d = xf[bf + st_of(2 * IX + 1, 2 * IY + 1, nxf)];
-  xc[e] = make_double2(0.25 * (((a.x + b.x) + c.x) + d.x), 0.25 * (((a.y + b.y) + c.y) + d.y));
+  int TW = min(32, nx), TH = TW >> 1;
+  const int N = nx * ny, tiles = N / (TW * TH), tpr = nx / TW;
+  const int s = blockIdx.x >> lg2(tiles), tile = blockIdx.x - s * tiles;
+  if (s >= B || !active[s]) return;
+  const int tx = tile & (tpr - 1), ty = tile >> lg2(tpr);
+  const double2* x = xf + (int64_t)s * N;
+  for (int k = 0; k < A.n; ++k) {
+    // the tile's TW/2 x TH/2 coarse cells from its TW x TH cells
+    const int cw = TW >> 1, ch = TH >> 1, t = threadIdx.x;
+    if (t < cw * ch) {
+      const int ly = t >> lg2(cw), lx = t - ly * cw;
+      double2 a, b, c, d;
+      if (k == 0) {
+        const int ix = tx * TW + 2 * lx, iy = ty * TH + 2 * ly;
+        a = x[st_of(ix, iy, nx)];
+        b = x[st_of(ix + 1, iy, nx)];
+        c = x[st_of(ix, iy + 1, nx)];
+        d = x[st_of(ix + 1, iy + 1, nx)];
+      } else {
+        const double2* q = buf[(k + 1) & 1] + 2 * ly * TW + 2 * lx;
+        a = q[0];
+        b = q[1];
+        c = q[TW];
+        d = q[TW + 1];
+      }
+      const double2 m = make_double2(0.25 * (((a.x + b.x) + c.x) + d.x), 0.25 * (((a.y + b.y) + c.y) + d.y));
+      buf[k & 1][t] = m;
+      const int ncx = nx >> (k + 1);
+      A.xc[k][(int64_t)s * (N >> (2 * (k + 1))) + st_of(tx * cw + lx, ty * ch + ly, ncx)] = m;
+    }
+    __syncthreads();
+    TW = cw;
+    TH = ch;
+  }
 }
 
 // a5 (Galerkin option): A_c = R A P with piecewise-constant P, R = P^T.
@@ -844,47 +921,71 @@ __global__ void __launch_bounds__(TPB) k_galerkin(int B, int ncx, int ncy, const
   Jc[5 * plane_c + e] = mkblk<B4>(d * idet, -b * idet, -c * idet, a * idet);
 }
 
-// Coarsest grid (2 x 1 cells, 4 unknowns): explicit inverse per sample by
-// Gauss-Jordan elimination with partial pivoting in FP64.
+// Gauss-Jordan elimination with partial pivoting in FP64 on an n x n matrix,
+// one column of [A | I] per lane (c = 0 .. 2n - 1 of a group of W lanes), rows in
+// registers: every step is one division and n multiply-adds deep, where one
+// thread per matrix runs all 2n columns one after another.  All lanes of the
+// warp take part.
+template <int N, int W>
+__device__ __forceinline__ void gauss_jordan_lanes(double (&M)[N]) {
+#pragma unroll
+  for (int col = 0; col < N; ++col) {
+    double v[N];  // column col
+#pragma unroll
+    for (int r = 0; r < N; ++r) v[r] = __shfl_sync(0xffffffffu, M[r], col, W);
+    int piv = col;
+    unsigned long long best = 0;
+#pragma unroll
+    for (int r = col; r < N; ++r) {  // largest magnitude, the first of equals
+      const unsigned long long m = (unsigned long long)__double_as_longlong(v[r]) & 0x7fffffffffffffffull;
+      if (r == col || m > best) {
+        best = m;
+        piv = r;
+      }
+    }
+#pragma unroll
+    for (int r = col + 1; r < N; ++r) {
+      if (r != piv) continue;
+      double t = M[r];
+      M[r] = M[col];
+      M[col] = t;
+      t = v[r];
+      v[r] = v[col];
+      v[col] = t;
+    }
+    M[col] *= 1.0 / v[col];
+#pragma unroll
+    for (int r = 0; r < N; ++r)
+      if (r != col) M[r] = fma(neg_(v[r]), M[col], M[r]);
+  }
+}
+
+// Coarsest grid (2 x 1 cells, 4 unknowns; cells st 0 = (0,0) colour 0, st 1 =
+// (1,0) colour 1): explicit inverse by eight lanes.  J: the sample's blocks, ps
+// their plane stride; lane c = 4 + j ends with column j of the inverse.
+template <typename B4>
+__device__ __forceinline__ void coarse_inverse_lanes(const B4* J, int64_t ps, int c, double (&M)[4]) {
+  // unknown c = 2 cell + var couples to the equations of cell 0 (rows 0, 1)
+  // and cell 1 (rows 2, 3)
+  const int cell = (c >> 1) & 1, var = c & 1;
+  const B4 up = cell == 0 ? J[0] : J[2 * ps];       // C of cell 0, E of cell 0
+  const B4 lo = cell == 0 ? J[ps + 1] : J[1];       // W of cell 1, C of cell 1
+  const double a[4] = {(double)(var ? up.a01 : up.a00), (double)(var ? up.a11 : up.a10),
+                       (double)(var ? lo.a01 : lo.a00), (double)(var ? lo.a11 : lo.a10)};
+#pragma unroll
+  for (int r = 0; r < 4; ++r) M[r] = c < 4 ? a[r] : (c - 4 == r ? 1.0 : 0.0);
+  gauss_jordan_lanes<4, 8>(M);
+}
 template <typename T>
 __global__ void k_coarse_inverse(int B, const typename VT<T>::b4* J, int64_t plane,
                                  T* __restrict__ Ainv, const int* active) {
   grid_enter();
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= B || !active[s]) return;
-  // cells: st 0 = (0,0) colour 0, st 1 = (1,0) colour 1
-  const int64_t a = (int64_t)s * 2, b = a + 1;
-  const auto Ca = J[a], Ea = J[2 * plane + a], Wb = J[plane + b], Cb = J[b];
-  double M[4][8];
-  const double blk[4][4] = {{Ca.a00, Ca.a01, Ea.a00, Ea.a01},
-                            {Ca.a10, Ca.a11, Ea.a10, Ea.a11},
-                            {Wb.a00, Wb.a01, Cb.a00, Cb.a01},
-                            {Wb.a10, Wb.a11, Cb.a10, Cb.a11}};
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) {
-      M[i][j] = blk[i][j];
-      M[i][4 + j] = (i == j) ? 1.0 : 0.0;
-    }
-  for (int col = 0; col < 4; ++col) {
-    int piv = col;
-    for (int r = col + 1; r < 4; ++r)
-      if (fabs(M[r][col]) > fabs(M[piv][col])) piv = r;
-    if (piv != col)
-      for (int j = 0; j < 8; ++j) {
-        const double t = M[col][j];
-        M[col][j] = M[piv][j];
-        M[piv][j] = t;
-      }
-    const double inv = 1.0 / M[col][col];
-    for (int j = 0; j < 8; ++j) M[col][j] *= inv;
-    for (int r = 0; r < 4; ++r) {
-      if (r == col) continue;
-      const double f = M[r][col];
-      for (int j = 0; j < 8; ++j) M[r][j] -= f * M[col][j];
-    }
-  }
-  for (int i = 0; i < 4; ++i)
-    for (int j = 0; j < 4; ++j) Ainv[(int64_t)s * 16 + i * 4 + j] = (T)M[i][4 + j];
+  const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3), c = threadIdx.x & 7;
+  const bool on = s < B && active[s];
+  double M[4];
+  coarse_inverse_lanes(J + 2 * (int64_t)(on ? s : 0), plane, c, M);
+  if (on && c >= 4)
+    for (int i = 0; i < 4; ++i) Ainv[(int64_t)s * 16 + i * 4 + c - 4] = (T)M[i];
 }
 
 template <typename T>
@@ -1515,51 +1616,50 @@ __global__ void __launch_bounds__(TPB) k_newton_step_max(int B, int N, double in
 }
 
 // Per sample: theta = min(1, dc_limit / max |dc|) (a step that would change a
-// mass fraction by more than dc_limit is shortened; dc_limit <= 0: theta = 1).
-__global__ void k_newton_theta(int B, int nct, double dc_limit, const double* dc_part,
-                               const int* newton_active, double* __restrict__ theta) {
+// mass fraction by more than dc_limit is shortened; dc_limit <= 0: theta = 1; 0
+// for a sample that does not iterate), and the update test on the full step:
+// at most dxtol ends the sample's iteration with this update.
+__global__ void k_newton_theta(int B, int nct, double dc_limit, const double* dc_part, double dxtol,
+                               const double* dmax_part, int* newton_active, int* status,
+                               double* __restrict__ theta) {
   grid_enter();
   // one warp per sample
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (s >= B || !newton_active[s]) return;
+  if (s >= B) return;
+  if (!newton_active[s]) {
+    if (lane == 0) theta[s] = 0.0;
+    return;
+  }
   double th = 1.0;
   if (dc_limit > 0.0) {
     const double mc = warp_sample_max(dc_part + (int64_t)s * nct, nct, lane);
     if (mc > dc_limit) th = dc_limit / mc;
   }
-  if (lane == 0) theta[s] = th;
-}
-
-// a9: x += theta dx.
-template <typename T>
-__global__ void __launch_bounds__(TPB) k_newton_update(int B, int N, double2* x, const typename VT<T>::v2* dx,
-                                                       const double* theta, const int* newton_active) {
-  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  const int s = blockIdx.x / (unsigned)(N / TPB);
-  grid_enter();
-  if (!newton_active[s]) return;
-  const double th = theta[s];
-  const auto d = dx[e];
-  double2 xx = x[e];
-  xx.x = fma(th, (double)d.x, xx.x);
-  xx.y = fma(th, (double)d.y, xx.y);
-  x[e] = xx;
-}
-
-__global__ void k_newton_dx_check(int B, int nct, double dxtol, const double* dmax_part,
-                                  int* newton_active, int* status) {
-  grid_enter();
-  // one warp per sample
-  const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (s >= B || !newton_active[s]) return;
   const double dm = warp_sample_max(dmax_part + (int64_t)s * nct, nct, lane);
   if (lane != 0) return;
+  theta[s] = th;
   if (!(dm <= 1.0e300)) {
     status[s] = 3;
     newton_active[s] = 0;
   } else if (dm <= dxtol) {
     newton_active[s] = 0;
   }
+}
+
+// a9: x += theta dx.
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_newton_update(int B, int N, double2* x, const typename VT<T>::v2* dx,
+                                                       const double* theta) {
+  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  const int s = blockIdx.x / (unsigned)(N / TPB);
+  grid_enter();
+  const double th = theta[s];
+  if (__double_as_longlong(th) == 0) return;  // the sample does not iterate
+  const auto d = dx[e];
+  double2 xx = x[e];
+  xx.x = fma(th, (double)d.x, xx.x);
+  xx.y = fma(th, (double)d.y, xx.y);
+  x[e] = xx;
 }
 
 // Start of a time step: old state = state; samples that have not failed iterate.
