@@ -1718,8 +1718,8 @@ int ensure_vc_tile_attr() {
   }
   CK(cudaFuncSetAttribute(k_vc_assemble_tile<T, true, true, VC_TILE_NT>,
                           cudaFuncAttributeMaxDynamicSharedMemorySize, vc_tile_smem<true, VC_TILE_NT>()));
-  CK(cudaFuncSetAttribute(k_vc_assemble_tile<T, false, true, VC_TILE_NT>,
-                          cudaFuncAttributeMaxDynamicSharedMemorySize, vc_tile_smem<true, VC_TILE_NT>()));
+  CK(cudaFuncSetAttribute(k_vc_assemble_levels<T, VC_TILE_NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                          vc_tile_smem<true, VC_TILE_NT>()));
   done[dev].store(1, std::memory_order_relaxed);
   return HENRY_OK;
 }
@@ -1788,15 +1788,24 @@ VcLevelArgs vc_args(const typename VcGroup<T>::Lv& L) {
 // States of the coarse levels by injection, level by level (old: the old state).
 template <typename T>
 int vc_inject(henry_handle* H, VcGroup<T>& G, int B, bool old, const int* active, cudaStream_t st) {
+  auto& L0 = G.lv[0];
+  VcInjectLevels A;
+  std::memset(&A, 0, sizeof A);
+  double nv = 0.0;
   for (int k = 1; k <= G.K; ++k) {
-    auto& Lf = G.lv[k - 1];
-    auto& Lc = G.lv[k];
-    launch(H, st, HENRY_K_STATE_RESTRICT, (double)H->nact * Lc.NV * 32.0, [&] {
-      chain(st, nblk((int64_t)B * Lc.NV), TPB, 0, k_vc_inject, B, Lc.nx, Lc.ny, Lf.stride, Lc.stride,
-                                                             old ? Lf.xo : Lf.x, old ? Lc.xo : Lc.x, active);
-    });
-    CKL();
+    auto& L = G.lv[k];
+    const int i = A.n++;
+    A.nx[i] = L.nx;
+    A.ny[i] = L.ny;
+    A.stride[i] = L.stride;
+    A.xc[i] = old ? L.xo : L.x;
+    A.first[i + 1] = A.first[i] + nblk((int64_t)B * L.NV);
+    nv += L.NV;
   }
+  launch(H, st, HENRY_K_STATE_RESTRICT, (double)H->nact * nv * 32.0, [&] {
+    chain(st, A.first[A.n], TPB, 0, k_vc_inject, B, L0.nx, L0.stride, old ? L0.xo : L0.x, A, active);
+  });
+  CKL();
   return HENRY_OK;
 }
 
@@ -1805,17 +1814,40 @@ int vc_inject(henry_handle* H, VcGroup<T>& G, int B, bool old, const int* active
 template <typename T>
 int vc_coarse_ops(henry_handle* H, VcGroup<T>& G, int B, double tau, double inv_s, cudaStream_t st) {
   typedef typename VT<T>::b4 B4;
-  for (int k = 1; k <= G.K; ++k) {
-    auto& L = G.lv[k];
-    launch(H, st, HENRY_K_COARSE_OPS, (double)H->nact * L.NV * (32.0 + 10.0 * sizeof(B4)), [&] {
-      vc_assemble_launch<T, false>(H->cfg, st, vc_params<T>(H->cfg, L, tau), G.coef, B, L.stride, L.plane, inv_s, L.x,
-                                   L.xo, G.lin_active, nullptr, (B4*)L.J, nullptr);
+  if (vc_use_tile(H->cfg)) {  // every level in one launch
+    VcAssembleLevels A;
+    std::memset(&A, 0, sizeof A);
+    double nv = 0.0;
+    for (int k = 1; k <= G.K; ++k) {
+      auto& L = G.lv[k];
+      const int i = A.n++;
+      A.P[i] = vc_params<T>(H->cfg, L, tau);
+      A.stride[i] = L.stride;
+      A.plane[i] = L.plane;
+      A.x[i] = L.x;
+      A.xo[i] = L.xo;
+      A.J[i] = L.J;
+      A.first[i + 1] = A.first[i] + nblk((int64_t)B * L.stride, VC_TILE_NT);
+      nv += L.NV;
+    }
+    launch(H, st, HENRY_K_COARSE_OPS, (double)H->nact * nv * (32.0 + 10.0 * sizeof(B4)), [&] {
+      chain(st, A.first[A.n], VC_TILE_NT, vc_tile_smem<true, VC_TILE_NT>(), k_vc_assemble_levels<T, VC_TILE_NT>, G.coef, A,
+            B, inv_s, G.lin_active);
     });
     CKL();
+  } else {
+    for (int k = 1; k <= G.K; ++k) {
+      auto& L = G.lv[k];
+      launch(H, st, HENRY_K_COARSE_OPS, (double)H->nact * L.NV * (32.0 + 10.0 * sizeof(B4)), [&] {
+        vc_assemble_launch<T, false>(H->cfg, st, vc_params<T>(H->cfg, L, tau), G.coef, B, L.stride, L.plane, inv_s, L.x,
+                                     L.xo, G.lin_active, nullptr, (B4*)L.J, nullptr);
+      });
+      CKL();
+    }
   }
   auto& Lc = G.lv[G.K];
   launch(H, st, HENRY_K_COARSE_OPS, (double)H->nact * (9.0 * 6 * sizeof(B4) + 144.0 * sizeof(T)), [&] {
-    chain(st, nblk(B, 64), 64, 0, k_vc_coarse_inverse<T>, B, vc_args<T>(Lc), (const B4*)Lc.J, G.Ainv, G.lin_active);
+    chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_vc_coarse_inverse<T>, B, vc_args<T>(Lc), (const B4*)Lc.J, G.Ainv, G.lin_active);
   });
   CKL();
   return HENRY_OK;

@@ -156,23 +156,20 @@ __device__ __forceinline__ void vc_eval_face(const VcParams& P, const VcCoef& C,
   vc_face<JAC>(P, C, p, c, f, ih, r.F, r.dF, r.G, r.dG);
 }
 
-template <typename T, bool FINE, bool JAC = true, int NT = 128>
-__global__ void __launch_bounds__(NT) k_vc_assemble_tile(VcParams P, const Coef* __restrict__ coef, int B,
-                                                          int stride, int64_t plane, double inv_s,
-                                                          const double2* x, const double2* xo,
-                                                          const int* active, double2* __restrict__ F,
-                                                          typename VT<T>::b4* __restrict__ J,
-                                                          double* __restrict__ rmax_part) {
+template <typename T, bool FINE, bool JAC, int NT>
+__device__ __forceinline__ void vc_assemble_tile(unsigned blk, const VcParams& P, const Coef* __restrict__ coef, int B,
+                                                 int stride, int64_t plane, double inv_s, const double2* x,
+                                                 const double2* xo, const int* active, double2* __restrict__ F,
+                                                 typename VT<T>::b4* __restrict__ J, double* __restrict__ rmax_part) {
   typedef typename VT<T>::b4 B4;
   typedef VcFaceRec<JAC> Rec;
   extern __shared__ __align__(16) unsigned char vc_smem[];
   Rec* rec = reinterpret_cast<Rec*>(vc_smem);  // [4][NT]: E1, E2, N1, N2
   __shared__ double sh[40];
   const int nxv = P.nx + 1, NV = nxv * (P.ny + 1);
-  const int64_t t0 = (int64_t)blockIdx.x * NT;
+  const int64_t t0 = (int64_t)blk * NT;
   const int64_t e = t0 + threadIdx.x;
   const int s = (int)(e / stride);
-  grid_enter();
   if (FINE) {
     if (!active[s]) return;  // uniform over the CTA (stride % NT == 0)
   }
@@ -278,27 +275,68 @@ __global__ void __launch_bounds__(NT) k_vc_assemble_tile(VcParams P, const Coef*
   }
 }
 
+template <typename T, bool FINE, bool JAC = true, int NT = 128>
+__global__ void __launch_bounds__(NT) k_vc_assemble_tile(VcParams P, const Coef* __restrict__ coef, int B,
+                                                          int stride, int64_t plane, double inv_s,
+                                                          const double2* x, const double2* xo,
+                                                          const int* active, double2* __restrict__ F,
+                                                          typename VT<T>::b4* __restrict__ J,
+                                                          double* __restrict__ rmax_part) {
+  grid_enter();
+  vc_assemble_tile<T, FINE, JAC, NT>(blockIdx.x, P, coef, B, stride, plane, inv_s, x, xo, active, F, J, rmax_part);
+}
+// All coarse levels in one launch (as k_assemble_levels: one level's assembly
+// is a dependent chain of some 700 FP64 operations, 25 us whatever its size).
+struct VcAssembleLevels {
+  static constexpr int MAX = 16;
+  int n;
+  unsigned first[MAX + 1];
+  VcParams P[MAX];
+  int stride[MAX];
+  int64_t plane[MAX];
+  const double2 *x[MAX], *xo[MAX];
+  void* J[MAX];
+};
+template <typename T, int NT = 128>
+__global__ void __launch_bounds__(NT) k_vc_assemble_levels(const Coef* __restrict__ coef,
+                                                            const __grid_constant__ VcAssembleLevels A, int B,
+                                                            double inv_s, const int* active) {
+  grid_enter();
+  int l = 0;
+  while (l + 1 < A.n && blockIdx.x >= A.first[l + 1]) ++l;
+  vc_assemble_tile<T, false, true, NT>(blockIdx.x - A.first[l], A.P[l], coef, B, A.stride[l], A.plane[l], inv_s, A.x[l],
+                                       A.xo[l], active, nullptr, (typename VT<T>::b4*)A.J[l], nullptr);
+}
+
 // Dynamic shared memory of k_vc_assemble_tile.
 template <bool JAC, int NT = 128>
 constexpr int vc_tile_smem() {
   return 4 * NT * (int)sizeof(VcFaceRec<JAC>);
 }
 
-// Coarse states by injection: x_c(J, I) = x_f(2J, 2I), for the iterate and
-// (old != 0) the old state.
-__global__ void __launch_bounds__(TPB) k_vc_inject(int B, int ncx, int ncy, int stride_f, int stride_c,
-                                                   const double2* xf, double2* __restrict__ xc,
-                                                   const int* active) {
+// Coarse states by injection, every level in one launch: level k's vertex (J,
+// I) is the fine vertex (2^k J, 2^k I).
+struct VcInjectLevels {
+  static constexpr int MAX = 16;
+  int n;
+  unsigned first[MAX + 1];
+  int nx[MAX], ny[MAX], stride[MAX];
+  double2* xc[MAX];
+};
+__global__ void __launch_bounds__(TPB) k_vc_inject(int B, int nfx, int stride_f, const double2* xf,
+                                                   const __grid_constant__ VcInjectLevels A, const int* active) {
   grid_enter();
-  const int ncxv = ncx + 1, NVc = ncxv * (ncy + 1), nfxv = 2 * ncx + 1;
-  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  int l = 0;
+  while (l + 1 < A.n && blockIdx.x >= A.first[l + 1]) ++l;
+  const int ncxv = A.nx[l] + 1, NVc = ncxv * (A.ny[l] + 1), r = nfx / A.nx[l];
+  const int64_t e = (int64_t)(blockIdx.x - A.first[l]) * TPB + threadIdx.x;
   if (e >= (int64_t)B * NVc) return;
   const int s = (int)(e / NVc);
   if (!active[s]) return;
   const int stc = (int)(e - (int64_t)s * NVc);
   int J, I;
   vxy(stc, ncxv, J, I);
-  xc[(int64_t)s * stride_c + stc] = xf[(int64_t)s * stride_f + vst(2 * J, 2 * I, nfxv)];
+  A.xc[l][(int64_t)s * A.stride[l] + stc] = xf[(int64_t)s * stride_f + vst(r * J, r * I, nfx + 1)];
 }
 
 // r = b - sum over the 9 blocks A_q x_nb for vertex (j, i) (sample-relative arrays).
@@ -459,54 +497,34 @@ __global__ void __launch_bounds__(TPB) k_vc_prolong_add(int B, VcLevelArgs Lf, V
 }
 
 // Coarsest grid (2 x 1 elements, 3 x 2 vertices, 12 unknowns u = 2 (j 3 + i)
-// + var): the dense matrix from the 9-point blocks, inverted per sample by
-// Gauss-Jordan elimination with partial pivoting in FP64; Ainv[s][12][12].
+// + var): the dense matrix from the 9-point blocks, inverted by one warp per
+// sample (gauss_jordan_lanes); Ainv[s][12][12].  One thread per sample, its
+// 12 x 24 matrix in local memory, was 3/5 of the coarse operators' time.
 template <typename T>
 __global__ void k_vc_coarse_inverse(int B, VcLevelArgs L, const typename VT<T>::b4* J,
                                     T* __restrict__ Ainv, const int* active) {
   grid_enter();
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= B || !active[s]) return;
+  const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), c = threadIdx.x & 31;
   constexpr int n = VC_COARSE_N;
-  double M[n][2 * n];
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < 2 * n; ++c) M[r][c] = (c - n == r) ? 1.0 : 0.0;
-  const int64_t base = (int64_t)s * L.stride;
-  for (int j = 0; j < 2; ++j)
-    for (int i = 0; i < 3; ++i) {
-      const int st = vst(j, i, 3), row = 2 * (j * 3 + i);
-      for (int q = 0; q < 9; ++q) {
-        const int jj = j + q / 3 - 1, ii = i + q % 3 - 1;
-        if (jj < 0 || jj >= 2 || ii < 0 || ii >= 3) continue;
-        const auto blk = J[q * L.plane + base + st];
-        const int col = 2 * (jj * 3 + ii);
-        M[row][col] = (double)blk.a00;
-        M[row][col + 1] = (double)blk.a01;
-        M[row + 1][col] = (double)blk.a10;
-        M[row + 1][col + 1] = (double)blk.a11;
-      }
-    }
-  for (int col = 0; col < n; ++col) {
-    int piv = col;
-    for (int r = col + 1; r < n; ++r)
-      if (fabs(M[r][col]) > fabs(M[piv][col])) piv = r;
-    if (piv != col)
-      for (int c = 0; c < 2 * n; ++c) {
-        const double tt = M[col][c];
-        M[col][c] = M[piv][c];
-        M[piv][c] = tt;
-      }
-    const double inv = 1.0 / M[col][col];
-    for (int c = 0; c < 2 * n; ++c) M[col][c] *= inv;
-    for (int r = 0; r < n; ++r) {
-      if (r == col) continue;
-      const double f = M[r][col];
-      if (f != 0.0)
-        for (int c = 0; c < 2 * n; ++c) M[r][c] -= f * M[col][c];
+  if (s >= B || !active[s]) return;  // uniform over the warp
+  double M[n];
+#pragma unroll
+  for (int r = 0; r < n; ++r) M[r] = c - n == r ? 1.0 : 0.0;
+  if (c < n) {  // column c: vertex (jc, ic), unknown var, in the rows of every vertex next to it
+    const int jc = (c >> 1) / 3, ic = (c >> 1) - 3 * jc, var = c & 1;
+    const int64_t base = (int64_t)s * L.stride;
+#pragma unroll
+    for (int v = 0; v < 6; ++v) {
+      const int j = v / 3, i = v % 3, dj = jc - j, di = ic - i;
+      if (di < -1 || di > 1) continue;
+      const auto blk = J[((dj + 1) * 3 + di + 1) * L.plane + base + vst(j, i, 3)];
+      M[2 * v] = (double)(var ? blk.a01 : blk.a00);
+      M[2 * v + 1] = (double)(var ? blk.a11 : blk.a10);
     }
   }
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < n; ++c) Ainv[(int64_t)s * n * n + r * n + c] = (T)M[r][n + c];
+  gauss_jordan_lanes<n, 32>(M);
+  if (c >= n && c < 2 * n)
+    for (int r = 0; r < n; ++r) Ainv[(int64_t)s * n * n + r * n + c - n] = (T)M[r];
 }
 
 template <typename T>
