@@ -910,24 +910,30 @@ int tail_level(const henry_config& c, const Group<T>& G, int B) {
 }
 
 // Launch one half-sweep of colour col (MODE as in sweep_cell) of a level.
+// b_is_new: the kernel before wrote b or the flags.
 template <typename T, int MODE>
 void launch_sweep(int mg_threads, int B, const Level& L, int col, const typename VT<T>::b4* J,
                   const typename VT<T>::v2* b, typename VT<T>::v2* x, const typename VT<T>::v2* xc, const int* act,
-                  cudaStream_t st) {
+                  cudaStream_t st, bool b_is_new = false) {
   const int64_t hn = (int64_t)B * L.N / 2;  // swept cells
   with_mg_threads(mg_cta<T>(mg_threads, hn), [&](auto nt) {
     constexpr int NT = decltype(nt)::value;
     with_preload(hn, [&](auto pre) {
-      chain(st, nblk(hn, NT), NT, 0, k_sweep<T, MODE, NT, decltype(pre)::value>, B, L.nx, L.ny, col, J, L.plane, b, x,
-            xc, act);
+      constexpr int PRE = decltype(pre)::value ? 1 : 0;
+      auto* k = &k_sweep<T, MODE, NT, PRE>;
+      if constexpr (PRE && MODE == 1)
+        if (b_is_new) k = &k_sweep<T, MODE, NT, 2>;
+      chain(st, nblk(hn, NT), NT, 0, k, B, L.nx, L.ny, col, J, L.plane, b, x, xc, act);
     });
   });
 }
 
-// One V(nu1, nu2) cycle: x0 = M^{-1} b0 on the fine level (active = lin_active).
+// One V(nu1, nu2) cycle: x0 = M^{-1} b0 on the fine level (active =
+// lin_active).  first_done: the caller has done the fine level's first red
+// half-sweep (k_bicg_p, k_bicg_s).
 template <typename T>
 int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, typename VT<T>::v2* x0,
-           cudaStream_t st, const void* J0 = nullptr) {
+           cudaStream_t st, const void* J0 = nullptr, bool first_done = false) {
   typedef typename VT<T>::v2 V2;
   typedef typename VT<T>::b4 B4;
   const int nu1 = H->cfg.nu1, nu2 = H->cfg.nu2;
@@ -945,14 +951,17 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
     const double hc = na * L.N / 2;  // swept cells per half-sweep
     const int sm = k == 0 ? HENRY_K_SMOOTH : HENRY_K_SMOOTH_COARSE;
     Level& Lc = G.lv[k + 1];
+    bool b_is_new = k == 0 && first_done;
     auto sweep = [&](int col, auto mode) {
-      launch_sweep<T, decltype(mode)::value>(mnt, B, L, col, J, b, x, nullptr, act, st);
+      launch_sweep<T, decltype(mode)::value>(mnt, B, L, col, J, b, x, nullptr, act, st, b_is_new);
     };
     if (nu1 > 0) {
-      launch(H, st, sm, hc * (b4 + 2 * v2), na * sweep_flops(L.nx, L.ny, 0),
-             [&] { sweep(0, std::integral_constant<int, 0>()); });
+      if (k > 0 || !first_done)
+        launch(H, st, sm, hc * (b4 + 2 * v2), na * sweep_flops(L.nx, L.ny, 0),
+               [&] { sweep(0, std::integral_constant<int, 0>()); });
       launch(H, st, sm, hc * (5 * b4 + 3 * v2), na * sweep_flops(L.nx, L.ny, 1),
              [&] { sweep(1, std::integral_constant<int, 1>()); });
+      b_is_new = false;
       for (int i = 1; i < nu1; ++i) {
         for (int col = 0; col < 2; ++col)
           launch(H, st, sm, hc * (5 * b4 + 3 * v2), na * sweep_flops(L.nx, L.ny, 1),
@@ -1004,6 +1013,7 @@ int vcycle(henry_handle* H, Group<T>& G, int B, const typename VT<T>::v2* b0, ty
     A.x = kt == 0 ? (void*)x0 : G.lv[kt].mgx;
     A.ainv = G.Ainv;
     A.active = act;
+    A.late = kt == 0;
     A.nu1 = nu1;
     A.nu2 = nu2;
     launch(H, st, HENRY_K_MG_TAIL, na * tb, na * (tf + 32.0), [&] {
@@ -1240,17 +1250,27 @@ struct Krylov : KrylovDrive<Krylov<T>> {
   int N;
   unsigned g;
   double* fin;  // large grids: each sample's partials reduced once, not in every CTA of the consumer kernel
+  const B4* Ci;     // the preconditioner's fine plane of inverse centre blocks
+  bool first;       // the cycles' first red half-sweep is done by k_bicg_p and k_bicg_s
+  bool black_known; // the cycles leave A x = b on the black cells (ended by a black sweep on the matvec's operator)
 
   Krylov(henry_handle* h, Group<T>& grp, int b, const void* jpre0, double rtol, int mi)
       : H(h), G(grp), B(b), Jpre0(jpre0), rtol2(rtol * rtol), maxit(mi), L(grp.lv[0]), N(grp.lv[0].N),
         g(nblk((int64_t)b * grp.lv[0].N)),
-        fin((h->cfg.finalize_nct > 0 && grp.nct >= h->cfg.finalize_nct) ? grp.fin : nullptr) {}
+        fin((h->cfg.finalize_nct > 0 && grp.nct >= h->cfg.finalize_nct) ? grp.fin : nullptr) {
+    Ci = (const B4*)(Jpre0 ? Jpre0 : L.J) + 5 * L.plane;
+    first = H->cfg.nu1 > 0 && tail_level<T>(H->cfg, G, B) != 0;
+    black_known = H->cfg.nu2 > 0 && !Jpre0;
+  }
 
   void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
            [&] { chain(ss, nblk((int64_t)B * 32, 128), 128, 0, k_finalize, B, G.nct, G.part, a, b, fin); });
   }
+  // Bytes of the matvec and of a first half-sweep per cell.
+  double spmv_bytes() const { return (black_known ? 0.5 : 1.0) * 5 * sizeof(B4) + 3 * sizeof(V2); }
+  double first_bytes() const { return first ? 0.5 * (sizeof(B4) + sizeof(V2)) : 0.0; }
   int init(cudaStream_t st, int* loop) {
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * sizeof(V2)), [&] {
       chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, loop);
@@ -1262,9 +1282,13 @@ struct Krylov : KrylovDrive<Krylov<T>> {
   // The convergence test and the new search direction of iteration `it` (or
   // *it_dev), counting the samples that go on in G.counter[1].
   int head(int it, const int* it_dev, cudaStream_t st) {
-    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * sizeof(V2), [&] {
-      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
-            G.iters, G.status, G.counter + 1, G.totals + 1, fin);
+    launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * ((it == 0 ? 2 : 4) * sizeof(V2) + first_bytes()), [&] {
+      auto go = [&](auto* k) {
+        chain(st, g, TPB, 0, k, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
+              G.status, G.counter + 1, G.totals + 1, fin, Ci, G.ph, L.nx);
+      };
+      if (first) go(&k_bicg_p<T, true>);
+      else go(&k_bicg_p<T, false>);
     });
     CKL();
     return HENRY_OK;
@@ -1273,25 +1297,30 @@ struct Krylov : KrylovDrive<Krylov<T>> {
   // updates (every argument fixed for this group and B; the samples' activity
   // is read from lin_active on the device).
   int body(int n_act, cudaStream_t ss) {
-    const double nc = (double)n_act * N, b4 = sizeof(B4), v2 = sizeof(V2);
-    int rc = vcycle<T>(H, G, B, G.p, G.ph, ss, Jpre0);
+    const double nc = (double)n_act * N, v2 = sizeof(V2);
+    int rc = vcycle<T>(H, G, B, G.p, G.ph, ss, Jpre0, first);
     if (rc) return rc;
-    launch(H, ss, HENRY_K_SPMV, nc * (5 * b4 + 3 * v2), n_act * spmv_flops(L.nx, L.ny, 1), [&] {
+    launch(H, ss, HENRY_K_SPMV, nc * spmv_bytes(), n_act * spmv_flops(L.nx, L.ny, 1), [&] {
       with_preload((int64_t)B * N, [&](auto pre) {
         chain(ss, g, TPB, 0, k_spmv<T, 1, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.ph, G.v, G.rh,
-              G.part, P_RV, 0, G.lin_active);
+              G.part, P_RV, 0, G.lin_active, black_known ? G.p : nullptr);
       });
     });
     finalize(P_RV, -1, ss);
-    launch(H, ss, HENRY_K_KRYLOV, nc * 3 * v2,
-           [&] { chain(ss, g, TPB, 0, k_bicg_s<T>, B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin); });
+    launch(H, ss, HENRY_K_KRYLOV, nc * (3 * v2 + first_bytes()), [&] {
+      auto go = [&](auto* k) {
+        chain(ss, g, TPB, 0, k, B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin, Ci, G.sh, L.nx);
+      };
+      if (first) go(&k_bicg_s<T, true>);
+      else go(&k_bicg_s<T, false>);
+    });
     CKL();
-    rc = vcycle<T>(H, G, B, G.s, G.sh, ss, Jpre0);
+    rc = vcycle<T>(H, G, B, G.s, G.sh, ss, Jpre0, first);
     if (rc) return rc;
-    launch(H, ss, HENRY_K_SPMV, nc * (5 * b4 + 3 * v2), n_act * spmv_flops(L.nx, L.ny, 2), [&] {
+    launch(H, ss, HENRY_K_SPMV, nc * spmv_bytes(), n_act * spmv_flops(L.nx, L.ny, 2), [&] {
       with_preload((int64_t)B * N, [&](auto pre) {
         chain(ss, g, TPB, 0, k_spmv<T, 2, decltype(pre)::value>, B, L.nx, L.ny, (const B4*)L.J, L.plane, G.sh, G.t, G.s,
-              G.part, P_TS, P_TT, G.lin_active);
+              G.part, P_TS, P_TT, G.lin_active, black_known ? G.s : nullptr);
       });
     });
     finalize(P_TS, P_TT, ss);
@@ -2008,8 +2037,8 @@ struct VcKrylov : KrylovDrive<VcKrylov<T>> {
   }
   int head(int it, const int* it_dev, cudaStream_t st) {
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * sizeof(V2), [&] {
-      chain(st, g, TPB, 0, k_bicg_p<T>, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
-            G.iters, G.status, G.counter + 1, G.totals + 1, fin);
+      chain(st, g, TPB, 0, k_bicg_p<T, false>, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
+            G.iters, G.status, G.counter + 1, G.totals + 1, fin, (const B4*)nullptr, (V2*)nullptr, 0);
     });
     CKL();
     return HENRY_OK;
@@ -2024,7 +2053,10 @@ struct VcKrylov : KrylovDrive<VcKrylov<T>> {
     });
     finalize(P_RV, -1, ss);
     launch(H, ss, HENRY_K_KRYLOV, nc * 3 * v2,
-           [&] { chain(ss, g, TPB, 0, k_bicg_s<T>, B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin); });
+           [&] {
+             chain(ss, g, TPB, 0, k_bicg_s<T, false>, B, N, G.r, G.v, G.s, G.part, G.sc, G.lin_active, fin,
+                   (const B4*)nullptr, (V2*)nullptr, 0);
+           });
     CKL();
     rc = vc_vcycle<T>(H, G, B, G.s, G.sh, ss);
     if (rc) return rc;
@@ -2613,7 +2645,7 @@ int step_entry(henry_handle* H, int which, int level, const double* xi, int n, c
     case 1:  // apply
       chain(st, nblk(n0), TPB, 0, k_to_storage<V2>, n, L.nx, L.ny, (const double2*)in, G->p);
       chain(st, nblk(n0), TPB, 0, k_spmv<T, 0>, n, L.nx, L.ny, (const B4*)L.J, L.plane, G->p, G->v, nullptr, nullptr, 0,
-            0, G->lin_active);
+            0, G->lin_active, nullptr);
       chain(st, nblk(n0), TPB, 0, k_from_storage<V2>, n, L.nx, L.ny, G->v, (double2*)out);
       break;
     case 2:  // precondition

@@ -60,6 +60,7 @@ struct Coef {
 // Per-sample scalars of BiCGStab.
 struct LinScal {
   double rho, alpha, omega, bnorm2;
+  double aow;  // alpha / omega
 };
 
 // Partial-sum slots of the fine-level reductions: [q][B][nct].
@@ -151,6 +152,23 @@ __device__ __forceinline__ double block_sum_tree(double v, double* sh) {
   __syncthreads();
   return sh[n];
 }
+// Two such sums side by side (CTAs of TPB threads, the same order of additions
+// each): the halves of the CTA take one each, so that their dependent
+// additions - 8 of 64 cycles - run on different warps.  The first sum is
+// returned to thread 0, the second to thread TPB / 2.  sh: 2 TPB doubles.
+__device__ __forceinline__ double block_sum_pair(double v1, double v2, double* sh) {
+  const int t = threadIdx.x, u = t & (TPB / 2 - 1);
+  sh[t] = v1;
+  sh[TPB + t] = v2;
+  __syncthreads();
+  double* q = sh + (t >= TPB / 2 ? TPB : 0);
+#pragma unroll
+  for (int s = TPB / 2; s >= 32; s >>= 1) {
+    if (u < s) q[u] += q[u + s];
+    __syncthreads();
+  }
+  return u < 32 ? warp_sum(q[u]) : 0.0;
+}
 // CTA-wide max of non-negative doubles without NaNs (+inf allowed) on the
 // integer pipes: for such values the IEEE-754 bit patterns order like the
 // values, so the max of the 64-bit patterns is the max of the values (the
@@ -179,26 +197,28 @@ __device__ __forceinline__ double block_max_nonneg(double v, double* sh) {
   __syncthreads();
   return __longlong_as_double((long long)su[32]);
 }
-// Sum of a sample's nct partials, computed identically by every CTA of the
-// sample (fixed order), returned to every thread.
-__device__ __forceinline__ double sample_sum(const double* p, int nct, double* sh) {
-  double v = 0.0;
-  if (threadIdx.x < 32) {
-    for (int i = threadIdx.x; i < nct; i += 32) v += p[i];
+// Two sums over a sample's nct partials (slots a and b), computed identically
+// by every CTA of the sample: warps 0 and 1 take one each, in a fixed order.
+// fin (large grids): the finalised per-sample values instead (one warp per
+// sample summed the partials in the same order).
+__device__ __forceinline__ void sample_sums(const double* part, const double* fin, int a, int b, int64_t stride, int s,
+                                            int nct, double* sh, double& va, double& vb) {
+  if (fin) {
+    va = fin[(int64_t)s * NPART + a];
+    vb = fin[(int64_t)s * NPART + b];
+    return;
+  }
+  const int w = threadIdx.x >> 5;
+  if (w < 2) {
+    const double* p = part + (w == 0 ? a : b) * stride + (int64_t)s * nct;
+    double v = 0.0;
+    for (int i = threadIdx.x & 31; i < nct; i += 32) v += p[i];
     v = warp_sum(v);
-    if (threadIdx.x == 0) sh[33] = v;
+    if ((threadIdx.x & 31) == 0) sh[w] = v;
   }
   __syncthreads();
-  v = sh[33];
-  __syncthreads();
-  return v;
-}
-// The same sum read from the finalised per-sample values when `fin` is set
-// (large grids: one warp per sample summed the partials in the same order).
-__device__ __forceinline__ double sample_sum_or_fin(const double* part, const double* fin,
-                                                    int slot, int64_t stride, int s, int nct, double* sh) {
-  if (fin) return fin[(int64_t)s * NPART + slot];
-  return sample_sum(part + slot * stride + (int64_t)s * nct, nct, sh);
+  va = sh[0];
+  vb = sh[1];  // the caller's next barrier comes before sh is written again
 }
 // One warp per sample: fin[s][slot] = sum of the sample's partials of up to
 // two slots (slot_b < 0: one), in the order sample_sum uses.
@@ -1049,10 +1069,12 @@ __device__ __forceinline__ typename VT<T>::v2 sweep_cell(int nx, int ny, int ix,
 // NT: threads per CTA (any multiple of 32 up to 1024; every thread owns one
 // cell).  Every sweep but the first of a level (MODE 0) follows another kernel
 // of the cycle, so its blocks and right-hand side are complete when it starts.
-// PRE: they are loaded before the wait, which leaves only the neighbours' x on
-// the critical path of a small launch but takes 76 registers instead of 32 in
-// FP64; the rule stands at preload (henry_engine.cu).
-template <typename T, int MODE, int NT = TPB, bool PRE = false>
+// PRE = 1: they are loaded before the wait, which leaves only the neighbours' x
+// on the critical path of a small launch but takes 76 registers instead of 32
+// in FP64; the rule stands at with_preload (henry_engine.cu).  PRE = 2: the
+// blocks alone, where b and the flags come from the kernel before (the black
+// sweep after k_bicg_p or k_bicg_s has done the red one).
+template <typename T, int MODE, int NT = TPB, int PRE = 0>
 __global__ void __launch_bounds__(NT) k_sweep(int B, int nx, int ny, int col, const typename VT<T>::b4* __restrict__ J,
                                                int64_t plane, const typename VT<T>::v2* b,
                                                typename VT<T>::v2* x, const typename VT<T>::v2* xc,
@@ -1074,7 +1096,7 @@ __global__ void __launch_bounds__(NT) k_sweep(int B, int nx, int ny, int col, co
     x[base + i] = sweep_cell<T, MODE>(nx, ny, ix, iy, i, J + base, plane, b + base, x + base,
                                       MODE == 2 ? xc + (int64_t)s * (N >> 2) : nullptr);
   } else {
-    const bool on = in && active[s];
+    bool on = in && (PRE == 2 || active[s]);
     const bool has[4] = {ix > 0, ix + 1 < nx, iy > 0, iy + 1 < ny};
     B4 A[4], Ci;
     V2 bb = mk2<V2>((T)0, (T)0);
@@ -1084,10 +1106,12 @@ __global__ void __launch_bounds__(NT) k_sweep(int B, int nx, int ny, int col, co
       for (int k = 0; k < 4; ++k)
         if (has[k]) A[k] = Js[(k + 1) * plane];
       Ci = Js[5 * plane];
-      bb = b[base + i];
+      if (PRE == 1) bb = b[base + i];
     }
     grid_enter();
+    if (PRE == 2) on = on && active[s];
     if (!on) return;
+    if (PRE == 2) bb = b[base + i];
     // sweep_cell's arithmetic
     const V2* xs = x + base;
     const V2* xcs = MODE == 2 ? xc + (int64_t)s * (N >> 2) : nullptr;
@@ -1282,26 +1306,46 @@ __device__ __forceinline__ typename VT<T>::v2 spmv_cell(int nx, int ny, int ix, 
 
 // y = A x (fine level, all cells) with per-CTA partial dot products:
 //   NDOT 1: <w1, y>;  NDOT 2: <w1, y>, <y, y>.
+// b (nullable): x is the result of a V-cycle on this operator for the right-
+// hand side b that ended with a black half-sweep.  Point Gauss-Seidel makes
+// the swept equations hold, (A x)_P = b_P on every black cell, so those cells
+// take b_P and only the red ones form the product: half the operations, and
+// 104 instead of 208 bytes a cell.  A warp's cells then have one colour (on 32
+// cells wide grids the CTA's eight rows are dealt out by colour).  8192 level-0
+// samples, FP64: 145 -> 94 us a call; with the first red half-sweeps in the
+// BiCGStab kernels the solve takes 364 instead of 386 ms (level 2 with
+// partners, 33 samples: 168 and 176 ms; level-3 mixed, 20 samples: 278 and 292).
 // PRE as in k_sweep (the kernel follows the sweep that ends a V-cycle).
 template <typename T, int NDOT, bool PRE = false>
 __global__ void __launch_bounds__(TPB) k_spmv(int B, int nx, int ny, const typename VT<T>::b4* __restrict__ J,
                                               int64_t plane, const typename VT<T>::v2* x,
                                               typename VT<T>::v2* __restrict__ y,
                                               const typename VT<T>::v2* w1, double* __restrict__ part,
-                                              int slot1, int slot2, const int* active) {
+                                              int slot1, int slot2, const int* active,
+                                              const typename VT<T>::v2* b) {
   typedef typename VT<T>::v2 V2;
   typedef typename VT<T>::b4 B4;
-  __shared__ double sh[TPB + 1];
+  __shared__ double sh[NDOT == 2 ? 2 * TPB : TPB + 1];
   const int N = nx * ny, nct = N / TPB;
-  const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
+  int lt = threadIdx.x;
+  if (b && nx == 32) lt = ((lt & 0x70) << 1) | ((lt >> 7) << 4) | (lt & 15);  // (colour, row, j) -> (row, colour, j)
+  const int64_t e = (int64_t)blockIdx.x * TPB + lt;
   const int s = sample_of(e, N);
   const bool on = active[s];  // uniform over the CTA
   const int st = (int)(e - (int64_t)s * N);
   int ix, iy;
   xy_of(st, nx, ix, iy);
   const int64_t base = e - st;
+  const bool black = b && (st & (nx - 1)) >= (nx >> 1);
   V2 ww = mk2<V2>((T)0, (T)0), yy;
-  if constexpr (PRE) {
+  if (black) {  // uniform over the warp
+    if (on) {
+      yy = b[e];
+      if (NDOT >= 1 && part) ww = w1[e];
+    }
+    grid_enter();
+    if (!on) return;
+  } else if constexpr (PRE) {
     const bool has[4] = {ix > 0, ix + 1 < nx, iy > 0, iy + 1 < ny};
     B4 A[5];
     if (on) {
@@ -1334,13 +1378,15 @@ __global__ void __launch_bounds__(TPB) k_spmv(int B, int nx, int ny, const typen
   y[e] = yy;
   if (NDOT >= 1 && part) {
     // per-cell products in T, widened once for the FP64 CTA reduction
-    const double d1 = block_sum_tree((double)fma_(ww.x, yy.x, ww.y * yy.y), sh);
-    double d2 = 0.0;
-    if (NDOT == 2) d2 = block_sum_tree((double)fma_(yy.x, yy.x, yy.y * yy.y), sh);
-    if (threadIdx.x == 0) {
-      const int64_t pi = (int64_t)s * nct + st / TPB, stride = (int64_t)B * nct;
-      part[slot1 * stride + pi] = d1;
-      if (NDOT == 2) part[slot2 * stride + pi] = d2;
+    const double w1y = (double)fma_(ww.x, yy.x, ww.y * yy.y);
+    const int64_t pi = (int64_t)s * nct + st / TPB, stride = (int64_t)B * nct;
+    if (NDOT == 2) {
+      const double d = block_sum_pair(w1y, (double)fma_(yy.x, yy.x, yy.y * yy.y), sh);
+      if (threadIdx.x == 0) part[slot1 * stride + pi] = d;
+      if (threadIdx.x == TPB / 2) part[slot2 * stride + pi] = d;
+    } else {
+      const double d = block_sum_tree(w1y, sh);
+      if (threadIdx.x == 0) part[slot1 * stride + pi] = d;
     }
   }
 }
@@ -1388,15 +1434,29 @@ __global__ void __launch_bounds__(TPB) k_bicg_init(int B, int N, const double2* 
 // A converged sample's CTA 0 clears lin_active; the last iteration counts
 // still-active samples in *n_active and per-sample iterations in iters.  it_dev
 // (nullable): the iteration index in device memory instead of `it`.
+// FIRST: the V-cycle that follows starts with a red half-sweep from zero, x_P =
+// C_P^-1 p_P; it is done here (Ci: the fine operator's plane of inverses, ph
+// the cycle's vector, nx the grid's width), one launch and one pass over the
+// red half of p less.
 template <typename T>
+__device__ __forceinline__ void first_sweep(const typename VT<T>::b4* Ci, typename VT<T>::v2* x, int nx, int64_t e,
+                                            typename VT<T>::v2 b) {
+  if (((int)e & (nx - 1)) >= (nx >> 1)) return;  // black
+  T y0, y1;
+  bmv(Ci[e], b.x, b.y, y0, y1);
+  x[e] = mk2<typename VT<T>::v2>(y0, y1);
+}
+template <typename T, bool FIRST = false>
 __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, const int* it_dev, int maxit, double rtol2,
                                                 const typename VT<T>::v2* r, typename VT<T>::v2* p,
                                                 const typename VT<T>::v2* v, const double* part, LinScal* sc,
                                                 int* lin_active, int* __restrict__ iters,
                                                 int* __restrict__ status, int* __restrict__ n_active,
-                                                unsigned long long* __restrict__ lin_total, const double* fin) {
+                                                unsigned long long* __restrict__ lin_total, const double* fin,
+                                                const typename VT<T>::b4* __restrict__ Ci, typename VT<T>::v2* ph,
+                                                int nx) {
   typedef typename VT<T>::v2 V2;
-  __shared__ double sh[40];
+  __shared__ double sh[2];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int s = blockIdx.x / (unsigned)nct;
@@ -1405,8 +1465,8 @@ __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, const int*
   if (it_dev) it = *it_dev;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
-  const double rho = sample_sum_or_fin(part, fin, P_RR, stride, s, nct, sh);
-  const double rn2 = sample_sum_or_fin(part, fin, P_RN, stride, s, nct, sh);
+  double rho, rn2;
+  sample_sums(part, fin, P_RR, P_RN, stride, s, nct, sh, rho, rn2);
   // The test and the Krylov scalars once per CTA, by thread 0 (an FP64
   // division is a long FP64-pipe sequence, and every thread would compute
   // the same values); bc = (stop code, beta, omega).
@@ -1431,7 +1491,7 @@ __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, const int*
       }
       if (it > 0) {
         const LinScal q = sc[s];
-        bc[1] = (rho / q.rho) * (q.alpha / q.omega);
+        bc[1] = (rho / q.rho) * q.aow;
         bc[2] = q.omega;
       }
     }
@@ -1439,23 +1499,26 @@ __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, const int*
   __syncthreads();
   if (bc[0] != -3.0) return;
   const V2 rr = r[e];
-  if (it == 0) {
-    p[e] = rr;
-    return;
+  V2 pn = rr;
+  if (it > 0) {
+    const V2 pp = p[e], vv = v[e];
+    const T bt = (T)bc[1], om = (T)bc[2];
+    pn = mk2<V2>(rr.x + bt * (pp.x - om * vv.x), rr.y + bt * (pp.y - om * vv.y));
   }
-  const double beta = bc[1], omega = bc[2];
-  const V2 pp = p[e], vv = v[e];
-  const T bt = (T)beta, om = (T)omega;
-  p[e] = mk2<V2>(rr.x + bt * (pp.x - om * vv.x), rr.y + bt * (pp.y - om * vv.y));
+  p[e] = pn;
+  if (FIRST) first_sweep<T>(Ci, ph, nx, e, pn);
 }
 
 // alpha = rho / <r_hat, v>; s = r - alpha v.  CTA 0 stores rho and alpha.
-template <typename T>
+// FIRST as in k_bicg_p.
+template <typename T, bool FIRST = false>
 __global__ void __launch_bounds__(TPB) k_bicg_s(int B, int N, const typename VT<T>::v2* r, const typename VT<T>::v2* v,
                                                 typename VT<T>::v2* __restrict__ sv, const double* part,
-                                                LinScal* sc, const int* lin_active, const double* fin) {
+                                                LinScal* sc, const int* lin_active, const double* fin,
+                                                const typename VT<T>::b4* __restrict__ Ci, typename VT<T>::v2* shv,
+                                                int nx) {
   typedef typename VT<T>::v2 V2;
-  __shared__ double sh[40];
+  __shared__ double sh[2];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int s = blockIdx.x / (unsigned)nct;
@@ -1463,8 +1526,8 @@ __global__ void __launch_bounds__(TPB) k_bicg_s(int B, int N, const typename VT<
   if (!lin_active[s]) return;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
-  const double rho = sample_sum_or_fin(part, fin, P_RR, stride, s, nct, sh);
-  const double rv = sample_sum_or_fin(part, fin, P_RV, stride, s, nct, sh);
+  double rho, rv;
+  sample_sums(part, fin, P_RR, P_RV, stride, s, nct, sh, rho, rv);
   __shared__ double bc;
   if (threadIdx.x == 0) bc = rho / rv;  // once per CTA
   __syncthreads();
@@ -1475,7 +1538,9 @@ __global__ void __launch_bounds__(TPB) k_bicg_s(int B, int N, const typename VT<
   }
   const V2 rr = r[e], vv = v[e];
   const T a = (T)alpha;
-  sv[e] = mk2<V2>(rr.x - a * vv.x, rr.y - a * vv.y);
+  const V2 sn = mk2<V2>(rr.x - a * vv.x, rr.y - a * vv.y);
+  sv[e] = sn;
+  if (FIRST) first_sweep<T>(Ci, shv, nx, e, sn);
 }
 
 // omega = <t, s> / <t, t>; dx += alpha p_hat + omega s_hat; r = s - omega t;
@@ -1488,7 +1553,7 @@ __global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T
                                                      typename VT<T>::v2* __restrict__ r, double* part, LinScal* sc,
                                                      const int* lin_active, const double* fin) {
   typedef typename VT<T>::v2 V2;
-  __shared__ double sh[TPB + 1];
+  __shared__ double sh[2 * TPB];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int s = blockIdx.x / (unsigned)nct;
@@ -1506,8 +1571,8 @@ __global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T
   if (!on) return;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
-  const double ts = sample_sum_or_fin(part, fin, P_TS, stride, s, nct, sh);
-  const double tt = sample_sum_or_fin(part, fin, P_TT, stride, s, nct, sh);
+  double ts, tt;
+  sample_sums(part, fin, P_TS, P_TT, stride, s, nct, sh, ts, tt);
   __shared__ double bc;
   if (threadIdx.x == 0) bc = (tt > 0.0) ? ts / tt : 0.0;  // once per CTA
   __syncthreads();
@@ -1520,13 +1585,11 @@ __global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T
   dx[e] = mk2<V2>(x0.x + a * p0.x + w * s0.x, x0.y + a * p0.y + w * s0.y);
   const V2 rn = mk2<V2>(sv0.x - w * t0.x, sv0.y - w * t0.y);
   r[e] = rn;
-  const double d1 = block_sum_tree((double)fma_(rh0.x, rn.x, rh0.y * rn.y), sh);
-  const double d2 = block_sum_tree((double)fma_(rn.x, rn.x, rn.y * rn.y), sh);
-  if (threadIdx.x == 0) {
-    const int64_t pi = (int64_t)s * nct + ct;
-    part[P_RR * stride + pi] = d1;
-    part[P_RN * stride + pi] = d2;
-  }
+  const double d = block_sum_pair((double)fma_(rh0.x, rn.x, rh0.y * rn.y), (double)fma_(rn.x, rn.x, rn.y * rn.y), sh);
+  const int64_t pi = (int64_t)s * nct + ct;
+  if (threadIdx.x == 0) part[P_RR * stride + pi] = d;
+  if (threadIdx.x == TPB / 2) part[P_RN * stride + pi] = d;
+  if (threadIdx.x == TPB - 1 && ct == 0) sc[s].aow = alpha / omega;
 }
 
 // One thread, after a kernel that counted the samples still iterating in

@@ -45,6 +45,7 @@ struct TailArgs {
   void* x;
   const void* ainv;
   const int* active;
+  int late;  // the kernel before sets the flags (a tail from the fine grid): read them after the wait
   int nu1, nu2;
 };
 
@@ -190,6 +191,7 @@ struct TailLevel {
     T b0, b1;
     if constexpr (FIRST) {
       grid_enter();
+      if (A.late && !A.active[s]) return;
       const T* bg = reinterpret_cast<const T*>(reinterpret_cast<const V2*>(A.b) + (int64_t)s * (NX * NY));
       b0 = bg[2 * st_of(ix0, iy0, NX) + row];
       b1 = bg[2 * st_of(ix1, iy1, NX) + row];
@@ -328,6 +330,7 @@ struct TailWide {
   }
   __device__ __forceinline__ void run(const TailArgs& A, int s, int Q, const T* ainv) {
     grid_enter();
+    if (A.late && !A.active[s]) return;
     const V2* bg = reinterpret_cast<const V2*>(A.b) + (int64_t)s * (NX * NY);
 #pragma unroll
     for (int col = 0; col < 2; ++col)
@@ -417,7 +420,7 @@ __global__ void __launch_bounds__(tail_threads(NX0)) k_vcycle_tail(const __grid_
   extern __shared__ __align__(16) unsigned char tail_smem[];
   V2* sm = reinterpret_cast<V2*>(tail_smem);
   const int s = blockIdx.x;
-  if (s >= B || !A.active[s]) {
+  if (s >= B || (!A.late && !A.active[s])) {
     grid_enter();
     return;
   }
