@@ -545,16 +545,16 @@ size_t bytes_per_sample(const henry_config& c, int level, bool light = false) {
 // host threads; every thread stores the same attribute value)
 std::atomic<int> g_smem_optin[64] = {};
 template <typename T>
-bool fused_eligible(const henry_config& c, int level, CtaLayout* L) {
+bool fused_eligible(const henry_config& c, int level) {
   // 1 (default): only with FP32 linear algebra, where it measured faster; on
-  // GB300 the FP64 variant (one CTA per SM for lack of shared memory) is
-  // FP64-latency bound and slower than the multi-kernel path.  2: always.
+  // GB300 the FP64 variant (one CTA per SM by its registers) keeps an SM's FP64
+  // pipe waiting on one sample's phases.  2: always.
   if (c.fused_small_grids <= 0 || has_fields(c) || c.qoi_set != HENRY_QOI_STANDARD ||
       c.scheme != HENRY_SCHEME_CELL)
     return false;
   if (c.fused_small_grids == 1 && sizeof(T) != sizeof(float)) return false;
   const LevelGeom lg = geom(c, level);
-  if (!cta_layout(lg.nx, lg.ny, (int)sizeof(T), L)) return false;
+  if (lg.nx != CTA_NX || lg.ny != CTA_NY) return false;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
   int optin = g_smem_optin[dev].load(std::memory_order_relaxed);
@@ -562,7 +562,7 @@ bool fused_eligible(const henry_config& c, int level, CtaLayout* L) {
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return false;
     g_smem_optin[dev].store(optin, std::memory_order_relaxed);
   }
-  return L->bytes <= optin;
+  return (int)sizeof(CtaShared<T>) <= optin;
 }
 
 // The device's opt-in shared memory per CTA (cached per device; 0 on error).
@@ -1663,13 +1663,11 @@ __global__ void k_first_bad(int n, const int* __restrict__ status, int* __restri
 // The whole scenario solve of B samples with the fused one-CTA-per-sample
 // kernel (coefficients and status set).
 template <typename T>
-int solve_group_fused(henry_handle* H, Group<T>& G, int B, const CtaLayout& L, double* qoi, cudaStream_t st) {
+int solve_group_fused(henry_handle* H, Group<T>& G, int B, double* qoi, cudaStream_t st) {
   const henry_config& c = H->cfg;
   const LevelGeom lg = geom(c, G.level);
   CtaParams P;
   P.ph = phys_of(c);
-  P.nx0 = lg.nx;
-  P.ny0 = lg.ny;
   P.steps = lg.steps;
   P.nu1 = c.nu1;
   P.nu2 = c.nu2;
@@ -1687,11 +1685,12 @@ int solve_group_fused(henry_handle* H, Group<T>& G, int B, const CtaLayout& L, d
   P.dc_limit = c.newton_dc_limit;
   P.rho0g = c.rho0 * c.g;
   P.Ly = c.Ly;
-  CK(cudaFuncSetAttribute(k_cta_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, L.bytes));
+  CK(cudaFuncSetAttribute(k_cta_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CtaShared<T>)));
   CK(cudaMemsetAsync(G.totals, 0, 4 * sizeof(unsigned long long), st));
   H->nact = B;
   launch(H, st, HENRY_K_FUSED, (double)B * (double)lg.nx * lg.ny * lg.steps * 64.0 + (double)B * 48.0, [&] {
-    k_cta_solve<T><<<B, CTA_THREADS, L.bytes, st>>>(P, L, B, G.coef, G.lv[0].xo, G.xoo, qoi, G.status, G.totals);
+    k_cta_solve<T><<<B, CTA_THREADS, sizeof(CtaShared<T>), st>>>(P, B, G.coef, G.lv[0].xo, G.xoo, qoi, G.status,
+                                                                 G.totals);
   });
   CKL();
   return HENRY_OK;
@@ -2363,8 +2362,7 @@ template <typename T>
 int batch_solve_level(henry_handle* H, int level, const double* xi, int n, double* qoi, int32_t* status, bool first,
                       henry_stats* stats, cudaStream_t st) {
   TuningScope tuning(H, level);
-  CtaLayout CL;
-  const bool fused = fused_eligible<T>(H->cfg, level, &CL);
+  const bool fused = fused_eligible<T>(H->cfg, level);
   const int Bmax = max_batch<T>(H->cfg, level, fused);
   const LevelGeom lg = geom(H->cfg, level);
   for (int off = 0; off < n; off += Bmax) {
@@ -2375,7 +2373,7 @@ int batch_solve_level(henry_handle* H, int level, const double* xi, int n, doubl
     rc = set_coefficients<T>(H, *G, xi + (int64_t)n_inputs(H->cfg) * off, B, st);
     if (rc) return rc;
     const int nq = qoi_count(H->cfg);
-    rc = fused ? solve_group_fused<T>(H, *G, B, CL, qoi + nq * (int64_t)off, st)
+    rc = fused ? solve_group_fused<T>(H, *G, B, qoi + nq * (int64_t)off, st)
                : solve_group<T>(H, *G, B, qoi + nq * (int64_t)off, st);
     if (rc) return rc;
     k_merge_status<<<nblk(B, 128), 128, 0, st>>>(B, G->status, status + off, first ? 1 : 0);
@@ -2874,9 +2872,8 @@ int henry_autotune(henry_handle* h, int level, int with_coarse, const double* xi
   std::vector<henry_tuning> cands;
   const double rts[3] = {1e-4, 1e-3, 1e-2};
   const int nus[3][2] = {{2, 2}, {1, 2}, {2, 1}};
-  CtaLayout CL;
-  const bool can_fuse = (c.precision == HENRY_MIXED ? fused_eligible<float>(c, level, &CL)
-                                                    : fused_eligible<double>(c, level, &CL)) ||
+  const bool can_fuse = (c.precision == HENRY_MIXED ? fused_eligible<float>(c, level)
+                                                    : fused_eligible<double>(c, level)) ||
                         (c.fused_small_grids == 0);
   for (double rt : rts)
     for (auto& nu : nus)
@@ -2950,7 +2947,7 @@ int henry_autotune(henry_handle* h, int level, int with_coarse, const double* xi
   if (best >= 0) {
     henry_config cb = c;
     cb.fused_small_grids = cands[best].fused_small_grids;
-    fused_won = c.precision == HENRY_MIXED ? fused_eligible<float>(cb, level, &CL) : fused_eligible<double>(cb, level, &CL);
+    fused_won = c.precision == HENRY_MIXED ? fused_eligible<float>(cb, level) : fused_eligible<double>(cb, level);
   }
   const bool cc = c.scheme == HENRY_SCHEME_CELL;  // the tail, tile and CTA-size stages are the cell scheme's
   if (!rc && best >= 0 && !fused_won) {

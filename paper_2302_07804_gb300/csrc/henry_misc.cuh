@@ -382,12 +382,6 @@ __global__ void k_permute_rows(int n, int w, const int* __restrict__ perm, const
   if (SCATTER) dst[j * w + k] = src[t];
   else dst[t] = src[j * w + k];
 }
-// Zero the rows perm[i], i in [0, n), of a [*][w] array.
-__global__ void k_zero_rows(int n, int w, const int* __restrict__ perm, double* __restrict__ dst) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)n * w) return;
-  dst[(int64_t)perm[t / w] * w + t % w] = 0.0;
-}
 
 __global__ void __launch_bounds__(TPB) k_scale_d2(int64_t n, double a, double2* x) {
   grid_enter();

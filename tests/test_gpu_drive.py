@@ -105,3 +105,20 @@ def test_vertex_step_graph_equals_host_driven_loops(hl, res_first, every, maxit)
     ok = out[0][2] == 0
     assert (maxit == 1) == bool((~ok).all())
     assert torch.equal(out[0][2], out[1][2]) and torch.equal(out[0][0][ok], out[1][0][ok]) and out[0][3] == out[1][3]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nu", [(2, 2), (1, 1), (3, 1), (0, 2), (2, 0)])
+def test_fused_level0_solver_with_other_sweep_counts(hl, precision, nu):
+    """The one-CTA-per-sample solver's V-cycle and matvec (red cells only where
+    a black half-sweep ends the cycle) with the sweep counts that change their
+    phases: the multi-kernel path solves to the same Newton tolerance."""
+    xi = torch.as_tensor(inputs.uniform_xi(9400, 3), device="cuda")
+    q = []
+    for fused in (2, 0):
+        s = hl.Solver(precision=precision, fused_small_grids=fused, nu1=nu[0], nu2=nu[1], steps0=6, T=6 * 360.0)
+        qf, _, st, _ = s.level_batch_solve(0, xi)
+        assert int(st.abs().sum()) == 0
+        q.append(qf)
+        s.close()
+    assert torch.allclose(q[0], q[1], rtol=1e-9, atol=1e-14)
