@@ -147,8 +147,8 @@ typedef struct {
   double newton_predictor; /* weight w in [0, 1] of the time predictor of Newton's first iterate of step
                               n+1 (0: x^n; default 1: the full extrapolation of newton_predictor_order) */
   double newton_dc_limit;  /* Newton steps with max |dc| > limit are scaled down to it (default 1; 0: off) */
-  int32_t fused_small_grids; /* grids of <= 512 cells solved by one CTA per sample with the whole hierarchy in
-                                shared memory: 1 (default) in HENRY_MIXED only, 2 also in HENRY_FP64,
+  int32_t fused_small_grids; /* grids of 512 cells solved by one CTA per sample with the whole hierarchy in
+                                registers and shared memory: 1 (default) in HENRY_MIXED only, 2 also in HENRY_FP64,
                                 0 never (always the multi-kernel path); not used by the field models */
   int32_t coef_model;        /* HENRY_MODEL_* */
   int32_t kl_terms;          /* KL terms per field (default 32) */
