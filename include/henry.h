@@ -159,10 +159,9 @@ typedef struct {
                            once per sample by a separate kernel (default 512; 0: never); same values */
   double adj_rtol;   /* henry_adjoint: relative residual of each adjoint solve J^T lam = rhs (default 1e-10) */
   int32_t adj_maxit; /* henry_adjoint: BiCGStab iteration cap of each adjoint solve (default 200) */
-  int32_t cuda_graphs; /* 1 (default): each implicit step (Newton and BiCGStab loops included, as conditional
-                          nodes) is captured once per workspace, batch size and settings into a CUDA graph
-                          and replayed without host synchronisation; 0: plain launches driven by the host.
-                          Same values either way; off while profiling */
+  int32_t cuda_graphs; /* 1 (default): a BiCGStab iteration's launches between two convergence tests are
+                          captured once per workspace, batch size and settings into a CUDA graph and replayed;
+                          0: plain launches. Same values either way; off while profiling */
   int32_t qoi_set;     /* HENRY_QOI_* (default STANDARD); sets other than STANDARD use the multi-kernel path */
   int32_t tile_assembly; /* 1 (default): face-once assembly in tiles of 256 cells (whole rows up to 256 cells
                             wide, else 128 x 2 blocks), every face inside a tile evaluated once; 0: every

@@ -11,11 +11,9 @@
 // arXiv 2302.07804); each step runs Newton iterations, each Newton iteration
 // assembles the residual and the Jacobian on the fine grid and the coarse
 // operators, and solves the Newton system with BiCGStab right-preconditioned
-// by one V-cycle.  Per-sample convergence decisions are taken on the device,
-// and so are the loops': a step is one CUDA graph with conditional nodes (see
-// "Device-driven loops"; with cuda_graphs = 0, the kernel timer on, or the
-// allocation-free entry point the host reads how many samples are still
-// iterating once per Newton and once per BiCGStab iteration instead).
+// by one V-cycle.  Per-sample convergence decisions are taken on the device;
+// the host reads how many samples are still iterating once per Newton and once
+// per BiCGStab iteration.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -72,8 +70,8 @@ inline unsigned nblk(int64_t n, int tpb = TPB) { return (unsigned)((n + tpb - 1)
 
 // Launch a kernel of the solve's chain with the programmatic-serialisation
 // attribute (the rules stand at grid_wait in henry_kernels.cuh).
-// Set before capturing nodes that follow a conditional node: the next kernel
-// is launched without the attribute (a full dependency).
+// Set before a capture: the first kernel captured is launched without the
+// attribute (a full dependency).
 thread_local bool g_full_dependency = false;
 template <typename... P, typename... A>
 void chain(cudaStream_t st, unsigned grid, unsigned tpb, size_t smem, void (*k)(P...), A&&... args) {
@@ -1081,69 +1079,17 @@ int read_counter(henry_handle* H, const int* dev, cudaStream_t st, int* out) {
 }
 
 // ---------------------------------------------------------------------------
-// Device-driven loops.  The Newton and BiCGStab loops of an implicit step run
-// as conditional (WHILE / IF) nodes of one CUDA graph: the kernels count the
-// samples still iterating and a one-thread kernel (k_loop_gate) sets the
-// node's condition, so the host launches one graph a step and never waits
-// for a count.  A host-driven turn costs some 19 us beyond its kernels (copy
-// of the count, synchronisation, launches), a WHILE turn 4.4 us, and the
-// launches outside the iteration's body 1.4 - 4 us each instead of ~1 us.
-// Against one graph per BiCGStab iteration between host turns: level-0 FP64
-// 64 samples 24.6 -> 20.3 ms, level 2 with partners (33 samples) 237 -> 219
-// ms, two-layer level 1 (50) 67 -> 59 ms, 8192 level-0 samples 444 -> 440 ms.
-// A graph under construction and the nodes its next node will follow.
-struct GraphBuild {
-  henry_handle* H;
-  cudaGraph_t g;
-  std::vector<cudaGraphNode_t> deps;
-
-  // Append the launches f(stream) makes.
-  template <typename F>
-  int seg(F&& f) {
-    cudaStream_t cs = H->cap_stream;
-    g_full_dependency = true;
-    CK(cudaStreamBeginCaptureToGraph(cs, g, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(),
-                                     cudaStreamCaptureModeThreadLocal));
-    int rc = f(cs);
-    g_full_dependency = false;
-    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-    const cudaGraphNode_t* d = nullptr;
-    const cudaGraphEdgeData* ed = nullptr;
-    size_t nd = 0;
-    const cudaError_t e1 = cudaStreamGetCaptureInfo(cs, &status, nullptr, nullptr, &d, &ed, &nd);
-    if (e1 == cudaSuccess && status == cudaStreamCaptureStatusActive) deps.assign(d, d + nd);
-    cudaGraph_t out = nullptr;
-    const cudaError_t e2 = cudaStreamEndCapture(cs, &out);
-    if (rc) return rc;
-    if (e1 != cudaSuccess || e2 != cudaSuccess || status != cudaStreamCaptureStatusActive)
-      return set_err(HENRY_ECUDA, "graph capture failed: %s", cudaGetErrorString(e2 != cudaSuccess ? e2 : e1));
-    return HENRY_OK;
-  }
-  int handle(cudaGraphConditionalHandle* h) {
-    CK(cudaGraphConditionalHandleCreate(h, g, 0, cudaGraphCondAssignDefault));
-    return HENRY_OK;
-  }
-  // Append a conditional node; *body is the graph it runs.
-  int cond(cudaGraphConditionalNodeType type, cudaGraphConditionalHandle h, GraphBuild* body) {
-    cudaGraphNodeParams p = {};
-    p.type = cudaGraphNodeTypeConditional;
-    p.conditional.handle = h;
-    p.conditional.type = type;
-    p.conditional.size = 1;
-    cudaGraphNode_t n = nullptr;
-    CK(cudaGraphAddNode(&n, g, deps.empty() ? nullptr : deps.data(), nullptr, deps.size(), &p));
-    deps.assign(1, n);
-    body->H = H;
-    body->g = p.conditional.phGraph_out[0];
-    body->deps.clear();
-    return HENRY_OK;
-  }
-};
-
-// Launch the graph that emit(GraphBuild&) describes on `st`, building it on
-// first use (key: what it is; the batch size and the configuration are added
-// here).  Captured on the handle's own stream, of st's priority (capturing the
-// legacy default stream is not allowed; capture executes nothing).
+// Launch the kernels that emit(stream) launches as one CUDA graph on `st`,
+// captured on first use (key: what they are; the batch size and the
+// configuration are added here).  Captured on the handle's own stream, of
+// st's priority (capturing the legacy default stream is not allowed; capture
+// executes nothing).
+//
+// The loops themselves stay on the host.  As conditional nodes of one graph
+// per implicit step they ran a third faster on small batches (level-0 FP64, 64
+// samples 20.3 against 24.6 ms then), but destroying such graphs while other
+// host threads worked on the device crashed inside cudaGraphDestroy now and
+// then (driver 580, also with every graph call of the process serialised).
 constexpr size_t MAX_GRAPHS = 16;
 template <typename GRP, typename F>
 int run_graph(henry_handle* H, GRP& G, int B, const std::string& what, cudaStream_t st, F&& emit) {
@@ -1162,12 +1108,14 @@ int run_graph(henry_handle* H, GRP& G, int B, const std::string& what, cudaStrea
       CK(cudaStreamCreateWithPriority(&H->cap_stream, cudaStreamNonBlocking, prio));
     }
     cudaGraph_t gr = nullptr;
-    CK(cudaGraphCreate(&gr, 0));
-    GraphBuild b{H, gr, {}};
-    const int rc = emit(b);
-    if (rc) {
-      cudaGraphDestroy(gr);
-      return rc;
+    CK(cudaStreamBeginCapture(H->cap_stream, cudaStreamCaptureModeThreadLocal));
+    g_full_dependency = true;
+    const int rc = emit(H->cap_stream);
+    g_full_dependency = false;
+    const cudaError_t ec = cudaStreamEndCapture(H->cap_stream, &gr);
+    if (rc || ec != cudaSuccess) {
+      if (ec == cudaSuccess && gr) cudaGraphDestroy(gr);
+      return rc ? rc : set_err(HENRY_ECUDA, "graph capture failed: %s", cudaGetErrorString(ec));
     }
     cudaGraphExec_t ex = nullptr;
     const cudaError_t e = cudaGraphInstantiate(&ex, gr, 0);
@@ -1185,49 +1133,26 @@ bool graphs_on(const henry_handle* H, const GRP& G) {
   return H->cfg.cuda_graphs && G.graphs && !H->prof.on;
 }
 
-// The BiCGStab loop over a solver D's pieces - init(stream, loop words), head
-// (iteration, its index in device memory, stream), body(samples, stream) - on
-// group D::G.
+// The BiCGStab loop over a solver D's pieces - init(stream), head(iteration,
+// stream), body(samples, stream) and what(), which names the body among the
+// group's graphs - on group D::G.
 template <typename D>
 struct KrylovDrive {
   D& d() { return static_cast<D&>(*this); }
-  // As nodes of a graph.
-  int emit(GraphBuild& b) {
-    auto& G = d().G;
-    cudaGraphConditionalHandle h;
-    int rc = b.handle(&h);
-    if (rc) return rc;
-    auto test = [&](cudaStream_t s) {
-      const int r = d().head(0, G.counter + 3, s);
-      chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 1, G.counter + 3);
-      return r;
-    };
-    rc = b.seg([&](cudaStream_t s) {
-      const int r = d().init(s, G.counter + 1);
-      return r ? r : test(s);
-    });
-    GraphBuild it;
-    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &it);
-    if (!rc)
-      rc = it.seg([&](cudaStream_t s) {
-        const int r = d().body(d().B, s);
-        return r ? r : test(s);
-      });
-    return rc;
-  }
-  // Driven from the host.
   int run(cudaStream_t st) {
     auto& G = d().G;
     henry_handle* H = d().H;
-    int rc = d().init(st, nullptr);
+    const bool graph = graphs_on(H, G);
+    int rc = d().init(st);
     for (int it = 0; !rc && it <= d().maxit; ++it) {
       CK(cudaMemsetAsync(G.counter + 1, 0, sizeof(int), st));
-      rc = d().head(it, nullptr, st);
+      rc = d().head(it, st);
       int n_act = 0;
       if (!rc) rc = read_counter(H, G.counter + 1, st, &n_act);
       if (rc || n_act == 0) return rc;
       H->nact = n_act;
-      rc = d().body(n_act, st);
+      rc = graph ? run_graph(H, G, d().B, d().what(), st, [&](cudaStream_t s) { return d().body(d().B, s); })
+                 : d().body(n_act, st);
     }
     return rc;
   }
@@ -1263,6 +1188,7 @@ struct Krylov : KrylovDrive<Krylov<T>> {
     black_known = H->cfg.nu2 > 0 && !Jpre0;
   }
 
+  std::string what() const { return std::string(reinterpret_cast<const char*>(&Jpre0), sizeof Jpre0); }
   void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
@@ -1271,20 +1197,20 @@ struct Krylov : KrylovDrive<Krylov<T>> {
   // Bytes of the matvec and of a first half-sweep per cell.
   double spmv_bytes() const { return (black_known ? 0.5 : 1.0) * 5 * sizeof(B4) + 3 * sizeof(V2); }
   double first_bytes() const { return first ? 0.5 * (sizeof(B4) + sizeof(V2)) : 0.0; }
-  int init(cudaStream_t st, int* loop) {
+  int init(cudaStream_t st) {
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * sizeof(V2)), [&] {
-      chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, loop);
+      chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
     });
     finalize(P_RR, P_RN, st);
     CKL();
     return HENRY_OK;
   }
-  // The convergence test and the new search direction of iteration `it` (or
-  // *it_dev), counting the samples that go on in G.counter[1].
-  int head(int it, const int* it_dev, cudaStream_t st) {
+  // The convergence test and the new search direction of iteration `it`,
+  // counting the samples that go on in G.counter[1].
+  int head(int it, cudaStream_t st) {
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * ((it == 0 ? 2 : 4) * sizeof(V2) + first_bytes()), [&] {
       auto go = [&](auto* k) {
-        chain(st, g, TPB, 0, k, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
+        chain(st, g, TPB, 0, k, B, N, it, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active, G.iters,
               G.status, G.counter + 1, G.totals + 1, fin, Ci, G.ph, L.nx);
       };
       if (first) go(&k_bicg_p<T, true>);
@@ -1343,19 +1269,14 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
   const double rt = rtol > 0.0 ? rtol : H->cfg.lin_rtol;
   const int mi = maxit > 0 ? maxit : H->cfg.lin_maxit;
   Krylov<T> k(H, G, B, Jpre0, rt, mi);
-  if (!graphs_on(H, G)) return k.run(st);
-  std::string what = "linear";
-  what.append(reinterpret_cast<const char*>(&Jpre0), sizeof Jpre0);
-  what.append(reinterpret_cast<const char*>(&rt), sizeof rt);
-  what.append(reinterpret_cast<const char*>(&mi), sizeof mi);
-  return run_graph(H, G, B, what, st, [&](GraphBuild& b) { return k.emit(b); });
+  return k.run(st);
 }
 
 // Newton's loop over a step D's pieces - start, evaluate(residual first, count,
 // stream), operators, krylov / solve(fallback), mark_retry and retry_operators
 // where retries(), update - on group D::G.
 //
-// Newton's choices (the same in both drives): the Jacobian and the coarse
+// Newton's choices: the Jacobian and the coarse
 // operators are assembled at iterations 0, k, 2k, ... of the step, k =
 // newton_jacobian_every (chord Newton; and after a fallback-preconditioner
 // retry, which rebuilt coarse operators for its samples), the others evaluate
@@ -1370,10 +1291,8 @@ struct NewtonDrive {
   explicit NewtonDrive(const henry_config& c)
       : jac_every(std::max(1, c.newton_jacobian_every)), res_from(c.newton_residual_first) {}
   D& d() { return static_cast<D&>(*this); }
-  bool jac_at(int it) const { return it % jac_every == 0; }
   bool res_first_at(int it, bool jac_now) const { return !jac_now || (res_from >= 0 && it >= res_from); }
 
-  // --- host-driven
   int run(cudaStream_t st) {
     D& n = d();
     henry_handle* H = n.H;
@@ -1416,83 +1335,6 @@ struct NewtonDrive {
     return rc;
   }
 
-  // --- as a graph
-  // From this iteration on the pattern of evaluations repeats every jac_every
-  // iterations.
-  int steady() const { return res_from <= 0 ? 0 : ((res_from + jac_every - 1) / jac_every) * jac_every; }
-  // Whether the step can run as one graph: few iterations before the steady
-  // pattern, and no retries that would shift a chord pattern.
-  bool graphable() { return steady() <= 6 && jac_every <= 8 && !(d().retries() && jac_every > 1); }
-  int emit_work(GraphBuild& b, int it) {
-    D& n = d();
-    auto& G = n.G;
-    int rc = HENRY_OK;
-    if (jac_at(it)) rc = b.seg([&](cudaStream_t s) { return n.operators(res_first_at(it, true), s); });
-    if (!rc) rc = n.krylov(false).emit(b);
-    if (!rc && n.retries()) {
-      cudaGraphConditionalHandle h;
-      rc = b.handle(&h);
-      if (!rc)
-        rc = b.seg([&](cudaStream_t s) {
-          const int r = n.mark_retry(s);
-          chain(s, 1, 1, 0, k_loop_gate, h, h, 0, G.counter + 2, (int*)nullptr);
-          return r;
-        });
-      GraphBuild r;
-      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &r);
-      if (!rc) rc = r.seg([&](cudaStream_t s) { return n.retry_operators(s); });
-      if (!rc) rc = n.krylov(true).emit(r);
-    }
-    return rc ? rc : b.seg([&](cudaStream_t s) { return n.update(n.B, s); });
-  }
-  // Iteration `it`: evaluate, then set the conditions h1 (and h2) to whether
-  // any sample goes on.
-  int emit_test(GraphBuild& b, int it, cudaGraphConditionalHandle h1, cudaGraphConditionalHandle h2, int two) {
-    return b.seg([&](cudaStream_t s) {
-      const int r = d().evaluate(res_first_at(it, jac_at(it)), d().G.counter, s);
-      chain(s, 1, 1, 0, k_loop_gate, h1, h2, two, d().G.counter, (int*)nullptr);
-      return r;
-    });
-  }
-  // The iterations from `it` on.  The first two run unconditionally (their
-  // kernels skip samples that have converged; hardly any step is done by
-  // then), the following ones up to the steady pattern inside IF nodes, then
-  // a WHILE node runs jac_every iterations a turn.
-  int emit_from(GraphBuild& b, int it) {
-    const int S = steady();
-    if (it < S && it < 2) {
-      int rc = b.seg([&](cudaStream_t s) { return d().evaluate(res_first_at(it, jac_at(it)), nullptr, s); });
-      if (!rc) rc = emit_work(b, it);
-      return rc ? rc : emit_from(b, it + 1);
-    }
-    cudaGraphConditionalHandle h;
-    int rc = b.handle(&h);
-    if (!rc) rc = emit_test(b, it, h, h, 0);
-    GraphBuild in;
-    if (it < S) {
-      if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
-      if (!rc) rc = emit_work(in, it);
-      return rc ? rc : emit_from(in, it + 1);
-    }
-    if (!rc) rc = b.cond(cudaGraphCondTypeWhile, h, &in);
-    return rc ? rc : emit_turn(in, S, 0, h);
-  }
-  // Iterations S + j .. S + jac_every - 1 of a turn of the WHILE node (condition w).
-  int emit_turn(GraphBuild& b, int S, int j, cudaGraphConditionalHandle w) {
-    int rc = emit_work(b, S + j);
-    if (rc) return rc;
-    if (j == jac_every - 1) return emit_test(b, S + j + 1, w, w, 0);
-    cudaGraphConditionalHandle h;
-    rc = b.handle(&h);
-    if (!rc) rc = emit_test(b, S + j + 1, h, w, 1);
-    GraphBuild in;
-    if (!rc) rc = b.cond(cudaGraphCondTypeIf, h, &in);
-    return rc ? rc : emit_turn(in, S, j + 1, w);
-  }
-  int emit(GraphBuild& b) {
-    const int rc = b.seg([&](cudaStream_t s) { return d().start(s); });
-    return rc ? rc : emit_from(b, 0);
-  }
 };
 
 // One implicit-Euler step (Sec. 2.3) of the B samples of a group: the state
@@ -1616,9 +1458,7 @@ int implicit_step(henry_handle* H, Group<T>& G, int B, int step, cudaStream_t st
   NewtonStep<T> n(H, G, B);
   const int rc = n.begin(step, st);
   if (rc) return rc;
-  if (!graphs_on(H, G) || !n.graphable()) return n.run(st);
-  if (step == 0) CK(cudaMemsetAsync(G.counter, 0, 4 * sizeof(int), st));
-  return run_graph(H, G, B, "step", st, [&](GraphBuild& b) { return n.emit(b); });
+  return n.run(st);
 }
 
 // Full scenario solves of B samples whose coefficients and status are set.
@@ -2021,22 +1861,23 @@ struct VcKrylov : KrylovDrive<VcKrylov<T>> {
       : H(h), G(grp), B(b), rtol2(h->cfg.lin_rtol * h->cfg.lin_rtol), maxit(h->cfg.lin_maxit), L(grp.lv[0]),
         N(grp.lv[0].stride), g(nblk((int64_t)b * grp.lv[0].stride)),
         fin((h->cfg.finalize_nct > 0 && grp.nct >= h->cfg.finalize_nct) ? grp.fin : nullptr) {}
+  std::string what() const { return "body"; }
   void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
            [&] { chain(ss, nblk((int64_t)B * 32, 128), 128, 0, k_finalize, B, G.nct, G.part, a, b, fin); });
   }
-  int init(cudaStream_t st, int* loop) {
+  int init(cudaStream_t st) {
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (16 + 5 * sizeof(V2)), [&] {
-      chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active, loop);
+      chain(st, g, TPB, 0, k_bicg_init<T>, B, N, G.F, G.r, G.rh, G.p, G.v, G.dx, G.part, G.lin_active);
     });
     finalize(P_RR, P_RN, st);
     CKL();
     return HENRY_OK;
   }
-  int head(int it, const int* it_dev, cudaStream_t st) {
+  int head(int it, cudaStream_t st) {
     launch(H, st, HENRY_K_KRYLOV, (double)H->nact * N * (it == 0 ? 2 : 4) * sizeof(V2), [&] {
-      chain(st, g, TPB, 0, k_bicg_p<T, false>, B, N, it, it_dev, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
+      chain(st, g, TPB, 0, k_bicg_p<T, false>, B, N, it, maxit, rtol2, G.r, G.p, G.v, G.part, G.sc, G.lin_active,
             G.iters, G.status, G.counter + 1, G.totals + 1, fin, (const B4*)nullptr, (V2*)nullptr, 0);
     });
     CKL();
@@ -2075,8 +1916,7 @@ struct VcKrylov : KrylovDrive<VcKrylov<T>> {
 template <typename T>
 int vc_linear_solve(henry_handle* H, VcGroup<T>& G, int B, cudaStream_t st) {
   VcKrylov<T> k(H, G, B);
-  if (!graphs_on(H, G)) return k.run(st);
-  return run_graph(H, G, B, "linear", st, [&](GraphBuild& b) { return k.emit(b); });
+  return k.run(st);
 }
 
 // Where the fine assembly leaves its per-CTA maxima of |F| and how many a
@@ -2203,9 +2043,7 @@ int vc_implicit_step(henry_handle* H, VcGroup<T>& G, int B, int step, cudaStream
   VcNewtonStep<T> n(H, G, B);
   const int rc = n.begin(step, st);
   if (rc) return rc;
-  if (!graphs_on(H, G) || !n.graphable()) return n.run(st);
-  if (step == 0) CK(cudaMemsetAsync(G.counter, 0, 4 * sizeof(int), st));
-  return run_graph(H, G, B, "step", st, [&](GraphBuild& b) { return n.emit(b); });
+  return n.run(st);
 }
 
 // Full scenario solves of B samples of the vertex-centred scheme whose

@@ -1395,23 +1395,20 @@ __global__ void __launch_bounds__(TPB) k_spmv(int B, int nx, int ny, const typen
 // a6: right-preconditioned BiCGStab (Templates book), per sample, on the fine
 // level; per-sample scalars live in LinScal, per-CTA partial sums in part.
 
-// r = r_hat = b (= -F), p = v = dx = 0; partials <r_hat, r>, <r, r>.  loop
-// (nullable): the device-driven loop's words, loop[0] = samples still
-// iterating, loop[2] = iteration index, set to 0.
+// r = r_hat = b (= -F), p = v = dx = 0; partials <r_hat, r>, <r, r>.
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_bicg_init(int B, int N, const double2* F,
                                                    typename VT<T>::v2* __restrict__ r,
                                                    typename VT<T>::v2* __restrict__ rh,
                                                    typename VT<T>::v2* __restrict__ p, typename VT<T>::v2* __restrict__ v,
                                                    typename VT<T>::v2* __restrict__ dx, double* __restrict__ part,
-                                                   const int* active, int* loop) {
+                                                   const int* active) {
   typedef typename VT<T>::v2 V2;
   __shared__ double sh[TPB + 1];
   const int nct = N / TPB;
   const int64_t e = (int64_t)blockIdx.x * TPB + threadIdx.x;
   const int s = blockIdx.x / (unsigned)nct;
   grid_enter();
-  if (loop && blockIdx.x == 0 && threadIdx.x == 0) loop[0] = loop[2] = 0;
   if (!active[s]) return;
   const double2 f = F[e];
   const V2 rr = mk2<V2>((T)(-f.x), (T)(-f.y));
@@ -1432,8 +1429,7 @@ __global__ void __launch_bounds__(TPB) k_bicg_init(int B, int N, const double2* 
 // Start of iteration `it`: rho_it = <r_hat, r>, convergence test on ||r||,
 // beta = (rho_it / rho_{it-1}) (alpha / omega), p = r + beta (p - omega v).
 // A converged sample's CTA 0 clears lin_active; the last iteration counts
-// still-active samples in *n_active and per-sample iterations in iters.  it_dev
-// (nullable): the iteration index in device memory instead of `it`.
+// still-active samples in *n_active and per-sample iterations in iters.
 // FIRST: the V-cycle that follows starts with a red half-sweep from zero, x_P =
 // C_P^-1 p_P; it is done here (Ci: the fine operator's plane of inverses, ph
 // the cycle's vector, nx the grid's width), one launch and one pass over the
@@ -1447,7 +1443,7 @@ __device__ __forceinline__ void first_sweep(const typename VT<T>::b4* Ci, typena
   x[e] = mk2<typename VT<T>::v2>(y0, y1);
 }
 template <typename T, bool FIRST = false>
-__global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, const int* it_dev, int maxit, double rtol2,
+__global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, int maxit, double rtol2,
                                                 const typename VT<T>::v2* r, typename VT<T>::v2* p,
                                                 const typename VT<T>::v2* v, const double* part, LinScal* sc,
                                                 int* lin_active, int* __restrict__ iters,
@@ -1462,7 +1458,6 @@ __global__ void __launch_bounds__(TPB) k_bicg_p(int B, int N, int it, const int*
   const int s = blockIdx.x / (unsigned)nct;
   grid_enter();
   if (!lin_active[s]) return;
-  if (it_dev) it = *it_dev;
   const int ct = (int)((e - (int64_t)s * N) / TPB);
   const int64_t stride = (int64_t)B * nct;
   double rho, rn2;
@@ -1590,21 +1585,6 @@ __global__ void __launch_bounds__(TPB) k_bicg_update(int B, int N, typename VT<T
   if (threadIdx.x == 0) part[P_RR * stride + pi] = d;
   if (threadIdx.x == TPB / 2) part[P_RN * stride + pi] = d;
   if (threadIdx.x == TPB - 1 && ct == 0) sc[s].aow = alpha / omega;
-}
-
-// One thread, after a kernel that counted the samples still iterating in
-// *n_active: the conditional nodes a (and b, if two) of the surrounding graph
-// run (again) while there are any.  Resets the count; *it (nullable) += 1.
-// The loops end because the counting kernels stop every sample at its
-// iteration cap.
-__global__ void k_loop_gate(cudaGraphConditionalHandle a, cudaGraphConditionalHandle b, int two, int* n_active,
-                            int* it) {
-  grid_enter();
-  const unsigned go = *n_active > 0 ? 1u : 0u;
-  *n_active = 0;
-  if (it) *it += 1;
-  cudaGraphSetConditional(a, go);
-  if (two) cudaGraphSetConditional(b, go);
 }
 
 // Samples whose BiCGStab did not converge (or broke down) in this Newton

@@ -1,6 +1,6 @@
 """How a solve is driven changes no value: the fused multigrid tail from the
-fine grid itself, and the device-driven step graphs, against separate kernels
-and host-driven loops, bit for bit, at the sizes and settings where the choice
+fine grid itself, and the captured BiCGStab iterations, against separate kernels
+and plain launches, bit for bit, at the sizes and settings where the choice
 changes."""
 import pytest
 import torch
@@ -47,7 +47,7 @@ def test_default_tail_start_is_bit_identical_to_separate_kernels(hl, precision, 
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("res_first,every,maxit", [(-1, 1, 30), (0, 1, 30), (1, 1, 30), (2, 1, 30), (3, 2, 30), (4, 3, 30),
                                                     (5, 1, 30), (9, 1, 30), (-1, 3, 30), (2, 1, 1), (2, 1, 2)])
-def test_step_graph_equals_host_driven_loops(hl, precision, res_first, every, maxit):
+def test_captured_iterations_equal_plain_launches(hl, precision, res_first, every, maxit):
     xi = torch.as_tensor(inputs.uniform_xi(9200, 5), device="cuda")
     out = []
     for graphs in (1, 0):
@@ -64,8 +64,8 @@ def test_step_graph_equals_host_driven_loops(hl, precision, res_first, every, ma
         assert o[3] == out[0][3]
 
 
-def test_step_graph_with_retries_equals_host_driven_loops(hl):
-    """KL inputs on which BiCGStab fails now and then: the fallback solve inside the graph."""
+def test_captured_iterations_with_retries_equal_plain_launches(hl):
+    """KL inputs on which BiCGStab fails now and then: the fallback solve's own graph."""
     xi = torch.as_tensor(1.6 * inputs.kl_inputs(9300, 6), device="cuda")
     xi[:, -1].clamp_(-1.0, 1.0)
     out = []
@@ -94,7 +94,7 @@ def test_vertex_tail_is_bit_identical_to_separate_kernels(hl, precision, level, 
 
 
 @pytest.mark.parametrize("res_first,every,maxit", [(2, 1, 30), (-1, 2, 30), (3, 2, 30), (2, 1, 1)])
-def test_vertex_step_graph_equals_host_driven_loops(hl, res_first, every, maxit):
+def test_vertex_captured_iterations_equal_plain_launches(hl, res_first, every, maxit):
     xi = torch.as_tensor(inputs.uniform_xi(9500, 4), device="cuda")
     out = []
     for graphs in (1, 0):
@@ -122,3 +122,21 @@ def test_fused_level0_solver_with_other_sweep_counts(hl, precision, nu):
         q.append(qf)
         s.close()
     assert torch.allclose(q[0], q[1], rtol=1e-9, atol=1e-14)
+
+
+def test_concurrent_levels_build_their_graphs_over_and_over(hl):
+    """Rounds of changing sizes: every level thread builds, replays and (past
+    the cache's bound) drops graphs while the others do the same."""
+    s = hl.Solver(steps0=2, T=720.0, max_level=2)
+    h = hl.Solver(steps0=2, T=720.0, max_level=2, cuda_graphs=0)
+    for k in range(60):
+        levels = [0] * (3 + k % 19) + [1] * (2 + k % 17) + [2] * (1 + k % 18)
+        xi = torch.as_tensor(inputs.uniform_xi(9500 + k, len(levels)), device="cuda")
+        levels = torch.tensor(levels, dtype=torch.int32)
+        qf, qc, st, _ = s.batch_solve_mixed(levels, xi, with_coarse=True)
+        assert int(st.abs().sum()) == 0
+        if k % 20 == 19:
+            rf, rc, _, _ = h.batch_solve_mixed(levels, xi, with_coarse=True)
+            assert torch.equal(qf, rf) and torch.equal(qc.nan_to_num(), rc.nan_to_num())
+    s.close()
+    h.close()
