@@ -136,7 +136,7 @@ struct Group {
   LinScal* sc;
   T* Ainv;
   void* Jp = nullptr;  // fine-level fallback preconditioner operator (field models only)
-  // Instantiated CUDA graphs (a whole implicit step, or a linear solve), by
+  // Instantiated CUDA graphs (a BiCGStab iteration each), by
   // what they run, the batch size and the whole configuration (every setting
   // that changes their launches); they hold this workspace's pointers and are
   // dropped with it.
@@ -1086,8 +1086,8 @@ int read_counter(henry_handle* H, const int* dev, cudaStream_t st, int* out) {
 // executes nothing).
 //
 // The loops themselves stay on the host.  As conditional nodes of one graph
-// per implicit step they ran a third faster on small batches (level-0 FP64, 64
-// samples 20.3 against 24.6 ms then), but destroying such graphs while other
+// per implicit step they ran faster on small batches (level-0 FP64, 64
+// samples 14.0 against 18.6 ms), but destroying such graphs while other
 // host threads worked on the device crashed inside cudaGraphDestroy now and
 // then (driver 580, also with every graph call of the process serialised).
 constexpr size_t MAX_GRAPHS = 16;
