@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
   constexpr int NW = ACC_THREADS / 32, RPW = 32 / CW, R = 8;  // R: rows a lane holds at a time
   __shared__ double part[4][NW][CW];
   __shared__ int cpart[NW][CW];
-  __shared__ double mom[2][CW][3];
+  __shared__ double mom[2][CW][4];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int col = lane % CW, q = blockIdx.x * CW + col;
   const int rank = blockIdx.y, ncta = gridDim.y;
@@ -507,28 +507,32 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
     const double d = m > 0 ? s1 / nn : 0.0;
     const double m2 = s2 - s1 * d;
     mom[which][col][0] = nn;
-    mom[which][col][1] = (which == 0 ? ky : kf) + d;
-    mom[which][col][2] = m2 < 0.0 ? 0.0 : m2;
+    mom[which][col][1] = which == 0 ? ky : kf;
+    mom[which][col][2] = d;
+    mom[which][col][3] = m2 < 0.0 ? 0.0 : m2;
   }
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();
   if (rank == 0 && which < 2 && lane < CW && on) {
-    // the batch's moments from the CTAs', then Chan's merge into the sums
-    double cb = 0.0, sb = 0.0;
+    // the batch's moments from the CTAs', then Chan's merge into the sums.
+    // The CTAs' means enter as distances from one CTA's pivot, (k - k0) + d:
+    // rounded to k + d they would put an error of eps |mean| sd into M2.
+    double cb = 0.0, sb = 0.0, k0 = 0.0;
     for (int k = 0; k < ncta; ++k) {
       const double* b = cl.map_shared_rank(&mom[which][col][0], k);
       if (b[0] == 0.0) continue;
+      if (cb == 0.0) k0 = b[1];
       cb += b[0];
-      sb = fma(b[0], b[1], sb);
+      sb = fma(b[0], (b[1] - k0) + b[2], sb);
     }
     if (cb > 0.0) {
-      const double mb = sb / cb;
+      const double off = sb / cb, mb = k0 + off;
       double m2 = 0.0;
       for (int k = 0; k < ncta; ++k) {
         const double* b = cl.map_shared_rank(&mom[which][col][0], k);
         if (b[0] == 0.0) continue;
-        const double d = b[1] - mb;
-        m2 += fma(b[0] * d, d, b[2]);
+        const double d = ((b[1] - k0) + b[2]) - off;
+        m2 += fma(b[0] * d, d, b[3]);
       }
       double* S = sums + ((int64_t)which * n_qoi + q) * 3;
       const double na = S[0], ma = S[1], m2a = S[2];
