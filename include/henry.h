@@ -365,7 +365,7 @@ int henry_adjoint(henry_handle* h, int level, const double* xi_dev, int n, const
  * sums_dev[2][n_qoi][3] holds (count, mean, M2) with M2 the centred sum of
  * squares; [0] for Y and [1] for qoi_fine itself; it is read and updated in
  * place (zero it before the first batch).  The batch's moments are formed
- * about a pivot inside the data and merged with Chan's pairwise update.  `level` is
+ * about a pivot close to their mean and merged with Chan's pairwise update.  `level` is
  * only checked (>= 0).  Asynchronous on `stream`. */
 int mlmc_accumulate(int level, int n, int n_qoi, const double* qoi_fine_dev, const double* qoi_coarse_dev,
                     const int32_t* status_dev, double* sums_dev, void* stream);

@@ -399,10 +399,15 @@ __global__ void __launch_bounds__(TPB) k_scale_d2(int64_t n, double a, double2* 
 //
 // The rows are read once, coalesced over CW neighbouring QoIs, by a cluster
 // of CTAs per group of CW columns: each CTA sums (y - k) and (y - k)^2 over
-// its rows about a pivot k, the mean of its first few used rows (so that k
-// lies in the data and s2 - s1^2 / n keeps its digits), and the cluster's
-// first CTA merges the CTAs' moments through distributed shared memory - no
-// workspace.  Bound by the FP64 pipe: 7 operations per row and QoI (the
+// its rows about a pivot k, and the cluster's first CTA merges the CTAs'
+// moments through distributed shared memory - no workspace.  The pivot is the
+// mean of the used ones among the first 8 rows of the CTA's first step that
+// has any there (0 if none has).  M2 = s2 - s1^2 / n keeps its digits while k
+// lies within a standard deviation or so of the mean; where it does not
+// (those rows failed, or lie far from the rest) a column's M2 comes out below
+// s2 / 4 and the CTA goes over its rows once more about the mean it then knows.
+// On normally distributed values that takes a mean of 8 more than 4.9 of its
+// own deviations off, one CTA and column in a million.  Bound by the FP64 pipe: 7 operations per row and QoI (the
 // difference Y, and a subtraction, an addition and a multiply-add for each
 // quantity), which at 17-19 cycles a warp instruction and SM is 145 us for
 // 20000 rows of 527 QoIs with their partners.  Measured there 180 us, against
@@ -461,55 +466,62 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
     kf = (m > 0 && fabs(kf) <= 1.0e300) ? kf / (double)m : 0.0;  // infinite or NaN values: pivot 0
     ky = (m > 0 && fabs(ky) <= 1.0e300) ? ky / (double)m : 0.0;
   }
-  int cnt = 0;
-  double s1y = 0.0, s2y = 0.0, s1f = 0.0, s2f = 0.0;
-  for (int64_t r0 = (rank * NW + w) * RPW; r0 < n; r0 += R * step) {
-    double f[R], c[R];
-    bool ok[R];
-    load(r0 + lane / CW, step, f, c, ok);
-#pragma unroll
-    for (int j = 0; j < R; ++j) {
-      if (r0 + j * step >= n) break;  // uniform over the warp
-      const double df = ok[j] ? f[j] - kf : 0.0, dy = ok[j] ? (f[j] - c[j]) - ky : 0.0;
-      cnt += ok[j];
-      s1f += df;
-      s2f = fma(df, df, s2f);
-      s1y += dy;
-      s2y = fma(dy, dy, s2y);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o >= CW; o >>= 1) {
-    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    s1y += __shfl_xor_sync(0xffffffffu, s1y, o);
-    s2y += __shfl_xor_sync(0xffffffffu, s2y, o);
-    s1f += __shfl_xor_sync(0xffffffffu, s1f, o);
-    s2f += __shfl_xor_sync(0xffffffffu, s2f, o);
-  }
-  if (lane < CW) {
-    cpart[w][col] = cnt;
-    part[0][w][col] = s1y;
-    part[1][w][col] = s2y;
-    part[2][w][col] = s1f;
-    part[3][w][col] = s2f;
-  }
-  __syncthreads();
   const int which = w;  // warps 0 and 1: Y and the fine QoI
-  if (which < 2 && lane < CW) {
-    int m = 0;
-    double s1 = 0.0, s2 = 0.0;
-    for (int k = 0; k < NW; ++k) {
-      m += cpart[k][col];
-      s1 += part[2 * which][k][col];
-      s2 += part[2 * which + 1][k][col];
+  for (int pass = 0;; ++pass) {
+    int cnt = 0;
+    double s1y = 0.0, s2y = 0.0, s1f = 0.0, s2f = 0.0;
+    for (int64_t r0 = (rank * NW + w) * RPW; r0 < n; r0 += R * step) {
+      double f[R], c[R];
+      bool ok[R];
+      load(r0 + lane / CW, step, f, c, ok);
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        if (r0 + j * step >= n) break;  // uniform over the warp
+        const double df = ok[j] ? f[j] - kf : 0.0, dy = ok[j] ? (f[j] - c[j]) - ky : 0.0;
+        cnt += ok[j];
+        s1f += df;
+        s2f = fma(df, df, s2f);
+        s1y += dy;
+        s2y = fma(dy, dy, s2y);
+      }
     }
-    const double nn = (double)m;
-    const double d = m > 0 ? s1 / nn : 0.0;
-    const double m2 = s2 - s1 * d;
-    mom[which][col][0] = nn;
-    mom[which][col][1] = which == 0 ? ky : kf;
-    mom[which][col][2] = d;
-    mom[which][col][3] = m2 < 0.0 ? 0.0 : m2;
+#pragma unroll
+    for (int o = 16; o >= CW; o >>= 1) {
+      cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      s1y += __shfl_xor_sync(0xffffffffu, s1y, o);
+      s2y += __shfl_xor_sync(0xffffffffu, s2y, o);
+      s1f += __shfl_xor_sync(0xffffffffu, s1f, o);
+      s2f += __shfl_xor_sync(0xffffffffu, s2f, o);
+    }
+    if (lane < CW) {
+      cpart[w][col] = cnt;
+      part[0][w][col] = s1y;
+      part[1][w][col] = s2y;
+      part[2][w][col] = s1f;
+      part[3][w][col] = s2f;
+    }
+    __syncthreads();
+    bool far = false;  // the pivot lies too far from this column's mean (infinite values have no better one)
+    if (which < 2 && lane < CW) {
+      int m = 0;
+      double s1 = 0.0, s2 = 0.0;
+      for (int k = 0; k < NW; ++k) {
+        m += cpart[k][col];
+        s1 += part[2 * which][k][col];
+        s2 += part[2 * which + 1][k][col];
+      }
+      const double nn = (double)m;
+      const double d = m > 0 ? s1 / nn : 0.0;
+      const double m2 = s2 - s1 * d;
+      mom[which][col][0] = nn;
+      mom[which][col][1] = which == 0 ? ky : kf;
+      mom[which][col][2] = d;
+      mom[which][col][3] = m2 < 0.0 ? 0.0 : m2;
+      far = pass == 0 && !(m2 >= 0.25 * s2) && fabs(d) <= 1.0e300;
+    }
+    if (!__syncthreads_or(far)) break;
+    if (fabs(mom[0][col][2]) <= 1.0e300) ky += mom[0][col][2];
+    if (fabs(mom[1][col][2]) <= 1.0e300) kf += mom[1][col][2];
   }
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();

@@ -64,3 +64,33 @@ def test_spread_far_below_the_mean(hl, n, n_qoi, mean, sd):
     qc = 0.25 * mean + sd * gen.standard_normal((n, n_qoi))
     _check(hl, qf, None, None)
     _check(hl, qf, qc, (gen.random(n) < 0.2).astype(np.int32))
+@pytest.mark.parametrize("n,n_qoi", [(100, 2), (513, 1), (20011, 2), (20011, 33), (20011, 257)])
+@pytest.mark.parametrize("head", [8, 16, "every", "outlier"])
+def test_first_rows_failed_or_far_from_the_rest(hl, n, n_qoi, head):
+    """The first rows of a CTA's share, which place the pivot, have failed (the
+    first 8 or 16 of the batch, or 8 of every step) or lie far from the rest."""
+    gen = inputs.rng(7400 + n + n_qoi)
+    qf = 0.999 + 1.0e-8 * gen.standard_normal((n, n_qoi))
+    qc = 0.25 + 1.0e-8 * gen.standard_normal((n, n_qoi))
+    _, rows, ctas = _shape(n, n_qoi)
+    status = np.zeros(n, dtype=np.int32)
+    if head == "every":
+        status[np.arange(n) % rows < 8] = 1
+    elif head == "outlier":  # one used row among each CTA's first 8, 1e4 standard deviations off
+        for r in range(ctas):
+            status[r * rows + 1:r * rows + 8] = 1
+            qf[r * rows] += 1.0e-4 * (1.0 + 0.1 * r)
+    else:
+        status[:head] = 1
+    _check(hl, qf, None, status)
+    _check(hl, qf, qc, status)
+
+
+def test_one_used_row_behind_failed_ones(hl):
+    qf = 0.999 + 1.0e-8 * inputs.rng(7500).standard_normal((100, 3))
+    status = np.ones(100, dtype=np.int32)
+    status[99] = 0
+    sums = torch.zeros((2, 3, 3), dtype=torch.float64, device=DEV)
+    hl.mlmc_accumulate(1, torch.as_tensor(qf, device=DEV), None, torch.as_tensor(status, device=DEV), sums)
+    S = sums.cpu().numpy()
+    assert np.all(S[:, :, 0] == 1) and np.all(S[:, :, 1] == qf[99]) and np.all(S[:, :, 2] == 0.0)
