@@ -1659,9 +1659,11 @@ __global__ void __launch_bounds__(TPB) k_newton_step_max(int B, int N, double in
 }
 
 // Per sample: theta = min(1, dc_limit / max |dc|) (a step that would change a
-// mass fraction by more than dc_limit is shortened; dc_limit <= 0: theta = 1; 0
-// for a sample that does not iterate), and the update test on the full step:
-// at most dxtol ends the sample's iteration with this update.
+// mass fraction by more than dc_limit is shortened; dc_limit <= 0: theta = 1;
+// -1 for a sample that does not iterate), and the update test on the full step:
+// at most dxtol ends the sample's iteration with this update.  An infinite or
+// NaN step has theta = 0 and is still applied, 0 * NaN: the failed sample's
+// state and QoIs become NaN.
 __global__ void k_newton_theta(int B, int nct, double dc_limit, const double* dc_part, double dxtol,
                                const double* dmax_part, int* newton_active, int* status,
                                double* __restrict__ theta) {
@@ -1670,7 +1672,7 @@ __global__ void k_newton_theta(int B, int nct, double dc_limit, const double* dc
   const int s = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (s >= B) return;
   if (!newton_active[s]) {
-    if (lane == 0) theta[s] = 0.0;
+    if (lane == 0) theta[s] = -1.0;
     return;
   }
   double th = 1.0;
@@ -1697,7 +1699,7 @@ __global__ void __launch_bounds__(TPB) k_newton_update(int B, int N, double2* x,
   const int s = blockIdx.x / (unsigned)(N / TPB);
   grid_enter();
   const double th = theta[s];
-  if (__double_as_longlong(th) == 0) return;  // the sample does not iterate
+  if (__double_as_longlong(th) < 0) return;  // the sample does not iterate
   const auto d = dx[e];
   double2 xx = x[e];
   xx.x = fma(th, (double)d.x, xx.x);
