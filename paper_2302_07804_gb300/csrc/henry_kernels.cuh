@@ -392,14 +392,9 @@ __device__ __forceinline__ void face_eval(S drho, S rho0, S ghh, const FaceCoef<
   f.G = fma_(Ff, cup, neg_(mul_(rs, mul_(k.PDh, cR - cL))));
   if constexpr (JAC) {
     const T rsT = (T)rs, cupT = (T)cup, FT = (T)Ff, khT = (T)k.kh, PDT = (T)k.PD, dT = (T)drho;
-    T rLT, rRT;
-    if constexpr (std::is_same<T, S>::value) {
-      rLT = rhoL;
-      rRT = rhoR;
-    } else {
-      rLT = (T)rhoL;
-      rRT = rsT - rLT;
-    }
+    // one rounding each; (T)rs - (T)rhoL carries two, one of them of a value twice as
+    // large (and saves a conversion: level 0, mixed, 1000 samples 16.93 against 17.01 ms)
+    const T rLT = (T)rhoL, rRT = (T)rhoR;
     const T dp = mul_(rsT, khT);
     const T dc = DROP ? (T)0 : mul_(dT, NORTH ? fma_(neg_((T)k.kg), rsT, (T)qh) : (T)qh);
     f.dp = dp;
