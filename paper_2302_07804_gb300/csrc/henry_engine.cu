@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -30,6 +31,7 @@
 #include "henry.h"
 #include "henry_kernels.cuh"
 #include "henry_misc.cuh"
+#include "henry_recent.cuh"
 #include "henry_cta.cuh"
 #include "henry_tail.cuh"
 #include "henry_kl.cuh"
@@ -114,6 +116,17 @@ struct Carver {
   }
 };
 
+// Instantiated CUDA graphs (a BiCGStab iteration each) of a group, by batch
+// size, preconditioner operator and every setting of a tuning table that
+// changes their launches (nu1, nu2, mg_tail_cells, mg_threads; the rest of a
+// handle's configuration is fixed).  They hold the group's pointers and are
+// dropped with it.  A caller that cycles through up to 256 batch sizes replays
+// them all (one step at 40 sizes in turn, against building each again: level
+// 2 13.47 against 13.64 ms a solve, vertex level 1 12.17 against 12.35); a
+// graph takes 0.1 MB on the device, 0.4 without the fused tails.
+typedef std::array<int64_t, 6> GraphKey;
+typedef RecentMap<GraphKey, cudaGraphExec_t, 256> GraphMap;
+
 template <typename T>
 struct Group {
   typedef typename VT<T>::v2 V2;
@@ -136,15 +149,10 @@ struct Group {
   LinScal* sc;
   T* Ainv;
   void* Jp = nullptr;  // fine-level fallback preconditioner operator (field models only)
-  // Instantiated CUDA graphs (a BiCGStab iteration each), by
-  // what they run, the batch size and the whole configuration (every setting
-  // that changes their launches); they hold this workspace's pointers and are
-  // dropped with it.
-  std::map<std::string, cudaGraphExec_t> gexec;
+  GraphMap gexec;
   bool graphs = true;  // false: never capture (the allocation-free entry point)
   void drop_graphs() {
-    for (auto& kv : gexec) cudaGraphExecDestroy(kv.second);
-    gexec.clear();
+    gexec.clear([](cudaGraphExec_t g) { cudaGraphExecDestroy(g); });
   }
 
   // Lay out (or size, with base == nullptr) the workspace for B samples.
@@ -249,11 +257,10 @@ struct VcGroup {
   unsigned long long* totals;
   LinScal* sc;
   T* Ainv;
-  std::map<std::string, cudaGraphExec_t> gexec;  // as Group's
+  GraphMap gexec;
   bool graphs = true;
   void drop_graphs() {
-    for (auto& kv : gexec) cudaGraphExecDestroy(kv.second);
-    gexec.clear();
+    gexec.clear([](cudaGraphExec_t g) { cudaGraphExecDestroy(g); });
   }
   size_t carve(char* base, int B, int nx0, int ny0, double h0) {
     Carver c{base, 0};
@@ -1080,28 +1087,22 @@ int read_counter(henry_handle* H, const int* dev, cudaStream_t st, int* out) {
 
 // ---------------------------------------------------------------------------
 // Launch the kernels that emit(stream) launches as one CUDA graph on `st`,
-// captured on first use (key: what they are; the batch size and the
-// configuration are added here).  Captured on the handle's own stream, of
-// st's priority (capturing the legacy default stream is not allowed; capture
-// executes nothing).
+// captured on first use (pre: the operator of their preconditioner, which with
+// the batch size and the settings names them).  Captured on the handle's own
+// stream, of st's priority (capturing the legacy default stream is not
+// allowed; capture executes nothing).
 //
 // The loops themselves stay on the host.  As conditional nodes of one graph
 // per implicit step they ran faster on small batches (level-0 FP64, 64
 // samples 14.0 against 18.6 ms), but destroying such graphs while other
 // host threads worked on the device crashed inside cudaGraphDestroy now and
 // then (driver 580, also with every graph call of the process serialised).
-constexpr size_t MAX_GRAPHS = 16;
 template <typename GRP, typename F>
-int run_graph(henry_handle* H, GRP& G, int B, const std::string& what, cudaStream_t st, F&& emit) {
-  std::string key = what;
-  key.append(reinterpret_cast<const char*>(&B), sizeof B);
-  key.append(reinterpret_cast<const char*>(&H->cfg), sizeof H->cfg);
-  auto f = G.gexec.find(key);
-  if (f == G.gexec.end()) {
-    if (G.gexec.size() >= MAX_GRAPHS) {  // e.g. an autotuner's candidates
-      CK(cudaStreamSynchronize(st));
-      G.drop_graphs();
-    }
+int run_graph(henry_handle* H, GRP& G, int B, const void* pre, cudaStream_t st, F&& emit) {
+  const henry_config& c = H->cfg;
+  const GraphKey key = {B, (int64_t)reinterpret_cast<intptr_t>(pre), c.nu1, c.nu2, c.mg_tail_cells, c.mg_threads};
+  cudaGraphExec_t* g = G.gexec.find(key);
+  if (!g) {
     if (!H->cap_stream) {
       int prio = 0;
       CK(cudaStreamGetPriority(st, &prio));
@@ -1121,9 +1122,10 @@ int run_graph(henry_handle* H, GRP& G, int B, const std::string& what, cudaStrea
     const cudaError_t e = cudaGraphInstantiate(&ex, gr, 0);
     cudaGraphDestroy(gr);
     if (e != cudaSuccess) return set_err(HENRY_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e));
-    f = G.gexec.emplace(key, ex).first;
+    // (the one given up has ended: a convergence test was read after each launch)
+    g = G.gexec.insert(key, ex, [](cudaGraphExec_t old) { cudaGraphExecDestroy(old); });
   }
-  CK(cudaGraphLaunch(f->second, st));
+  CK(cudaGraphLaunch(*g, st));
   return HENRY_OK;
 }
 // Graphs are used unless the configuration says no, the workspace may not
@@ -1134,8 +1136,8 @@ bool graphs_on(const henry_handle* H, const GRP& G) {
 }
 
 // The BiCGStab loop over a solver D's pieces - init(stream), head(iteration,
-// stream), body(samples, stream) and what(), which names the body among the
-// group's graphs - on group D::G.
+// stream), body(samples, stream) and pre(), the body's preconditioner operator
+// (NULL: the Jacobian) - on group D::G.
 template <typename D>
 struct KrylovDrive {
   D& d() { return static_cast<D&>(*this); }
@@ -1151,7 +1153,7 @@ struct KrylovDrive {
       if (!rc) rc = read_counter(H, G.counter + 1, st, &n_act);
       if (rc || n_act == 0) return rc;
       H->nact = n_act;
-      rc = graph ? run_graph(H, G, d().B, d().what(), st, [&](cudaStream_t s) { return d().body(d().B, s); })
+      rc = graph ? run_graph(H, G, d().B, d().pre(), st, [&](cudaStream_t s) { return d().body(d().B, s); })
                  : d().body(n_act, st);
     }
     return rc;
@@ -1188,7 +1190,7 @@ struct Krylov : KrylovDrive<Krylov<T>> {
     black_known = H->cfg.nu2 > 0 && !Jpre0;
   }
 
-  std::string what() const { return std::string(reinterpret_cast<const char*>(&Jpre0), sizeof Jpre0); }
+  const void* pre() const { return Jpre0; }
   void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
@@ -1861,7 +1863,7 @@ struct VcKrylov : KrylovDrive<VcKrylov<T>> {
       : H(h), G(grp), B(b), rtol2(h->cfg.lin_rtol * h->cfg.lin_rtol), maxit(h->cfg.lin_maxit), L(grp.lv[0]),
         N(grp.lv[0].stride), g(nblk((int64_t)b * grp.lv[0].stride)),
         fin((h->cfg.finalize_nct > 0 && grp.nct >= h->cfg.finalize_nct) ? grp.fin : nullptr) {}
-  std::string what() const { return "body"; }
+  const void* pre() const { return nullptr; }
   void finalize(int a, int b, cudaStream_t ss) {
     if (!fin) return;
     launch(H, ss, HENRY_K_KRYLOV, (double)B * G.nct * 16.0,
