@@ -183,7 +183,8 @@ typedef struct {
                             16 elements unless this is 0.  Same values either way */
   int32_t mg_tail_batch_cells; /* ... only while the batch times that level's cells per sample is at most this
                                   (default 2^20; 0: no limit): larger batches run those levels as separate,
-                                  large launches.  The default start with FP32 linear algebra has no limit */
+                                  large launches.  The default start with FP32 linear algebra is limited by
+                                  a stated value (any other than the default) only */
   int32_t scheme; /* HENRY_SCHEME_CELL (default) or HENRY_SCHEME_VERTEX */
   int32_t newton_jacobian_every; /* Newton assembles the Jacobian and the coarse operators at
                                     iterations 0, k, 2k, ... of a time step and reuses them in between (chord

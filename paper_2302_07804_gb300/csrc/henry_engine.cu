@@ -889,6 +889,9 @@ int restrict_states(henry_handle* H, Group<T>& G, int B, bool old, const int* ac
 // timer: FP64 from 16 x 8 cells 42.4 -> 18.6 us (64 samples) and 404 -> 182 us
 // (8192 samples); FP32 from 64 x 32 cells 54.9 -> 18.7 us (2 samples), 55 ->
 // 21 us (20 to 50 samples).
+// The default rule for FP32 has no batch limit of its own (above); a stated
+// mg_tail_batch_cells, any value but the default, limits it like every other.
+constexpr int TAIL_BATCH_CELLS = 1 << 20;
 template <typename T>
 int tail_level(const henry_config& c, const Group<T>& G, int B) {
   const int N0 = G.lv[0].N;
@@ -899,7 +902,7 @@ int tail_level(const henry_config& c, const Group<T>& G, int B) {
       const bool all = N0 > 512 || B <= 1024;
       cells = all ? 2048 : 128;
       k0 = all ? 0 : 1;
-      limit = !all;
+      limit = !all || c.mg_tail_batch_cells != TAIL_BATCH_CELLS;
     } else {
       cells = B <= 304 ? 512 : 128;
       k0 = B <= 152 ? 0 : 1;
@@ -2626,7 +2629,7 @@ void henry_default_config(henry_config* c) {
   c->newton_jacobian_every = 1;
   c->level_priority = 1;
   c->mg_tail_cells = -1;
-  c->mg_tail_batch_cells = 1 << 20;
+  c->mg_tail_batch_cells = TAIL_BATCH_CELLS;
   c->scheme = HENRY_SCHEME_CELL;
   c->assembly_tile_w = 0;
   c->mg_threads = 0;
