@@ -2848,8 +2848,9 @@ int henry_autotune(henry_handle* h, int level, int with_coarse, const double* xi
     // kernels (small batches of mid-size grids fill more SMs with smaller CTAs).
     const int b5 = best;
     for (int v : {64, 128, 256, 512}) {
-      const int cur = cands[b5].mg_threads == 0 ? TPB : cands[b5].mg_threads;
-      if (v == cur || rc) continue;
+      // (with FP32 linear algebra 0 is 256 threads; in FP64 it is a rule of its own, see mg_cta)
+      const bool is256 = cands[b5].mg_threads == 0 && c.precision == HENRY_MIXED;
+      if (v == (is256 ? TPB : cands[b5].mg_threads) || rc) continue;
       henry_tuning t = cands[b5];
       t.mg_threads = v;
       cands.push_back(t);
