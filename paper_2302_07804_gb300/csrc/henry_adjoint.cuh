@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(TPB) k_adj_project(AdjModel M, int B, int nx, 
   const double* Sq = S + ((int64_t)s * A_NPLANE + A_Q) * N;
   double q = 0.0;
   for (int i = threadIdx.x; i < N; i += blockDim.x) q += Sq[i];
-  q = block_reduce<false>(q, sh);
+  q = block_reduce(q, sh);
   if (threadIdx.x == 0) out[M.n_in - 1] = -q * M.qin_mean * M.qin_amp;
   if (M.model == 0) {
     double a = 0.0, k = 0.0;
@@ -295,8 +295,8 @@ __global__ void __launch_bounds__(TPB) k_adj_project(AdjModel M, int B, int nx, 
       a += v.x;
       k += v.y;
     }
-    a = block_reduce<false>(a, sh);
-    k = block_reduce<false>(k, sh);
+    a = block_reduce(a, sh);
+    k = block_reduce(k, sh);
     if (threadIdx.x == 0) {
       out[0] = a * M.phi_mean * M.phi_amp;
       out[1] = k * coef[s].kmu * M.mu * M.logK_amp;
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(TPB) k_adj_project(AdjModel M, int B, int nx, 
         else d = (c.x > M.phi_lo && c.x < M.phi_hi) ? v.x * M.sigma_phi : 0.0;
         a = fma(d, px[ix] * py[iy], a);
       }
-      a = block_reduce<false>(a, sh);
+      a = block_reduce(a, sh);
       if (threadIdx.x == 0) out[t] = a * sl[tt];
     }
   } else {
@@ -341,8 +341,8 @@ __global__ void __launch_bounds__(TPB) k_adj_project(AdjModel M, int B, int nx, 
       a1 = fma(gp, M.phi_mean * (0.15 * cos(2.0 * pi * x) * c0 + wv * dc0), a1);
       a2 = fma(gp, M.phi_mean * 0.15 * (cos(pi * x / 2.0) + sin(2.0 * pi * yp)) * c0, a2);
     }
-    a1 = block_reduce<false>(a1, sh);
-    a2 = block_reduce<false>(a2, sh);
+    a1 = block_reduce(a1, sh);
+    a2 = block_reduce(a2, sh);
     if (threadIdx.x == 0) {
       out[0] = a1;
       out[1] = a2;

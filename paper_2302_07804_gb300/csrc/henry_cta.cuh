@@ -16,7 +16,7 @@
 // Bound by latency (dependent phases between barriers) and, in the assembly,
 // by the FP64 pipe.  With FP32 linear algebra, 1000 samples of 20 steps: 27.3
 // ms with all blocks and vectors in 111 KB of shared memory and one thread per
-// cell on the coarse levels, 16.8 ms in this form (41 KB; two CTAs per SM by
+// cell on the coarse levels, 17.0 ms in this form (41 KB; two CTAs per SM by
 // registers either way).
 // The per-cell arithmetic is the multi-kernel path's and the steps follow the
 // same order, so both paths compute the same iterates up to the summation

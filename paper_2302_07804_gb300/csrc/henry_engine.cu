@@ -142,7 +142,7 @@ struct Group {
   Coef* coef;
   double* part;
   int *newton_active, *lin_active, *newton_it, *status, *iters;
-  int* counter;  // samples iterating: [0] Newton, [1] BiCGStab, [2] retries; [3] the BiCGStab iteration index
+  int* counter;  // samples iterating: [0] Newton, [1] BiCGStab, [2] retries
   double* theta;  // per-sample Newton step factor
   double* fin;    // finalised per-sample reduction values [B][NPART] (large grids)
   unsigned long long* totals;  // [0] Newton iterations, [1] BiCGStab iterations
@@ -458,9 +458,9 @@ auto assemble_kernel(const henry_config& c, int nx, int ny) -> decltype(&k_assem
 // Whether a launch of `threads` threads (one per cell) takes the PRE form of
 // its kernel, which loads the operands that the previous kernel does not write
 // before it waits for that kernel.  That shortens a launch of one wave (level
-// 2 with partners, 33 samples, FP64: 268 -> 237 ms; with the line at 3 CTAs an
-// SM 252 ms; level-5 KL mixed, 2 samples: 149 -> 133 ms) and costs a large one
-// occupancy (level 0, 8192 samples, FP64: 445 -> 456 ms), so the line is what
+// 2 with partners, 33 samples, FP64: 215 -> 188 ms; with the line at 3 CTAs an
+// SM 201 ms; level-5 KL mixed, 2 samples: 147 -> 132 ms) and costs a large one
+// occupancy (level 0, 8192 samples, FP64: 370 -> 376 ms), so the line is what
 // 8 CTAs of 256 threads on each of 152 SMs hold.
 constexpr int64_t PRELOAD_THREADS = (int64_t)152 * 8 * TPB;
 template <typename F>
@@ -472,10 +472,9 @@ void with_preload(int64_t threads, F&& f) {
 // CTA size of the multigrid kernels where mg_threads leaves it open.  Small FP64
 // launches take small CTAs: an SM's FP64 pipe needs 19 cycles for a warp
 // instruction, so a launch of few CTAs is faster on more SMs (against 256
-// threads everywhere: level 2 with partners, 33 samples, 206 -> 193 ms; two-
-// layer level 1, 50 samples, 55.6 -> 51.2 ms; level 0, 64 samples, 18.8 -> 18.0
-// ms).  FP32 launches gain nothing (level 3, 20 samples: 311 ms either way; 64
-// threads up to the PRELOAD_THREADS line: 319 ms).
+// threads everywhere: level 2 with partners, 33 samples, 195 -> 187 ms; two-
+// layer level 1, 50 samples, 52.2 -> 50.5 ms).  FP32 launches lose (level 3, 20
+// samples: 252 ms, with 64 threads 266 ms).
 template <typename T>
 int mg_cta(int mg_threads, int64_t threads) {
   if (mg_threads || sizeof(T) == sizeof(float)) return mg_threads;
@@ -877,14 +876,15 @@ int restrict_states(henry_handle* H, Group<T>& G, int B, bool old, const int* ac
 //  * FP32: from 64 x 32 cells, the whole cycle where that is the fine grid -
 //    the kernel reads a sample's operator once where the separate sweeps read
 //    it nine times - for any batch (level 1 against a tail from 16 x 8: 200
-//    samples 25.9 / 30.4 ms, 884 80.8 / 97.3, 2500 208 / 256; level 2: 500
-//    samples 351 / 368 ms); fine grids of 32 x 16 up to 1024 samples, beyond
-//    that from 16 x 8 (4000 samples: 106 against 116 ms).
+//    samples 45.6 / 51.9 ms, 884 144 / 166, 2500 367 / 430; level 2: 500
+//    samples 611 / 643 ms); fine grids of 32 x 16 up to 1024 samples (1000:
+//    30.8 / 32.3 ms), beyond that from 16 x 8 (4000 samples: 105 against 115 ms).
 //  * FP64: from 32 x 16 cells while every sample's CTA has an SM or half of
 //    one to itself (its half-sweep there keeps the SM's FP64 pipe busy for
-//    1.5 us; level 1: 300 samples 46.4 against 48.6 ms from 16 x 8), the whole
-//    cycle of a 32 x 16 fine grid up to 152 samples (7.9 against 9.8 ms); else
-//    from 16 x 8 within mg_tail_batch_cells.
+//    1.5 us; level 1 against 16 x 8: 300 samples 124 / 130 ms, 320 142 / 141), the
+//    whole cycle of a 32 x 16 fine grid while every sample has an SM, up to 152
+//    samples (64: 18.4 / 19.8 ms, 152: 20.8 / 25.7; two to an SM would still gain:
+//    304 29.4 / 33.4); else from 16 x 8 within mg_tail_batch_cells.
 // The kernel itself against the one-thread-per-cell one it replaced, by event
 // timer: FP64 from 16 x 8 cells 42.4 -> 18.6 us (64 samples) and 404 -> 182 us
 // (8192 samples); FP32 from 64 x 32 cells 54.9 -> 18.7 us (2 samples), 55 ->
@@ -1277,9 +1277,9 @@ int linear_solve(henry_handle* H, Group<T>& G, int B, cudaStream_t st, const voi
   return k.run(st);
 }
 
-// Newton's loop over a step D's pieces - start, evaluate(residual first, count,
-// stream), operators, krylov / solve(fallback), mark_retry and retry_operators
-// where retries(), update - on group D::G.
+// Newton's loop over a step D's pieces - start, evaluate(residual first,
+// stream), operators, solve(fallback), mark_retry and retry_operators where
+// retries(), update - on group D::G.
 //
 // Newton's choices: the Jacobian and the coarse
 // operators are assembled at iterations 0, k, 2k, ... of the step, k =
@@ -1310,7 +1310,7 @@ struct NewtonDrive {
       const bool jac_now = force_jac || last_jac < 0 || it - last_jac >= jac_every;
       const bool res_first = res_first_at(it, jac_now);
       CK(cudaMemsetAsync(G.counter, 0, sizeof(int), st));
-      rc = n.evaluate(res_first, G.counter, st);
+      rc = n.evaluate(res_first, st);
       int n_act = 0;
       if (!rc) rc = read_counter(H, G.counter, st, &n_act);
       if (rc || n_act == 0) return rc;
@@ -1409,15 +1409,14 @@ struct NewtonStep : NewtonDrive<NewtonStep<T>> {
     CKL();
     return HENRY_OK;
   }
-  Krylov<T> krylov(bool fallback) { return Krylov<T>(H, G, B, fallback ? G.Jp : nullptr, c.lin_rtol, c.lin_maxit); }
   int solve(bool fallback, cudaStream_t st) { return linear_solve<T>(H, G, B, st, fallback ? G.Jp : nullptr); }
-  // The evaluation of an iteration and its residual test; `count` (nullable):
-  // the samples that go on are added to it.
-  int evaluate(bool res_first, int* count, cudaStream_t st) {
+  // The evaluation of an iteration and its residual test; the samples that go
+  // on are added to G.counter[0].
+  int evaluate(bool res_first, cudaStream_t st) {
     const int rc = assemble(!res_first, st);
     launch(H, st, HENRY_K_NEWTON, (double)B * 8 * G.nct, [&] {
       chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, G.nct, c.newton_atol, c.newton_maxit, pmax,
-            G.newton_active, G.lin_active, G.newton_it, G.status, count, G.totals);
+            G.newton_active, G.lin_active, G.newton_it, G.status, G.counter, G.totals);
     });
     CKL();
     return rc;
@@ -1658,7 +1657,8 @@ VcLevelArgs vc_args(const typename VcGroup<T>::Lv& L) {
   return VcLevelArgs{L.nx, L.ny, L.stride, L.plane};
 }
 
-// States of the coarse levels by injection, level by level (old: the old state).
+// States of the coarse levels by injection, all of them in one launch (old: the
+// old state).
 template <typename T>
 int vc_inject(henry_handle* H, VcGroup<T>& G, int B, bool old, const int* active, cudaStream_t st) {
   auto& L0 = G.lv[0];
@@ -1727,10 +1727,10 @@ int vc_coarse_ops(henry_handle* H, VcGroup<T>& G, int B, double tau, double inv_
 }
 
 // The first level of the fused tail (henry_vc_tail.cuh), -1 for none: the first
-// coarse one of at most 32 x 16 elements, whatever the batch (10 steps of
-// level 1, 400 samples, FP64: 235 ms, 246 ms from 16 x 8 elements, 290 ms
-// without; 4096 samples of level 0, whose first coarse grid is 16 x 8: 351 and
-// 353 ms); mg_tail_cells = 0: none.
+// coarse one of at most 32 x 16 elements, whatever the batch (FP64, level 1: 64
+// samples 188 ms, 217 ms from 16 x 8 elements, 322 ms without; 10 steps of 400
+// samples 371, 387 and 463 ms; 10 steps of 4096 samples of level 0, whose first
+// coarse grid is 16 x 8: 592 and 607 ms without); mg_tail_cells = 0: none.
 template <typename T>
 int vc_tail_level(const henry_config& c, const VcGroup<T>& G) {
   if (c.mg_tail_cells == 0 || !vc_tail_fits<T>()) return -1;
@@ -2010,15 +2010,14 @@ struct VcNewtonStep : NewtonDrive<VcNewtonStep<T>> {
     CKL();
     return vc_inject<T>(H, G, B, true, G.newton_active, st);
   }
-  VcKrylov<T> krylov(bool) { return VcKrylov<T>(H, G, B); }
   int solve(bool, cudaStream_t st) { return vc_linear_solve<T>(H, G, B, st); }
-  int evaluate(bool res_first, int* count, cudaStream_t st) {
+  int evaluate(bool res_first, cudaStream_t st) {
     const int rc = vc_assemble_fine<T>(H, G, B, lg.tau, inv_s, st, !res_first);
     int nct_f = 0;
     const double* fmax_parts = vc_max_parts<T>(H, G, B, &nct_f);
     launch(H, st, HENRY_K_NEWTON, (double)B * 8 * nct_f, [&] {
       chain(st, nblk((int64_t)B * 32, 128), 128, 0, k_newton_res_check, B, nct_f, c.newton_atol, c.newton_maxit,
-            fmax_parts, G.newton_active, G.lin_active, G.newton_it, G.status, count, G.totals);
+            fmax_parts, G.newton_active, G.lin_active, G.newton_it, G.status, G.counter, G.totals);
     });
     CKL();
     return rc;

@@ -110,22 +110,15 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-// Deterministic CTA-wide sum / max; the result is returned to every thread.
-template <bool MAX>
+// Deterministic CTA-wide sum; the result is returned to every thread.
 __device__ __forceinline__ double block_reduce(double v, double* sh) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  v = MAX ? warp_max(v) : warp_sum(v);
+  v = warp_sum(v);
   __syncthreads();
   if (lane == 0) sh[w] = v;
   __syncthreads();
   if (w == 0) {
-    double u = lane < nw ? sh[lane] : (MAX ? -INFINITY : 0.0);
-    u = MAX ? warp_max(u) : warp_sum(u);
+    const double u = warp_sum(lane < nw ? sh[lane] : 0.0);
     if (lane == 0) sh[32] = u;
   }
   __syncthreads();
@@ -171,8 +164,8 @@ __device__ __forceinline__ double block_sum_pair(double v1, double v2, double* s
 }
 // CTA-wide max of non-negative doubles without NaNs (+inf allowed) on the
 // integer pipes: for such values the IEEE-754 bit patterns order like the
-// values, so the max of the 64-bit patterns is the max of the values (the
-// same result as block_reduce<true>, with no FP64 instruction).
+// values, so the max of the 64-bit patterns is the max of the values, with no
+// FP64 instruction.
 __device__ __forceinline__ double block_max_nonneg(double v, double* sh) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   unsigned long long u = (unsigned long long)__double_as_longlong(v);
@@ -348,7 +341,8 @@ __device__ __forceinline__ double abs_max_or_inf(double a, double b) {
 // in FP32 from FP64 fluxes.
 //
 // Scaled coefficients of one sample on one multigrid level of the constant-
-// coefficient model (k_level_coefs), inv_s included.
+// coefficient model (formed by level_coef: k_coefficients for every level, the
+// fused solver its own), inv_s included.
 struct __align__(64) LevelCoef {
   double kh, kg;    // K / (2 mu), kh g h / 2
   double PD, PDh;   // phi Dm, half of it
@@ -1307,9 +1301,10 @@ __device__ __forceinline__ typename VT<T>::v2 spmv_cell(int nx, int ny, int ix, 
 // take b_P and only the red ones form the product: half the operations, and
 // 104 instead of 208 bytes a cell.  A warp's cells then have one colour (on 32
 // cells wide grids the CTA's eight rows are dealt out by colour).  8192 level-0
-// samples, FP64: 145 -> 94 us a call; with the first red half-sweeps in the
-// BiCGStab kernels the solve takes 364 instead of 386 ms (level 2 with
-// partners, 33 samples: 168 and 176 ms; level-3 mixed, 20 samples: 278 and 292).
+// samples, FP64: 145 -> 94 us a call, the solve 384 -> 369 ms (level 2 with
+// partners, 33 samples: 192 -> 188; level 3 with partners, mixed, 20 samples:
+// 316 -> 314); with the first red half-sweeps in the BiCGStab kernels as well
+// 370, 187 and 312 ms.
 // PRE as in k_sweep (the kernel follows the sweep that ends a V-cycle).
 template <typename T, int NDOT, bool PRE = false>
 __global__ void __launch_bounds__(TPB) k_spmv(int B, int nx, int ny, const typename VT<T>::b4* __restrict__ J,
@@ -1620,7 +1615,7 @@ __global__ void k_newton_res_check(int B, int nct, double atol, int maxit, const
       act = 0;
     } else {
       newton_it[s] += 1;
-      if (n_active) atomicAdd(n_active, 1);
+      atomicAdd(n_active, 1);
       atomicAdd(it_total, 1ULL);
     }
   }

@@ -258,8 +258,8 @@ __global__ void __launch_bounds__(TPB) k_qoi(int B, int nx, int ny, double h, do
     acc += w * (rho0 + drho * c) * c;
     fresh += (c <= 0.012178) ? 1.0 : 0.0;
   }
-  acc = block_reduce<false>(acc, sh);
-  if (Q.set >= 1) fresh = block_reduce<false>(fresh, sh);
+  acc = block_reduce(acc, sh);
+  if (Q.set >= 1) fresh = block_reduce(fresh, sh);
   if (threadIdx.x == 0) {
     const int ix0 = (3 * ny) / 2 - 1, iy0 = ny / 4 - 1;
     const double c00 = xs[st_of(ix0, iy0, nx)].y, c10 = xs[st_of(ix0 + 1, iy0, nx)].y;
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(TPB) k_qfw(int B, int N, double h, const doubl
   const double2* xs = x + (int64_t)s * N;
   double fresh = 0.0;
   for (int i = threadIdx.x; i < N; i += blockDim.x) fresh += (xs[i].y <= 0.012178) ? 1.0 : 0.0;
-  fresh = block_reduce<false>(fresh, sh);
+  fresh = block_reduce(fresh, sh);
   if (threadIdx.x == 0) out[(int64_t)s * stride] = status[s] == 0 ? fresh * h * h : 0.0;
 }
 

@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(TPB) k_vc_qoi(int B, int nx, int ny, int strid
     const double c = xs[st].y;
     acc += nel * (rho0 + drho * c) * c;
   }
-  const double tot = block_reduce<false>(acc, sh);
+  const double tot = block_reduce(acc, sh);
   if (threadIdx.x == 0) {
     const bool bad = status[s] != 0;
     qoi[2 * (int64_t)s] = bad ? NAN : coef[s].phi * 0.25 * h * h * tot;

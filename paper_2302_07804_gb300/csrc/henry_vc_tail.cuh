@@ -14,9 +14,8 @@
 // operations (36 with one thread per vertex), which in FP64 take 64 cycles
 // each.  The arithmetic and its order are vc_offdiag's, k_vc_restrict's,
 // k_vc_prolong_add's and k_vc_coarse_solve's: bit-identical to the
-// level-by-level kernels.  Level 1, 64 samples, with every kernel of the
-// scheme in the programmatic chain and the step as one graph: 350 -> 221 ms
-// FP64 (131 against 81 ms over 5 steps without and with this kernel).
+// level-by-level kernels.  Level 1, 64 samples, FP64: 188 ms, 322 ms with the
+// same levels as separate kernels.
 #pragma once
 #include "henry_tail.cuh"
 #include "henry_vc_solve.cuh"
@@ -144,7 +143,8 @@ struct VcTailLevel {
       m.on[col] = vertex(col, tt >> 1, m.i[col], m.j[col]) && t < ITEMS;
       if (!m.on[col]) vertex(col, 0, m.i[col], m.j[col]);  // read along with the first vertex
     }
-    // slots of vertices the thread does not have are its own first one's: see blk
+    // (the slots of vertices the thread does not have hold the zeros of the initial
+    // clear, and nothing is stored for them)
     const V2* bg = reinterpret_cast<const V2*>(A.b) + (int64_t)s * A.stride[0];
     if constexpr (FIRST) grid_enter();
 #pragma unroll
