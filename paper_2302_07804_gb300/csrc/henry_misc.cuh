@@ -410,34 +410,31 @@ __global__ void __launch_bounds__(TPB) k_scale_d2(int64_t n, double a, double2* 
 // own deviations off, one CTA and column in a million.  Bound by the FP64 pipe: 7 operations per row and QoI (the
 // difference Y, and a subtraction, an addition and a multiply-add for each
 // quantity), which at 17-19 cycles a warp instruction and SM is 145 us for
-// 20000 rows of 527 QoIs with their partners.  Measured there 180 us, against
-// 307 us for one CTA of 1024 threads per QoI and quantity with two strided
-// passes; 20000 x 15: 49 -> 19 us, 81675 x 2: 148 -> 33 us, 500 x 527: 63 -> 19
-// us, 50 x 2: 11 -> 10 us.
+// 20000 rows of 527 QoIs with their partners.  Measured there 187 us, against
+// 314 us for one CTA of 1024 threads per QoI and quantity with two strided
+// passes; 20000 x 15: 54 -> 27 us, 81675 x 2: 160 -> 44 us, 500 x 527: 68 -> 27
+// us, 50 x 2: 15 -> 17 us (event timer around the call, L2 flushed before it).
 // A CTA takes columns in groups of CW (1 .. 16); few QoIs take narrow groups
 // so that the rows still spread over many CTAs.
 constexpr int ACC_THREADS = 256, ACC_MAX_CLUSTER = 8;
 
+constexpr int ACC_WARPS = ACC_THREADS / 32, ACC_R = 8;  // ACC_R: rows a lane holds at a time
 template <int CW>
-__global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n_qoi, const double* __restrict__ qf,
-                                                                 const double* __restrict__ qc,
-                                                                 const int32_t* __restrict__ status,
-                                                                 double* __restrict__ sums) {
-  namespace cg = cooperative_groups;
-  constexpr int NW = ACC_THREADS / 32, RPW = 32 / CW, R = 8;  // R: rows a lane holds at a time
-  __shared__ double part[4][NW][CW];
-  __shared__ int cpart[NW][CW];
-  __shared__ double mom[2][CW][4];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int col = lane % CW, q = blockIdx.x * CW + col;
-  const int rank = blockIdx.y, ncta = gridDim.y;
-  const bool on = q < n_qoi;
-  const int qq = on ? q : n_qoi - 1;  // lanes beyond the last QoI read along
-  // R rows from r0 on, `inc` apart: every load is issued before the first use,
+struct AccShared {
+  double part[4][ACC_WARPS][CW];
+  int cpart[ACC_WARPS][CW];
+  double mom[2][CW][4];  // of Y and the fine QoI: count, pivot, mean less the pivot, M2
+};
+// A CTA's share of the batch: its steps of ACC_THREADS / CW rows of CW columns.
+struct AccRows {
+  int n, n_qoi, rank, ncta, qq;
+  const double *qf, *qc;
+  const int32_t* status;
+  // ACC_R rows from r0 on, `inc` apart: every load is issued before the first use,
   // the status decides afterwards (a failed sample's NaN is dropped by it)
-  auto load = [&](int64_t r0, int64_t inc, double* f, double* c, bool* ok) {
+  __device__ __forceinline__ void load(int64_t r0, int64_t inc, double* f, double* c, bool* ok) const {
 #pragma unroll
-    for (int j = 0; j < R; ++j) {
+    for (int j = 0; j < ACC_R; ++j) {
       const int64_t i = r0 + j * inc;
       ok[j] = i < n;
       const int64_t at = (ok[j] ? i : 0) * n_qoi + qq;
@@ -445,18 +442,97 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
       c[j] = qc ? qc[at] : 0.0;
       if (status) ok[j] = ok[j] && status[ok[j] ? i : 0] == 0;
     }
-  };
-  // pivot: the mean of the CTA's first used rows
-  const int64_t per_cta = NW * RPW, step = ncta * per_cta;
-  double ky = 0.0, kf = 0.0;
-  {
+  }
+};
+// The CTA's moments about the pivots ky and kf into S.mom; true in a thread
+// whose column's pivot lies too far from its mean (infinite values have no
+// better one).
+template <int CW>
+__device__ __forceinline__ bool acc_moments(const AccRows& A, double ky, double kf, AccShared<CW>& S) {
+  constexpr int NW = ACC_WARPS, RPW = 32 / CW, R = ACC_R;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, col = lane % CW;
+  const int64_t step = (int64_t)A.ncta * NW * RPW;
+  int cnt = 0;
+  double s1y = 0.0, s2y = 0.0, s1f = 0.0, s2f = 0.0;
+  for (int64_t r0 = (A.rank * NW + w) * RPW; r0 < A.n; r0 += R * step) {
     double f[R], c[R];
     bool ok[R];
-    int m = 0;
-    for (int64_t b = rank * per_cta; b < n && m == 0; b += step) {
-      load(b, 1, f, c, ok);
+    A.load(r0 + lane / CW, step, f, c, ok);
 #pragma unroll
-      for (int j = 0; j < R; ++j)
+    for (int j = 0; j < R; ++j) {
+      if (r0 + j * step >= A.n) break;  // uniform over the warp
+      const double df = ok[j] ? f[j] - kf : 0.0, dy = ok[j] ? (f[j] - c[j]) - ky : 0.0;
+      cnt += ok[j];
+      s1f += df;
+      s2f = fma(df, df, s2f);
+      s1y += dy;
+      s2y = fma(dy, dy, s2y);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o >= CW; o >>= 1) {
+    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    s1y += __shfl_xor_sync(0xffffffffu, s1y, o);
+    s2y += __shfl_xor_sync(0xffffffffu, s2y, o);
+    s1f += __shfl_xor_sync(0xffffffffu, s1f, o);
+    s2f += __shfl_xor_sync(0xffffffffu, s2f, o);
+  }
+  if (lane < CW) {
+    S.cpart[w][col] = cnt;
+    S.part[0][w][col] = s1y;
+    S.part[1][w][col] = s2y;
+    S.part[2][w][col] = s1f;
+    S.part[3][w][col] = s2f;
+  }
+  __syncthreads();
+  if (w >= 2 || lane >= CW) return false;
+  int m = 0;  // warps 0 and 1: Y and the fine QoI
+  double s1 = 0.0, s2 = 0.0;
+  for (int k = 0; k < NW; ++k) {
+    m += S.cpart[k][col];
+    s1 += S.part[2 * w][k][col];
+    s2 += S.part[2 * w + 1][k][col];
+  }
+  const double nn = (double)m;
+  const double d = m > 0 ? s1 / nn : 0.0;
+  const double m2 = s2 - s1 * d;
+  S.mom[w][col][0] = nn;
+  S.mom[w][col][1] = w == 0 ? ky : kf;
+  S.mom[w][col][2] = d;
+  S.mom[w][col][3] = m2 < 0.0 ? 0.0 : m2;
+  return !(m2 >= 0.25 * s2) && fabs(d) <= 1.0e300;
+}
+// The second pass, out of line: as a second turn of one loop it slowed the first
+// pass down (81675 x 2: 56 us, 44 in this form and without any second pass).
+template <int CW>
+__device__ __noinline__ void acc_moments_again(const AccRows& A, double ky, double kf, AccShared<CW>& S) {
+  acc_moments<CW>(A, ky, kf, S);
+}
+
+template <int CW>
+__global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n_qoi, const double* __restrict__ qf,
+                                                                 const double* __restrict__ qc,
+                                                                 const int32_t* __restrict__ status,
+                                                                 double* __restrict__ sums) {
+  namespace cg = cooperative_groups;
+  constexpr int per_cta = ACC_THREADS / CW;
+  __shared__ AccShared<CW> S;
+  const int lane = threadIdx.x & 31, which = threadIdx.x >> 5;  // warps 0 and 1 merge: Y and the fine QoI
+  const int col = lane % CW, q = blockIdx.x * CW + col;
+  const int rank = blockIdx.y, ncta = gridDim.y;
+  const bool on = q < n_qoi;
+  // lanes beyond the last QoI read along
+  const AccRows A = {n, n_qoi, rank, ncta, on ? q : n_qoi - 1, qf, qc, status};
+  // pivot: the mean of the CTA's first used rows
+  double ky = 0.0, kf = 0.0;
+  {
+    double f[ACC_R], c[ACC_R];
+    bool ok[ACC_R];
+    int m = 0;
+    for (int64_t b = rank * per_cta; b < n && m == 0; b += (int64_t)ncta * per_cta) {
+      A.load(b, 1, f, c, ok);
+#pragma unroll
+      for (int j = 0; j < ACC_R; ++j)
         if (ok[j] && j < per_cta) {
           kf += f[j];
           ky += f[j] - c[j];
@@ -466,62 +542,9 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
     kf = (m > 0 && fabs(kf) <= 1.0e300) ? kf / (double)m : 0.0;  // infinite or NaN values: pivot 0
     ky = (m > 0 && fabs(ky) <= 1.0e300) ? ky / (double)m : 0.0;
   }
-  const int which = w;  // warps 0 and 1: Y and the fine QoI
-  for (int pass = 0;; ++pass) {
-    int cnt = 0;
-    double s1y = 0.0, s2y = 0.0, s1f = 0.0, s2f = 0.0;
-    for (int64_t r0 = (rank * NW + w) * RPW; r0 < n; r0 += R * step) {
-      double f[R], c[R];
-      bool ok[R];
-      load(r0 + lane / CW, step, f, c, ok);
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        if (r0 + j * step >= n) break;  // uniform over the warp
-        const double df = ok[j] ? f[j] - kf : 0.0, dy = ok[j] ? (f[j] - c[j]) - ky : 0.0;
-        cnt += ok[j];
-        s1f += df;
-        s2f = fma(df, df, s2f);
-        s1y += dy;
-        s2y = fma(dy, dy, s2y);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o >= CW; o >>= 1) {
-      cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-      s1y += __shfl_xor_sync(0xffffffffu, s1y, o);
-      s2y += __shfl_xor_sync(0xffffffffu, s2y, o);
-      s1f += __shfl_xor_sync(0xffffffffu, s1f, o);
-      s2f += __shfl_xor_sync(0xffffffffu, s2f, o);
-    }
-    if (lane < CW) {
-      cpart[w][col] = cnt;
-      part[0][w][col] = s1y;
-      part[1][w][col] = s2y;
-      part[2][w][col] = s1f;
-      part[3][w][col] = s2f;
-    }
-    __syncthreads();
-    bool far = false;  // the pivot lies too far from this column's mean (infinite values have no better one)
-    if (which < 2 && lane < CW) {
-      int m = 0;
-      double s1 = 0.0, s2 = 0.0;
-      for (int k = 0; k < NW; ++k) {
-        m += cpart[k][col];
-        s1 += part[2 * which][k][col];
-        s2 += part[2 * which + 1][k][col];
-      }
-      const double nn = (double)m;
-      const double d = m > 0 ? s1 / nn : 0.0;
-      const double m2 = s2 - s1 * d;
-      mom[which][col][0] = nn;
-      mom[which][col][1] = which == 0 ? ky : kf;
-      mom[which][col][2] = d;
-      mom[which][col][3] = m2 < 0.0 ? 0.0 : m2;
-      far = pass == 0 && !(m2 >= 0.25 * s2) && fabs(d) <= 1.0e300;
-    }
-    if (!__syncthreads_or(far)) break;
-    if (fabs(mom[0][col][2]) <= 1.0e300) ky += mom[0][col][2];
-    if (fabs(mom[1][col][2]) <= 1.0e300) kf += mom[1][col][2];
+  if (__syncthreads_or(acc_moments<CW>(A, ky, kf, S))) {
+    const double dy = S.mom[0][col][2], df = S.mom[1][col][2];
+    acc_moments_again<CW>(A, fabs(dy) <= 1.0e300 ? ky + dy : ky, fabs(df) <= 1.0e300 ? kf + df : kf, S);
   }
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();
@@ -531,7 +554,7 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
     // rounded to k + d they would put an error of eps |mean| sd into M2.
     double cb = 0.0, sb = 0.0, k0 = 0.0;
     for (int k = 0; k < ncta; ++k) {
-      const double* b = cl.map_shared_rank(&mom[which][col][0], k);
+      const double* b = cl.map_shared_rank(&S.mom[which][col][0], k);
       if (b[0] == 0.0) continue;
       if (cb == 0.0) k0 = b[1];
       cb += b[0];
@@ -541,18 +564,18 @@ __global__ void __launch_bounds__(ACC_THREADS, 4) k_mlmc_accumulate(int n, int n
       const double off = sb / cb, mb = k0 + off;
       double m2 = 0.0;
       for (int k = 0; k < ncta; ++k) {
-        const double* b = cl.map_shared_rank(&mom[which][col][0], k);
+        const double* b = cl.map_shared_rank(&S.mom[which][col][0], k);
         if (b[0] == 0.0) continue;
         const double d = ((b[1] - k0) + b[2]) - off;
         m2 += fma(b[0] * d, d, b[3]);
       }
-      double* S = sums + ((int64_t)which * n_qoi + q) * 3;
-      const double na = S[0], ma = S[1], m2a = S[2];
+      double* out = sums + ((int64_t)which * n_qoi + q) * 3;
+      const double na = out[0], ma = out[1], m2a = out[2];
       const double nn = na + cb;
       const double d = mb - ma;
-      S[0] = nn;
-      S[1] = ma + d * (cb / nn);
-      S[2] = m2a + m2 + d * d * (na * cb / nn);
+      out[0] = nn;
+      out[1] = ma + d * (cb / nn);
+      out[2] = m2a + m2 + d * d * (na * cb / nn);
     }
   }
   cl.sync();  // the other CTAs' shared memory stays until it has been read
